@@ -1381,13 +1381,15 @@ __global__ void advance_steps_kernel(InstDev *const *insts, int32_t n_inst, int6
 // ------------------------------------------------------------ diagnostics
 // Conservation sums of the SDs inside the domain (slots [0, n_in)): live
 // count, sum of xi (128-bit, exact) and sum of xi v (binary64).  Each thread
-// adds its slots in index order, then warps and blocks combine in a fixed
+// adds its slot pairs in index order, then warps and blocks combine in a fixed
 // tree, so that a given grid gives the same bits every time.
 struct DiagPart {
     unsigned long long live, xi_lo, xi_hi;
     double xv;
 };
 constexpr int kDiagNT = 256;
+constexpr int kDiagBlocks = 152 * 4;
+constexpr int kDiagU = 4; // slot pairs per thread and round, all loaded first
 
 __device__ __forceinline__ void add128(unsigned long long &lo, unsigned long long &hi, unsigned long long blo,
                                        unsigned long long bhi)
@@ -1437,13 +1439,29 @@ __global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(const InstDev *__
                                                                DiagPart *__restrict__ parts)
 {
     DiagPart a{0ull, 0ull, 0ull, 0.0};
-    const int64_t stride = (int64_t)gridDim.x * kDiagNT;
-    for (int64_t i = (int64_t)blockIdx.x * kDiagNT + threadIdx.x; i < n_in; i += stride) {
-        const int64_t x = P->xi[i];
+    const longlong2 *__restrict__ gxi = reinterpret_cast<const longlong2 *>(P->xi);
+    const double2 *__restrict__ gv = reinterpret_cast<const double2 *>(P->v);
+    const int64_t stride = (int64_t)gridDim.x * kDiagNT, np = n_in / 2; // every group has an even number of slots
+    auto add = [&](int64_t x, double v) {
         if (x > 0) {
             a.live += 1ull;
             add128(a.xi_lo, a.xi_hi, (unsigned long long)x, 0ull);
-            a.xv = __fma_rn(xi2d(x), P->v[i], a.xv);
+            a.xv = __fma_rn(xi2d(x), v, a.xv);
+        }
+    };
+    for (int64_t q0 = (int64_t)blockIdx.x * kDiagNT + threadIdx.x; q0 < np; q0 += kDiagU * stride) {
+        longlong2 x[kDiagU];
+        double2 v[kDiagU];
+#pragma unroll
+        for (int u = 0; u < kDiagU; ++u) {
+            const int64_t q = q0 + u * stride;
+            x[u] = q < np ? gxi[q] : make_longlong2(0, 0);
+            v[u] = q < np ? gv[q] : make_double2(0.0, 0.0);
+        }
+#pragma unroll
+        for (int u = 0; u < kDiagU; ++u) {
+            add(x[u].x, v[u].x);
+            add(x[u].y, v[u].y);
         }
     }
     a = diag_block_reduce(a);
@@ -1502,29 +1520,6 @@ __device__ __forceinline__ int spectrum_bin(double v, const double *s_edges, con
     return a;
 }
 
-// The same with a fixed-step search over at most MAXE - 1 edges (unrolled,
-// so that the searches of neighbouring SDs interleave).
-template <int MAXE>
-__device__ __forceinline__ int spectrum_bin_fixed(double v, const double *s_edges, const float *s_lo,
-                                                  const float *s_hi, int n_edges)
-{
-    const int nb = n_edges - 1;
-    bool in_range;
-    const float rf = cbrt_filter(hi2f((uint32_t)__double2hiint(v), in_range) * kVolToR3F);
-    int lo = -1; // largest lo with lower(edge[lo]) <= rf
-#pragma unroll
-    for (int step = MAXE / 2; step > 0; step >>= 1) {
-        const int mid = lo + step;
-        if (mid < n_edges && s_lo[mid] <= rf)
-            lo = mid;
-    }
-    const bool clear_below = lo >= 0 && rf > s_hi[lo];
-    const bool clear_above = lo + 1 >= n_edges || rf < s_lo[lo + 1];
-    if (in_range && (lo < 0 || clear_below) && clear_above)
-        return (lo < 0 || lo >= nb) ? -1 : lo;
-    return spectrum_bin(v, s_edges, s_lo, s_hi, n_edges);
-}
-
 // Edges into shared memory with their binary32 images widened by 2^-14.
 __device__ __forceinline__ void spectrum_edges_to_smem(const double *edges, int n_edges, double *s_edges, float *s_lo,
                                                        float *s_hi)
@@ -1574,87 +1569,252 @@ __global__ void __launch_bounds__(kSpecNT) spectrum_kernel(const InstDev *__rest
     }
 }
 
-// Total spectrum without atomics: a grid-stride pass over every storage slot
-// (padding and dead SDs hold xi = 0); each thread adds into its own column
-// of a bins x threads shared array, then each block sums its columns in a
-// fixed order into partial[bin][block].  Results repeat bit for bit.
-constexpr int kSpecTotNT = 128;
-constexpr int kSpecTotMaxBins = 32;
+// ---- spectra of at most 32 bins (total and per cell): warps, fixed point.
+//
+// binary64 adds are what a spectrum must not spend here (16 cycles of an SM
+// per warp instruction): the columns of binary64 sums this replaced spent two
+// thirds of their time adding 31 x 128 columns per block (49 us for the total
+// of 4.19M SDs), and shared-memory binary64 atomics, which are compare-and-
+// swap loops, took 236 us for its 16,384 cells.  A warp now takes 256 slots
+// at a time and adds xi v per bin in fixed point, in three 21-bit limbs by
+// native 32-bit shared-memory atomics:
+//   1. bins by a table over the top bits of v (its high word orders as v);
+//      per bin the greatest e = floor(log2 xi) + floor(log2 v);
+//   2. the top 64 bits of the exact product xi v, shifted so that the bin's
+//      least bit weighs 2^(e_max - 61); 256 values below 2^63 leave 32-bit
+//      limb sums below 2^29.
+// Truncation loses less than 2^-61 of the bin's greatest term per SD, so 256
+// of them less than 2^-53 of the sum: below the rounding of one binary64 add,
+// where the columns rounded once per SD.  Integer sums have no order: the
+// chunk's sums, one binary64 add per bin and chunk in a fixed order, repeat
+// bit for bit.
+constexpr int kSpecMaxBins = 32;
+constexpr int kSpecChunk = 256; // slots per warp and round (8 per lane)
+constexpr int kSpecTabMax = 512;
+constexpr int kSpecWarps = 4;   // warps per block
+constexpr uint32_t kSpecLimb = (1u << 21) - 1u;
 
-__global__ void __launch_bounds__(kSpecTotNT) spectrum_total_kernel(const InstDev *__restrict__ P, int64_t n_slots,
-                                                                    const double *__restrict__ edges, int32_t n_edges,
-                                                                    double *__restrict__ partial)
+// Edges as the kernels use them, made on the host per call and passed by
+// value.  key[i]: high words of volumes certainly below (.x) and certainly
+// above (.y: greater) the volume of edge i; one sentinel after the last.
+// start[k]: the last edge certainly below every v whose high word >> shift
+// is base + k (0: below all of the table; -1 as 255).
+struct SpecTab {
+    double edge[kSpecMaxBins + 1];
+    double den[kSpecMaxBins]; // volume of air x width of the bin in ln r
+    uint2 key[kSpecMaxBins + 2];
+    int32_t n_edges, shift, base, nt;
+    uint8_t start[kSpecTabMax];
+};
+
+struct SpecSmem {
+    uint2 key[kSpecMaxBins + 2];
+    uint8_t start[kSpecTabMax];
+    uint32_t acc[kSpecWarps][3][kSpecMaxBins];
+    uint32_t emax[kSpecWarps][kSpecMaxBins];
+    double part[kSpecWarps][kSpecMaxBins];
+};
+
+__device__ __forceinline__ void spec_smem_init(SpecSmem &S, const SpecTab &T)
 {
-    __shared__ double s_col[kSpecTotMaxBins * kSpecTotNT];
-    __shared__ double s_edges[kSpecTotMaxBins + 1];
-    __shared__ float s_lo[kSpecTotMaxBins + 1], s_hi[kSpecTotMaxBins + 1];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int nb = n_edges - 1;
-    spectrum_edges_to_smem(edges, n_edges, s_edges, s_lo, s_hi);
-    for (int b = 0; b < nb; ++b)
-        s_col[b * kSpecTotNT + t] = 0.0;
+    for (int i = threadIdx.x; i < T.n_edges + 1; i += blockDim.x)
+        S.key[i] = T.key[i];
+    for (int i = threadIdx.x; i < T.nt; i += blockDim.x)
+        S.start[i] = T.start[i];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+        S.acc[warp][l][lane] = 0u;
+    S.emax[warp][lane] = 0u;
     __syncthreads();
-    const int64_t *__restrict__ gxi = P->xi;
-    const double *__restrict__ gv = P->v;
-    // four slots per iteration, all loads issued before any is used
-    constexpr int U = 4;
-    const int64_t stride = (int64_t)gridDim.x * kSpecTotNT;
-    for (int64_t i0 = (int64_t)blockIdx.x * kSpecTotNT + t; i0 < n_slots; i0 += U * stride) {
-        int64_t x[U];
-        double v[U];
+}
+
+// Bin whose radius range holds the exact radius of v, when v lies within
+// 2^-17 of the volume of edge lo + 1 (rare).
+__device__ __noinline__ int spec_bin_exact(const SpecSmem &S, const double *edge, int n_edges, uint32_t key, int lo,
+                                           double v)
+{
+    const double r = radius_exact(v);
+    while (lo + 1 < n_edges && key >= S.key[lo + 1].x && r >= edge[lo + 1])
+        ++lo;
+    return lo;
+}
+
+// Bin of a live SD, outside [0, n_edges - 1) when outside the edges.
+__device__ __forceinline__ int spec_bin(const SpecSmem &S, const SpecTab &T, double v)
+{
+    const uint32_t key = (uint32_t)__double2hiint(v);
+    const int k = min(max((int)(key >> T.shift) - T.base, 0), T.nt - 1);
+    int lo = (int)(int8_t)S.start[k];
+    uint2 nx = S.key[lo + 1];
+    while (key > nx.y) { // at most the edges inside one table entry, rarely one
+        ++lo;
+        nx = S.key[lo + 1];
+    }
+    if (key >= nx.x)
+        lo = spec_bin_exact(S, T.edge, T.n_edges, key, lo, v);
+    return lo;
+}
+
+// Adds the SDs of slots [lo, lo + n), n <= kSpecChunk, lo even, and returns
+// the sum of bin `lane`.  Every lane of the warp calls it.
+__device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, const int64_t *__restrict__ gxi,
+                                             const double *__restrict__ gv, int n)
+{
+    constexpr int Q = kSpecChunk / 64; // slot pairs per lane
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nb = T.n_edges - 1;
+    uint64_t x[2 * Q];
+    double v[2 * Q];
+    int bin[2 * Q];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t i = i0 + u * stride;
-            x[u] = i < n_slots ? gxi[i] : 0;
-            v[u] = i < n_slots ? gv[i] : 1.0;
+    for (int i = 0; i < Q; ++i) { // every load first
+        const int q = lane + 32 * i;
+        longlong2 xx = make_longlong2(0, 0);
+        double2 vv = make_double2(1.0, 1.0);
+        if (2 * q < n) {
+            xx = reinterpret_cast<const longlong2 *>(gxi)[q];
+            vv = reinterpret_cast<const double2 *>(gv)[q];
         }
+        x[2 * i] = (uint64_t)xx.x;
+        x[2 * i + 1] = (uint64_t)xx.y;
+        v[2 * i] = vv.x;
+        v[2 * i + 1] = vv.y;
+    }
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (x[u] <= 0)
-                continue;
-            const int bin = spectrum_bin_fixed<2 * kSpecTotMaxBins>(v[u], s_edges, s_lo, s_hi, n_edges);
-            if (bin >= 0) // xi v added with one rounding
-                s_col[bin * kSpecTotNT + t] = __fma_rn(xi2d(x[u]), v[u], s_col[bin * kSpecTotNT + t]);
+    for (int i = 0; i < 2 * Q; ++i) {
+        bin[i] = -1;
+        if ((int64_t)x[i] > 0) {
+            const int b = spec_bin(S, T, v[i]);
+            if ((unsigned)b < (unsigned)nb) {
+                bin[i] = b;
+                const uint32_t e = (63u - (uint32_t)__clzll((long long)x[i])) +
+                                   (((uint32_t)__double2hiint(v[i]) >> 20) & 0x7FFu);
+                atomicMax(&S.emax[warp][b], e);
+            }
         }
     }
-    __syncthreads();
-    // Bins that no thread of the block touched hold zeros only: they skip the
-    // binary64 adds (adding +0.0 changes no sum, so the result is the same).
-    for (int b = warp; b < nb; b += kSpecTotNT / 32) {
-        bool any = false;
-        for (int j = lane; j < kSpecTotNT; j += 32)
-            any |= s_col[b * kSpecTotNT + j] != 0.0;
-        double sum = 0.0;
-        if (__any_sync(0xFFFFFFFFu, any)) {
-            for (int j = lane; j < kSpecTotNT; j += 32)
-                sum = __dadd_rn(sum, s_col[b * kSpecTotNT + j]);
+    __syncwarp();
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1)
-                sum = __dadd_rn(sum, __shfl_down_sync(0xFFFFFFFFu, sum, d));
-        }
-        if (lane == 0)
-            partial[(int64_t)b * gridDim.x + blockIdx.x] = sum;
+    for (int i = 0; i < 2 * Q; ++i) {
+        if (bin[i] < 0)
+            continue;
+        const uint32_t lz = (uint32_t)__clzll((long long)x[i]);
+        const uint64_t bits = (uint64_t)__double_as_longlong(v[i]);
+        const uint32_t e = (63u - lz) + ((uint32_t)(bits >> 52) & 0x7FFu);
+        const uint64_t m = (bits << 11) | (1ull << 63); // the mantissa, leading one at bit 63
+        const uint64_t h = __umul64hi(x[i] << lz, m);   // in [2^62, 2^64): xi v = h 2^(e - 62)
+        const uint32_t d = S.emax[warp][bin[i]] - e + 1u;
+        const uint64_t val = d < 64u ? h >> d : 0ull;
+        atomicAdd(&S.acc[warp][0][bin[i]], (uint32_t)val & kSpecLimb);
+        atomicAdd(&S.acc[warp][1][bin[i]], (uint32_t)(val >> 21) & kSpecLimb);
+        atomicAdd(&S.acc[warp][2][bin[i]], (uint32_t)(val >> 42));
+    }
+    __syncwarp();
+    const uint32_t e = S.emax[warp][lane];
+    const uint32_t a0 = S.acc[warp][0][lane], a1 = S.acc[warp][1][lane], a2 = S.acc[warp][2][lane];
+    S.emax[warp][lane] = 0u;
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+        S.acc[warp][l][lane] = 0u;
+    __syncwarp();
+    if (e == 0u)
+        return 0.0;
+    // a2 2^42 and a1 2^21 + a0 as binary64, exactly (below 2^52: placed under
+    // the leading one of 2^94 and 2^52), then one rounding
+    const uint64_t low = ((uint64_t)a1 << 21) + a0;
+    const double hi = __dsub_rn(__hiloint2double(0x43300000 + (42 << 20), (int)a2), 0x1p94);
+    const double lo = __dsub_rn(__longlong_as_double((long long)(0x4330000000000000ull | low)), 0x1p52);
+    const uint32_t sc = min(max((int)e - 61, 1), 2046); // 2^(e_max - 61), biased exponent
+    return __dmul_rn(__dadd_rn(hi, lo), __hiloint2double((int)(sc << 20), 0));
+}
+
+// Sums of every bin over all slots [0, n_slots) (padding and dead SDs hold
+// xi = 0): partial[bin][block].
+__global__ void __launch_bounds__(32 * kSpecWarps) spectrum_total_kernel(const InstDev *__restrict__ P, int64_t n_slots,
+                                                                         const __grid_constant__ SpecTab T,
+                                                                         double *__restrict__ partial)
+{
+    __shared__ SpecSmem S;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    spec_smem_init(S, T);
+    const int64_t *__restrict__ gxi = P->xi;
+    const double *__restrict__ gv = P->v;
+    double acc = 0.0;
+    const int64_t step = (int64_t)gridDim.x * kSpecWarps * kSpecChunk;
+    for (int64_t at = ((int64_t)blockIdx.x * kSpecWarps + warp) * kSpecChunk; at < n_slots; at += step)
+        acc = __dadd_rn(acc, spec_chunk(S, T, gxi + at, gv + at, (int)min((int64_t)kSpecChunk, n_slots - at)));
+    S.part[warp][lane] = acc;
+    __syncthreads();
+    if (warp == 0) {
+        double sum = S.part[0][lane];
+        for (int w = 1; w < kSpecWarps; ++w)
+            sum = __dadd_rn(sum, S.part[w][lane]);
+        partial[(int64_t)lane * gridDim.x + blockIdx.x] = sum;
     }
 }
 
-// out[b] = (sum over blocks of partial[b][block], fixed order) / vol / dln[b],
-// dln[b] = ln e[b+1] - ln e[b] (from the host); one warp (block) per bin.
+// out[b] = (sum over blocks of partial[b][block], fixed order) / den[b]; one
+// warp (block) per bin.
 __global__ void spectrum_total_finalize_kernel(const double *__restrict__ partial, int32_t n_blocks,
-                                               const double *__restrict__ dln, int32_t nb, double vol,
-                                               double *__restrict__ out)
+                                               const __grid_constant__ SpecTab T, double *__restrict__ out)
 {
     const int b = blockIdx.x;
     const int lane = threadIdx.x & 31;
-    if (b >= nb)
-        return;
     double sum = 0.0;
-    for (int j = lane; j < n_blocks; j += 32)
-        sum = __dadd_rn(sum, partial[(int64_t)b * n_blocks + j]);
+    for (int j0 = lane; j0 < n_blocks; j0 += 8 * 32) { // eight loads in flight
+        double p[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            p[u] = j0 + 32 * u < n_blocks ? partial[(int64_t)b * n_blocks + j0 + 32 * u] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (j0 + 32 * u < n_blocks)
+                sum = __dadd_rn(sum, p[u]);
+    }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1)
         sum = __dadd_rn(sum, __shfl_down_sync(0xFFFFFFFFu, sum, d));
     if (lane == 0)
-        out[b] = sum / vol / dln[b];
+        out[b] = sum / T.den[b];
+}
+
+// dv/dlnr of every cell, cell-major.  One warp per cell, or (block_cells)
+// one block per cell: its warps take the cell's chunks in turn.
+__global__ void __launch_bounds__(32 * kSpecWarps) spectrum_cells_kernel(const InstDev *__restrict__ P, int32_t n_cells,
+                                                                         const __grid_constant__ SpecTab T,
+                                                                         int32_t block_cells, double *__restrict__ out)
+{
+    __shared__ SpecSmem S;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    spec_smem_init(S, T);
+    const int nb = T.n_edges - 1;
+    const int64_t *__restrict__ gxi = P->xi;
+    const double *__restrict__ gv = P->v;
+    const int32_t *__restrict__ off = P->cell_off;
+    const int unit = block_cells ? (int)blockIdx.x : (int)blockIdx.x * kSpecWarps + warp;
+    const int units = block_cells ? (int)gridDim.x : (int)gridDim.x * kSpecWarps;
+    const double den = T.den[lane < nb ? lane : 0];
+    for (int c = unit; c < n_cells; c += units) {
+        const int32_t lo = off[c], hi = off[c + 1];
+        double acc = 0.0;
+        for (int32_t at = lo + (block_cells ? warp * kSpecChunk : 0); at < hi;
+             at += block_cells ? kSpecWarps * kSpecChunk : kSpecChunk)
+            acc = __dadd_rn(acc, spec_chunk(S, T, gxi + at, gv + at, min(kSpecChunk, hi - at)));
+        if (block_cells) { // uniform over the block
+            S.part[warp][lane] = acc;
+            __syncthreads();
+            if (warp == 0)
+                for (int w = 1; w < kSpecWarps; ++w)
+                    acc = __dadd_rn(acc, S.part[w][lane]);
+            __syncthreads();
+            if (warp != 0)
+                continue;
+        }
+        // most bins of a small cell are empty: only the others divide
+        if (lane < nb)
+            out[(int64_t)c * nb + lane] = acc != 0.0 ? acc / den : 0.0;
+    }
 }
 
 // out[i] = acc[i] / vol / dln[i mod nb]

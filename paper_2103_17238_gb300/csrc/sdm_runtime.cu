@@ -417,7 +417,8 @@ struct DevGrids {
     int variant[kNumVariants] = {};
     int fused[kNumFused] = {};
     int mid[3] = {}; // clusters of the mid-size-cell kernel resident at once, K = 1, 2, 4
-    int spec = 1;    // blocks of the total-spectrum kernel
+    int spec = 1;    // blocks of the total-spectrum kernel resident at once
+    int spec_cells = 1; // the same of the per-cell spectrum kernel
 };
 std::mutex g_dev_mutex;
 DevGrids g_dev[kMaxDevices];
@@ -566,10 +567,14 @@ cudaError_t configure_kernels()
         X(64) X(128) X(256) X(512)
 #undef X
         int spec_per_sm = 0;
-        if ((r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&spec_per_sm, spectrum_total_kernel, kSpecTotNT, 0)) !=
-            cudaSuccess)
+        if ((r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&spec_per_sm, spectrum_total_kernel, 32 * kSpecWarps,
+                                                               0)) != cudaSuccess)
             e = r;
         G.spec = std::max(1, spec_per_sm) * sms;
+        if ((r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&spec_per_sm, spectrum_cells_kernel, 32 * kSpecWarps,
+                                                               0)) != cudaSuccess)
+            e = r;
+        G.spec_cells = std::max(1, spec_per_sm) * sms;
         const int hb = (int)big_hist_smem(kBigMaxLB);
         if ((r = cudaFuncSetAttribute(big_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess) e = r;
         if ((r = cudaFuncSetAttribute(big_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess) e = r;
@@ -1260,6 +1265,45 @@ void set_prefilter(InstDev &d)
     d.pre_v[1] = down(4.0 / 3.0 * pi * d.r2 * d.r2 * d.r2);
 }
 
+// The edges of a spectrum of at most kSpecMaxBins bins as its kernels use
+// them (n_edges finite, increasing, > 0).
+SpecTab spec_table(const double *e, int32_t n_edges, double vol)
+{
+    SpecTab T{};
+    T.n_edges = n_edges;
+    auto high_word = [](double x) {
+        uint64_t b;
+        std::memcpy(&b, &x, sizeof b);
+        return (uint32_t)(b >> 32);
+    };
+    for (int32_t i = 0; i < n_edges; ++i) {
+        T.edge[i] = e[i];
+        const double v = 4.0 / 3.0 * 3.141592653589793 * e[i] * e[i] * e[i]; // may be 0 or infinite
+        const uint32_t lo = high_word(v * (1.0 - 0x1p-17));
+        T.key[i] = make_uint2(lo, std::isfinite(v) ? high_word(v * (1.0 + 0x1p-17)) + 1u : 0xFFFFFFFFu);
+    }
+    T.key[n_edges] = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
+    for (int32_t b = 0; b + 1 < n_edges; ++b)
+        T.den[b] = vol * (std::log(e[b + 1]) - std::log(e[b]));
+    // entry 0 below the first edge, the last one above the last edge
+    T.shift = 15;
+    const uint32_t k0 = T.key[0].x, k1 = std::min(T.key[n_edges - 1].y, 0x7FF00000u);
+    do {
+        ++T.shift;
+        T.base = (int32_t)(k0 >> T.shift) - 1;
+        T.nt = (int32_t)(k1 >> T.shift) + 2 - T.base;
+    } while (T.nt > kSpecTabMax);
+    int lo = -1;
+    for (int32_t k = 0; k < T.nt; ++k) {
+        // high words of entry k are >= first (entry 0 also takes all below)
+        const int64_t first = k == 0 ? 0 : (int64_t)(T.base + k) << T.shift;
+        while (lo + 1 < n_edges && (int64_t)T.key[lo + 1].y < first)
+            ++lo;
+        T.start[k] = (uint8_t)(int8_t)lo;
+    }
+    return T;
+}
+
 InstDev make_inst(const sdm_ctx *c)
 {
     InstDev d{};
@@ -1633,16 +1677,27 @@ sdm_status sdm_spectrum(sdm_ctx *ctx, const double *r_edges, int32_t n_edges, in
     const int64_t n_out = per_cell ? (int64_t)ctx->cfg.n_cells * nb : nb;
     cudaStream_t s = ctx->stream;
     CTX_CUDA(ctx, configure_kernels());
-    // the total over all cells with few bins: the atomic-free kernel
-    const bool total = !per_cell && nb <= kSpecTotMaxBins;
-    const int grid = dev_grids().spec;
+    // up to 32 bins: the warp kernels, the edges passed by value; more: one
+    // block per cell with shared-memory atomics, the edges copied to the device
+    const bool few = nb <= kSpecMaxBins;
+    // one cell's spectrum is the total's
+    const bool total = few && (!per_cell || ctx->cfg.n_cells == 1);
+    const int64_t n_in = ctx->h_cell_off[ctx->cfg.n_cells];
+    const double vol = per_cell ? ctx->cfg.dv : ctx->cfg.dv * (double)ctx->cfg.n_cells;
+    const int grid = total ? (int)std::max<int64_t>(1, std::min<int64_t>(dev_grids().spec,
+                                                                         (n_in + kSpecWarps * kSpecChunk - 1) /
+                                                                             (kSpecWarps * kSpecChunk)))
+                           : 0;
     // edges, then dln[b] = ln e[b+1] - ln e[b] (host logarithms), in one copy
-    std::vector<double> host_e(r_edges, r_edges + n_edges);
-    for (int32_t b = 0; b < nb; ++b)
-        host_e.push_back(std::log(r_edges[b + 1]) - std::log(r_edges[b]));
-    const size_t b_edges = sizeof(double) * host_e.size(), b_acc = sizeof(double) * n_out;
-    const size_t b_part = total ? sizeof(double) * (size_t)grid * nb : b_acc;
-    const size_t b_tmp = b_edges + b_part + b_acc;
+    std::vector<double> host_e;
+    if (!few) {
+        host_e.assign(r_edges, r_edges + n_edges);
+        for (int32_t b = 0; b < nb; ++b)
+            host_e.push_back(std::log(r_edges[b + 1]) - std::log(r_edges[b]));
+    }
+    const size_t b_edges = sizeof(double) * host_e.size(), b_out = sizeof(double) * n_out;
+    const size_t b_part = total ? sizeof(double) * (size_t)grid * kSpecMaxBins : (few ? 0 : b_out);
+    const size_t b_tmp = b_edges + b_part + (out_on_device ? 0 : b_out);
     // host result: the edges go out of, and the status word comes back into,
     // page-locked staging (the call synchronises before it returns, so the
     // next call finds the staging free)
@@ -1657,30 +1712,37 @@ sdm_status sdm_spectrum(sdm_ctx *ctx, const double *r_edges, int32_t n_edges, in
     char *tmp = (char *)ctx->mem.get(b_tmp);
     if (!tmp)
         return fail(&ctx->error, SDM_ENOMEM, "allocation failed");
-    double *d_edges = (double *)tmp;
-    const double *d_dln = d_edges + n_edges;
-    double *d_acc = (double *)(tmp + b_edges);
+    double *d_part = (double *)(tmp + b_edges);
     double *d_out = out_on_device ? out : (double *)(tmp + b_edges + b_part);
-    const double *src_e = host_e.data();
-    if (!out_on_device) {
-        std::memcpy(ctx->h_spec, host_e.data(), b_edges);
-        src_e = (const double *)ctx->h_spec;
-    }
-    CTX_CUDA(ctx, cudaMemcpyAsync(d_edges, src_e, b_edges, cudaMemcpyHostToDevice, s));
-    const double vol = per_cell ? ctx->cfg.dv : ctx->cfg.dv * (double)ctx->cfg.n_cells;
-    if (total) {
-        spectrum_total_kernel<<<grid, kSpecTotNT, 0, s>>>(ctx->d_inst, ctx->h_cell_off[ctx->cfg.n_cells], d_edges,
-                                                          n_edges, d_acc);
-        spectrum_total_finalize_kernel<<<nb, 32, 0, s>>>(d_acc, grid, d_dln, nb, vol, d_out);
+    if (few) {
+        const SpecTab T = spec_table(r_edges, n_edges, vol);
+        if (total) {
+            spectrum_total_kernel<<<grid, 32 * kSpecWarps, 0, s>>>(ctx->d_inst, n_in, T, d_part);
+            spectrum_total_finalize_kernel<<<nb, 32, 0, s>>>(d_part, grid, T, d_out);
+        } else {
+            // a block per cell where a warp alone would take many rounds
+            const int block_cells = n_in / ctx->cfg.n_cells > 4 * kSpecChunk ? 1 : 0;
+            const int units = block_cells ? ctx->cfg.n_cells : (ctx->cfg.n_cells + kSpecWarps - 1) / kSpecWarps;
+            spectrum_cells_kernel<<<std::min(units, dev_grids().spec_cells), 32 * kSpecWarps, 0, s>>>(
+                ctx->d_inst, ctx->cfg.n_cells, T, block_cells, d_out);
+        }
     } else {
-        CTX_CUDA(ctx, cudaMemsetAsync(d_acc, 0, b_acc, s));
-        spectrum_kernel<<<ctx->cfg.n_cells, kSpecNT, 0, s>>>(ctx->d_inst, d_edges, n_edges, per_cell ? 1 : 0, d_acc);
-        spectrum_finalize_kernel<<<(unsigned)((n_out + 255) / 256), 256, 0, s>>>(d_acc, d_dln, nb, n_out, vol, d_out);
+        double *d_edges = (double *)tmp;
+        const double *src_e = host_e.data();
+        if (!out_on_device) {
+            std::memcpy(ctx->h_spec, host_e.data(), b_edges);
+            src_e = (const double *)ctx->h_spec;
+        }
+        CTX_CUDA(ctx, cudaMemcpyAsync(d_edges, src_e, b_edges, cudaMemcpyHostToDevice, s));
+        CTX_CUDA(ctx, cudaMemsetAsync(d_part, 0, b_out, s));
+        spectrum_kernel<<<ctx->cfg.n_cells, kSpecNT, 0, s>>>(ctx->d_inst, d_edges, n_edges, per_cell ? 1 : 0, d_part);
+        spectrum_finalize_kernel<<<(unsigned)((n_out + 255) / 256), 256, 0, s>>>(d_part, d_edges + n_edges, nb, n_out,
+                                                                                 vol, d_out);
     }
     CTX_CUDA(ctx, cudaGetLastError());
     if (!out_on_device) {
         uint32_t *h_status = (uint32_t *)(ctx->h_spec + sizeof(double) * 2 * kMaxEdges);
-        CTX_CUDA(ctx, cudaMemcpyAsync(out, d_out, b_acc, cudaMemcpyDeviceToHost, s));
+        CTX_CUDA(ctx, cudaMemcpyAsync(out, d_out, b_out, cudaMemcpyDeviceToHost, s));
         CTX_CUDA(ctx, cudaMemcpyAsync(h_status, &ctx->d_inst->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         CTX_CUDA(ctx, cudaStreamSynchronize(s));
         ctx->mem.put(tmp, b_tmp);
@@ -1868,7 +1930,7 @@ sdm_status sdm_diagnostics(sdm_ctx *ctx, sdm_diag *out)
         return fail(&ctx->error, SDM_ESTATE, "no attributes set");
     const int64_t n_in = ctx->h_cell_off[ctx->cfg.n_cells]; // slots of the cells (not the SDs outside)
     // the grid depends on the size only: the same state gives the same bits
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(1216, (n_in + kDiagNT * 8 - 1) / (kDiagNT * 8)));
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(kDiagBlocks, (n_in + 2 * kDiagU * kDiagNT - 1) / (2 * kDiagU * kDiagNT)));
     const size_t bytes = sizeof(DiagPart) * ((size_t)blocks + 1);
     DiagPart *d = (DiagPart *)ctx->mem.get(bytes);
     if (!d)
