@@ -1831,66 +1831,98 @@ __global__ void spectrum_finalize_kernel(const double *__restrict__ acc, const d
 // Validation and per-group counts of set_attributes (groups: the cells, then
 // n_cells for the SDs outside the domain, cell id -1).  flags bit 0: an
 // invalid attribute (first bad SD index in *bad); bit 1: groups not sorted.
-// Each warp takes 32 consecutive SDs at a time and adds one count per run of
-// equal groups (one or two atomics per warp for sorted input).
+// Each warp takes 128 consecutive SDs at a time, 32 by 32, and adds one count
+// per run of equal groups (one or two atomics per 32 for sorted input).
 __global__ void validate_count_kernel(int64_t lo, int64_t hi, const int64_t *__restrict__ xi,
                                       const double *__restrict__ v, const int32_t *__restrict__ cell, int32_t n_cells,
                                       uint32_t *__restrict__ counts, uint32_t *__restrict__ flags,
                                       unsigned long long *__restrict__ bad)
 {
     constexpr unsigned FULL = 0xFFFFFFFFu;
+    constexpr int U = 4; // runs of 32 SDs per warp and round, every load first
     const int lane = threadIdx.x & 31;
-    const int64_t wstride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = lo + (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < hi; base += wstride) {
-        const int64_t i = base + lane;
-        const bool in = i < hi;
-        const int32_t c_in = in ? cell[i] : INT32_MAX;
-        const int32_t craw = c_in == -1 ? n_cells : c_in; // the group; outside sorts last
-        int32_t c = -1;                                     // counted group, -1: none
-        if (in) {
-            const double vi = v[i];
-            if (xi[i] >= 0 && vi >= 1e-30 && vi <= 1e30 && c_in >= -1 && c_in < n_cells) {
-                c = craw;
-            } else {
-                atomicOr(flags, 1u);
-                atomicMin(bad, (unsigned long long)i);
+    const int64_t wstride = (int64_t)gridDim.x * blockDim.x * U;
+    for (int64_t base = lo + ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) * U; base < hi;
+         base += wstride) {
+        int32_t c_in[U];
+        int64_t x[U];
+        double vol[U];
+        const int32_t before = base > 0 && lane == 0 ? cell[base - 1] : -2;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = base + 32 * u + lane;
+            const bool in = i < hi;
+            c_in[u] = in ? cell[i] : INT32_MAX;
+            x[u] = in ? xi[i] : 0;
+            vol[u] = in ? v[i] : 1.0;
+        }
+        int32_t last = before == -1 ? n_cells : (before == -2 ? INT32_MIN : before); // lane 0: the SD before
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = base + 32 * u + lane;
+            const bool in = i < hi;
+            const int32_t craw = c_in[u] == -1 ? n_cells : c_in[u]; // the group; outside sorts last
+            int32_t c = -1;                                           // counted group, -1: none
+            if (in) {
+                if (x[u] >= 0 && vol[u] >= 1e-30 && vol[u] <= 1e30 && c_in[u] >= -1 && c_in[u] < n_cells) {
+                    c = craw;
+                } else {
+                    atomicOr(flags, 1u);
+                    atomicMin(bad, (unsigned long long)i);
+                }
             }
-        }
-        int32_t prev = __shfl_up_sync(FULL, craw, 1);
-        if (lane == 0) {
-            prev = INT32_MIN;
-            if (in && i > 0)
-                prev = cell[i - 1] == -1 ? n_cells : cell[i - 1];
-        }
-        if (__any_sync(FULL, in && prev > craw) && lane == 0)
-            atomicOr(flags, 2u);
-        const int32_t next = __shfl_down_sync(FULL, c, 1);
-        const bool end = lane == 31 || next != c;
-        const unsigned ends = __ballot_sync(FULL, end);
-        if (end && c >= 0) {
-            const unsigned below = ends & ((1u << lane) - 1u);
-            const int start = below ? 32 - __clz(below) : 0;
-            atomicAdd(&counts[c], (uint32_t)(lane - start + 1));
+            int32_t prev = __shfl_up_sync(FULL, craw, 1);
+            if (lane == 0)
+                prev = last;
+            if (__any_sync(FULL, in && prev > craw) && lane == 0)
+                atomicOr(flags, 2u);
+            last = __shfl_sync(FULL, craw, 31);
+            const int32_t next = __shfl_down_sync(FULL, c, 1);
+            const bool end = lane == 31 || next != c;
+            const unsigned ends = __ballot_sync(FULL, end);
+            if (end && c >= 0) {
+                const unsigned below = ends & ((1u << lane) - 1u);
+                const int start = below ? 32 - __clz(below) : 0;
+                atomicAdd(&counts[c], (uint32_t)(lane - start + 1));
+            }
         }
     }
 }
 
 // Group-sorted input: SD i goes to padded slot poff[g] + (i - uoff[g]), g its
-// group (cell id -1: n_cells, outside the domain).  Otherwise pos[i] gives
-// the slot.
+// group (cell id -1: n_cells, outside the domain).
 __global__ void scatter_kernel(int64_t n_sd, const int64_t *__restrict__ xi, const double *__restrict__ v,
                                const int32_t *__restrict__ cell, int32_t n_cells, const int32_t *__restrict__ poff,
-                               const int32_t *__restrict__ uoff, const int32_t *__restrict__ pos,
-                               int64_t *__restrict__ sxi, double *__restrict__ sv, int32_t *__restrict__ id_of_slot)
+                               const int32_t *__restrict__ uoff, int64_t *__restrict__ sxi, double *__restrict__ sv,
+                               int32_t *__restrict__ id_of_slot)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_sd; i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t p;
-        if (pos) {
-            p = pos[i];
-        } else {
-            const int32_t c = cell[i] < 0 ? n_cells : cell[i];
-            p = poff[c] + (int32_t)(i - uoff[c]);
-        }
+        const int32_t c = cell[i] < 0 ? n_cells : cell[i];
+        const int32_t p = poff[c] + (int32_t)(i - uoff[c]);
+        sxi[p] = xi[i];
+        sv[p] = v[i];
+        id_of_slot[p] = (int32_t)i;
+    }
+}
+
+// Input in no order: the groups as sort keys in id order, then, with the
+// sorted (group, id) pairs, the j-th one's SD to slot poff[g] + (j - uoff[g]).
+__global__ void group_keys_kernel(int64_t n_sd, const int32_t *__restrict__ cell, int32_t n_cells,
+                                  uint32_t *__restrict__ key)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_sd; i += (int64_t)gridDim.x * blockDim.x)
+        key[i] = (uint32_t)(cell[i] < 0 ? n_cells : cell[i]);
+}
+
+__global__ void place_sorted_kernel(int64_t n_sd, const uint32_t *__restrict__ group, const uint32_t *__restrict__ id,
+                                    const int64_t *__restrict__ xi, const double *__restrict__ v,
+                                    const int32_t *__restrict__ poff, const int32_t *__restrict__ uoff,
+                                    int64_t *__restrict__ sxi, double *__restrict__ sv,
+                                    int32_t *__restrict__ id_of_slot)
+{
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n_sd; j += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t g = group[j], i = id[j];
+        const int32_t p = poff[g] + (int32_t)(j - uoff[g]);
         sxi[p] = xi[i];
         sv[p] = v[i];
         id_of_slot[p] = (int32_t)i;

@@ -17,6 +17,7 @@
 #include "../../include/sdm.h"
 #include "sdm_kernels.cuh"
 #include "sdm_mid.cuh"
+#include "sdm_radix.cuh"
 
 using namespace sdm;
 
@@ -1560,22 +1561,12 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
     }
     poff[n_groups] = (int32_t)ps;
     uoff[n_groups] = (int32_t)us;
-    // slot positions for unsorted input (stable by id)
-    std::vector<int32_t> pos;
-    if (flags & 2u) {
-        std::vector<int32_t> hcell(n_sd);
-        if (on_device) {
-            CTX_CUDA(ctx, cudaMemcpyAsync(hcell.data(), cell_id, b_c, cudaMemcpyDeviceToHost, s));
-            CTX_CUDA(ctx, cudaStreamSynchronize(s));
-        } else {
-            std::memcpy(hcell.data(), cell_id, b_c);
-        }
-        pos.resize(n_sd);
-        std::vector<int32_t> fill(poff, poff + n_groups);
-        for (int64_t i = 0; i < n_sd; ++i)
-            pos[i] = fill[hcell[i] < 0 ? n_cells : hcell[i]]++;
-    }
-    const size_t b_aux = sizeof(int32_t) * 2 * (n_groups + 1) + (pos.empty() ? 0 : b_c);
+    // cells in no order: the groups are sorted on the device (stable, so SDs
+    // keep increasing id within a cell) and the layout gathered
+    const bool unsorted = (flags & 2u) != 0;
+    auto a256 = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t b_off = a256(sizeof(int32_t) * 2 * (n_groups + 1)), b_key = a256(sizeof(uint32_t) * n_sd);
+    const size_t b_aux = b_off + (unsorted ? 2 * b_key + radix_hist_bytes(n_sd) : 0);
     void *aux = mem.get(b_aux);
     if (!aux) {
         mem.put(meta, b_counts);
@@ -1584,11 +1575,8 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
     }
     int32_t *d_poff = (int32_t *)aux;
     int32_t *d_uoff = d_poff + (n_groups + 1);
-    int32_t *d_pos = pos.empty() ? nullptr : d_uoff + (n_groups + 1);
     // poff and uoff lie back to back in both buffers: one copy
     CTX_CUDA(ctx, cudaMemcpyAsync(d_poff, poff, sizeof(int32_t) * 2 * (n_groups + 1), cudaMemcpyHostToDevice, s));
-    if (d_pos)
-        CTX_CUDA(ctx, cudaMemcpyAsync(d_pos, pos.data(), b_c, cudaMemcpyHostToDevice, s));
     // a context's own launch plan depends only on the padded layout and the
     // launch tuning: kept when both are unchanged
     std::vector<int32_t> cell_off(poff, poff + n_cells + 1);
@@ -1609,10 +1597,28 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
     // scratch is released in stream order: nothing waits for the kernels.
     CTX_CUDA(ctx, cudaMemcpyAsync(ctx->d_cell_off, poff, sizeof(int32_t) * (n_cells + 1), cudaMemcpyHostToDevice, s));
     CTX_CUDA(ctx, cudaMemcpyAsync(ctx->d_inst, inst, sizeof *inst, cudaMemcpyHostToDevice, s));
+    if (unsorted) {
+        char *w = (char *)aux + b_off;
+        const int bits = 32 - __builtin_clz((unsigned)n_cells | 1u);
+        // the pair of arrays that ends with the result in scratch, the other
+        // one where the new multiplicities will be written after it
+        const int res = radix_result(bits);
+        uint32_t *keys[2], *vals[2];
+        keys[res] = (uint32_t *)w;
+        vals[res] = (uint32_t *)(w + b_key);
+        keys[res ^ 1] = (uint32_t *)ctx->d_xi;
+        vals[res ^ 1] = keys[res ^ 1] + n_sd;
+        group_keys_kernel<<<1216, 256, 0, s>>>(n_sd, dcell, n_cells, keys[0]);
+        const int cur = radix_sort(keys, vals, true, n_sd, bits, (uint32_t *)(w + 2 * b_key), s);
+        place_sorted_kernel<<<1216, 256, 0, s>>>(n_sd, keys[cur], vals[cur], dxi, dv, d_poff, d_uoff, ctx->d_xi,
+                                                 ctx->d_v, ctx->d_id_of_slot);
+    } else {
+        scatter_kernel<<<1216, 256, 0, s>>>(n_sd, dxi, dv, dcell, n_cells, d_poff, d_uoff, ctx->d_xi, ctx->d_v,
+                                            ctx->d_id_of_slot);
+    }
+    // after the sort, whose other pair of arrays lies over the padding too
     fill_padding_kernel<<<(n_groups + 255) / 256, 256, 0, s>>>(n_groups, d_poff, d_uoff, ctx->d_xi, ctx->d_v,
                                                                 ctx->d_id_of_slot);
-    scatter_kernel<<<1216, 256, 0, s>>>(n_sd, dxi, dv, dcell, n_cells, d_poff, d_uoff, d_pos, ctx->d_xi, ctx->d_v,
-                                        ctx->d_id_of_slot);
     CTX_CUDA(ctx, cudaGetLastError());
     mem.put(aux, b_aux);
     mem.put(meta, b_counts);

@@ -15,10 +15,9 @@
 //                        group, the water that leaves through the bottom;
 //   sed_scan_kernel      new group offsets (unpadded and padded to even
 //                        slots) and the precipitated total, in fixed order;
-//   radix_*_kernel       stable LSD radix sort of the keys, 8-bit digits
-//                        (SD-id order in, so equal groups keep increasing
-//                        id): per-tile digit counts, a scan of each digit's
-//                        row, a scan of the digit totals, a ranked scatter;
+//   radix_sort           (sdm_radix.cuh) of the keys: per-tile digit counts, a
+//                        scan of each digit's row, a scan of the digit totals,
+//                        a ranked scatter;
 //   sed_gather_kernel    the new layout, gathered from the old one;
 //   sed_pad_kernel       its padding slots.
 // The scan, the padding, the refresh of the context's own launch plan and
@@ -31,10 +30,6 @@
 namespace {
 
 constexpr int kSedNT = 256;
-constexpr int kRadixNT = 256;
-constexpr int kRadixRounds = 16;
-constexpr int kRadixTile = kRadixNT * kRadixRounds; // keys per block and pass
-constexpr int kRadixBuckets = 256;                  // 8-bit digits
 
 // ------------------------------------------------------------------ kernels
 // zeta of every slot from z (SD-id order): z - (level) dz with level =
@@ -353,126 +348,6 @@ __global__ void __launch_bounds__(1024) sed_scan_kernel(const uint32_t *__restri
     }
 }
 
-// hist[d * n_tiles + tile] = keys of the tile whose digit (key >> shift) & 255 is d.
-__global__ void __launch_bounds__(kRadixNT) radix_hist_kernel(const uint32_t *__restrict__ keys, int64_t n, int shift,
-                                                              uint32_t *__restrict__ hist, int32_t n_tiles)
-{
-    __shared__ uint32_t h[kRadixBuckets];
-    const int t = threadIdx.x;
-    h[t] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRadixTile;
-    uint32_t k[kRadixRounds]; // every load of the thread in flight at once
-#pragma unroll
-    for (int r = 0; r < kRadixRounds; ++r) {
-        const int64_t i = base + (int64_t)r * kRadixNT + t;
-        k[r] = i < n ? keys[i] : 0xFFFFFFFFu;
-    }
-#pragma unroll
-    for (int r = 0; r < kRadixRounds; ++r)
-        if (base + (int64_t)r * kRadixNT + t < n)
-            atomicAdd(&h[(k[r] >> shift) & 255u], 1u);
-    __syncthreads();
-    hist[(int64_t)t * n_tiles + blockIdx.x] = h[t];
-}
-
-// Block d: exclusive scan, in place, of the counts of digit d over the
-// tiles (one contiguous row of hist), in chunks of 1024 with a running
-// carry; total[d] = the row's sum.
-__global__ void __launch_bounds__(1024) radix_row_scan_kernel(uint32_t *__restrict__ hist, int32_t n_tiles,
-                                                              uint32_t *__restrict__ total)
-{
-    __shared__ uint32_t s[1024];
-    __shared__ uint32_t s_warp[32];
-    const int t = threadIdx.x;
-    uint32_t *row = hist + (int64_t)blockIdx.x * n_tiles;
-    uint32_t carry = 0;
-    for (int32_t c0 = 0; c0 < n_tiles; c0 += 1024) {
-        const int32_t i = c0 + t;
-        s[t] = i < n_tiles ? row[i] : 0u;
-        __syncthreads();
-        const uint32_t sum = block_exclusive_scan<1024, 1024>(s, s_warp);
-        if (i < n_tiles)
-            row[i] = carry + s[t];
-        carry += sum;
-        __syncthreads();
-    }
-    if (t == 0)
-        total[blockIdx.x] = carry;
-}
-
-// One block of 256: exclusive scan of the digit totals, in place.
-__global__ void __launch_bounds__(kRadixBuckets) radix_digit_scan_kernel(uint32_t *__restrict__ total)
-{
-    __shared__ uint32_t s[kRadixBuckets];
-    __shared__ uint32_t s_warp[32];
-    s[threadIdx.x] = total[threadIdx.x];
-    __syncthreads();
-    block_exclusive_scan<kRadixBuckets, kRadixBuckets>(s, s_warp);
-    total[threadIdx.x] = s[threadIdx.x];
-}
-
-// Stable scatter of one pass: tile keys in index order (round-major, thread
-// minor); within a round, lanes of a warp with equal digits are ranked by
-// __match_any_sync, warps by their per-digit counts in shared memory.
-__global__ void __launch_bounds__(kRadixNT) radix_scatter_kernel(const uint32_t *__restrict__ keys_in,
-                                                                 const uint32_t *__restrict__ vals_in, int64_t n,
-                                                                 int shift, const uint32_t *__restrict__ offs,
-                                                                 const uint32_t *__restrict__ digit_base,
-                                                                 int32_t n_tiles, uint32_t *__restrict__ keys_out,
-                                                                 uint32_t *__restrict__ vals_out)
-{
-    constexpr int NW = kRadixNT / 32;
-    __shared__ uint32_t s_base[kRadixBuckets + 1];
-    __shared__ uint32_t s_wcnt[NW][kRadixBuckets + 1];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    s_base[t] = digit_base[t] + offs[(int64_t)t * n_tiles + blockIdx.x];
-    for (int i = t; i < NW * (kRadixBuckets + 1); i += kRadixNT)
-        (&s_wcnt[0][0])[i] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRadixTile;
-    const unsigned lt = (1u << lane) - 1u;
-    uint32_t kk[kRadixRounds], vv[kRadixRounds]; // every load of the thread in flight at once
-#pragma unroll
-    for (int r = 0; r < kRadixRounds; ++r) {
-        const int64_t i = base + (int64_t)r * kRadixNT + t;
-        kk[r] = i < n ? keys_in[i] : 0u;
-        vv[r] = i < n ? vals_in[i] : 0u;
-    }
-#pragma unroll
-    for (int r = 0; r < kRadixRounds; ++r) {
-        const int64_t i = base + (int64_t)r * kRadixNT + t;
-        const bool valid = i < n;
-        const uint32_t k = kk[r];
-        const uint32_t v = vv[r];
-        const uint32_t d = valid ? ((k >> shift) & 255u) : (uint32_t)kRadixBuckets;
-        const unsigned peers = __match_any_sync(0xFFFFFFFFu, d);
-        const uint32_t rank = (uint32_t)__popc(peers & lt);
-        if (rank == 0)
-            s_wcnt[warp][d] = (uint32_t)__popc(peers);
-        __syncthreads();
-        if (valid) {
-            uint32_t before = 0;
-            for (int w = 0; w < warp; ++w)
-                before += s_wcnt[w][d];
-            const uint32_t pos = s_base[d] + before + rank;
-            keys_out[pos] = k;
-            vals_out[pos] = v;
-        }
-        __syncthreads();
-        for (int dd = t; dd <= kRadixBuckets; dd += kRadixNT) {
-            uint32_t sum = 0;
-            for (int w = 0; w < NW; ++w) {
-                sum += s_wcnt[w][dd];
-                s_wcnt[w][dd] = 0;
-            }
-            if (dd < kRadixBuckets)
-                s_base[dd] += sum;
-        }
-        __syncthreads();
-    }
-}
-
 // The new layout: the j-th SD in (group, id) order goes to slot
 // poff[g] + (j - ustart[g]).
 __global__ void sed_gather_kernel(int64_t n_sd, const uint32_t *__restrict__ keys, const uint32_t *__restrict__ vals,
@@ -750,18 +625,7 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     CTX_CUDA(ctx, cudaEventRecord(b.join, b.side));
     // stable sort of the new groups, SD-id order in
     const int bits = 32 - __builtin_clz((unsigned)nc | 1u);
-    const int passes = (bits + 7) / 8;
-    const int32_t tiles = (int32_t)((n + kRadixTile - 1) / kRadixTile);
-    int cur = 0;
-    for (int p = 0; p < passes; ++p) {
-        uint32_t *digit_total = b.hist + (size_t)kRadixBuckets * tiles;
-        radix_hist_kernel<<<tiles, kRadixNT, 0, s>>>(b.keys[cur], n, 8 * p, b.hist, tiles);
-        radix_row_scan_kernel<<<kRadixBuckets, 1024, 0, s>>>(b.hist, tiles, digit_total);
-        radix_digit_scan_kernel<<<1, kRadixBuckets, 0, s>>>(digit_total);
-        radix_scatter_kernel<<<tiles, kRadixNT, 0, s>>>(b.keys[cur], b.vals[cur], n, 8 * p, b.hist, digit_total,
-                                                         tiles, b.keys[cur ^ 1], b.vals[cur ^ 1]);
-        cur ^= 1;
-    }
+    const int cur = radix_sort(b.keys, b.vals, false, n, bits, b.hist, s);
     CTX_CUDA(ctx, cudaStreamWaitEvent(s, b.join, 0));
     sed_gather_kernel<<<1216, 256, 0, s>>>(n, b.keys[cur], b.vals[cur], b.ustart, b.cell_off2, ctx->d_xi, ctx->d_v,
                                            b.zeta_new, ctx->d_id_of_slot, b.xi2, b.v2, b.zeta2, b.id2, b.group2);
