@@ -138,101 +138,119 @@ __global__ void selftest_wait_kernel(uint32_t max_polls, uint32_t *out)
 }
 
 // -------------------------------------------------------------- cell step
-// A pair the filter could not decide, waiting for the exact evaluation.
-struct QEntry {
-    int64_t xj, xk;
-    double vj, vk;
-    uint32_t slot_j, slot_k; // storage slots in the run's arrays
-    uint32_t wa, wb;         // the pair's uniform words
-    uint32_t n_c;            // live SDs of its cell
-    int32_t inst;            // its run
-    int32_t gamma;           // certain collision count (>= 1), or -1: evaluate exactly
-    int32_t pad_;
+// Where a cell kernel finds its work: the plan's items and the runs' records
+// in device memory, or one cell whose record is a kernel argument (the
+// allocation-free step).
+struct PlanCells {
+    const WorkItem *items;
+    int32_t n_items;
+    InstDev *const *insts;
+    __device__ __forceinline__ WorkItem item(int i) const { return items[i]; }
+    __device__ __forceinline__ const InstDev *record(int inst) const { return insts[inst]; }
+    __device__ __forceinline__ void give_up(int inst) const { atomicOr(&insts[inst]->status, 1u); }
 };
 
-constexpr int kQueueFlush = 64; // flush once this many pairs wait
-
-template <int CAP>
-struct QueueCap {
-    static constexpr int value = (kQueueFlush + CAP / 2) < 512 ? (kQueueFlush + CAP / 2) : 512;
+struct OneCell {
+    const InstDev *P;
+    int32_t n, n_items;
+    uint32_t *status;
+    __device__ __forceinline__ WorkItem item(int) const { return WorkItem{0, 0, 0, n}; }
+    __device__ __forceinline__ const InstDev *record(int) const { return P; }
+    __device__ __forceinline__ void give_up(int) const { atomicOr(status, 1u); }
 };
 
 template <int CAP, int STAGES>
 struct CellSmem {
-    // STAGES x (xi, v) staging + key, bucket, rank, perm work arrays + queue
-    static constexpr size_t bytes =
-        (size_t)CAP * (16 * STAGES + 8 + 4 + 2 + 2) + sizeof(QEntry) * (size_t)QueueCap<CAP>::value;
+    // STAGES x (xi, v) staging + sort word, bucket start, permutation
+    static constexpr size_t bytes = (size_t)CAP * (16 * STAGES + 4 + 4 + 2) + 16;
 };
 
-// Persistent: CTA b handles work items b, b + gridDim.x, ...  Thread 0
-// streams the next STAGES - 1 cells into shared memory with bulk copies
-// while the CTA works on the current one.  Pairs the binary32 filter cannot
-// decide wait in a shared-memory queue (across cells) and are evaluated
-// exactly, one per lane, when kQueueFlush of them have gathered and at the
-// end: every SD belongs to one pair per step and nothing reads it again in
-// this launch, so deferring its update is safe.
-template <int CAP, int NT, int STAGES>
-__global__ void __launch_bounds__(NT, (1024 / NT > 0 ? 1024 / NT : 1)) cell_step_kernel(const WorkItem *__restrict__ items, int32_t n_items,
-                                                       InstDev *const *__restrict__ insts, int64_t step_offset)
+// Position, among the n words of one bucket, of the SD of rank rk in full
+// (key, rank) order; the keys are drawn again.  Taken only where two keys of
+// a bucket share the bits above the rank field of their words.
+__device__ __noinline__ uint32_t rank_in_bucket_full(uint64_t seed, uint32_t cell, int64_t s, const uint32_t *w,
+                                                     uint32_t n, uint32_t rk, uint32_t rank_mask)
+{
+    auto full_key = [&](uint32_t r) {
+        const uint4 k = draw4(seed, r >> 1, cell, s, 0u);
+        return (r & 1u) ? (((uint64_t)k.z << 32) | k.w) : (((uint64_t)k.x << 32) | k.y);
+    };
+    const uint64_t kk = full_key(rk);
+    uint32_t c = 0;
+    for (uint32_t m = 0; m < n; ++m) {
+        const uint32_t r = w[m] & rank_mask;
+        c += key_less(full_key(r), r, kk, rk) ? 1u : 0u;
+    }
+    return c;
+}
+
+// Cells of 513 .. 4096 SDs (and smaller ones where the tuning or the
+// allocation-free step asks for a block): one block per cell.  Persistent:
+// CTA b handles items b, b + gridDim.x, ...  Thread 0 streams the next
+// STAGES - 1 cells into shared memory with bulk copies while the CTA works
+// on the current one.
+//
+// A step is six phases between block barriers, and a lone cell (the paper's
+// box of 2^12) is bound by their latency and by the one SM's issue slots, so
+// each phase is short and every thread keeps what it drew in registers:
+//   keys       a thread's Philox blocks and the block of its two pairs
+//              together (the pairs' uniforms depend on nothing but their
+//              index), one shared atomic per live SD on the key's top LB bits;
+//   starts     a block scan of the bucket counts (two barriers);
+//   words      the key's next 32 - LB bits above the rank, into bucket order;
+//   order      a thread counts the smaller words of its SDs' buckets (about
+//              one each); words that share their key bits (32 of them with
+//              the bucket's) take the full keys;
+//   pairs      the bound, the certified filter and the exact evaluation as in
+//              the warp kernel, one thread per two pairs.
+// FUSED: the cell stays in its stage for n_fused consecutive steps, its
+// updates go to the stage, which returns to global memory at the end.
+template <int CAP, int NT, int STAGES, bool FUSED, typename SRC>
+__device__ __forceinline__ void block_cell_steps(const SRC src, int64_t step_offset, int32_t n_fused)
 {
     constexpr int NB = CAP;
     constexpr int LB = ilog2_c(CAP);
     constexpr int RP = (CAP / 2 + NT - 1) / NT; // rank pairs per thread
-    static_assert((1 << LB) == CAP, "CAP must be a power of two");
-    static_assert(CAP <= 65536, "ranks are stored in 16 bits");
+    constexpr int BPT = NB / NT;                // buckets per thread in the scan
+    constexpr int NW = NT / 32;
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    constexpr uint32_t RM = (uint32_t)CAP - 1u; // rank mask of a word
+    static_assert((1 << LB) == CAP && CAP <= 4096, "CAP: a power of two, ranks in LB bits");
+    static_assert(BPT == 2 || BPT == 4, "threads: half or a quarter of the buckets");
+    static_assert(CAP / 4 <= NT, "one thread per two pairs");
 
     extern __shared__ __align__(128) unsigned char smem_raw[];
     int64_t *st_xi = reinterpret_cast<int64_t *>(smem_raw);          // [STAGES][CAP]
     double *st_v = reinterpret_cast<double *>(st_xi + STAGES * CAP); // [STAGES][CAP]
-    uint64_t *s_key = reinterpret_cast<uint64_t *>(st_v + STAGES * CAP);
-    uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_key + CAP);
-    uint16_t *s_rank = reinterpret_cast<uint16_t *>(s_hist + NB);
-    uint16_t *s_perm = s_rank + CAP;
-    QEntry *s_q = reinterpret_cast<QEntry *>(s_perm + CAP);
-    constexpr uint32_t QCAP = QueueCap<CAP>::value;
-    __shared__ uint32_t s_qn;
+    uint32_t *s_word = reinterpret_cast<uint32_t *>(st_v + STAGES * CAP);
+    uint32_t *s_start = s_word + CAP; // NB + 1 bucket counts, then starts
+    uint16_t *s_perm = reinterpret_cast<uint16_t *>(s_start + NB + 4);
     __shared__ uint64_t s_bar[STAGES];
     __shared__ int4 s_meta[STAGES]; // off, n, cell, inst
     __shared__ uint32_t s_warp[32];
 
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (t == 0) {
         for (int i = 0; i < STAGES; ++i)
             mbar_init(&s_bar[i], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        s_qn = 0;
     }
-    __syncthreads();
-
-    auto flush = [&]() { // all threads; the queue's contents are visible to all
-        const uint32_t nq = s_qn < QCAP ? s_qn : QCAP;
-        for (uint32_t e = t; e < nq; e += NT) {
-            QEntry E = s_q[e];
-            InstDev *Pq = insts[E.inst];
-            const int64_t g = E.gamma > 0 ? cap_gamma(E.gamma, E.xj, E.xk)
-                                          : pair_gamma_exact(Pq, E.n_c, E.xj, E.xk, E.vj, E.vk, E.wa, E.wb);
-            if (g > 0) {
-                const bool split = shima_update(g, E.xj, E.xk, E.vj, E.vk);
-                Pq->xi[E.slot_j] = E.xj;
-                Pq->xi[E.slot_k] = E.xk;
-                Pq->v[E.slot_k] = E.vk;
-                if (split)
-                    Pq->v[E.slot_j] = E.vj;
-            }
-        }
-        __syncthreads();
-        if (t == 0)
-            s_qn = 0;
-        __syncthreads();
+    auto clear = [&]() {
+        if constexpr (BPT == 4)
+            reinterpret_cast<uint4 *>(s_start)[t] = make_uint4(0u, 0u, 0u, 0u);
+        else
+            reinterpret_cast<uint2 *>(s_start)[t] = make_uint2(0u, 0u);
     };
+    clear();
+    __syncthreads();
 
     auto issue = [&](int k) { // thread 0: start loading the k-th cell of this CTA
         const int i = blockIdx.x + k * gridDim.x;
-        if (i >= n_items)
+        if (i >= src.n_items)
             return;
         const int sg = k % STAGES;
-        const WorkItem it = items[i];
-        const InstDev *P = insts[it.inst];
+        const WorkItem it = src.item(i);
+        const InstDev *P = src.record(it.inst);
         s_meta[sg] = make_int4(it.off, it.n, it.cell, it.inst);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive_expect_tx(&s_bar[sg], (uint32_t)it.n * 16u);
@@ -243,7 +261,7 @@ __global__ void __launch_bounds__(NT, (1024 / NT > 0 ? 1024 / NT : 1)) cell_step
         for (int k = 0; k < STAGES - 1; ++k)
             issue(k);
 
-    for (int k = 0; blockIdx.x + k * gridDim.x < n_items; ++k) {
+    for (int k = 0; blockIdx.x + k * gridDim.x < src.n_items; ++k) {
         if (t == 0)
             issue(k + STAGES - 1);
         const int sg = k % STAGES;
@@ -252,9 +270,9 @@ __global__ void __launch_bounds__(NT, (1024 / NT > 0 ? 1024 / NT : 1)) cell_step
             // a copy never completed: report, wait (bounded) for the copies
             // still in flight, leave
             if (t == 0) {
-                atomicOr(&insts[s_meta[sg].w]->status, 1u);
+                src.give_up(s_meta[sg].w);
                 for (int kk = k; kk < k + STAGES; ++kk) // copies issued and not consumed
-                    if (blockIdx.x + kk * gridDim.x < n_items)
+                    if (blockIdx.x + kk * gridDim.x < src.n_items)
                         mbar_wait_bounded(&s_bar[kk % STAGES], (uint32_t)(kk / STAGES) & 1u);
             }
             return;
@@ -262,139 +280,192 @@ __global__ void __launch_bounds__(NT, (1024 / NT > 0 ? 1024 / NT : 1)) cell_step
         const int4 meta = s_meta[sg];
         const int n = meta.y;
         const uint32_t cell = (uint32_t)meta.z;
-        InstDev *__restrict__ P = insts[meta.w];
-        const int64_t s = P->step + step_offset;
+        const InstDev *__restrict__ P = src.record(meta.w);
+        const int64_t s0 = P->step + step_offset;
         const uint64_t seed = P->seed;
-        const int64_t *xs = st_xi + sg * CAP;
-        const double *vs = st_v + sg * CAP;
+        int64_t *xs = st_xi + sg * CAP;
+        double *vs = st_v + sg * CAP;
+        const uint32_t *vs_words = reinterpret_cast<const uint32_t *>(vs);
         int64_t *__restrict__ gxi = P->xi + meta.x;
         double *__restrict__ gv = P->v + meta.x;
-
-        for (int i = t; i < NB; i += NT)
-            s_hist[i] = 0u;
-        __syncthreads();
-
-        // sort keys of live SDs and their bucket slots
-        uint64_t key[2 * RP];
-        uint32_t slot[2 * RP];
+        const PairConsts C = pair_consts(P);
+        const int n_rep = FUSED ? n_fused : 1;
+        for (int rep = 0; rep < n_rep; ++rep) { // uniform over the block
+            const int64_t s = s0 + rep;
+            uint4 kw[RP];
 #pragma unroll
-        for (int r = 0; r < RP; ++r) {
-            const int q = t + r * NT;
-            slot[2 * r] = 0xFFFFFFFFu;
-            slot[2 * r + 1] = 0xFFFFFFFFu;
-            key[2 * r] = 0;
-            key[2 * r + 1] = 0;
-            if (2 * q < n) {
-                const bool la = xs[2 * q] > 0, lb = xs[2 * q + 1] > 0;
-                if (la | lb) {
-                    const uint4 w = draw4(seed, (uint32_t)q, cell, s, 0u);
-                    if (la) {
-                        key[2 * r] = ((uint64_t)w.x << 32) | w.y;
-                        slot[2 * r] = atomicAdd(&s_hist[key[2 * r] >> (64 - LB)], 1u);
-                    }
-                    if (lb) {
-                        key[2 * r + 1] = ((uint64_t)w.z << 32) | w.w;
-                        slot[2 * r + 1] = atomicAdd(&s_hist[key[2 * r + 1] >> (64 - LB)], 1u);
-                    }
-                }
-            }
-        }
-        __syncthreads();
-
-        // bucket starts; the total is the live count n_c
-        const uint32_t n_c = block_exclusive_scan<NT, NB>(s_hist, s_warp);
-        if (n_c >= 2) {
-            // scatter into bucket order
+            for (int r = 0; r < RP; ++r)
+                kw[r] = draw4(seed, (uint32_t)(t + r * NT), cell, s, 0u);
+            const uint4 pw = draw4(seed, (uint32_t)t, cell, s, 1u); // of pairs 2 t and 2 t + 1
+            uint32_t word[2 * RP], at[2 * RP]; // at: bucket above slot, all ones for a dead SD
 #pragma unroll
             for (int r = 0; r < RP; ++r) {
+                const int q = t + r * NT;
+                longlong2 x2 = make_longlong2(0, 0);
+                if (2 * q < n)
+                    x2 = reinterpret_cast<const longlong2 *>(xs)[q];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    if (slot[2 * r + h] != 0xFFFFFFFFu) {
-                        const uint32_t pos = s_hist[key[2 * r + h] >> (64 - LB)] + slot[2 * r + h];
-                        s_key[pos] = key[2 * r + h];
-                        s_rank[pos] = (uint16_t)(2 * (t + r * NT) + h);
+                    const uint32_t k1 = h ? kw[r].z : kw[r].x, k0 = h ? kw[r].w : kw[r].y;
+                    word[2 * r + h] = (__funnelshift_l(k0, k1, LB) & ~RM) | (uint32_t)(2 * q + h);
+                    at[2 * r + h] = 0xFFFFFFFFu;
+                    if ((h ? x2.y : x2.x) > 0) {
+                        const uint32_t b = k1 >> (32 - LB);
+                        at[2 * r + h] = (b << 16) | atomicAdd(&s_start[b], 1u);
                     }
                 }
             }
             __syncthreads();
 
-            // order within each bucket by (key, rank)
-            for (uint32_t pos = t; pos < n_c; pos += NT) {
-                const uint64_t kk = s_key[pos];
-                const uint32_t rk = s_rank[pos];
-                const uint32_t b = (uint32_t)(kk >> (64 - LB));
-                const uint32_t lo = s_hist[b];
-                const uint32_t hi = (b + 1 < (uint32_t)NB) ? s_hist[b + 1] : n_c;
-                uint32_t cnt = 0;
-                for (uint32_t m = lo; m < hi; ++m)
-                    cnt += key_less(s_key[m], s_rank[m], kk, rk) ? 1u : 0u;
-                s_perm[lo + cnt] = (uint16_t)rk;
+            // bucket starts; the total is the live count n_c
+            uint32_t cnt[BPT], sum = 0;
+            if constexpr (BPT == 4) {
+                const uint4 c = reinterpret_cast<const uint4 *>(s_start)[t];
+                cnt[0] = c.x;
+                cnt[1] = c.y;
+                cnt[2] = c.z;
+                cnt[3] = c.w;
+            } else {
+                const uint2 c = reinterpret_cast<const uint2 *>(s_start)[t];
+                cnt[0] = c.x;
+                cnt[1] = c.y;
             }
-            __syncthreads();
-
-            // pairs (l = 2q, 2q + 1 share one Philox block): the filter
-            // settles almost all; the rest join the queue
-            const uint32_t n_pairs = n_c / 2;
-            const float ratio_f = u32_to_f32_rn((n_c & 1u) ? n_c : n_c - 1u);
-            const PairConsts C = pair_consts(P);
-            for (uint32_t q = t; 2 * q < n_pairs; q += NT) {
-                const uint4 w = draw4(seed, q, cell, s, 1u);
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t l = 2 * q + h;
-                    if (l >= n_pairs)
-                        break;
-                    int a = s_perm[2 * l], b = s_perm[2 * l + 1];
-                    int64_t xa = xs[a], xb = xs[b];
-                    if (xa < xb) { // j holds the larger multiplicity; ties keep the earlier
-                        const int tmp = a;
-                        a = b;
-                        b = tmp;
-                        const int64_t tx = xa;
-                        xa = xb;
-                        xb = tx;
+            for (int i = 0; i < BPT; ++i)
+                sum += cnt[i];
+            uint32_t incl = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULL, incl, d);
+                if (lane >= d)
+                    incl += y;
+            }
+            if (lane == 31)
+                s_warp[warp] = incl;
+            __syncthreads();
+            const uint32_t ws = lane < NW ? s_warp[lane] : 0u;
+            const uint32_t n_c = __reduce_add_sync(FULL, ws);
+            uint32_t run = __reduce_add_sync(FULL, lane < warp ? ws : 0u) + incl - sum;
+#pragma unroll
+            for (int i = 0; i < BPT; ++i) {
+                const uint32_t c = cnt[i];
+                cnt[i] = run;
+                run += c;
+            }
+            if constexpr (BPT == 4)
+                reinterpret_cast<uint4 *>(s_start)[t] = make_uint4(cnt[0], cnt[1], cnt[2], cnt[3]);
+            else
+                reinterpret_cast<uint2 *>(s_start)[t] = make_uint2(cnt[0], cnt[1]);
+            if (t == 0)
+                s_start[NB] = n_c;
+            __syncthreads();
+            if (n_c >= 2) { // uniform over the block
+                uint32_t lo[2 * RP];
+#pragma unroll
+                for (int i = 0; i < 2 * RP; ++i) {
+                    lo[i] = 0;
+                    if (at[i] != 0xFFFFFFFFu) {
+                        lo[i] = s_start[at[i] >> 16];
+                        s_word[lo[i] + (at[i] & 0xFFFFu)] = word[i];
                     }
-                    double va = vs[a], vb = vs[b];
-                    const uint32_t wa = h ? w.z : w.x, wb = h ? w.w : w.y;
-                    const int32_t gf = pair_gamma_filter(C, ratio_f, xa, va, vb, wa);
-                    if (gf == 0)
+                }
+                __syncthreads();
+#pragma unroll
+                for (int i = 0; i < 2 * RP; ++i) {
+                    if (at[i] == 0xFFFFFFFFu)
                         continue;
-                    const uint32_t qi = atomicAdd(&s_qn, 1u);
-                    if (qi < QCAP) {
-                        QEntry E;
-                        E.xj = xa;
-                        E.xk = xb;
-                        E.vj = va;
-                        E.vk = vb;
-                        E.slot_j = (uint32_t)(meta.x + a);
-                        E.slot_k = (uint32_t)(meta.x + b);
-                        E.wa = wa;
-                        E.wb = wb;
-                        E.n_c = n_c;
-                        E.inst = meta.w;
-                        E.gamma = gf;
-                        s_q[qi] = E;
-                    } else { // queue full: update here
+                    const uint32_t hi = s_start[(at[i] >> 16) + 1u];
+                    uint32_t c = 0;
+                    bool tie = false;
+                    for (uint32_t m = lo[i]; m < hi; ++m) {
+                        const uint32_t wm = s_word[m];
+                        c += wm < word[i] ? 1u : 0u;
+                        tie |= ((wm ^ word[i]) - 1u) < RM; // another word with the same key bits
+                    }
+                    if (tie)
+                        c = rank_in_bucket_full(seed, cell, s, s_word + lo[i], hi - lo[i], word[i] & RM, RM);
+                    s_perm[lo[i] + c] = (uint16_t)(word[i] & RM);
+                }
+                __syncthreads();
+                const uint32_t n_pairs = n_c / 2;
+                if (2u * (uint32_t)t < n_pairs) {
+                    const float ratio_f = u32_to_f32_rn((n_c & 1u) ? n_c : n_c - 1u);
+                    const float sc = C.dtdvf * ratio_f;
+                    const uint2 ab2 = reinterpret_cast<const uint2 *>(s_perm)[t];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (2u * (uint32_t)t + h >= n_pairs)
+                            break;
+                        const uint32_t ab = h ? ab2.y : ab2.x;
+                        uint32_t a = ab & 0xFFFFu, b = ab >> 16;
+                        int64_t xa = xs[a], xb = xs[b];
+                        const uint32_t wa = h ? pw.z : pw.x, wb = h ? pw.w : pw.y;
+                        if (pair_prefilter_zero(C, sc, xa > xb ? xa : xb, vs_words[2 * a + 1], vs_words[2 * b + 1], wa))
+                            continue;
+                        if (xa < xb) { // j holds the larger multiplicity; ties keep the earlier
+                            const uint32_t tmp = a;
+                            a = b;
+                            b = tmp;
+                            const int64_t tx = xa;
+                            xa = xb;
+                            xb = tx;
+                        }
+                        const int32_t gf = pair_gamma_filter(C, ratio_f, xa, vs_words[2 * a + 1], vs_words[2 * b + 1],
+                                                             wa);
+                        if (gf == 0)
+                            continue;
+                        double va = vs[a], vb = vs[b];
                         const int64_t g = gf > 0 ? cap_gamma(gf, xa, xb)
                                                  : pair_gamma_exact(P, n_c, xa, xb, va, vb, wa, wb);
                         if (g > 0) {
                             const bool split = shima_update(g, xa, xb, va, vb);
-                            gxi[a] = xa;
-                            gxi[b] = xb;
-                            gv[b] = vb;
-                            if (split)
-                                gv[a] = va;
+                            if constexpr (FUSED) { // nothing else reads this pair in this step
+                                xs[a] = xa;
+                                xs[b] = xb;
+                                vs[b] = vb;
+                                if (split)
+                                    vs[a] = va;
+                            } else {
+                                gxi[a] = xa;
+                                gxi[b] = xb;
+                                gv[b] = vb;
+                                if (split)
+                                    gv[a] = va;
+                            }
                         }
                     }
                 }
             }
+            clear(); // read last in the ordering
+            __syncthreads();
         }
-        __syncthreads(); // stage sg and the work arrays are free again
-        if (s_qn >= (uint32_t)kQueueFlush)
-            flush();
+        if constexpr (FUSED) { // the cell back to global memory
+            for (int i = t; 2 * i < n; i += NT) {
+                reinterpret_cast<longlong2 *>(gxi)[i] = reinterpret_cast<const longlong2 *>(xs)[i];
+                reinterpret_cast<double2 *>(gv)[i] = reinterpret_cast<const double2 *>(vs)[i];
+            }
+            // the stage was written through the generic proxy; the next bulk
+            // copy into it goes through the async proxy
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncthreads();
+        }
     }
-    if (s_qn > 0)
-        flush();
+}
+
+template <int CAP, int NT, int STAGES, bool FUSED>
+__global__ void __launch_bounds__(NT, (1024 / NT > 0 ? 1024 / NT : 1)) cell_step_kernel(const WorkItem *__restrict__ items, int32_t n_items,
+                                                       InstDev *const *__restrict__ insts, int64_t step_offset,
+                                                       int32_t n_fused)
+{
+    block_cell_steps<CAP, NT, STAGES, FUSED>(PlanCells{items, n_items, insts}, step_offset, n_fused);
+}
+
+// One step of one cell whose record is an argument: one launch, nothing to
+// set up in device memory.
+template <int CAP, int NT>
+__global__ void __launch_bounds__(NT) one_cell_step_kernel(const __grid_constant__ InstDev P, int32_t n, uint32_t *status)
+{
+    block_cell_steps<CAP, NT, 1, false>(OneCell{&P, n, 1, status}, 0, 1);
 }
 
 // ------------------------------------------------------ warp-per-cell step
@@ -523,26 +594,6 @@ __device__ __forceinline__ void sort_net(uint32_t (&v)[E])
 // Swap rounds of the lane-block sort before the per-element fixup takes
 // over (one to three rounds suffice for bucket-ordered random words).
 constexpr int kMaxSwapRounds = 32;
-
-// Position, among the n words of one bucket, of the SD of rank rk in full
-// (key, rank) order; the keys are drawn again.  Taken only by buckets in
-// which two keys share the bits above the rank field (about one cell in 500
-// at 256 SDs, one in 60 at 512).
-__device__ __noinline__ uint32_t rank_in_bucket_full(uint64_t seed, uint32_t cell, int64_t s, const uint32_t *w,
-                                                     uint32_t n, uint32_t rk, uint32_t rank_mask)
-{
-    auto full_key = [&](uint32_t r) {
-        const uint4 k = draw4(seed, r >> 1, cell, s, 0u);
-        return (r & 1u) ? (((uint64_t)k.z << 32) | k.w) : (((uint64_t)k.x << 32) | k.y);
-    };
-    const uint64_t kk = full_key(rk);
-    uint32_t c = 0;
-    for (uint32_t m = 0; m < n; ++m) {
-        const uint32_t r = w[m] & rank_mask;
-        c += key_less(full_key(r), r, kk, rk) ? 1u : 0u;
-    }
-    return c;
-}
 
 // FUSED: every cell stays in its stage for n_fused consecutive steps (its
 // updates go to the stage, which returns to global memory at the end), for

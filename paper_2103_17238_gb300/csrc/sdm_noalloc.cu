@@ -8,13 +8,16 @@
 // This entry point serves them: the caller passes the cell's arrays, and the
 // large-cell kernels' scratch (sort keys, ranks, permutation, bucket counts)
 // together with their work lists and run record live in one fixed-size,
-// file-scope device array, set up once per device.
+// file-scope device array, set up once per device.  A cell of up to 4096 SDs
+// needs none of it: one block steps it in one launch, its record a kernel
+// argument.
 //
 // Compiled as part of the library's single translation unit (included at the
 // end of sdm_runtime.cu), after the kernels it launches.
 
 #include <initializer_list>
 #include <mutex>
+#include <type_traits>
 
 namespace {
 
@@ -39,7 +42,8 @@ constexpr size_t kNaPairs = na_align(kNaBuckets + sizeof(BigBucket) * ((size_t)1
 constexpr size_t kNaInst = na_align(kNaPairs + sizeof(BigPairs) * (size_t)kNaMaxPairBlocks);
 constexpr size_t kNaInsts = na_align(kNaInst + sizeof(InstDev));
 constexpr size_t kNaCellOff = na_align(kNaInsts + sizeof(InstDev *));
-constexpr size_t kNaBytes = na_align(kNaCellOff + 2 * sizeof(int32_t));
+constexpr size_t kNaStatus = na_align(kNaCellOff + 2 * sizeof(int32_t));
+constexpr size_t kNaBytes = na_align(kNaStatus + sizeof(uint32_t));
 
 // About 8.6 MiB; every GPU that loads the library holds it until exit.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaBytes];
@@ -100,10 +104,7 @@ sdm_status noalloc_base(unsigned char **out)
         e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e != cudaSuccess)
             return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: cudaGetSymbolAddress: %s", cudaGetErrorString(e));
-        const int hb = (int)big_hist_smem(kBigMaxLB);
-        if ((e = cudaFuncSetAttribute(big_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(big_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(big_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess)
+        if ((e = configure_kernels()) != cudaSuccess)
             return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: kernel set-up: %s", cudaGetErrorString(e));
         g_na_base[dev] = static_cast<unsigned char *>(p);
     }
@@ -188,6 +189,28 @@ extern "C" sdm_status sdm_cell_step_noalloc(const sdm_config *cfg, int64_t step,
     inst.precision = cfg->precision;
     inst.n_cells = 1;
     const int n = (int)n_sd;
+    if (n <= 4096) { // one block, one launch, the record as an argument
+        uint32_t *status = reinterpret_cast<uint32_t *>(base + kNaStatus);
+        auto one = [&](auto cap, auto nt) {
+            constexpr int CAP = decltype(cap)::value, NT = decltype(nt)::value;
+            one_cell_step_kernel<CAP, NT><<<1, NT, CellSmem<CAP, 1>::bytes, s>>>(inst, n, status);
+        };
+        int cls = 0;
+        while (kClassCap[cls] < n)
+            ++cls;
+        switch (cls) {
+#define X(CAP, NT, ST)                                                                                                 \
+    case ilog2_c(CAP) - 6:                                                                                             \
+        one(std::integral_constant<int, CAP>{}, std::integral_constant<int, NT>{});                                    \
+        break;
+            SDM_BLOCK_VARIANTS(X)
+#undef X
+        }
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess)
+            return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: launch: %s", cudaGetErrorString(e));
+        return SDM_OK;
+    }
     const int lb = big_lb(n);
     if (lb > kNaMaxLb) // cannot happen for n <= kNaMaxSd; the tables are sized for kNaMaxLb
         return fail(nullptr, SDM_EINVAL, "sdm_cell_step_noalloc: %d buckets exceed the static tables", 1 << lb);

@@ -376,7 +376,15 @@ void launch_warp_fused(int grid, int n, const WorkItem *items, InstDev *const *i
 template <int CAP, int NT, int ST>
 void launch_block(int grid, int n, const WorkItem *items, InstDev *const *insts, int64_t off, cudaStream_t st)
 {
-    cell_step_kernel<CAP, NT, ST><<<grid, NT, CellSmem<CAP, ST>::bytes, st>>>(items, n, insts, off);
+    cell_step_kernel<CAP, NT, ST, false><<<grid, NT, CellSmem<CAP, ST>::bytes, st>>>(items, n, insts, off, 1);
+}
+
+// One stage: a block loads a cell once per nf steps.
+template <int CAP, int NT>
+void launch_block_fused(int grid, int n, const WorkItem *items, InstDev *const *insts, int64_t off, int32_t nf,
+                        cudaStream_t st)
+{
+    cell_step_kernel<CAP, NT, 1, true><<<grid, NT, CellSmem<CAP, 1>::bytes, st>>>(items, n, insts, off, nf);
 }
 
 typedef void (*fused_fn)(int grid, int n, const WorkItem *, InstDev *const *, int64_t, int32_t, cudaStream_t);
@@ -387,15 +395,19 @@ struct Variant {
     launch_fn launch;
 };
 
-// the fused warp kernels by capacity 64 .. 512
+// the fused kernels: warp per cell by size class (capacity 64 .. 512), and
+// block per cell for every class
 struct FusedVariant {
-    int cap;
+    int per_block; // cells of a block
     fused_fn launch;
 };
-const FusedVariant g_fused[] = {{64, launch_warp_fused<64>},
-                                {128, launch_warp_fused<128>},
-                                {256, launch_warp_fused<256>},
-                                {512, launch_warp_fused<512>}};
+const FusedVariant g_fused[] = {
+    {2, launch_warp_fused<64>}, {2, launch_warp_fused<128>}, {2, launch_warp_fused<256>}, {2, launch_warp_fused<512>},
+#define X(CAP, NT, ST) {1, launch_block_fused<CAP, NT>},
+    SDM_BLOCK_VARIANTS(X)
+#undef X
+};
+constexpr int kFusedWarp = 4; // then the block kernels by class
 
 const Variant g_variants[] = {
 #define X(CAP, WARPS) {CAP, WARPS, launch_warp<CAP, WARPS>},
@@ -541,12 +553,12 @@ cudaError_t configure_kernels()
 #define X(CAP, NT, ST)                                                                                                 \
     {                                                                                                                  \
         const int bytes = (int)CellSmem<CAP, ST>::bytes;                                                               \
-        if ((r = cudaFuncSetAttribute(cell_step_kernel<CAP, NT, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
-                                      bytes)) != cudaSuccess)                                                          \
+        if ((r = cudaFuncSetAttribute(cell_step_kernel<CAP, NT, ST, false>,                                            \
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess)             \
             e = r;                                                                                                     \
         int per_sm = 0;                                                                                                \
-        if ((r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cell_step_kernel<CAP, NT, ST>, NT, bytes)) != \
-            cudaSuccess)                                                                                               \
+        if ((r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cell_step_kernel<CAP, NT, ST, false>, NT,      \
+                                                               bytes)) != cudaSuccess)                                 \
             e = r;                                                                                                     \
         G.variant[v++] = std::max(1, per_sm) * sms;                                                                   \
     }
@@ -566,6 +578,23 @@ cudaError_t configure_kernels()
         G.fused[v++] = std::max(1, per_sm) * sms;                                                                      \
     }
         X(64) X(128) X(256) X(512)
+#undef X
+#define X(CAP, NT, ST)                                                                                                 \
+    {                                                                                                                  \
+        const int bytes = (int)CellSmem<CAP, 1>::bytes;                                                                \
+        if ((r = cudaFuncSetAttribute(cell_step_kernel<CAP, NT, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                      bytes)) != cudaSuccess)                                                          \
+            e = r;                                                                                                     \
+        if ((r = cudaFuncSetAttribute(one_cell_step_kernel<CAP, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
+                                      bytes)) != cudaSuccess)                                                          \
+            e = r;                                                                                                     \
+        int per_sm = 0;                                                                                                \
+        if ((r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cell_step_kernel<CAP, NT, 1, true>, NT,        \
+                                                               bytes)) != cudaSuccess)                                 \
+            e = r;                                                                                                     \
+        G.fused[v++] = std::max(1, per_sm) * sms;                                                                      \
+    }
+        SDM_BLOCK_VARIANTS(X)
 #undef X
         int spec_per_sm = 0;
         if ((r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&spec_per_sm, spectrum_total_kernel, 32 * kSpecWarps,
@@ -1049,8 +1078,8 @@ struct ClassFork {
 
 // Enqueues n steps (offsets off .. off + n - 1) of every cell.  Cells are
 // independent, so each one may take its n steps apart from the others: with
-// fusion on (tuning fuse_steps f >= 2) the warp-per-cell classes take up to f
-// steps per launch, the other cells one launch per step.
+// fusion on (tuning fuse_steps f >= 2) the shared-memory classes take up to f
+// steps per launch, the larger cells one launch per step.
 void enqueue_steps(const Plan &pl, int64_t off, int32_t n, cudaStream_t st)
 {
     // one fork and one join for all n steps: every class's launches follow
@@ -1064,9 +1093,10 @@ void enqueue_steps(const Plan &pl, int64_t off, int32_t n, cudaStream_t st)
         if (!pl.n_items[k])
             continue;
         const Variant &x = g_variants[pl.variant[k]];
-        if (fuse && x.warps > 0) {
-            const FusedVariant &fv = g_fused[k];
-            const int grid = std::min((pl.n_items[k] + 1) / 2, dev_grids().fused[k]);
+        if (fuse) {
+            const int fi = x.warps > 0 ? k : kFusedWarp + k;
+            const FusedVariant &fv = g_fused[fi];
+            const int grid = std::min((pl.n_items[k] + fv.per_block - 1) / fv.per_block, dev_grids().fused[fi]);
             for (int32_t i = 0; i < n; i += f)
                 fv.launch(grid, pl.n_items[k], pl.d_items[k], pl.d_insts, off + i, std::min(f, n - i), cf.of(k));
         } else {
