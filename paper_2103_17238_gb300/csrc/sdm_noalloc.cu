@@ -10,7 +10,7 @@
 // together with their work lists and run record live in one fixed-size,
 // file-scope device array, set up once per device.  A cell of up to 4096 SDs
 // needs none of it: one block steps it in one launch, its record a kernel
-// argument.
+// argument.  Up to 2^18 SDs take two launches (sdm_spread.cuh).
 //
 // Compiled as part of the library's single translation unit (included at the
 // end of sdm_runtime.cu), after the kernels it launches.
@@ -43,7 +43,12 @@ constexpr size_t kNaInst = na_align(kNaPairs + sizeof(BigPairs) * (size_t)kNaMax
 constexpr size_t kNaInsts = na_align(kNaInst + sizeof(InstDev));
 constexpr size_t kNaCellOff = na_align(kNaInsts + sizeof(InstDev *));
 constexpr size_t kNaStatus = na_align(kNaCellOff + 2 * sizeof(int32_t));
-constexpr size_t kNaBytes = na_align(kNaStatus + sizeof(uint32_t));
+// the bucketed path's counts (zero between calls; its rooms lie over the
+// multi-pass path's arrays)
+constexpr int kNaSpreadMax = 1 << 18;
+constexpr size_t kNaSpreadCnt = na_align(kNaStatus + sizeof(uint32_t));
+constexpr size_t kNaBytes = na_align(kNaSpreadCnt + sizeof(uint32_t) * (spread_words(kNaSpreadMax / kSpreadMean + 1) + 4));
+static_assert((size_t)(kNaSpreadMax / kSpreadMean + 1) * kSpreadRoom * sizeof(uint2) <= kNaBstart, "rooms");
 
 // About 8.6 MiB; every GPU that loads the library holds it until exit.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaBytes];
@@ -206,6 +211,21 @@ extern "C" sdm_status sdm_cell_step_noalloc(const sdm_config *cfg, int64_t step,
             SDM_BLOCK_VARIANTS(X)
 #undef X
         }
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess)
+            return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: launch: %s", cudaGetErrorString(e));
+        return SDM_OK;
+    }
+    if (n <= kNaSpreadMax) { // the bucketed path: two launches
+        int64_t counters = 0, rooms = 0;
+        const SpreadCell c = spread_cell(nullptr, 0, 0, n, counters, rooms);
+        SpreadScratch S;
+        S.cnt = reinterpret_cast<uint32_t *>(base + kNaSpreadCnt);
+        S.rooms = reinterpret_cast<uint2 *>(base);
+        uint32_t *status = reinterpret_cast<uint32_t *>(base + kNaStatus);
+        launch_chained(one_spread_scatter_kernel, (n / 2 + kSpreadNT - 1) / kSpreadNT, kSpreadNT, s, false, inst, c, S,
+                       status);
+        launch_chained(one_spread_pairs_kernel, c.groups, kSpreadNT, s, true, inst, c, S, status);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess)
             return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: launch: %s", cudaGetErrorString(e));

@@ -18,6 +18,7 @@
 #include "sdm_kernels.cuh"
 #include "sdm_mid.cuh"
 #include "sdm_radix.cuh"
+#include "sdm_spread.cuh"
 
 using namespace sdm;
 
@@ -166,6 +167,11 @@ struct Plan {
     int mid_clusters[3] = {};    // clusters of each launch: the SMs dealt in proportion to the classes' SDs
     cudaStream_t mid_side[3] = {}; // the cluster launches run beside each other and the multi-pass path
     cudaEvent_t mid_fork = nullptr, mid_join[3] = {};
+    // the larger cells when they hold few SDs in all (sdm_spread.cuh); then no
+    // cell takes the cluster or the multi-pass path
+    SpreadCell *d_spread_scatter = nullptr, *d_spread_pairs = nullptr; // an item per block
+    int n_spread_scatter = 0, n_spread_pairs = 0;
+    SpreadScratch spread{};
     BigCell *d_bigs = nullptr;
     int n_big = 0;
     BigChunk *d_chunks = nullptr;
@@ -516,6 +522,24 @@ cudaError_t launch_mid(int clusters, int n, const WorkItem *items, InstDev *cons
     return cudaLaunchKernelEx(&cfg, mid_cell_kernel<K>, items, (int32_t)n, insts, off);
 }
 
+// A launch whose blocks may become resident before the kernel before it on
+// the stream is complete (programmatic dependent launch); both kernels wait
+// with chain_wait() before they touch what the other writes.
+template <typename... KARGS, typename... ARGS>
+cudaError_t launch_chained(void (*kernel)(KARGS...), int grid, int nt, cudaStream_t st, bool chain, ARGS... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(nt, 1, 1);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = chain ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KARGS>(args)...);
+}
+
 // Configures the current device once (the first context, batch or spectrum
 // call on each device does it, with that device current).
 cudaError_t configure_kernels()
@@ -688,6 +712,25 @@ cudaError_t plan_refresh(Plan &pl, const int32_t *d_cell_off, int32_t n_cells, i
     return cudaGetLastError();
 }
 
+// Whether a plan's cells above the shared-memory classes take the bucketed
+// path (sdm_spread.cuh): `total` SDs in `count` cells, the largest of `most`.
+// Measured per step (us, bucketed | cluster | multi-pass): one box of 12,000
+// 8.4 | 46 | 37, of 2^17 15 | - | 43, of 524,288 36 | - | 52, of 900,000
+// 59 | - | 62, of 2^20 73 | - | 66; 8 of 2^17 52 | - | 58; 76 of 12,000
+// 41 | 50 | 53; 180 of 5000 40 | 42 | 58; but 150 of 5000 34 | 24 | 45.  So up
+// to 15 x 2^16 SDs, except where the cluster path takes every cell at once, one
+// CTA each, in less time (about 4 + 3.8 n / 1000 us for its largest cell
+// against 7 + 0.037 total / 1000).
+constexpr int64_t kSpreadMaxSd = (int64_t)15 << 16;
+
+bool spread_cells(int64_t total, int64_t count, int32_t most, const sdm_tuning &t, int sms)
+{
+    if (total == 0 || total > kSpreadMaxSd || t.mid_max_sd != SDM_MID_MAX_SD_DEFAULT)
+        return false;
+    const bool one_round = most <= std::min(t.mid_max_sd, kMidSdPerCta) && count <= sms;
+    return !(one_round && 4.0 + 3.8e-3 * most < 7.0 + 3.7e-5 * (double)total);
+}
+
 // Work lists of every run in the batch, split by cell size.
 sdm_status build_plan(sdm_batch *b)
 {
@@ -703,6 +746,7 @@ sdm_status build_plan(sdm_batch *b)
         std::vector<BigChunk> chunks;
         std::vector<BigBucket> buckets;
         std::vector<BigPairs> pairs;
+        std::vector<SpreadCell> sp_scatter, sp_pairs;
         std::vector<InstDev *> insts;
         std::vector<int8_t> cls; // per cell of a run: its class, -1 above them, -2 fewer than 2 SDs
     };
@@ -722,12 +766,28 @@ sdm_status build_plan(sdm_batch *b)
     chunks.clear();
     buckets.clear();
     pairs.clear();
+    scr.sp_scatter.clear();
+    scr.sp_pairs.clear();
+    int64_t sp_counters = 0, sp_rooms = 0;
     insts.assign(n_inst, nullptr);
     int64_t hist_total = 0, sd_total = 0, bkt_total = 0;
     const sdm_tuning tun = current_tuning();
     pl.tuning = tun;
     for (int k = 0; k < kNumClass; ++k)
         pl.variant[k] = variant_for(kClassCap[k], tun);
+    // the cells above the shared-memory classes
+    int64_t above_sd = 0, above_cells = 0;
+    int32_t above_most = 0;
+    for (sdm_ctx *c : b->ctxs)
+        for (int32_t cell = 0; c->largest_cell > tun.smem_max_sd && cell < c->cfg.n_cells; ++cell) {
+            const int32_t n = c->h_cell_off[cell + 1] - c->h_cell_off[cell];
+            if (n > tun.smem_max_sd) {
+                above_sd += n;
+                ++above_cells;
+                above_most = std::max(above_most, n);
+            }
+        }
+    const bool spread = spread_cells(above_sd, above_cells, above_most, tun, dev_grids().mid[0]);
     for (int i = 0; i < n_inst; ++i) {
         sdm_ctx *c = b->ctxs[i];
         insts[i] = c->d_inst;
@@ -765,6 +825,14 @@ sdm_status build_plan(sdm_batch *b)
             if (cls[cell] != -1)
                 continue;
             const int n = off[cell + 1] - off[cell];
+            if (spread) {
+                SpreadCell sc = spread_cell(c->d_inst, cb + cell, off[cell], n, sp_counters, sp_rooms);
+                for (sc.first = 0; 2 * sc.first < n; sc.first += kSpreadNT)
+                    scr.sp_scatter.push_back(sc);
+                for (sc.first = 0; sc.first < sc.nb; sc.first += kSpreadW)
+                    scr.sp_pairs.push_back(sc);
+                continue;
+            }
             if (n <= tun.mid_max_sd) { // the cluster path, K = 1, 2 or 4 CTAs (sorted below)
                 const int km = n <= kMidSdPerCta ? 0 : (n <= 2 * kMidSdPerCta ? 1 : 2);
                 mid[km].push_back(WorkItem{i, c->cfg.cell_base + cell, c->h_cell_off[cell], n});
@@ -811,6 +879,10 @@ sdm_status build_plan(sdm_batch *b)
         off_mid[k] = sz;
         sz += a16(sizeof(WorkItem) * mid[k].size());
     }
+    const size_t off_sps = sz;
+    sz += a16(sizeof(SpreadCell) * scr.sp_scatter.size());
+    const size_t off_spp = sz;
+    sz += a16(sizeof(SpreadCell) * scr.sp_pairs.size());
     const size_t off_bigs = sz;
     sz += a16(sizeof(BigCell) * bigs.size());
     const size_t off_chunks = sz;
@@ -856,6 +928,10 @@ sdm_status build_plan(sdm_batch *b)
     for (int k = 0; k < 3; ++k)
         if (!mid[k].empty())
             std::memcpy(h + off_mid[k], mid[k].data(), sizeof(WorkItem) * mid[k].size());
+    if (!scr.sp_pairs.empty()) {
+        std::memcpy(h + off_sps, scr.sp_scatter.data(), sizeof(SpreadCell) * scr.sp_scatter.size());
+        std::memcpy(h + off_spp, scr.sp_pairs.data(), sizeof(SpreadCell) * scr.sp_pairs.size());
+    }
     if (!bigs.empty()) {
         std::memcpy(h + off_bigs, bigs.data(), sizeof(BigCell) * bigs.size());
         std::memcpy(h + off_chunks, chunks.data(), sizeof(BigChunk) * chunks.size());
@@ -872,7 +948,20 @@ sdm_status build_plan(sdm_batch *b)
     }
     // a context's own plan of shared-memory classes only: items with room
     // for every cell in every class, built on the device like later refreshes
-    if (own && n_inst == 1 && bigs.empty() && mid[0].empty() && mid[1].empty() && mid[2].empty()) {
+    if (!scr.sp_pairs.empty()) {
+        pl.d_spread_scatter = reinterpret_cast<SpreadCell *>(d + off_sps);
+        pl.d_spread_pairs = reinterpret_cast<SpreadCell *>(d + off_spp);
+        pl.n_spread_scatter = (int)scr.sp_scatter.size();
+        pl.n_spread_pairs = (int)scr.sp_pairs.size();
+        pl.spread.cnt = plan_alloc<uint32_t>(pl, mem, (size_t)sp_counters);
+        pl.spread.rooms = plan_alloc<uint2>(pl, mem, (size_t)sp_rooms * kSpreadRoom);
+        if (!pl.spread.cnt || !pl.spread.rooms)
+            return fail(&b->error, SDM_ENOMEM, "batch plan: bucket scratch allocation failed");
+        const cudaError_t e = cudaMemsetAsync(pl.spread.cnt, 0, sizeof(uint32_t) * (size_t)sp_counters, b->stream);
+        if (e != cudaSuccess)
+            return cuda_fail(b, e, "batch plan: bucket counts");
+    }
+    if (own && n_inst == 1 && scr.sp_pairs.empty() && bigs.empty() && mid[0].empty() && mid[1].empty() && mid[2].empty()) {
         const int32_t nc = own->cfg.n_cells;
         pl.d_items_all = plan_alloc<WorkItem>(pl, mem, (size_t)kNumClass * std::max(nc, 1));
         pl.d_refresh = plan_alloc<uint32_t>(pl, mem, kNumClass + 1);
@@ -909,7 +998,7 @@ sdm_status build_plan(sdm_batch *b)
             const int share = (int)((double)sms * (double)work[k] / (double)total) / ks[k];
             pl.mid_clusters[k] = std::max(1, std::min({share, pl.n_mid[k], G.mid[k]}));
         }
-        int classes = bigs.empty() ? 0 : 1;
+        int classes = bigs.empty() && scr.sp_pairs.empty() ? 0 : 1;
         for (int k = 0; k < 3; ++k)
             classes += pl.n_mid[k] ? 1 : 0;
         if (classes > 1) {
@@ -1008,6 +1097,12 @@ void enqueue_big_steps(const Plan &pl, int64_t off, int32_t n, cudaStream_t st)
                 cudaStreamWaitEvent(pl.mid_side[k], pl.mid_fork, 0);
     }
     auto side = [&](int k) { return fork ? pl.mid_side[k] : st; };
+    for (int32_t i = 0; pl.n_spread_pairs && i < n; ++i) {
+        const PlanSpread sc{pl.d_spread_scatter}, sp{pl.d_spread_pairs};
+        // chained but for the first, whose predecessor may be any work
+        launch_chained(spread_scatter_kernel, pl.n_spread_scatter, kSpreadNT, st, i > 0, sc, pl.spread, off + i);
+        launch_chained(spread_pairs_kernel, pl.n_spread_pairs, kSpreadNT, st, true, sp, pl.spread, off + i);
+    }
     for (int32_t i = 0; i < n; ++i) {
         if (pl.n_mid[2])
             launch_mid<4>(pl.mid_clusters[2], pl.n_mid[2], pl.d_mid[2], pl.d_insts, off + i, side(2));
@@ -1375,8 +1470,8 @@ sdm_status check_device_status(sdm_ctx *ctx)
         return fail(&ctx->error, SDM_ETIMEOUT, "a device-side wait for a bulk copy gave up; results are incomplete");
     if (status & 2u)
         return fail(&ctx->error, SDM_ESTATE,
-                    "a sort bucket of a mid-size cell outgrew its room (more than 2048 of the cell's keys in one "
-                    "bucket): that cell was not stepped; results are incomplete");
+                    "a sort bucket of a large cell outgrew its room (its keys are far from uniform): that cell was not "
+                    "stepped; results are incomplete");
     return SDM_OK;
 }
 
@@ -1423,7 +1518,12 @@ int64_t sdm_footprint_bytes(int64_t capacity_sd, int32_t n_cells, int32_t larges
         // liveness bits per chunk
         const int lb = big_lb(largest_cell);
         const int64_t chunks = (capacity_sd + kBigChunk - 1) / kBigChunk + n_cells;
-        bytes += capacity_sd * (4 + 4) + (chunks << lb) * 4 + ((int64_t)n_cells << lb) * 4 + chunks * kLiveWords * 4;
+        int64_t big = capacity_sd * (4 + 4) + (chunks << lb) * 4 + ((int64_t)n_cells << lb) * 4 + chunks * kLiveWords * 4;
+        if (slots <= kSpreadMaxSd + n_cells + 1) { // or the bucketed path's rooms and counts
+            const int64_t nb = slots / kSpreadMean + std::min<int64_t>(n_cells, slots / largest_cell + 1) + 1;
+            big = std::max<int64_t>(big, nb * (kSpreadRoom * (int64_t)sizeof(uint2) + 2 * kSpreadStride * (int64_t)sizeof(uint32_t) + 48));
+        }
+        bytes += big;
     }
     return bytes;
 }
