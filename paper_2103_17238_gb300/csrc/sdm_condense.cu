@@ -16,12 +16,12 @@
 // Multiplicities do not change.  The per-cell condensed water sum(xi dV) is
 // an optional output.
 //
-// One step on the device (one warp per work item of up to 256 slots of one
-// cell, 16-byte loads of xi and v, the binary32 arithmetic per SD, one
-// binary64 add per SD to update v):
-//   condense_kernel       the update, and per work item the partial sum of
-//                         xi dV (one fused multiply-add per SD, lanes in a
-//                         fixed shuffle order);
+// One step on the device (a warp takes up to 256 slots of one cell at a time:
+// 16-byte loads of xi and v, the binary32 arithmetic per SD, one binary64 add
+// per SD to update v, the sum of xi dV in fixed point):
+//   condense_by_cell_kernel one warp per cell, its water at once; or, when
+//                         the largest cell is above 1024 slots,
+//   condense_kernel       one warp per work item of up to 256 slots, and
 //   condense_cells_kernel per cell, its items' partials in item order.
 // HBM traffic: 16 B read and 8 B written per live SD.
 //
@@ -32,6 +32,8 @@ namespace {
 
 constexpr int kCondItem = 256; // slots per work item (a multiple of 2: cells start at even slots)
 constexpr int kCondNT = 256;
+constexpr int kCondByCell = 1024; // largest cell that one warp takes (4 rounds)
+constexpr int kCondStage = 4;     // calls whose fields may be on their way at once
 constexpr float kR3ToVolF = (float)(4.0 * kPi / 3.0); // 4 pi / 3 (binary64 pi) rounded to binary32
 
 struct __align__(16) CondItem {
@@ -49,9 +51,10 @@ struct CondBuffers {
     float *cf = nullptr;           // n_cells: c of each cell, binary32
     double *partial = nullptr;     // n_items
     double *cond = nullptr;        // n_cells
-    float *h_cf = nullptr;         // page-locked staging of cf
-    cudaEvent_t cf_done = nullptr; // the last copy out of h_cf
-    std::vector<float> last_cf;    // cf on the device (no copy when a call repeats it)
+    float *h_cf = nullptr;         // page-locked staging of cf, kCondStage fields in turn
+    cudaEvent_t cf_done[kCondStage] = {}; // the last copy out of each
+    int stage = 0;                 // the next one
+    const float *last_cf = nullptr; // the field on the device (no copy when a call repeats it)
 };
 
 // f2d_exact (sdm_sediment.cu): the exact widening of a binary32 on the
@@ -59,7 +62,9 @@ struct CondBuffers {
 
 // dV of one live SD (the reading above), binary32.  The binary32 image of
 // v is rounded on the integer pipe (d2f_rn): the conversion instruction would
-// take the narrow binary64 pipe, which then bounds the kernel.
+// take the narrow binary64 pipe, which then bounds the kernel.  sqrt(x) is r
+// itself: in binary arithmetic rounded to nearest the square root of a
+// rounded square is the number again (Boldo 2015; r^2 is far from underflow).
 __device__ __forceinline__ float condense_dv(double v, float cf, float xminf)
 {
     bool in_range;
@@ -74,73 +79,123 @@ __device__ __forceinline__ float condense_dv(double v, float cf, float xminf)
     }
     if (d == 0.0f)
         return 0.0f;
-    const float a = __fsqrt_rn(xn), b = __fsqrt_rn(x);
-    const float num = __fmul_rn(d, __fadd_rn(__fadd_rn(xn, __fmul_rn(a, b)), x));
-    return __fmul_rn(kR3ToVolF, __fdiv_rn(num, __fadd_rn(a, b)));
+    const float a = __fsqrt_rn(xn);
+    const float num = __fmul_rn(d, __fadd_rn(__fadd_rn(xn, __fmul_rn(a, r)), x));
+    return __fmul_rn(kR3ToVolF, __fdiv_rn(num, __fadd_rn(a, r)));
 }
 
+// |dV|'s exponent field (1 for subnormals) and mantissa.
+__device__ __forceinline__ uint32_t dv_exponent(float dv) { return max((__float_as_uint(dv) >> 23) & 0xFFu, 1u); }
+__device__ __forceinline__ uint32_t dv_mantissa(float dv)
+{
+    const uint32_t b = __float_as_uint(dv);
+    return (b & 0x7FFFFFu) | ((b & 0x7F800000u) ? 0x800000u : 0u);
+}
+
+// One warp's round: up to kCondItem slots of one cell (n even) grow, and with
+// WATER the sum of xi |dV| is returned (every dV of a cell has the sign of its
+// cf).  xi |dV| is exact below xi 2^39 and is cut to 63 bits below the round's
+// greatest: FixedSum.
+template <bool WATER>
+__device__ __forceinline__ double condense_round(const int64_t *__restrict__ xi, double *__restrict__ v, int n, float c,
+                                                 float xminf)
+{
+    constexpr int PAIRS = kCondItem / 64; // SD pairs per lane
+    const int lane = threadIdx.x & 31;
+    const longlong2 *x2 = reinterpret_cast<const longlong2 *>(xi);
+    double2 *v2 = reinterpret_cast<double2 *>(v);
+    const int np = n / 2;
+    longlong2 xs[PAIRS];
+    double2 vs[PAIRS];
+#pragma unroll
+    for (int k = 0; k < PAIRS; ++k) { // every load of the round first
+        const int q = lane + 32 * k;
+        xs[k] = q < np ? x2[q] : make_longlong2(0, 0);
+        vs[k] = q < np ? v2[q] : make_double2(1.0, 1.0);
+    }
+    float dv[2 * PAIRS];
+    uint32_t emax = 0u;
+#pragma unroll
+    for (int k = 0; k < PAIRS; ++k) {
+        double2 w = vs[k];
+        dv[2 * k] = xs[k].x > 0 ? condense_dv(w.x, c, xminf) : 0.0f;
+        dv[2 * k + 1] = xs[k].y > 0 ? condense_dv(w.y, c, xminf) : 0.0f;
+        if (dv[2 * k] != 0.0f || dv[2 * k + 1] != 0.0f) { // adding 0 changes nothing
+            w.x = __dadd_rn(w.x, f2d_exact(dv[2 * k]));
+            w.y = __dadd_rn(w.y, f2d_exact(dv[2 * k + 1]));
+            v2[lane + 32 * k] = w;
+        }
+        if constexpr (WATER) {
+            if (dv[2 * k] != 0.0f)
+                emax = max(emax, 63u - (uint32_t)__clzll(xs[k].x) + dv_exponent(dv[2 * k]));
+            if (dv[2 * k + 1] != 0.0f)
+                emax = max(emax, 63u - (uint32_t)__clzll(xs[k].y) + dv_exponent(dv[2 * k + 1]));
+        }
+    }
+    if constexpr (!WATER)
+        return 0.0;
+    emax = __reduce_max_sync(0xFFFFFFFFu, emax);
+    FixedSum f;
+#pragma unroll
+    for (int k = 0; k < 2 * PAIRS; ++k) {
+        if (dv[k] == 0.0f)
+            continue;
+        const uint64_t x = (uint64_t)((k & 1) ? xs[k / 2].y : xs[k / 2].x);
+        const uint32_t m = dv_mantissa(dv[k]);
+        // the product below 2^63 in units of 2^(emax - 188)
+        const int sh = (int)dv_exponent(dv[k]) - (int)emax + 38;
+        if (x >> 39) { // xi above 5e11: the product's top 64 bits
+            const uint32_t lz = (uint32_t)__clzll((long long)x);
+            const uint64_t h = __umul64hi(x << lz, (uint64_t)m << 40); // the product times 2^(lz - 24)
+            const int r = sh + 24 - (int)lz;
+            f.add(r >= 0 ? h << r : (r > -64 ? h >> -r : 0ull));
+        } else {
+            const uint64_t pr = x * m;
+            f.add(sh >= 0 ? pr << sh : (sh > -64 ? pr >> -sh : 0ull));
+        }
+    }
+    return f.warp_sum((int)emax - 188);
+}
+
+// Every cell by one warp: no work list, nothing to rebuild when the layout
+// changes, no second pass.  56 + 10 us per call of the 4.19M-SD grid as two
+// kernels with binary64 sums (the binary64 pipe 68% busy).
+template <bool WATER>
+__global__ void __launch_bounds__(kCondNT) condense_by_cell_kernel(const int32_t *__restrict__ cell_off, int32_t n_cells,
+                                                                   const int64_t *__restrict__ xi,
+                                                                   double *__restrict__ v, const float *__restrict__ cf,
+                                                                   float xminf, double *__restrict__ out)
+{
+    const int lane = threadIdx.x & 31;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int cell = gw; cell < n_cells; cell += nw) {
+        const int32_t lo = cell_off[cell], hi = cell_off[cell + 1];
+        const float c = cf[cell];
+        double acc = 0.0;
+        for (int32_t at = lo; at < hi; at += kCondItem) {
+            const double w = condense_round<WATER>(xi + at, v + at, min(kCondItem, hi - at), c, xminf);
+            acc = at == lo ? w : __dadd_rn(acc, w);
+        }
+        if (WATER && lane == 0)
+            out[cell] = c < 0.0f ? 0.0 - acc : acc;
+    }
+}
+
+// Cells above kCondByCell slots: work items of up to kCondItem slots.
+template <bool WATER>
 __global__ void __launch_bounds__(kCondNT) condense_kernel(const CondItem *__restrict__ items, int32_t n_items,
                                                            const int64_t *__restrict__ xi, double *__restrict__ v,
                                                            const float *__restrict__ cf, float xminf,
                                                            double *__restrict__ partial)
 {
-    constexpr int PAIRS = kCondItem / 64; // SD pairs per lane
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     for (int it = gw; it < n_items; it += nw) {
         const CondItem I = items[it];
         const float c = cf[I.cell];
-        const longlong2 *x2 = reinterpret_cast<const longlong2 *>(xi + I.begin);
-        double2 *v2 = reinterpret_cast<double2 *>(v + I.begin);
-        const int np = I.n / 2;
-        longlong2 xs[PAIRS];
-        double2 vs[PAIRS];
-#pragma unroll
-        for (int k = 0; k < PAIRS; ++k) { // every load of the item first
-            const int q = lane + 32 * k;
-            if (q < np) {
-                xs[k] = x2[q];
-                vs[k] = v2[q];
-            }
-        }
-        double acc = 0.0;
-#pragma unroll
-        for (int k = 0; k < PAIRS; ++k) {
-            const int q = lane + 32 * k;
-            if (q >= np)
-                continue;
-            double2 w = vs[k];
-            bool changed = false;
-            if (xs[k].x > 0) {
-                const float dv = condense_dv(w.x, c, xminf);
-                if (dv != 0.0f) {
-                    const double dd = f2d_exact(dv);
-                    w.x = __dadd_rn(w.x, dd);
-                    if (partial)
-                        acc = __fma_rn(xi2d(xs[k].x), dd, acc);
-                    changed = true;
-                }
-            }
-            if (xs[k].y > 0) {
-                const float dv = condense_dv(w.y, c, xminf);
-                if (dv != 0.0f) {
-                    const double dd = f2d_exact(dv);
-                    w.y = __dadd_rn(w.y, dd);
-                    if (partial)
-                        acc = __fma_rn(xi2d(xs[k].y), dd, acc);
-                    changed = true;
-                }
-            }
-            if (changed)
-                v2[q] = w;
-        }
-        if (partial) {
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1)
-                acc = __dadd_rn(acc, __shfl_down_sync(0xFFFFFFFFu, acc, d));
-            if (lane == 0)
-                partial[it] = acc;
-        }
+        const double w = condense_round<WATER>(xi + I.begin, v + I.begin, I.n, c, xminf);
+        if (WATER && lane == 0)
+            partial[it] = c < 0.0f ? -w : w;
     }
 }
 
@@ -171,10 +226,11 @@ void cond_release(sdm_ctx *ctx)
     void *bufs[] = {b.items, b.item_start, b.cf, b.partial, b.cond};
     for (void *p : bufs)
         ctx->mem.put(p, 0);
-    if (b.cf_done) {
-        cudaEventSynchronize(b.cf_done);
-        cudaEventDestroy(b.cf_done);
-    }
+    for (cudaEvent_t ev : b.cf_done)
+        if (ev) {
+            cudaEventSynchronize(ev);
+            cudaEventDestroy(ev);
+        }
     if (b.h_cf)
         cudaFreeHost(b.h_cf);
     delete ctx->cond;
@@ -195,9 +251,10 @@ sdm_status cond_prepare(sdm_ctx *ctx)
             cond_release(ctx);
             return fail(&ctx->error, SDM_ENOMEM, "condensation: device allocation failed");
         }
-        cudaError_t e = cudaMallocHost(&b.h_cf, sizeof(float) * nc);
-        if (e == cudaSuccess)
-            e = cudaEventCreateWithFlags(&b.cf_done, cudaEventDisableTiming);
+        cudaError_t e = cudaMallocHost(&b.h_cf, sizeof(float) * nc * kCondStage);
+        for (cudaEvent_t &ev : b.cf_done)
+            if (e == cudaSuccess)
+                e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
         if (e != cudaSuccess) {
             cudaGetLastError();
             cond_release(ctx);
@@ -205,7 +262,7 @@ sdm_status cond_prepare(sdm_ctx *ctx)
         }
     }
     CondBuffers &b = *ctx->cond;
-    if (b.layout_version == ctx->layout_version)
+    if (ctx->largest_cell <= kCondByCell || b.layout_version == ctx->layout_version)
         return SDM_OK;
     std::vector<CondItem> items;
     std::vector<int32_t> start(nc + 1);
@@ -253,7 +310,22 @@ extern "C" sdm_status sdm_condensation_step(sdm_ctx *ctx, const double *G, const
         return fail(&ctx->error, SDM_EINVAL, "r_min = %g outside [1e-9, 1e-3] m", r_min);
     const int32_t nc = ctx->cfg.n_cells;
     const double dt = ctx->cfg.dt;
+    st = cond_prepare(ctx);
+    if (st != SDM_OK)
+        return st;
+    CondBuffers &b = *ctx->cond;
+    cudaStream_t cs = ctx->stream;
+    CTX_CUDA(ctx, cudaEventSynchronize(b.cf_done[b.stage])); // the staging's last copy has left
+    float *cf = b.h_cf + (size_t)b.stage * nc;
+    // one pass without branches; what it finds wrong is named by a second
+    int bad = 0;
     for (int32_t c = 0; c < nc; ++c) {
+        const double g = ((2.0 * G[c]) * s[c]) * dt;
+        bad |= (int)!(G[c] >= 0.0) | (int)!(s[c] >= -1.0) | (int)!(s[c] <= 1.0) | (int)!(std::fabs(g) <= 1e-6) |
+               (int)!(G[c] <= 1.7976931348623157e308);
+        cf[c] = (float)g;
+    }
+    for (int32_t c = 0; bad && c < nc; ++c) {
         if (!(std::isfinite(G[c]) && G[c] >= 0.0) || !(std::isfinite(s[c]) && s[c] >= -1.0 && s[c] <= 1.0))
             return fail(&ctx->error, SDM_EINVAL, "cell %d: G = %g must be finite and >= 0, s = %g in [-1, 1]", c, G[c],
                         s[c]);
@@ -261,39 +333,38 @@ extern "C" sdm_status sdm_condensation_step(sdm_ctx *ctx, const double *G, const
             return fail(&ctx->error, SDM_EINVAL, "cell %d: |2 G s dt| = %g m^2 above 1e-6 m^2", c,
                         std::fabs(((2.0 * G[c]) * s[c]) * dt));
     }
-    st = cond_prepare(ctx);
-    if (st != SDM_OK)
-        return st;
-    CondBuffers &b = *ctx->cond;
-    cudaStream_t cs = ctx->stream;
-    std::vector<float> cf(nc);
-    for (int32_t c = 0; c < nc; ++c)
-        cf[c] = (float)(((2.0 * G[c]) * s[c]) * dt);
-    if (cf != b.last_cf) { // a new field (a repeated one is on the device already)
-        CTX_CUDA(ctx, cudaEventSynchronize(b.cf_done)); // the staging's last copy has left
-        std::memcpy(b.h_cf, cf.data(), sizeof(float) * nc);
-        CTX_CUDA(ctx, cudaMemcpyAsync(b.cf, b.h_cf, sizeof(float) * nc, cudaMemcpyHostToDevice, cs));
-        CTX_CUDA(ctx, cudaEventRecord(b.cf_done, cs));
-        b.last_cf.swap(cf);
+    if (!b.last_cf || std::memcmp(cf, b.last_cf, sizeof(float) * nc)) { // a new field (a repeated one is on the device)
+        b.last_cf = nullptr;
+        CTX_CUDA(ctx, cudaMemcpyAsync(b.cf, cf, sizeof(float) * nc, cudaMemcpyHostToDevice, cs));
+        CTX_CUDA(ctx, cudaEventRecord(b.cf_done[b.stage], cs));
+        b.last_cf = cf;
+        b.stage = (b.stage + 1) % kCondStage;
     }
     const float xminf = (float)(r_min * r_min);
-    if (b.n_items > 0) {
+    const int cells_grid = (int)std::min<int64_t>((nc + kCondNT / 32 - 1) / (kCondNT / 32), 152 * 8);
+    double *out = condensed && condensed_on_device ? condensed : b.cond;
+    if (ctx->largest_cell <= kCondByCell) {
+        if (condensed)
+            condense_by_cell_kernel<true><<<cells_grid, kCondNT, 0, cs>>>(ctx->d_cell_off, nc, ctx->d_xi, ctx->d_v, b.cf,
+                                                                          xminf, out);
+        else
+            condense_by_cell_kernel<false><<<cells_grid, kCondNT, 0, cs>>>(ctx->d_cell_off, nc, ctx->d_xi, ctx->d_v,
+                                                                           b.cf, xminf, nullptr);
+    } else {
         const int grid = (int)std::min<int64_t>((b.n_items + kCondNT / 32 - 1) / (kCondNT / 32), 152 * 8);
-        condense_kernel<<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, b.cf, xminf,
-                                                  condensed ? b.partial : nullptr);
-    }
-    if (condensed) {
-        const int grid = (int)std::min<int64_t>((nc + kCondNT / 32 - 1) / (kCondNT / 32), 152 * 8);
-        condense_cells_kernel<<<grid, kCondNT, 0, cs>>>(b.item_start, nc, b.partial, b.cond);
+        if (condensed) {
+            condense_kernel<true><<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, b.cf, xminf,
+                                                            b.partial);
+            condense_cells_kernel<<<cells_grid, kCondNT, 0, cs>>>(b.item_start, nc, b.partial, out);
+        } else {
+            condense_kernel<false><<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, b.cf, xminf,
+                                                             nullptr);
+        }
     }
     CTX_CUDA(ctx, cudaGetLastError());
-    if (condensed) {
-        if (condensed_on_device) {
-            CTX_CUDA(ctx, cudaMemcpyAsync(condensed, b.cond, sizeof(double) * nc, cudaMemcpyDeviceToDevice, cs));
-        } else {
-            CTX_CUDA(ctx, cudaMemcpyAsync(condensed, b.cond, sizeof(double) * nc, cudaMemcpyDeviceToHost, cs));
-            CTX_CUDA(ctx, cudaStreamSynchronize(cs));
-        }
+    if (condensed && !condensed_on_device) {
+        CTX_CUDA(ctx, cudaMemcpyAsync(condensed, b.cond, sizeof(double) * nc, cudaMemcpyDeviceToHost, cs));
+        CTX_CUDA(ctx, cudaStreamSynchronize(cs));
     }
     return SDM_OK;
 }

@@ -72,6 +72,73 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t *s, uint32_t *
     return total;
 }
 
+// ------------------------------------------------------ fixed-point sums
+// A binary64 instruction holds an SM's pipe for 32 cycles per warp here (as
+// long as 128 integer instructions of its four schedulers), so sums of one
+// product per SD are kept in integers: a round's products, as 64-bit integers
+// below 2^63 whose unit comes from the round's greatest, add up without
+// order or rounding, and one binary64 number leaves the round.
+
+// n 2^w rounded to nearest even, on the integer pipe; n > 0, w such that the
+// result is normal; sticky: the number is a little above n.
+__device__ __forceinline__ double u64_to_double(uint64_t n, bool sticky, int w)
+{
+    const int lz = __clzll((long long)n);
+    n <<= lz;
+    const uint64_t m = n >> 11;
+    const uint32_t rest = (((uint32_t)n & 0x7FFu) << 1) | (sticky ? 1u : 0u); // below the last place
+    const uint32_t up = rest > 0x800u || (rest == 0x800u && (m & 1u)) ? 1u : 0u;
+    return __longlong_as_double((long long)(((uint64_t)(uint32_t)(1023 + 52 + 11 - 1 - lz + w) << 52) + m + up));
+}
+
+// (a 2^B + l) 2^w, not zero, a < 2^(64 - B + 9), l < 2^52 (a sum of 2^61 and
+// more keeps 53 bits).
+template <int B>
+__device__ __forceinline__ double fixed_to_double(uint64_t a, uint64_t l, int w)
+{
+    if (a == 0)
+        return u64_to_double(l, false, w);
+    return u64_to_double((a << (B - 9)) + (l >> 9), (l & 511u) != 0, w + 9);
+}
+
+// A lane's sum of up to 2^8 values below 2^63, and the warp's as binary64
+// (in units of 2^w; 0 when nothing was added).
+struct FixedSum {
+    uint64_t s = 0;
+    uint32_t carry = 0;
+    __device__ __forceinline__ void add(uint64_t v)
+    {
+        s += v;
+        carry += s < v ? 1u : 0u;
+    }
+    __device__ __forceinline__ double warp_sum(int w) const
+    {
+        constexpr unsigned FULL = 0xFFFFFFFFu;
+        const uint32_t t0 = __reduce_add_sync(FULL, (uint32_t)s & 0x7FFFFFu);
+        const uint32_t t1 = __reduce_add_sync(FULL, (uint32_t)(s >> 23) & 0x7FFFFFu);
+        const uint32_t t2 = __reduce_add_sync(FULL, (uint32_t)(s >> 46) | (carry << 18));
+        if ((t0 | t1 | t2) == 0u)
+            return 0.0;
+        return fixed_to_double<46>(t2, ((uint64_t)t1 << 23) + t0, w);
+    }
+};
+
+// xi v: floor(log2 xi) + floor(log2 v) with v's biased exponent, and the
+// product (its top 62 or 63 bits) in units of 2^(emax - 61 - 1023).
+__device__ __forceinline__ uint32_t xiv_exponent(uint64_t x, double v)
+{
+    return (63u - (uint32_t)__clzll((long long)x)) + (((uint32_t)__double2hiint(v) >> 20) & 0x7FFu);
+}
+
+__device__ __forceinline__ uint64_t xiv_fixed(uint64_t x, double v, uint32_t emax)
+{
+    const uint32_t lz = (uint32_t)__clzll((long long)x);
+    const uint64_t bits = (uint64_t)__double_as_longlong(v);
+    const uint64_t h = __umul64hi(x << lz, (bits << 11) | (1ull << 63)); // in [2^62, 2^64)
+    const uint32_t d = emax - ((63u - lz) + ((uint32_t)(bits >> 52) & 0x7FFu)) + 1u;
+    return d < 64u ? h >> d : 0ull;
+}
+
 __device__ __forceinline__ bool key_less(uint64_t ka, uint32_t ra, uint64_t kb, uint32_t rb)
 {
     return (ka < kb) | ((ka == kb) & (ra < rb));
@@ -1431,8 +1498,8 @@ __global__ void advance_steps_kernel(InstDev *const *insts, int32_t n_inst, int6
 
 // ------------------------------------------------------------ diagnostics
 // Conservation sums of the SDs inside the domain (slots [0, n_in)): live
-// count, sum of xi (128-bit, exact) and sum of xi v (binary64).  Each thread
-// adds its slot pairs in index order, then warps and blocks combine in a fixed
+// count, sum of xi (128-bit, exact) and sum of xi v: in fixed point over a
+// warp's 256 slots, in binary64 over its rounds, then warps and blocks in a fixed
 // tree, so that a given grid gives the same bits every time.
 struct DiagPart {
     unsigned long long live, xi_lo, xi_hi;
@@ -1440,7 +1507,7 @@ struct DiagPart {
 };
 constexpr int kDiagNT = 256;
 constexpr int kDiagBlocks = 152 * 4;
-constexpr int kDiagU = 4; // slot pairs per thread and round, all loaded first
+constexpr int kDiagChunk = 256; // slots per warp and round
 
 __device__ __forceinline__ void add128(unsigned long long &lo, unsigned long long &hi, unsigned long long blo,
                                        unsigned long long bhi)
@@ -1489,32 +1556,44 @@ __device__ __forceinline__ DiagPart diag_block_reduce(DiagPart a)
 __global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(const InstDev *__restrict__ P, int64_t n_in,
                                                                DiagPart *__restrict__ parts)
 {
+    constexpr int Q = kDiagChunk / 64; // slot pairs per lane and round
+    const int lane = threadIdx.x & 31;
     DiagPart a{0ull, 0ull, 0ull, 0.0};
-    const longlong2 *__restrict__ gxi = reinterpret_cast<const longlong2 *>(P->xi);
-    const double2 *__restrict__ gv = reinterpret_cast<const double2 *>(P->v);
-    const int64_t stride = (int64_t)gridDim.x * kDiagNT, np = n_in / 2; // every group has an even number of slots
-    auto add = [&](int64_t x, double v) {
-        if (x > 0) {
-            a.live += 1ull;
-            add128(a.xi_lo, a.xi_hi, (unsigned long long)x, 0ull);
-            a.xv = __fma_rn(xi2d(x), v, a.xv);
-        }
-    };
-    for (int64_t q0 = (int64_t)blockIdx.x * kDiagNT + threadIdx.x; q0 < np; q0 += kDiagU * stride) {
-        longlong2 x[kDiagU];
-        double2 v[kDiagU];
+    double xv = 0.0;
+    const int64_t gw = ((int64_t)blockIdx.x * kDiagNT + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * kDiagNT) >> 5;
+    for (int64_t at = gw * kDiagChunk; at < n_in; at += nw * kDiagChunk) {
+        const int n = (int)min((int64_t)kDiagChunk, n_in - at); // even: every group has an even number of slots
+        const longlong2 *gx = reinterpret_cast<const longlong2 *>(P->xi + at);
+        const double2 *gv = reinterpret_cast<const double2 *>(P->v + at);
+        longlong2 xx[Q];
+        double2 vv[Q];
 #pragma unroll
-        for (int u = 0; u < kDiagU; ++u) {
-            const int64_t q = q0 + u * stride;
-            x[u] = q < np ? gxi[q] : make_longlong2(0, 0);
-            v[u] = q < np ? gv[q] : make_double2(0.0, 0.0);
+        for (int i = 0; i < Q; ++i) { // every load first
+            const bool in = 2 * (lane + 32 * i) < n;
+            xx[i] = in ? gx[lane + 32 * i] : make_longlong2(0, 0);
+            vv[i] = in ? gv[lane + 32 * i] : make_double2(1.0, 1.0);
         }
+        uint32_t e = 0u;
 #pragma unroll
-        for (int u = 0; u < kDiagU; ++u) {
-            add(x[u].x, v[u].x);
-            add(x[u].y, v[u].y);
+        for (int i = 0; i < 2 * Q; ++i) {
+            const int64_t x = (i & 1) ? xx[i / 2].y : xx[i / 2].x;
+            if (x > 0) {
+                a.live += 1ull;
+                add128(a.xi_lo, a.xi_hi, (unsigned long long)x, 0ull);
+                e = max(e, xiv_exponent((uint64_t)x, (i & 1) ? vv[i / 2].y : vv[i / 2].x));
+            }
         }
+        e = __reduce_max_sync(0xFFFFFFFFu, e);
+        FixedSum f;
+#pragma unroll
+        for (int i = 0; i < 2 * Q; ++i) {
+            const int64_t x = (i & 1) ? xx[i / 2].y : xx[i / 2].x;
+            if (x > 0)
+                f.add(xiv_fixed((uint64_t)x, (i & 1) ? vv[i / 2].y : vv[i / 2].x, e));
+        }
+        xv = __dadd_rn(xv, f.warp_sum((int)e - 61 - 1023));
     }
+    a.xv = lane == 0 ? xv : 0.0;
     a = diag_block_reduce(a);
     if (threadIdx.x == 0)
         parts[blockIdx.x] = a;
@@ -1644,6 +1723,9 @@ constexpr int kSpecChunk = 256; // slots per warp and round (8 per lane)
 constexpr int kSpecTabMax = 512;
 constexpr int kSpecWarps = 4;   // warps per block
 constexpr uint32_t kSpecLimb = (1u << 21) - 1u;
+// Lanes of one bin meet on its limbs' addresses: four copies, by lane, each
+// eight banks further, share them out.
+constexpr int kSpecRep = 4;
 
 // Edges as the kernels use them, made on the host per call and passed by
 // value.  key[i]: high words of volumes certainly below (.x) and certainly
@@ -1652,7 +1734,9 @@ constexpr uint32_t kSpecLimb = (1u << 21) - 1u;
 // is base + k (0: below all of the table; -1 as 255).
 struct SpecTab {
     double edge[kSpecMaxBins + 1];
-    double den[kSpecMaxBins]; // volume of air x width of the bin in ln r
+    double den[kSpecMaxBins];      // volume of air x width of the bin in ln r
+    uint64_t recip[kSpecMaxBins];  // 1 / den = recip 2^recip_w, recip's top bit set
+    int32_t recip_w[kSpecMaxBins];
     uint2 key[kSpecMaxBins + 2];
     int32_t n_edges, shift, base, nt;
     uint8_t start[kSpecTabMax];
@@ -1661,10 +1745,20 @@ struct SpecTab {
 struct SpecSmem {
     uint2 key[kSpecMaxBins + 2];
     uint8_t start[kSpecTabMax];
-    uint32_t acc[kSpecWarps][3][kSpecMaxBins];
+    uint32_t acc[kSpecWarps][kSpecRep][3][kSpecMaxBins];
     uint32_t emax[kSpecWarps][kSpecMaxBins];
     double part[kSpecWarps][kSpecMaxBins];
 };
+
+__device__ __forceinline__ void spec_clear(SpecSmem &S, int warp, int lane)
+{
+#pragma unroll
+    for (int r = 0; r < kSpecRep; ++r)
+#pragma unroll
+        for (int l = 0; l < 3; ++l)
+            S.acc[warp][r][l][lane] = 0u;
+    S.emax[warp][lane] = 0u;
+}
 
 __device__ __forceinline__ void spec_smem_init(SpecSmem &S, const SpecTab &T)
 {
@@ -1673,10 +1767,7 @@ __device__ __forceinline__ void spec_smem_init(SpecSmem &S, const SpecTab &T)
     for (int i = threadIdx.x; i < T.nt; i += blockDim.x)
         S.start[i] = T.start[i];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int l = 0; l < 3; ++l)
-        S.acc[warp][l][lane] = 0u;
-    S.emax[warp][lane] = 0u;
+    spec_clear(S, warp, lane);
     __syncthreads();
 }
 
@@ -1739,9 +1830,9 @@ __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, cons
             const int b = spec_bin(S, T, v[i]);
             if ((unsigned)b < (unsigned)nb) {
                 bin[i] = b;
-                const uint32_t e = (63u - (uint32_t)__clzll((long long)x[i])) +
-                                   (((uint32_t)__double2hiint(v[i]) >> 20) & 0x7FFu);
-                atomicMax(&S.emax[warp][b], e);
+                const uint32_t e = xiv_exponent(x[i], v[i]);
+                if (e > S.emax[warp][b]) // most are not, once one round of lanes is in
+                    atomicMax(&S.emax[warp][b], e);
             }
         }
     }
@@ -1750,34 +1841,41 @@ __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, cons
     for (int i = 0; i < 2 * Q; ++i) {
         if (bin[i] < 0)
             continue;
-        const uint32_t lz = (uint32_t)__clzll((long long)x[i]);
-        const uint64_t bits = (uint64_t)__double_as_longlong(v[i]);
-        const uint32_t e = (63u - lz) + ((uint32_t)(bits >> 52) & 0x7FFu);
-        const uint64_t m = (bits << 11) | (1ull << 63); // the mantissa, leading one at bit 63
-        const uint64_t h = __umul64hi(x[i] << lz, m);   // in [2^62, 2^64): xi v = h 2^(e - 62)
-        const uint32_t d = S.emax[warp][bin[i]] - e + 1u;
-        const uint64_t val = d < 64u ? h >> d : 0ull;
-        atomicAdd(&S.acc[warp][0][bin[i]], (uint32_t)val & kSpecLimb);
-        atomicAdd(&S.acc[warp][1][bin[i]], (uint32_t)(val >> 21) & kSpecLimb);
-        atomicAdd(&S.acc[warp][2][bin[i]], (uint32_t)(val >> 42));
+        const uint64_t val = xiv_fixed(x[i], v[i], S.emax[warp][bin[i]]);
+        uint32_t(*acc)[kSpecMaxBins] = S.acc[warp][lane % kSpecRep];
+        const int at = (bin[i] + 8 * (lane % kSpecRep)) & 31;
+        atomicAdd(&acc[0][at], (uint32_t)val & kSpecLimb);
+        atomicAdd(&acc[1][at], (uint32_t)(val >> 21) & kSpecLimb);
+        atomicAdd(&acc[2][at], (uint32_t)(val >> 42));
     }
     __syncwarp();
     const uint32_t e = S.emax[warp][lane];
-    const uint32_t a0 = S.acc[warp][0][lane], a1 = S.acc[warp][1][lane], a2 = S.acc[warp][2][lane];
-    S.emax[warp][lane] = 0u;
+    uint32_t a0 = 0, a1 = 0, a2 = 0;
 #pragma unroll
-    for (int l = 0; l < 3; ++l)
-        S.acc[warp][l][lane] = 0u;
+    for (int r = 0; r < kSpecRep; ++r) {
+        const int at = (lane + 8 * r) & 31;
+        a0 += S.acc[warp][r][0][at];
+        a1 += S.acc[warp][r][1][at];
+        a2 += S.acc[warp][r][2][at];
+    }
+    __syncwarp();
+    spec_clear(S, warp, lane);
     __syncwarp();
     if (e == 0u)
         return 0.0;
-    // a2 2^42 and a1 2^21 + a0 as binary64, exactly (below 2^52: placed under
-    // the leading one of 2^94 and 2^52), then one rounding
-    const uint64_t low = ((uint64_t)a1 << 21) + a0;
-    const double hi = __dsub_rn(__hiloint2double(0x43300000 + (42 << 20), (int)a2), 0x1p94);
-    const double lo = __dsub_rn(__longlong_as_double((long long)(0x4330000000000000ull | low)), 0x1p52);
-    const uint32_t sc = min(max((int)e - 61, 1), 2046); // 2^(e_max - 61), biased exponent
-    return __dmul_rn(__dadd_rn(hi, lo), __hiloint2double((int)(sc << 20), 0));
+    return fixed_to_double<42>(a2, ((uint64_t)a1 << 21) + a0, (int)e - 61 - 1023);
+}
+
+// x / den by the 64-bit reciprocal (x >= 0): within 0.5 + 2^-9 ulp, where the
+// binary64 division would cost as much as everything else of a small cell.
+__device__ __forceinline__ double spec_divide(const SpecTab &T, int b, double x)
+{
+    const uint64_t bits = (uint64_t)__double_as_longlong(x);
+    const int e = (int)(bits >> 52);
+    const int w = e - 1075 + T.recip_w[b] + 53;
+    if (e == 0 || (unsigned)(w + 64 + 1000) > 2000u) // zero, or a result near the ends of the range
+        return x == 0.0 ? 0.0 : x / T.den[b];
+    return u64_to_double(__umul64hi((bits << 11) | (1ull << 63), T.recip[b]), true, w);
 }
 
 // Sums of every bin over all slots [0, n_slots) (padding and dead SDs hold
@@ -1845,7 +1943,6 @@ __global__ void __launch_bounds__(32 * kSpecWarps) spectrum_cells_kernel(const I
     const int32_t *__restrict__ off = P->cell_off;
     const int unit = block_cells ? (int)blockIdx.x : (int)blockIdx.x * kSpecWarps + warp;
     const int units = block_cells ? (int)gridDim.x : (int)gridDim.x * kSpecWarps;
-    const double den = T.den[lane < nb ? lane : 0];
     for (int c = unit; c < n_cells; c += units) {
         const int32_t lo = off[c], hi = off[c + 1];
         double acc = 0.0;
@@ -1862,9 +1959,8 @@ __global__ void __launch_bounds__(32 * kSpecWarps) spectrum_cells_kernel(const I
             if (warp != 0)
                 continue;
         }
-        // most bins of a small cell are empty: only the others divide
         if (lane < nb)
-            out[(int64_t)c * nb + lane] = acc != 0.0 ? acc / den : 0.0;
+            out[(int64_t)c * nb + lane] = spec_divide(T, lane, acc);
     }
 }
 

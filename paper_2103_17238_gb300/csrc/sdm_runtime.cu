@@ -1340,6 +1340,10 @@ sdm_status batch_step(sdm_batch *b, int32_t n_steps)
     return SDM_OK;
 }
 
+// Blocks of 256 threads for n items, a thread each, at most eight per SM (the
+// kernel's loop takes the rest).
+int grid_of(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>(1216, (n + 255) / 256)); }
+
 bool finite_pos(double x) { return std::isfinite(x) && x > 0.0; }
 
 sdm_status check_config(const sdm_config *cfg, std::string *err)
@@ -1409,8 +1413,14 @@ SpecTab spec_table(const double *e, int32_t n_edges, double vol)
         T.key[i] = make_uint2(lo, std::isfinite(v) ? high_word(v * (1.0 + 0x1p-17)) + 1u : 0xFFFFFFFFu);
     }
     T.key[n_edges] = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
-    for (int32_t b = 0; b + 1 < n_edges; ++b)
-        T.den[b] = vol * (std::log(e[b + 1]) - std::log(e[b]));
+    for (int32_t b = 0; b + 1 < n_edges; ++b) {
+        const double dln = std::log(e[b + 1]) - std::log(e[b]);
+        T.den[b] = vol * dln;
+        int w = 0;
+        const long double r = std::frexp(1.0L / ((long double)vol * (long double)dln), &w); // in [1/2, 1)
+        T.recip[b] = (uint64_t)std::ldexp(r, 64);
+        T.recip_w[b] = w - 64;
+    }
     // entry 0 below the first edge, the last one above the last edge
     T.shift = 15;
     const uint32_t k0 = T.key[0].x, k1 = std::min(T.key[n_edges - 1].y, 0x7FF00000u);
@@ -1659,7 +1669,8 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
         if (!on_device)
             CTX_CUDA(ctx, cudaStreamWaitEvent(s, ctx->in_ev[k], 0));
         if (piece[k + 1] > piece[k])
-            validate_count_kernel<<<1216, 256, 0, s>>>(piece[k], piece[k + 1], dxi, dv, dcell, n_cells, d_counts,
+            validate_count_kernel<<<grid_of((piece[k + 1] - piece[k] + 3) / 4), 256, 0, s>>>(
+                piece[k], piece[k + 1], dxi, dv, dcell, n_cells, d_counts,
                                                         d_flags, d_bad);
     }
     // one copy of the whole block (counts, flags, first bad index)
@@ -1738,12 +1749,12 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
         vals[res] = (uint32_t *)(w + b_key);
         keys[res ^ 1] = (uint32_t *)ctx->d_xi;
         vals[res ^ 1] = keys[res ^ 1] + n_sd;
-        group_keys_kernel<<<1216, 256, 0, s>>>(n_sd, dcell, n_cells, keys[0]);
+        group_keys_kernel<<<grid_of(n_sd), 256, 0, s>>>(n_sd, dcell, n_cells, keys[0]);
         const int cur = radix_sort(keys, vals, true, n_sd, bits, (uint32_t *)(w + 2 * b_key), s);
-        place_sorted_kernel<<<1216, 256, 0, s>>>(n_sd, keys[cur], vals[cur], dxi, dv, d_poff, d_uoff, ctx->d_xi,
+        place_sorted_kernel<<<grid_of(n_sd), 256, 0, s>>>(n_sd, keys[cur], vals[cur], dxi, dv, d_poff, d_uoff, ctx->d_xi,
                                                  ctx->d_v, ctx->d_id_of_slot);
     } else {
-        scatter_kernel<<<1216, 256, 0, s>>>(n_sd, dxi, dv, dcell, n_cells, d_poff, d_uoff, ctx->d_xi, ctx->d_v,
+        scatter_kernel<<<grid_of(n_sd), 256, 0, s>>>(n_sd, dxi, dv, dcell, n_cells, d_poff, d_uoff, ctx->d_xi, ctx->d_v,
                                             ctx->d_id_of_slot);
     }
     // after the sort, whose other pair of arrays lies over the padding too
@@ -1903,7 +1914,7 @@ sdm_status sdm_get_attributes(sdm_ctx *ctx, int64_t *xi, double *volume, int on_
     cudaStream_t s = ctx->stream;
     const int64_t n = ctx->n_sd;
     if (on_device) {
-        gather_kernel<<<1216, 256, 0, s>>>(ctx->n_slots, ctx->d_xi, ctx->d_v, ctx->d_id_of_slot, xi, volume);
+        gather_kernel<<<grid_of(ctx->n_slots), 256, 0, s>>>(ctx->n_slots, ctx->d_xi, ctx->d_v, ctx->d_id_of_slot, xi, volume);
         CTX_CUDA(ctx, cudaGetLastError());
         return SDM_OK;
     }
@@ -1911,7 +1922,7 @@ sdm_status sdm_get_attributes(sdm_ctx *ctx, int64_t *xi, double *volume, int on_
     char *tmp = (char *)ctx->mem.get(bx + bv);
     if (!tmp)
         return fail(&ctx->error, SDM_ENOMEM, "allocation failed");
-    gather_kernel<<<1216, 256, 0, s>>>(ctx->n_slots, ctx->d_xi, ctx->d_v, ctx->d_id_of_slot,
+    gather_kernel<<<grid_of(ctx->n_slots), 256, 0, s>>>(ctx->n_slots, ctx->d_xi, ctx->d_v, ctx->d_id_of_slot,
                                        xi ? (int64_t *)tmp : nullptr, volume ? (double *)(tmp + bx) : nullptr);
     CTX_CUDA(ctx, cudaGetLastError());
     if (xi)
@@ -2066,7 +2077,7 @@ sdm_status sdm_diagnostics(sdm_ctx *ctx, sdm_diag *out)
         return fail(&ctx->error, SDM_ESTATE, "no attributes set");
     const int64_t n_in = ctx->h_cell_off[ctx->cfg.n_cells]; // slots of the cells (not the SDs outside)
     // the grid depends on the size only: the same state gives the same bits
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(kDiagBlocks, (n_in + 2 * kDiagU * kDiagNT - 1) / (2 * kDiagU * kDiagNT)));
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(kDiagBlocks, (n_in + kDiagChunk * (kDiagNT / 32) - 1) / (kDiagChunk * (kDiagNT / 32))));
     const size_t bytes = sizeof(DiagPart) * ((size_t)blocks + 1);
     DiagPart *d = (DiagPart *)ctx->mem.get(bytes);
     if (!d)
