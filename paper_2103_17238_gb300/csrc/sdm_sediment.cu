@@ -8,7 +8,26 @@
 // and the distance widened exactly to binary64; positions are heights above
 // the bottom of the SD's cell, so a step needs no division.
 //
-// One step on the device:
+// One step on the device, for layouts whose largest cell holds up to 1024
+// slots.  Most SDs stay in their cell (over 95% per second on a cloud's
+// grid), both layouts keep a cell's SDs in increasing id, and a cell receives
+// from few others: so nothing is sorted as a whole.
+//   sed_fall_kernel      one warp per cell: the fall; per slot its new height
+//                        (negative: leaves the cell), the movers of the cell
+//                        (new group, id, slot, place among the group's
+//                        arrivals), the water that leaves through the bottom;
+//   sed_offsets_kernel   the new cells' offsets (even) and their arrivals', the
+//                        precipitated total in a fixed order;
+//   sed_deal_kernel      the movers to their group's arrivals;
+//   sed_merge_kernel     one warp per new cell: its arrivals sorted by id, its
+//                        stayers streamed through, each moved up by the
+//                        arrivals of lower id; the new layout with its padding.
+// 112 B per SD (xi, v, heights; heights out; the layout in and out).  The
+// refresh of the context's own launch plan and the read-back run on a side
+// stream beside the last two; the host waits for the read-back only.
+// Measured on the 4.19M-SD grid: SED_FIGURES
+//
+// With larger cells (a warp would take too long), a stable sort of all SDs:
 //   sed_move_kernel      per slot (four per thread): the fall, the new group
 //                        of every SD (the cells, then n_cells for outside the
 //                        domain) as a key in SD-id order, counts per new
@@ -20,8 +39,6 @@
 //                        a ranked scatter;
 //   sed_gather_kernel    the new layout, gathered from the old one;
 //   sed_pad_kernel       its padding slots.
-// The scan, the padding, the refresh of the context's own launch plan and
-// the read-back run on a side stream beside the radix sort.
 // The two layouts swap; the host reads the new offsets for the launch plan.
 //
 // Compiled as part of the library's single translation unit (included at the
@@ -35,12 +52,15 @@ constexpr int kSedNT = 256;
 // zeta of every slot from z (SD-id order): z - (level) dz with level =
 // (cbase + c) / nx, which must lie in [0, dz) (zeta_in: z already holds
 // zeta); flags bit 0 and the first bad id on failure.  SDs outside the
-// domain and padding slots get zeta 0.  group[slot] = the slot's group.
+// domain and padding slots get zeta 0.  A warp takes 128 slots of a group at a
+// time, the ids and then the heights of all in flight together (43 us for
+// 4.19M SDs one by one).
+constexpr int kSedRun = 4; // times 32 slots per warp and round
+
 __global__ void __launch_bounds__(kSedNT) sed_set_kernel(const int32_t *__restrict__ cell_off, int32_t n_cells,
                                                          int64_t n_slots, const int32_t *__restrict__ id_of_slot,
                                                          const double *__restrict__ z, int32_t nx, double dz,
-                                                         int32_t cbase, int zeta_in,
-                                                         double *__restrict__ zeta, int32_t *__restrict__ group,
+                                                         int32_t cbase, int zeta_in, double *__restrict__ zeta,
                                                          uint32_t *__restrict__ flags,
                                                          unsigned long long *__restrict__ bad)
 {
@@ -49,21 +69,46 @@ __global__ void __launch_bounds__(kSedNT) sed_set_kernel(const int32_t *__restri
     for (int g = gw; g <= n_cells; g += nw) {
         const int64_t lo = cell_off[g], hi = g < n_cells ? cell_off[g + 1] : n_slots;
         const double base = zeta_in ? 0.0 : __dmul_rn((double)((g + cbase) / nx), dz);
-        for (int64_t s = lo + lane; s < hi; s += 32) {
-            const int32_t id = id_of_slot[s];
-            double zt = 0.0;
-            if (id >= 0 && g < n_cells) {
-                // + 0 turns a -0 height into +0 (the fall tests signs bitwise)
-                zt = __dadd_rn(__dsub_rn(z[id], base), 0.0);
-                if (!(zt >= 0.0 && zt < dz)) {
-                    atomicOr(flags, 1u);
-                    atomicMin(bad, (unsigned long long)id);
-                    zt = 0.0;
+        for (int64_t s0 = lo; s0 < hi; s0 += 32 * kSedRun) {
+            int32_t id[kSedRun];
+            double zz[kSedRun];
+#pragma unroll
+            for (int u = 0; u < kSedRun; ++u)
+                id[u] = s0 + 32 * u + lane < hi ? id_of_slot[s0 + 32 * u + lane] : -1;
+#pragma unroll
+            for (int u = 0; u < kSedRun; ++u)
+                zz[u] = id[u] >= 0 && g < n_cells ? z[id[u]] : 0.0;
+#pragma unroll
+            for (int u = 0; u < kSedRun; ++u) {
+                const int64_t s = s0 + 32 * u + lane;
+                if (s >= hi)
+                    break;
+                double zt = 0.0;
+                if (id[u] >= 0 && g < n_cells) {
+                    // + 0 turns a -0 height into +0 (the fall tests signs bitwise)
+                    zt = __dadd_rn(__dsub_rn(zz[u], base), 0.0);
+                    if (!(zt >= 0.0 && zt < dz)) {
+                        atomicOr(flags, 1u);
+                        atomicMin(bad, (unsigned long long)id[u]);
+                        zt = 0.0;
+                    }
                 }
+                zeta[s] = zt;
             }
-            zeta[s] = zt;
-            group[s] = g;
         }
+    }
+}
+
+// group[slot] = the slot's group, for the sorted path.
+__global__ void __launch_bounds__(kSedNT) sed_group_kernel(const int32_t *__restrict__ cell_off, int32_t n_cells,
+                                                           int64_t n_slots, int32_t *__restrict__ group)
+{
+    const int lane = threadIdx.x & 31;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int g = gw; g <= n_cells; g += nw) {
+        const int64_t lo = cell_off[g], hi = g < n_cells ? cell_off[g + 1] : n_slots;
+        for (int64_t s = lo + lane; s < hi; s += 32)
+            group[s] = g;
     }
 }
 
@@ -81,21 +126,32 @@ __global__ void __launch_bounds__(kSedNT) sed_get_kernel(const int32_t *__restri
 {
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    const bool heights = z || zeta_out;
     for (int g = gw; g <= n_cells; g += nw) {
         const int64_t lo = cell_off[g], hi = g < n_cells ? cell_off[g + 1] : n_slots;
         const double base = g < n_cells && z ? __dmul_rn((double)((g + cbase) / nx), dz) : 0.0;
-        for (int64_t s = lo + lane; s < hi; s += 32) {
-            const int32_t id = id_of_slot[s];
-            if (id < 0)
-                continue;
-            if (z)
-                z[id] = g < n_cells ? __dadd_rn(base, zeta[s]) : 0.0;
-            if (cell)
-                cell[id] = g < n_cells ? g : -1;
-            if (zeta_out)
-                zeta_out[id] = zeta[s];
-            if (gcell)
-                gcell[id] = g < n_cells ? g + cbase : (emig ? emig[id] : -1);
+        for (int64_t s0 = lo; s0 < hi; s0 += 32 * kSedRun) {
+            int32_t id[kSedRun];
+            double zt[kSedRun];
+#pragma unroll
+            for (int u = 0; u < kSedRun; ++u) { // every load first
+                const int64_t s = s0 + 32 * u + lane;
+                id[u] = s < hi ? id_of_slot[s] : -1;
+                zt[u] = s < hi && heights ? zeta[s] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kSedRun; ++u) {
+                if (id[u] < 0)
+                    continue;
+                if (z)
+                    z[id[u]] = g < n_cells ? __dadd_rn(base, zt[u]) : 0.0;
+                if (cell)
+                    cell[id[u]] = g < n_cells ? g : -1;
+                if (zeta_out)
+                    zeta_out[id[u]] = zt[u];
+                if (gcell)
+                    gcell[id[u]] = g < n_cells ? g + cbase : (emig ? emig[id[u]] : -1);
+            }
         }
     }
 }
@@ -135,6 +191,54 @@ __device__ __forceinline__ bool dge_pos(double x, double y)
     return __double_as_longlong(x) >= __double_as_longlong(y);
 }
 
+// The fall of one live SD of cell g: its new cell c (negative, or another
+// piece's when c + cbase < 0 ends the fall: out of the grid) and height.
+struct Fall {
+    int32_t c;
+    double z;
+};
+
+__device__ __forceinline__ Fall sed_fall(const PairConsts &C, double v, double zt, float dt32, int32_t g, int32_t nx,
+                                         double dz, int32_t cbase)
+{
+    bool in_range;
+    const float vf = d2f_rn(v, in_range);
+    const double d = f2d_exact(__fmul_rn(vt32c(C, radius32(vf)), dt32));
+    double zz = __dsub_rn(zt, d);
+    // crossing k levels takes cell c to c - k nx; below the grid's level 0
+    // exactly when cbase + c is negative (0 <= column < nx)
+    int32_t c = g;
+    while (dneg(zz)) { // at most as many levels as the SD falls through
+        c -= nx;
+        if (c + cbase < 0)
+            return Fall{c, 0.0};
+        zz = __dadd_rn(zz, dz);
+    }
+    if (dge_pos(zz, dz)) { // zeta + dz rounded up to dz: on the boundary, level above
+        c += nx;
+        zz = 0.0;
+    }
+    return Fall{c, zz};
+}
+
+// precip_part[block] = the block's sum of pr (lanes, then warps, in a fixed tree).
+__device__ __forceinline__ void sed_precip(double pr, double *precip_part)
+{
+    __shared__ double s_pr[kSedNT / 32];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1)
+        pr = __dadd_rn(pr, __shfl_down_sync(0xFFFFFFFFu, pr, d));
+    if ((threadIdx.x & 31) == 0)
+        s_pr[threadIdx.x >> 5] = pr;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < kSedNT / 32; ++w)
+            t = __dadd_rn(t, s_pr[w]);
+        precip_part[blockIdx.x] = t;
+    }
+}
+
 __global__ void __launch_bounds__(kSedNT) sed_move_kernel(const InstDev *__restrict__ P, int32_t n_cells, int64_t n_slots,
                                                           int32_t nx, double dz, float dt32,
                                                           const double *__restrict__ zeta,
@@ -146,7 +250,6 @@ __global__ void __launch_bounds__(kSedNT) sed_move_kernel(const InstDev *__restr
                                                           int32_t *__restrict__ emig)
 {
     constexpr unsigned FULL = 0xFFFFFFFFu;
-    __shared__ double s_pr[kSedNT / 32];
     const PairConsts C = pair_consts(P);
     const int lane = threadIdx.x & 31;
     const int64_t *__restrict__ gxi = P->xi;
@@ -177,32 +280,15 @@ __global__ void __launch_bounds__(kSedNT) sed_move_kernel(const InstDev *__restr
                 int32_t em = -1;
                 ng = n_cells;
                 if (g[u] < n_cells && x[u] > 0) {
-                    bool in_range;
-                    const float vf = d2f_rn(vv[u], in_range);
-                    const double d = f2d_exact(__fmul_rn(vt32c(C, radius32(vf)), dt32));
-                    double zz = __dsub_rn(zt[u], d);
-                    // crossing k levels takes cell c to c - k nx; below the
-                    // grid's level 0 exactly when cbase + c is negative
-                    // (0 <= column < nx)
-                    int32_t c = g[u];
-                    while (dneg(zz)) { // at most as many levels as the SD falls through
-                        c -= nx;
-                        if (c + cbase < 0)
-                            break;
-                        zz = __dadd_rn(zz, dz);
-                    }
-                    if (c + cbase < 0) {
+                    const Fall f = sed_fall(C, vv[u], zt[u], dt32, g[u], nx, dz, cbase);
+                    if (f.c + cbase < 0) {
                         pr = __dadd_rn(pr, __dmul_rn(xi2d(x[u]), vv[u]));
                     } else {
-                        if (dge_pos(zz, dz)) { // zeta + dz rounded up to dz: on the boundary, level above
-                            c += nx;
-                            zz = 0.0;
-                        }
-                        zn = zz;
-                        if (c >= 0)
-                            ng = c;
+                        zn = f.z;
+                        if (f.c >= 0)
+                            ng = f.c;
                         else // into another piece of the grid
-                            em = c + cbase;
+                            em = f.c + cbase;
                     }
                 }
                 key[id[u]] = (uint32_t)ng;
@@ -220,17 +306,42 @@ __global__ void __launch_bounds__(kSedNT) sed_move_kernel(const InstDev *__restr
             }
         }
     }
+    sed_precip(pr, precip_part);
+}
+
+// *precip_total = the sum of precip[0 .. n_parts), by one block of 1024:
+// thread t sums parts t, t + 1024, ... in order, then a fixed tree over the
+// threads (the loads of four parts in flight at once, the sums in the same
+// order).
+__device__ __forceinline__ void sed_precip_total(const double *__restrict__ precip, int32_t n_parts,
+                                                 double *__restrict__ precip_total)
+{
+    __shared__ double s_pr[32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    double pr = 0.0;
+    for (int i0 = t; i0 < n_parts; i0 += 4 * 1024) {
+        double q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            q[u] = i0 + u * 1024 < n_parts ? precip[i0 + u * 1024] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i0 + u * 1024 < n_parts)
+                pr = __dadd_rn(pr, q[u]);
+    }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1)
-        pr = __dadd_rn(pr, __shfl_down_sync(FULL, pr, d));
+        pr = __dadd_rn(pr, __shfl_down_sync(0xFFFFFFFFu, pr, d));
     if (lane == 0)
-        s_pr[threadIdx.x >> 5] = pr;
+        s_pr[warp] = pr;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kSedNT / 32; ++w)
-            t = __dadd_rn(t, s_pr[w]);
-        precip_part[blockIdx.x] = t;
+    if (warp == 0) {
+        pr = s_pr[lane];
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1)
+            pr = __dadd_rn(pr, __shfl_down_sync(0xFFFFFFFFu, pr, d));
+        if (lane == 0)
+            *precip_total = pr;
     }
 }
 
@@ -247,7 +358,6 @@ __global__ void __launch_bounds__(1024) sed_scan_kernel(const uint32_t *__restri
     constexpr int E = 8, TILE = 1024 * E;
     __shared__ uint32_t s_c[TILE];
     __shared__ unsigned long long s_w[32];
-    __shared__ double s_pr[32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     unsigned long long carry = 0;
     for (int32_t g0 = 0; g0 < n_groups; g0 += TILE) {
@@ -318,34 +428,7 @@ __global__ void __launch_bounds__(1024) sed_scan_kernel(const uint32_t *__restri
         ustart[n_groups] = (int32_t)(uint32_t)carry;
         poff[n_groups] = (int32_t)(uint32_t)(carry >> 32);
     }
-    // the precipitated water: thread t sums parts t, t + 1024, ... in order,
-    // then a fixed tree over the threads (the loads of four parts in flight
-    // at once, the sums in the same order)
-    double pr = 0.0;
-    for (int i0 = t; i0 < n_parts; i0 += 4 * 1024) {
-        double q[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            q[u] = i0 + u * 1024 < n_parts ? precip[i0 + u * 1024] : 0.0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (i0 + u * 1024 < n_parts)
-                pr = __dadd_rn(pr, q[u]);
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1)
-        pr = __dadd_rn(pr, __shfl_down_sync(0xFFFFFFFFu, pr, d));
-    if (lane == 0)
-        s_pr[warp] = pr;
-    __syncthreads();
-    if (warp == 0) {
-        pr = s_pr[lane];
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1)
-            pr = __dadd_rn(pr, __shfl_down_sync(0xFFFFFFFFu, pr, d));
-        if (lane == 0)
-            *precip_total = pr;
-    }
+    sed_precip_total(precip, n_parts, precip_total);
 }
 
 // The new layout: the j-th SD in (group, id) order goes to slot
@@ -387,17 +470,378 @@ __global__ void sed_pad_kernel(int32_t n_groups, const int32_t *__restrict__ ust
 // -------------------------------------------------------------------- host
 // The second layout (swapped with the context's after every step, so both
 // sets are freed through their current pointers) and the scratch.
+// ------------------------------------------------- cells of up to kSedByCell
+constexpr int kSedByCell = 1024;  // slots of the largest cell that a warp takes
+constexpr int kSedArrive = 512;   // arrivals of a cell sorted in shared memory
+constexpr int kSedMergeNT = 128;
+
+// What the movers of the cells and the arrivals of the groups are kept in.
+// Cell c's movers take places [cell_off[c], + left[c]) of the mover arrays;
+// group g's arrivals [first[g], + arr[g]) of the arrival arrays.
+struct SedMoves {
+    uint32_t *group, *id, *slot, *place; // per mover: new group, id, slot, place among the group's arrivals
+    uint32_t *a_id, *a_slot;             // per arrival
+    uint32_t *stay, *arr, *left;         // per group: SDs that stay, that arrive; per cell: movers
+    int32_t *first;                      // n_groups
+};
+
+__global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restrict__ P,
+                                                          const int32_t *__restrict__ cell_off, int32_t n_cells,
+                                                          int64_t n_slots, int32_t nx, double dz, float dt32,
+                                                          const double *__restrict__ zeta,
+                                                          const int32_t *__restrict__ id_of_slot,
+                                                          double *__restrict__ zeta_new, SedMoves M,
+                                                          double *__restrict__ precip_part, int32_t cbase,
+                                                          int32_t *__restrict__ emig)
+{
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    const PairConsts C = pair_consts(P);
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int64_t *__restrict__ gxi = P->xi;
+    const double *__restrict__ gv = P->v;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    double pr = 0.0;
+    for (int g = gw; g < n_cells; g += nw) { // uniform over the warp
+        const int32_t lo = cell_off[g], hi = cell_off[g + 1];
+        uint32_t stay = 0, left = 0;
+        for (int32_t s0 = lo; s0 < hi; s0 += 32 * kSedRun) {
+            int64_t x[kSedRun];
+            double vv[kSedRun], zt[kSedRun];
+#pragma unroll
+            for (int u = 0; u < kSedRun; ++u) { // every load first
+                const int32_t sl = s0 + 32 * u + lane;
+                const bool in = sl < hi;
+                x[u] = in ? gxi[sl] : 0;
+                vv[u] = in ? gv[sl] : 1.0;
+                zt[u] = in ? zeta[sl] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kSedRun; ++u) {
+                const int32_t sl = s0 + 32 * u + lane;
+                if (s0 + 32 * u >= hi) // uniform over the warp
+                    break;
+                int32_t ng = n_cells, em = -1;
+                double zn = 0.0;
+                if (x[u] > 0) {
+                    const Fall f = sed_fall(C, vv[u], zt[u], dt32, g, nx, dz, cbase);
+                    if (f.c + cbase < 0) {
+                        pr = __dadd_rn(pr, __dmul_rn(xi2d(x[u]), vv[u]));
+                    } else {
+                        zn = f.z;
+                        if (f.c >= 0)
+                            ng = f.c;
+                        else // into another piece of the grid
+                            em = f.c + cbase;
+                    }
+                }
+                // stayers +zn, the others (padding too) with the sign bit set
+                const bool keep = ng == g;
+                stay += (uint32_t)__popc(__ballot_sync(FULL, keep));
+                int32_t id = -1;
+                if (sl < hi) {
+                    zeta_new[sl] = keep ? zn : __hiloint2double(__double2hiint(zn) | (int)0x80000000, __double2loint(zn));
+                    if (!keep)
+                        id = id_of_slot[sl];
+                }
+                const unsigned mv = __ballot_sync(FULL, id >= 0);
+                if (mv == 0u)
+                    continue;
+                const unsigned out = __ballot_sync(FULL, id >= 0 && ng == n_cells);
+                uint32_t place = 0;
+                if (out && lane == __ffs(out) - 1) // one counter for all that leave the domain
+                    place = atomicAdd(&M.arr[n_cells], (uint32_t)__popc(out));
+                place = __shfl_sync(FULL, place, out ? __ffs(out) - 1 : 0) + (uint32_t)__popc(out & lt);
+                if (id >= 0) {
+                    if (ng != n_cells)
+                        place = atomicAdd(&M.arr[ng], 1u);
+                    const uint32_t at = (uint32_t)lo + left + (uint32_t)__popc(mv & lt);
+                    M.group[at] = (uint32_t)ng;
+                    M.id[at] = (uint32_t)id;
+                    M.slot[at] = (uint32_t)sl;
+                    M.place[at] = place;
+                    if (em >= 0)
+                        emig[id] = em;
+                }
+                left += (uint32_t)__popc(mv);
+            }
+        }
+        if (lane == 0) {
+            M.stay[g] = stay;
+            M.left[g] = left;
+        }
+    }
+    if (gw == 0 && lane == 0) { // those outside stay there (their last slot may be padding)
+        const int32_t lo = cell_off[n_cells];
+        M.stay[n_cells] = (uint32_t)(n_slots - lo) - (n_slots > lo && id_of_slot[n_slots - 1] < 0 ? 1u : 0u);
+    }
+    sed_precip(pr, precip_part);
+}
+
+// Sums over the groups of a block of 1024, for sed_offsets_kernel over many.
+__device__ __forceinline__ unsigned long long sed_sizes(const SedMoves &M, int g)
+{
+    const uint32_t a = M.arr[g];
+    return (unsigned long long)((M.stay[g] + a + 1u) & ~1u) | ((unsigned long long)a << 32);
+}
+
+__device__ __forceinline__ unsigned long long sed_block_sum(unsigned long long x, unsigned long long *s_w)
+{
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1)
+        x += __shfl_down_sync(0xFFFFFFFFu, x, d);
+    if ((threadIdx.x & 31) == 0)
+        s_w[threadIdx.x >> 5] = x;
+    __syncthreads();
+    unsigned long long t = s_w[threadIdx.x & 31];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1)
+        t += __shfl_xor_sync(0xFFFFFFFFu, t, d);
+    __syncthreads();
+    return t;
+}
+
+__global__ void __launch_bounds__(1024) sed_totals_kernel(SedMoves M, int32_t n_groups,
+                                                          unsigned long long *__restrict__ totals)
+{
+    __shared__ unsigned long long s_w[32];
+    const int g = blockIdx.x * 1024 + threadIdx.x;
+    const unsigned long long t = sed_block_sum(g < n_groups ? sed_sizes(M, g) : 0ull, s_w);
+    if (threadIdx.x == 0)
+        totals[blockIdx.x] = t;
+}
+
+// poff[g] = first slot of group g (every group an even number), M.first[g] =
+// its first arrival; block 0 also sums the precipitated water.  The groups
+// before a block are summed by the block itself (up to 64 blocks: totals
+// null), or their blocks' totals.
+__global__ void __launch_bounds__(1024) sed_offsets_kernel(SedMoves M, int32_t n_groups,
+                                                           const unsigned long long *__restrict__ totals,
+                                                           int32_t *__restrict__ poff,
+                                                           const double *__restrict__ precip, int32_t n_parts,
+                                                           double *__restrict__ precip_total)
+{
+    __shared__ unsigned long long s_w[32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int g = blockIdx.x * 1024 + t;
+    unsigned long long before = 0;
+    if (totals)
+        for (int i = t; i < (int)blockIdx.x; i += 1024)
+            before += totals[i];
+    else
+        for (int i = t; i < (int)blockIdx.x * 1024; i += 4 * 1024) { // four loads in flight
+            unsigned long long q[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                q[u] = i + u * 1024 < (int)blockIdx.x * 1024 ? sed_sizes(M, i + u * 1024) : 0ull;
+            before += (q[0] + q[1]) + (q[2] + q[3]);
+        }
+    const unsigned long long mine = g < n_groups ? sed_sizes(M, g) : 0ull;
+    before = sed_block_sum(before, s_w);
+    unsigned long long x = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, d);
+        if (lane >= d)
+            x += y;
+    }
+    if (lane == 31)
+        s_w[warp] = x;
+    __syncthreads();
+    unsigned long long w = lane < warp ? s_w[lane] : 0ull;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1)
+        w += __shfl_xor_sync(0xFFFFFFFFu, w, d);
+    const unsigned long long at = before + w + x - mine;
+    if (g < n_groups) {
+        poff[g] = (int32_t)(uint32_t)at;
+        M.first[g] = (int32_t)(uint32_t)(at >> 32);
+        if (g == n_groups - 1)
+            poff[n_groups] = (int32_t)(uint32_t)(at + mine);
+    }
+    if (blockIdx.x == 0)
+        sed_precip_total(precip, n_parts, precip_total);
+}
+
+__global__ void __launch_bounds__(kSedNT) sed_deal_kernel(const int32_t *__restrict__ cell_off, int32_t n_cells,
+                                                          SedMoves M)
+{
+    const int lane = threadIdx.x & 31;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int g = gw; g < n_cells; g += nw) {
+        const uint32_t lo = (uint32_t)cell_off[g], n = M.left[g];
+        for (uint32_t i = lane; i < n; i += 32) {
+            const uint32_t at = (uint32_t)M.first[M.group[lo + i]] + M.place[lo + i];
+            M.a_id[at] = M.id[lo + i];
+            M.a_slot[at] = M.slot[lo + i];
+        }
+    }
+}
+
+// A layout's arrays.
+struct SedLayout {
+    int64_t *xi;
+    double *v, *zeta;
+    int32_t *id;
+    __device__ __forceinline__ void put(int64_t p, int64_t x, double w, double z, int32_t i) const
+    {
+        xi[p] = x;
+        v[p] = w;
+        zeta[p] = z;
+        id[p] = i;
+    }
+};
+
+__global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *__restrict__ cell_off, int32_t n_cells,
+                                                                SedMoves M, const int64_t *__restrict__ xi,
+                                                                const double *__restrict__ v,
+                                                                const double *__restrict__ zeta_new,
+                                                                const int32_t *__restrict__ id_of_slot,
+                                                                const int32_t *__restrict__ poff, SedLayout L)
+{
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    constexpr int W = kSedMergeNT / 32;
+    __shared__ unsigned long long s_key[W][kSedArrive]; // arrivals: id above slot, in order
+    __shared__ uint32_t s_below[W][kSedArrive];         // stayers that follow t arrivals and no more
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned long long *key = s_key[warp];
+    uint32_t *below = s_below[warp];
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int g = gw; g < n_cells; g += nw) { // uniform over the warp
+        const int32_t lo = cell_off[g], hi = cell_off[g + 1];
+        const int32_t p0 = poff[g], p1 = poff[g + 1];
+        const uint32_t A = M.arr[g], a0 = (uint32_t)M.first[g];
+        const uint32_t n_stay = M.stay[g];
+        const bool sorted = A <= (uint32_t)kSedArrive;
+        if (A > 0 && sorted) {
+            uint32_t P2 = 1;
+            while (P2 < A)
+                P2 <<= 1;
+            for (uint32_t i = lane; i < P2; i += 32) {
+                key[i] = i < A ? ((unsigned long long)M.a_id[a0 + i] << 32) | M.a_slot[a0 + i] : ~0ull;
+                below[i] = 0u;
+            }
+            __syncwarp();
+            for (uint32_t k = 2; k <= P2; k <<= 1) // bitonic
+                for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+                    for (uint32_t i = lane; i < P2 / 2; i += 32) {
+                        const uint32_t a = 2 * i - (i & (j - 1)), b = a + j;
+                        const unsigned long long ka = key[a], kb = key[b];
+                        if ((ka > kb) == ((a & k) == 0)) {
+                            key[a] = kb;
+                            key[b] = ka;
+                        }
+                    }
+                    __syncwarp();
+                }
+        }
+        uint32_t done = 0; // stayers so far
+        for (int32_t s0 = lo; s0 < hi; s0 += 32 * kSedRun) {
+            int64_t x[kSedRun];
+            double w[kSedRun], z[kSedRun];
+            int32_t id[kSedRun];
+#pragma unroll
+            for (int u = 0; u < kSedRun; ++u) { // every load first
+                const int32_t sl = s0 + 32 * u + lane;
+                const bool in = sl < hi;
+                z[u] = in ? zeta_new[sl] : -1.0;
+                x[u] = in ? xi[sl] : 0;
+                w[u] = in ? v[sl] : 1.0;
+                id[u] = in ? id_of_slot[sl] : -1;
+            }
+#pragma unroll
+            for (int u = 0; u < kSedRun; ++u) {
+                if (s0 + 32 * u >= hi) // uniform over the warp
+                    break;
+                const bool keep = !dneg(z[u]);
+                const unsigned km = __ballot_sync(FULL, keep);
+                uint32_t t = 0; // arrivals of lower id
+                if (A > 0 && sorted) {
+                    uint32_t end = A;
+                    while (t < end) { // first arrival above this id
+                        const uint32_t mid = (t + end) >> 1;
+                        if ((uint32_t)(key[mid] >> 32) < (uint32_t)id[u])
+                            t = mid + 1;
+                        else
+                            end = mid;
+                    }
+                    // stayers before each arrival: t does not fall along the kept lanes, one
+                    // addition per run of equal t (those after the last need none)
+                    const unsigned same = __match_any_sync(FULL, keep ? t : 0xFFFFFFFFu);
+                    if (keep && t < A && (same & lt) == 0u)
+                        below[t] += (uint32_t)__popc(same);
+                    __syncwarp();
+                } else if (A > 0 && keep) {
+                    for (uint32_t k = 0; k < A; ++k)
+                        t += M.a_id[a0 + k] < (uint32_t)id[u] ? 1u : 0u;
+                }
+                if (keep)
+                    L.put((int64_t)p0 + done + (uint32_t)__popc(km & lt) + t, x[u], w[u], z[u], id[u]);
+                done += (uint32_t)__popc(km);
+            }
+        }
+        uint32_t carry = 0; // stayers before the arrivals of this round
+        for (uint32_t j0 = 0; j0 < A; j0 += 32) {
+            const uint32_t j = j0 + lane;
+            uint32_t slot = 0, id = 0, at = 0;
+            if (sorted) {
+                uint32_t c = j < A ? below[j] : 0u;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t y = __shfl_up_sync(FULL, c, d);
+                    if (lane >= d)
+                        c += y;
+                }
+                if (j < A) {
+                    id = (uint32_t)(key[j] >> 32);
+                    slot = (uint32_t)key[j];
+                    at = j + carry + c;
+                }
+                carry += __shfl_sync(FULL, c, 31);
+            } else if (j < A) { // more arrivals than the sort takes: by counting
+                id = M.a_id[a0 + j];
+                slot = M.a_slot[a0 + j];
+                for (uint32_t k = 0; k < A; ++k)
+                    at += M.a_id[a0 + k] < id ? 1u : 0u;
+                for (int32_t s = lo; s < hi; ++s)
+                    at += !dneg(zeta_new[s]) && (uint32_t)id_of_slot[s] < id ? 1u : 0u;
+            }
+            if (j < A)
+                L.put((int64_t)p0 + at, xi[slot], v[slot], fabs(zeta_new[slot]), (int32_t)id);
+        }
+        if (lane == 0 && p0 + (int32_t)(n_stay + A) < p1) // the padding slot of an odd cell
+            L.put(p1 - 1, 0, 1.0, 0.0, -1);
+        __syncwarp();
+    }
+    // outside the domain: those that were, in their order, then the arrivals
+    const int32_t lo = cell_off[n_cells], p0 = poff[n_cells], p1 = poff[n_cells + 1];
+    const uint32_t n_out = M.stay[n_cells], A = M.arr[n_cells], a0 = (uint32_t)M.first[n_cells];
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p1 - p0; i += (int64_t)gridDim.x * blockDim.x) {
+        if (i < n_out) {
+            L.put(p0 + i, xi[lo + i], v[lo + i], 0.0, id_of_slot[lo + i]);
+        } else if (i < (int64_t)n_out + A) {
+            const uint32_t s = M.a_slot[a0 + (i - n_out)];
+            L.put(p0 + i, xi[s], v[s], fabs(zeta_new[s]), (int32_t)M.a_id[a0 + (i - n_out)]);
+        } else {
+            L.put(p0 + i, 0, 1.0, 0.0, -1);
+        }
+    }
+}
+
 struct SedBuffers {
     int64_t *xi2 = nullptr;
     double *v2 = nullptr;
     double *zeta2 = nullptr;
     int32_t *id2 = nullptr;
-    int32_t *group = nullptr;     // group of every slot of the current layout
-    int32_t *group2 = nullptr;
+    int32_t *group = nullptr;     // sorted path: group of every slot of the current layout;
+    int32_t *group2 = nullptr;    //   else the arrivals' ids and slots
+    bool group_valid = false;     // group holds the current layout's
     int32_t *cell_off2 = nullptr; // n_cells + 2
     double *zeta_new = nullptr;   // per slot of the old layout
-    uint32_t *keys[2] = {};
-    uint32_t *vals[2] = {};
+    uint32_t *keys[2] = {}; // sorted path: keys and slots; else the movers' new groups, ids,
+    uint32_t *vals[2] = {}; //   slots and places
+    uint32_t *moves = nullptr; // per group: stayers, arrivals, movers, first arrival; then block totals
     uint32_t *counts = nullptr; // n_cells + 1
     int32_t *ustart = nullptr;  // n_cells + 2
     double *precip = nullptr;   // per-block parts of the move kernel, then the total
@@ -419,7 +863,8 @@ void sed_release(sdm_ctx *ctx)
         SedBuffers &b = *ctx->sed;
         void *bufs[] = {b.xi2,      b.v2,       b.zeta2,    b.id2,    b.group,  b.group2,
                         b.cell_off2, b.zeta_new, b.keys[0], b.keys[1], b.vals[0], b.vals[1],
-                        b.counts,   b.ustart,   b.precip,   b.hist,   b.flags,  b.emig};
+                        b.counts,   b.ustart,   b.precip,   b.hist,   b.flags,  b.emig,
+                        b.moves};
         for (void *p : bufs)
             ctx->mem.put(p, 0);
         if (b.h_read || b.side) {
@@ -448,6 +893,10 @@ T *sed_get(sdm_ctx *ctx, size_t count)
     return static_cast<T *>(ctx->mem.get(sizeof(T) * (count > 0 ? count : 1)));
 }
 
+// Words of one of the per-group arrays of SedBuffers::moves (a multiple of 2:
+// the totals behind them are 8-byte words).
+size_t sed_stride(int32_t n_cells) { return ((size_t)n_cells + 3) & ~(size_t)1; }
+
 sdm_status sed_alloc(sdm_ctx *ctx)
 {
     if (ctx->sed)
@@ -469,14 +918,15 @@ sdm_status sed_alloc(sdm_ctx *ctx)
     b.cell_off2 = sed_get<int32_t>(ctx, (size_t)nc + 2);
     b.zeta_new = sed_get<double>(ctx, slots);
     for (int i = 0; i < 2; ++i) {
-        b.keys[i] = sed_get<uint32_t>(ctx, cap);
-        b.vals[i] = sed_get<uint32_t>(ctx, cap);
+        b.keys[i] = sed_get<uint32_t>(ctx, slots);
+        b.vals[i] = sed_get<uint32_t>(ctx, slots);
     }
     b.counts = sed_get<uint32_t>(ctx, (size_t)nc + 1);
     b.ustart = sed_get<int32_t>(ctx, (size_t)nc + 2);
     b.precip = sed_get<double>(ctx, (size_t)kSedMaxBlocks + 1);
     b.hist = sed_get<uint32_t>(ctx, (size_t)kRadixBuckets * tiles + kRadixBuckets);
     b.flags = sed_get<uint32_t>(ctx, 4);
+    b.moves = sed_get<uint32_t>(ctx, 4 * sed_stride(nc) + 2 * ((size_t)nc / 1024 + 1));
     b.emig = sed_get<int32_t>(ctx, cap);
     if (cudaMallocHost(&b.h_read, sed_read_bytes(nc)) != cudaSuccess) {
         cudaGetLastError();
@@ -491,12 +941,12 @@ sdm_status sed_alloc(sdm_ctx *ctx)
     }
     const bool ok = ctx->d_zeta && b.xi2 && b.v2 && b.zeta2 && b.id2 && b.group && b.group2 && b.cell_off2 &&
                     b.zeta_new && b.keys[0] && b.keys[1] && b.vals[0] && b.vals[1] && b.counts && b.ustart &&
-                    b.precip && b.hist && b.flags && b.emig && b.h_read;
+                    b.precip && b.hist && b.flags && b.emig && b.moves && b.h_read;
     if (!ok) {
         sed_release(ctx);
         return fail(&ctx->error, SDM_ENOMEM, "sedimentation buffers: device allocation failed");
     }
-    ctx->device_bytes += slots * (8 + 8 + 8 + 8 + 4 + 4 + 4 + 8) + cap * 20 + ((int64_t)nc + 2) * 16 +
+    ctx->device_bytes += slots * (8 + 8 + 8 + 8 + 4 + 4 + 4 + 8 + 16) + cap * 4 + ((int64_t)nc + 2) * 32 +
                          (int64_t)kRadixBuckets * (tiles + 1) * 4;
     return SDM_OK;
 }
@@ -544,8 +994,9 @@ sdm_status set_positions_impl(sdm_ctx *ctx, const double *z, int32_t nx, double 
     CTX_CUDA(ctx, cudaMemsetAsync(d_flags, 0, sizeof(uint32_t), s));
     CTX_CUDA(ctx, cudaMemsetAsync(d_bad, 0xFF, sizeof(unsigned long long), s));
     sed_set_kernel<<<sed_grid(nc + 1), kSedNT, 0, s>>>(ctx->d_cell_off, nc, ctx->n_slots, ctx->d_id_of_slot, dz_arr,
-                                                        nx, dz, ctx->cfg.cell_base, zeta_in, ctx->d_zeta,
-                                                        ctx->sed->group, d_flags, d_bad);
+                                                        nx, dz, ctx->cfg.cell_base, zeta_in, ctx->d_zeta, d_flags,
+                                                        d_bad);
+    ctx->sed->group_valid = false;
     CTX_CUDA(ctx, cudaMemsetAsync(ctx->sed->emig, 0xFF, sizeof(int32_t) * ctx->n_sd, s));
     uint32_t flags = 0;
     unsigned long long bad = 0;
@@ -592,45 +1043,96 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     cudaStream_t s = ctx->stream;
     const int32_t nc = ctx->cfg.n_cells, n_groups = nc + 1;
     const int64_t n = ctx->n_sd;
-    CTX_CUDA(ctx, cudaMemsetAsync(b.counts, 0, sizeof(uint32_t) * n_groups, s));
-    const int move_blocks = (int)std::max<int64_t>(
-        1, std::min<int64_t>(kSedMaxBlocks, (ctx->n_slots + (int64_t)kSedNT * kSedU - 1) / ((int64_t)kSedNT * kSedU)));
-    sed_move_kernel<<<move_blocks, kSedNT, 0, s>>>(ctx->d_inst, nc, ctx->n_slots, ctx->nx, ctx->dz, (float)ctx->cfg.dt,
-                                                   ctx->d_zeta, b.group, ctx->d_id_of_slot, b.keys[0], b.vals[0],
-                                                   b.zeta_new, b.counts, b.precip, ctx->cfg.cell_base, b.emig);
-    // the offset scan, the refresh of the context's own launch plan (when
-    // refreshable: rebuilt on the device for the new layout) and the read-back
-    // into the pinned buffer (offsets, precipitated total, class counts) on
-    // the side stream, beside the radix sort, which needs none of them
     sdm_batch *sb = ctx->self_batch;
     const bool refresh = sb && sb->plan.refreshable && same_tuning(sb->plan.tuning, current_tuning());
     unsigned char *hr = static_cast<unsigned char *>(b.h_read);
     const int32_t *off = reinterpret_cast<const int32_t *>(hr);
     const size_t at_pr = (((size_t)nc + 2) * 4 + 7) / 8 * 8;
     const uint32_t *rc = reinterpret_cast<const uint32_t *>(hr + at_pr + 8);
-    CTX_CUDA(ctx, cudaEventRecord(b.fork, s));
-    CTX_CUDA(ctx, cudaStreamWaitEvent(b.side, b.fork, 0));
-    sed_scan_kernel<<<1, 1024, 0, b.side>>>(b.counts, n_groups, b.ustart, b.cell_off2, b.precip, move_blocks,
-                                            b.precip + kSedMaxBlocks);
-    // the new layout's padding slots (the gather writes only the others)
-    sed_pad_kernel<<<(n_groups + 255) / 256, 256, 0, b.side>>>(n_groups, b.ustart, b.cell_off2, b.xi2, b.v2, b.zeta2,
-                                                                b.id2, b.group2);
-    if (refresh) {
-        CTX_CUDA(ctx, plan_refresh(sb->plan, b.cell_off2, nc, ctx->cfg.cell_base, b.side));
-        CTX_CUDA(ctx, cudaMemcpyAsync(hr + at_pr + 8, sb->plan.d_refresh, sizeof(uint32_t) * (kNumClass + 1),
-                                      cudaMemcpyDeviceToHost, b.side));
+    // on the side stream, beside what follows the new offsets: the refresh of
+    // the context's own launch plan (when refreshable: rebuilt on the device for
+    // the new layout) and the read-back into the pinned buffer (offsets,
+    // precipitated total, class counts)
+    auto side_work = [&]() -> sdm_status {
+        if (refresh) {
+            CTX_CUDA(ctx, plan_refresh(sb->plan, b.cell_off2, nc, ctx->cfg.cell_base, b.side));
+            CTX_CUDA(ctx, cudaMemcpyAsync(hr + at_pr + 8, sb->plan.d_refresh, sizeof(uint32_t) * (kNumClass + 1),
+                                          cudaMemcpyDeviceToHost, b.side));
+        }
+        CTX_CUDA(ctx, cudaMemcpyAsync(hr, b.cell_off2, sizeof(int32_t) * (n_groups + 1), cudaMemcpyDeviceToHost, b.side));
+        CTX_CUDA(ctx, cudaMemcpyAsync(hr + at_pr, b.precip + kSedMaxBlocks, sizeof(double), cudaMemcpyDeviceToHost,
+                                      b.side));
+        CTX_CUDA(ctx, cudaEventRecord(b.join, b.side));
+        return SDM_OK;
+    };
+    const bool by_cell = ctx->largest_cell <= kSedByCell;
+    if (by_cell) {
+        const size_t st_ = sed_stride(nc);
+        SedMoves M{b.keys[0], b.vals[0],      b.keys[1],          b.vals[1],   (uint32_t *)b.group, (uint32_t *)b.group2,
+                   b.moves,   b.moves + st_, b.moves + 2 * st_, (int32_t *)(b.moves + 3 * st_)};
+        unsigned long long *totals = (unsigned long long *)(b.moves + 4 * st_);
+        b.group_valid = false;
+        CTX_CUDA(ctx, cudaMemsetAsync(M.arr, 0, sizeof(uint32_t) * n_groups, s));
+        if (ctx->cfg.cell_base > 0) // the emigrants of the step before are none of this one's
+            CTX_CUDA(ctx, cudaMemsetAsync(b.emig, 0xFF, sizeof(int32_t) * n, s));
+        const int warps = kSedNT / 32;
+        const int fall_blocks = std::max(1, std::min((nc + warps - 1) / warps, 152 * 4));
+        sed_fall_kernel<<<fall_blocks, kSedNT, 0, s>>>(ctx->d_inst, ctx->d_cell_off, nc, ctx->n_slots, ctx->nx, ctx->dz,
+                                                       (float)ctx->cfg.dt, ctx->d_zeta, ctx->d_id_of_slot, b.zeta_new, M,
+                                                       b.precip, ctx->cfg.cell_base, b.emig);
+        const int blocks = (n_groups + 1023) / 1024;
+        if (blocks > 64)
+            sed_totals_kernel<<<blocks, 1024, 0, s>>>(M, n_groups, totals);
+        sed_offsets_kernel<<<blocks, 1024, 0, s>>>(M, n_groups, blocks > 64 ? totals : nullptr, b.cell_off2, b.precip,
+                                                   fall_blocks, b.precip + kSedMaxBlocks);
+        CTX_CUDA(ctx, cudaEventRecord(b.fork, s));
+        CTX_CUDA(ctx, cudaStreamWaitEvent(b.side, b.fork, 0));
+        st = side_work();
+        if (st != SDM_OK)
+            return st;
+        sed_deal_kernel<<<std::max(1, std::min((nc + warps - 1) / warps, 152 * 8)), kSedNT, 0, s>>>(ctx->d_cell_off, nc, M);
+        const int mw = kSedMergeNT / 32;
+        const int64_t units = std::max<int64_t>((nc + mw - 1) / mw, (ctx->n_slots - ctx->h_cell_off[nc]) / kSedMergeNT + 1);
+        sed_merge_kernel<<<(int)std::min<int64_t>(units, 152 * 9), kSedMergeNT, 0, s>>>(
+            ctx->d_cell_off, nc, M, ctx->d_xi, ctx->d_v, b.zeta_new, ctx->d_id_of_slot, b.cell_off2,
+            SedLayout{b.xi2, b.v2, b.zeta2, b.id2});
+        CTX_CUDA(ctx, cudaGetLastError());
+        CTX_CUDA(ctx, cudaStreamWaitEvent(s, b.join, 0)); // later work may write what the side stream reads
+    } else {
+        if (!b.group_valid)
+            sed_group_kernel<<<sed_grid(n_groups), kSedNT, 0, s>>>(ctx->d_cell_off, nc, ctx->n_slots, b.group);
+        CTX_CUDA(ctx, cudaMemsetAsync(b.counts, 0, sizeof(uint32_t) * n_groups, s));
+        const int move_blocks = (int)std::max<int64_t>(
+            1,
+            std::min<int64_t>(kSedMaxBlocks, (ctx->n_slots + (int64_t)kSedNT * kSedU - 1) / ((int64_t)kSedNT * kSedU)));
+        sed_move_kernel<<<move_blocks, kSedNT, 0, s>>>(ctx->d_inst, nc, ctx->n_slots, ctx->nx, ctx->dz,
+                                                       (float)ctx->cfg.dt, ctx->d_zeta, b.group, ctx->d_id_of_slot,
+                                                       b.keys[0], b.vals[0], b.zeta_new, b.counts, b.precip,
+                                                       ctx->cfg.cell_base, b.emig);
+        // the offset scan, the padding and the rest of the side stream's work
+        // beside the radix sort, which needs none of them
+        CTX_CUDA(ctx, cudaEventRecord(b.fork, s));
+        CTX_CUDA(ctx, cudaStreamWaitEvent(b.side, b.fork, 0));
+        sed_scan_kernel<<<1, 1024, 0, b.side>>>(b.counts, n_groups, b.ustart, b.cell_off2, b.precip, move_blocks,
+                                                b.precip + kSedMaxBlocks);
+        // the new layout's padding slots (the gather writes only the others)
+        sed_pad_kernel<<<(n_groups + 255) / 256, 256, 0, b.side>>>(n_groups, b.ustart, b.cell_off2, b.xi2, b.v2,
+                                                                    b.zeta2, b.id2, b.group2);
+        st = side_work();
+        if (st != SDM_OK)
+            return st;
+        // stable sort of the new groups, SD-id order in
+        const int bits = 32 - __builtin_clz((unsigned)nc | 1u);
+        const int cur = radix_sort(b.keys, b.vals, false, n, bits, b.hist, s);
+        CTX_CUDA(ctx, cudaStreamWaitEvent(s, b.join, 0));
+        sed_gather_kernel<<<1216, 256, 0, s>>>(n, b.keys[cur], b.vals[cur], b.ustart, b.cell_off2, ctx->d_xi, ctx->d_v,
+                                               b.zeta_new, ctx->d_id_of_slot, b.xi2, b.v2, b.zeta2, b.id2, b.group2);
+        CTX_CUDA(ctx, cudaGetLastError());
+        std::swap(b.group, b.group2);
+        b.group_valid = true;
     }
-    CTX_CUDA(ctx, cudaMemcpyAsync(hr, b.cell_off2, sizeof(int32_t) * (n_groups + 1), cudaMemcpyDeviceToHost, b.side));
-    CTX_CUDA(ctx, cudaMemcpyAsync(hr + at_pr, b.precip + kSedMaxBlocks, sizeof(double), cudaMemcpyDeviceToHost, b.side));
-    CTX_CUDA(ctx, cudaEventRecord(b.join, b.side));
-    // stable sort of the new groups, SD-id order in
-    const int bits = 32 - __builtin_clz((unsigned)nc | 1u);
-    const int cur = radix_sort(b.keys, b.vals, false, n, bits, b.hist, s);
-    CTX_CUDA(ctx, cudaStreamWaitEvent(s, b.join, 0));
-    sed_gather_kernel<<<1216, 256, 0, s>>>(n, b.keys[cur], b.vals[cur], b.ustart, b.cell_off2, ctx->d_xi, ctx->d_v,
-                                           b.zeta_new, ctx->d_id_of_slot, b.xi2, b.v2, b.zeta2, b.id2, b.group2);
-    CTX_CUDA(ctx, cudaGetLastError());
-    CTX_CUDA(ctx, cudaStreamSynchronize(s));
+    // the read-back only: what writes the new layout goes on behind it
+    CTX_CUDA(ctx, cudaEventSynchronize(b.join));
     double precip = 0.0;
     std::memcpy(&precip, hr + at_pr, sizeof precip);
     // the new layout becomes the state; the old one the next scratch
@@ -639,7 +1141,6 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     std::swap(ctx->d_zeta, b.zeta2);
     std::swap(ctx->d_id_of_slot, b.id2);
     std::swap(ctx->d_cell_off, b.cell_off2);
-    std::swap(b.group, b.group2);
     int32_t largest = 0;
     for (int32_t c = 0; c < nc; ++c)
         largest = std::max(largest, off[c + 1] - off[c]);
