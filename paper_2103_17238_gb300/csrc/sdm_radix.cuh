@@ -9,11 +9,17 @@
 namespace sdm {
 
 constexpr int kRadixNT = 256;
-constexpr int kRadixRounds = 16;
-constexpr int kRadixTile = kRadixNT * kRadixRounds; // keys per block and pass
+// Keys per block and pass: 4096 (1,024 tiles of 4.19M keys make one wave; tiles
+// of 2048 or 8192 took 0.224 and 0.241 ms against 0.210 per sort there), or 1024
+// below 2^21 keys, where tiles of 4096 leave SMs with one or none (975,000 keys:
+// RADIX_FIGURES).
+constexpr int kRadixRounds = 16, kRadixRoundsFew = 4;
+constexpr int64_t kRadixFew = (int64_t)1 << 21;
+constexpr int radix_rounds(int64_t n) { return n < kRadixFew ? kRadixRoundsFew : kRadixRounds; }
 constexpr int kRadixBuckets = 256;                  // 8-bit digits
 
 // hist[d * n_tiles + tile] = keys of the tile whose digit (key >> shift) & 255 is d.
+template <int ROUNDS>
 __global__ void __launch_bounds__(kRadixNT) radix_hist_kernel(const uint32_t *__restrict__ keys, int64_t n, int shift,
                                                               uint32_t *__restrict__ hist, int32_t n_tiles)
 {
@@ -21,15 +27,15 @@ __global__ void __launch_bounds__(kRadixNT) radix_hist_kernel(const uint32_t *__
     const int t = threadIdx.x;
     h[t] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRadixTile;
-    uint32_t k[kRadixRounds]; // every load of the thread in flight at once
+    const int64_t base = (int64_t)blockIdx.x * (kRadixNT * ROUNDS);
+    uint32_t k[ROUNDS]; // every load of the thread in flight at once
 #pragma unroll
-    for (int r = 0; r < kRadixRounds; ++r) {
+    for (int r = 0; r < ROUNDS; ++r) {
         const int64_t i = base + (int64_t)r * kRadixNT + t;
         k[r] = i < n ? keys[i] : 0xFFFFFFFFu;
     }
 #pragma unroll
-    for (int r = 0; r < kRadixRounds; ++r)
+    for (int r = 0; r < ROUNDS; ++r)
         if (base + (int64_t)r * kRadixNT + t < n)
             atomicAdd(&h[(k[r] >> shift) & 255u], 1u);
     __syncthreads();
@@ -76,6 +82,7 @@ __global__ void __launch_bounds__(kRadixBuckets) radix_digit_scan_kernel(uint32_
 // minor); within a round, lanes of a warp with equal digits are ranked by
 // __match_any_sync, warps by their per-digit counts in shared memory.
 // vals_in null: the values are the indices.
+template <int ROUNDS>
 __global__ void __launch_bounds__(kRadixNT) radix_scatter_kernel(const uint32_t *__restrict__ keys_in,
                                                                  const uint32_t *__restrict__ vals_in, int64_t n,
                                                                  int shift, const uint32_t *__restrict__ offs,
@@ -91,17 +98,17 @@ __global__ void __launch_bounds__(kRadixNT) radix_scatter_kernel(const uint32_t 
     for (int i = t; i < NW * (kRadixBuckets + 1); i += kRadixNT)
         (&s_wcnt[0][0])[i] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRadixTile;
+    const int64_t base = (int64_t)blockIdx.x * (kRadixNT * ROUNDS);
     const unsigned lt = (1u << lane) - 1u;
-    uint32_t kk[kRadixRounds], vv[kRadixRounds]; // every load of the thread in flight at once
+    uint32_t kk[ROUNDS], vv[ROUNDS]; // every load of the thread in flight at once
 #pragma unroll
-    for (int r = 0; r < kRadixRounds; ++r) {
+    for (int r = 0; r < ROUNDS; ++r) {
         const int64_t i = base + (int64_t)r * kRadixNT + t;
         kk[r] = i < n ? keys_in[i] : 0u;
         vv[r] = i < n ? (vals_in ? vals_in[i] : (uint32_t)i) : 0u;
     }
 #pragma unroll
-    for (int r = 0; r < kRadixRounds; ++r) {
+    for (int r = 0; r < ROUNDS; ++r) {
         const int64_t i = base + (int64_t)r * kRadixNT + t;
         const bool valid = i < n;
         const uint32_t k = kk[r];
@@ -145,24 +152,31 @@ inline int radix_sort(uint32_t *const keys[2], uint32_t *const vals[2], bool iot
                       cudaStream_t s)
 {
     const int passes = (bits + 7) / 8;
-    const int32_t tiles = (int32_t)((n + kRadixTile - 1) / kRadixTile);
+    const int tile = kRadixNT * radix_rounds(n);
+    const int32_t tiles = (int32_t)((n + tile - 1) / tile);
+    const auto count = n < kRadixFew ? radix_hist_kernel<kRadixRoundsFew> : radix_hist_kernel<kRadixRounds>;
+    const auto place = n < kRadixFew ? radix_scatter_kernel<kRadixRoundsFew> : radix_scatter_kernel<kRadixRounds>;
     uint32_t *digit_total = hist + (size_t)kRadixBuckets * tiles;
     int cur = 0;
     for (int p = 0; p < passes; ++p) {
-        radix_hist_kernel<<<tiles, kRadixNT, 0, s>>>(keys[cur], n, 8 * p, hist, tiles);
+        count<<<tiles, kRadixNT, 0, s>>>(keys[cur], n, 8 * p, hist, tiles);
         radix_row_scan_kernel<<<kRadixBuckets, 1024, 0, s>>>(hist, tiles, digit_total);
         radix_digit_scan_kernel<<<1, kRadixBuckets, 0, s>>>(digit_total);
-        radix_scatter_kernel<<<tiles, kRadixNT, 0, s>>>(keys[cur], p == 0 && iota ? nullptr : vals[cur], n, 8 * p, hist,
-                                                         digit_total, tiles, keys[cur ^ 1], vals[cur ^ 1]);
+        place<<<tiles, kRadixNT, 0, s>>>(keys[cur], p == 0 && iota ? nullptr : vals[cur], n, 8 * p, hist, digit_total,
+                                         tiles, keys[cur ^ 1], vals[cur ^ 1]);
         cur ^= 1;
     }
     return cur;
 }
 
-// Bytes of radix_sort's hist for n pairs.
-inline size_t radix_hist_bytes(int64_t n)
+// Words of radix_sort's hist for up to n pairs.
+inline size_t radix_hist_words(int64_t n)
 {
-    return sizeof(uint32_t) * (size_t)kRadixBuckets * (size_t)((n + kRadixTile - 1) / kRadixTile + 1);
+    auto words = [](int64_t m) {
+        const int64_t tile = kRadixNT * radix_rounds(m);
+        return (size_t)kRadixBuckets * (size_t)((m + tile - 1) / tile + 1);
+    };
+    return std::max(words(n), words(std::min(n, kRadixFew - 1)));
 }
 
 } // namespace sdm

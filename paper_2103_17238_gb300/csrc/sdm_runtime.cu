@@ -478,6 +478,21 @@ int variant_for(int cap, const sdm_tuning &t)
     return -1;
 }
 
+// The variant of class k for a plan's n cells of it.  With the default tuning,
+// classes that leave most of the device idle take a block per cell where that
+// is faster than a warp (fused steps, us, warp | block): 500 SDs, 1 cell 5.2 |
+// 2.7, 304 cells 5.6 | 3.3, 608 5.7 | 4.6, 912 6.4 | 7.5; 250 SDs, 1 cell 2.7 | 2.5,
+// 304 3.0 | 2.9, 608 3.2 | 3.2; smaller cells never (120 SDs, 1 cell 1.7 | 2.4).
+int variant_of_class(int k, int n, const sdm_tuning &t)
+{
+    constexpr int kFew512 = 608, kFew256 = 304;
+    const bool standard = t.warp_cell_max == 512 && t.warps_per_block == 2;
+    sdm_tuning u = t;
+    if (standard && n <= (kClassCap[k] == 512 ? kFew512 : (kClassCap[k] == 256 ? kFew256 : 0)))
+        u.warp_cell_max = kClassCap[k] / 2;
+    return variant_for(kClassCap[k], u);
+}
+
 // The mid-size-cell kernel with K CTAs per cluster: its shared-memory limit,
 // and how many clusters fit on the device at once (its persistent grid).
 template <int K>
@@ -773,8 +788,6 @@ sdm_status build_plan(sdm_batch *b)
     int64_t hist_total = 0, sd_total = 0, bkt_total = 0;
     const sdm_tuning tun = current_tuning();
     pl.tuning = tun;
-    for (int k = 0; k < kNumClass; ++k)
-        pl.variant[k] = variant_for(kClassCap[k], tun);
     // the cells above the shared-memory classes
     int64_t above_sd = 0, above_cells = 0;
     int32_t above_most = 0;
@@ -944,6 +957,7 @@ sdm_status build_plan(sdm_batch *b)
     pl.d_insts = reinterpret_cast<InstDev **>(d);
     for (int k = 0; k < kNumClass; ++k) {
         pl.n_items[k] = (int)items[k].size();
+        pl.variant[k] = variant_of_class(k, pl.n_items[k], tun);
         pl.d_items[k] = pl.n_items[k] ? reinterpret_cast<WorkItem *>(d + off_items[k]) : nullptr;
     }
     // a context's own plan of shared-memory classes only: items with room
@@ -1669,7 +1683,7 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
         if (!on_device)
             CTX_CUDA(ctx, cudaStreamWaitEvent(s, ctx->in_ev[k], 0));
         if (piece[k + 1] > piece[k])
-            validate_count_kernel<<<grid_of((piece[k + 1] - piece[k] + 3) / 4), 256, 0, s>>>(
+            validate_count_kernel<<<(int)std::min<int64_t>((piece[k + 1] - piece[k] + 1023) / 1024, 1 << 20), 256, 0, s>>>(
                 piece[k], piece[k + 1], dxi, dv, dcell, n_cells, d_counts,
                                                         d_flags, d_bad);
     }
@@ -1707,7 +1721,7 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
     const bool unsorted = (flags & 2u) != 0;
     auto a256 = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t b_off = a256(sizeof(int32_t) * 2 * (n_groups + 1)), b_key = a256(sizeof(uint32_t) * n_sd);
-    const size_t b_aux = b_off + (unsorted ? 2 * b_key + radix_hist_bytes(n_sd) : 0);
+    const size_t b_aux = b_off + (unsorted ? 2 * b_key + sizeof(uint32_t) * radix_hist_words(n_sd) : 0);
     void *aux = mem.get(b_aux);
     if (!aux) {
         mem.put(meta, b_counts);
@@ -1754,7 +1768,7 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
         place_sorted_kernel<<<grid_of(n_sd), 256, 0, s>>>(n_sd, keys[cur], vals[cur], dxi, dv, d_poff, d_uoff, ctx->d_xi,
                                                  ctx->d_v, ctx->d_id_of_slot);
     } else {
-        scatter_kernel<<<grid_of(n_sd), 256, 0, s>>>(n_sd, dxi, dv, dcell, n_cells, d_poff, d_uoff, ctx->d_xi, ctx->d_v,
+        scatter_kernel<<<grid_of((n_sd + 3) / 4), 256, 0, s>>>(n_sd, dxi, dv, dcell, n_cells, d_poff, d_uoff, ctx->d_xi, ctx->d_v,
                                             ctx->d_id_of_slot);
     }
     // after the sort, whose other pair of arrays lies over the padding too

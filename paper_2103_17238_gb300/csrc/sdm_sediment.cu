@@ -85,9 +85,12 @@ __global__ void __launch_bounds__(kSedNT) sed_set_kernel(const int32_t *__restri
                     break;
                 double zt = 0.0;
                 if (id[u] >= 0 && g < n_cells) {
-                    // + 0 turns a -0 height into +0 (the fall tests signs bitwise)
-                    zt = __dadd_rn(__dsub_rn(zz[u], base), 0.0);
-                    if (!(zt >= 0.0 && zt < dz)) {
+                    zt = zeta_in ? zz[u] : __dsub_rn(zz[u], base);
+                    // a -0 height becomes +0 (the fall tests signs bitwise)
+                    if (__double_as_longlong(zt) == (long long)0x8000000000000000ll)
+                        zt = 0.0;
+                    // in [0, dz): by the bit patterns (NaN and negative ones are above)
+                    if ((unsigned long long)__double_as_longlong(zt) >= (unsigned long long)__double_as_longlong(dz)) {
                         atomicOr(flags, 1u);
                         atomicMin(bad, (unsigned long long)id[u]);
                         zt = 0.0;
@@ -198,13 +201,16 @@ struct Fall {
     double z;
 };
 
-__device__ __forceinline__ Fall sed_fall(const PairConsts &C, double v, double zt, float dt32, int32_t g, int32_t nx,
-                                         double dz, int32_t cbase)
+// The height after the fall (negative: below the cell's bottom).
+__device__ __forceinline__ double sed_drop(const PairConsts &C, double v, double zt, float dt32)
 {
     bool in_range;
     const float vf = d2f_rn(v, in_range);
-    const double d = f2d_exact(__fmul_rn(vt32c(C, radius32(vf)), dt32));
-    double zz = __dsub_rn(zt, d);
+    return __dsub_rn(zt, f2d_exact(__fmul_rn(vt32c(C, radius32(vf)), dt32)));
+}
+
+__device__ __forceinline__ Fall sed_levels(double zz, int32_t g, int32_t nx, double dz, int32_t cbase)
+{
     // crossing k levels takes cell c to c - k nx; below the grid's level 0
     // exactly when cbase + c is negative (0 <= column < nx)
     int32_t c = g;
@@ -219,6 +225,12 @@ __device__ __forceinline__ Fall sed_fall(const PairConsts &C, double v, double z
         zz = 0.0;
     }
     return Fall{c, zz};
+}
+
+__device__ __forceinline__ Fall sed_fall(const PairConsts &C, double v, double zt, float dt32, int32_t g, int32_t nx,
+                                         double dz, int32_t cbase)
+{
+    return sed_levels(sed_drop(C, v, zt, dt32), g, nx, dz, cbase);
 }
 
 // precip_part[block] = the block's sum of pr (lanes, then warps, in a fixed tree).
@@ -474,6 +486,7 @@ __global__ void sed_pad_kernel(int32_t n_groups, const int32_t *__restrict__ ust
 constexpr int kSedByCell = 1024;  // slots of the largest cell that a warp takes
 constexpr int kSedArrive = 512;   // arrivals of a cell sorted in shared memory
 constexpr int kSedMergeNT = 128;
+constexpr int kSedFew = 12;       // arrivals up to which each is compared with every stayer, by ballots
 
 // What the movers of the cells and the arrivals of the groups are kept in.
 // Cell c's movers take places [cell_off[c], + left[c]) of the mover arrays;
@@ -485,6 +498,12 @@ struct SedMoves {
     int32_t *first;                      // n_groups
 };
 
+// A warp first takes every SD's height down; the few that leave their cell (or
+// are dead, or padding) wait in shared memory and are followed 32 at a time, so
+// that their levels, each a binary64 addition, and their places are not paid by
+// every 32 slots that hold one.
+constexpr int kSedWait = 64; // entries: below 32 left from before, and up to 32 new ones
+
 __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restrict__ P,
                                                           const int32_t *__restrict__ cell_off, int32_t n_cells,
                                                           int64_t n_slots, int32_t nx, double dz, float dt32,
@@ -495,8 +514,10 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
                                                           int32_t *__restrict__ emig)
 {
     constexpr unsigned FULL = 0xFFFFFFFFu;
+    __shared__ double s_z[kSedNT / 32][kSedWait];
+    __shared__ int32_t s_slot[kSedNT / 32][kSedWait]; // with the sign bit for an SD that does not fall (dead, padding)
     const PairConsts C = pair_consts(P);
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int64_t *__restrict__ gxi = P->xi;
     const double *__restrict__ gv = P->v;
@@ -504,7 +525,52 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
     double pr = 0.0;
     for (int g = gw; g < n_cells; g += nw) { // uniform over the warp
         const int32_t lo = cell_off[g], hi = cell_off[g + 1];
-        uint32_t stay = 0, left = 0;
+        uint32_t stay = 0, left = 0, wait = 0; // uniform
+        auto follow = [&](uint32_t n) {        // the first n <= 32 waiting entries
+            int32_t ng = n_cells, em = -1, id = -1, sl = 0;
+            double zn = 0.0;
+            if (lane < (int)n) {
+                const int32_t e = s_slot[warp][lane];
+                sl = e & 0x7FFFFFFF;
+                id = id_of_slot[sl];
+                if (e >= 0) {
+                    const Fall f = sed_levels(s_z[warp][lane], g, nx, dz, cbase);
+                    if (f.c + cbase < 0) {
+                        pr = __dadd_rn(pr, __dmul_rn(xi2d(gxi[sl]), gv[sl]));
+                    } else {
+                        zn = f.z;
+                        if (f.c >= 0)
+                            ng = f.c;
+                        else // into another piece of the grid
+                            em = f.c + cbase;
+                    }
+                }
+            }
+            // (level 0 dz above: zeta + dz rounded up to dz, so it stays after all)
+            const bool keep = lane < (int)n && ng == g;
+            stay += (uint32_t)__popc(__ballot_sync(FULL, keep));
+            if (lane < (int)n) // stayers +zn, the others (padding too) with the sign bit set
+                zeta_new[sl] = keep ? zn : __hiloint2double(__double2hiint(zn) | (int)0x80000000, __double2loint(zn));
+            const bool go = id >= 0 && !keep;
+            const unsigned mv = __ballot_sync(FULL, go);
+            const unsigned out = __ballot_sync(FULL, go && ng == n_cells);
+            uint32_t place = 0;
+            if (out && lane == __ffs(out) - 1) // one counter for all that leave the domain
+                place = atomicAdd(&M.arr[n_cells], (uint32_t)__popc(out));
+            place = __shfl_sync(FULL, place, out ? __ffs(out) - 1 : 0) + (uint32_t)__popc(out & lt);
+            if (go) {
+                if (ng != n_cells)
+                    place = atomicAdd(&M.arr[ng], 1u);
+                const uint32_t at = (uint32_t)lo + left + (uint32_t)__popc(mv & lt);
+                M.group[at] = (uint32_t)ng;
+                M.id[at] = (uint32_t)id;
+                M.slot[at] = (uint32_t)sl;
+                M.place[at] = place;
+                if (em >= 0)
+                    emig[id] = em;
+            }
+            left += (uint32_t)__popc(mv);
+        };
         for (int32_t s0 = lo; s0 < hi; s0 += 32 * kSedRun) {
             int64_t x[kSedRun];
             double vv[kSedRun], zt[kSedRun];
@@ -518,54 +584,38 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
             }
 #pragma unroll
             for (int u = 0; u < kSedRun; ++u) {
-                const int32_t sl = s0 + 32 * u + lane;
                 if (s0 + 32 * u >= hi) // uniform over the warp
                     break;
-                int32_t ng = n_cells, em = -1;
-                double zn = 0.0;
-                if (x[u] > 0) {
-                    const Fall f = sed_fall(C, vv[u], zt[u], dt32, g, nx, dz, cbase);
-                    if (f.c + cbase < 0) {
-                        pr = __dadd_rn(pr, __dmul_rn(xi2d(x[u]), vv[u]));
-                    } else {
-                        zn = f.z;
-                        if (f.c >= 0)
-                            ng = f.c;
-                        else // into another piece of the grid
-                            em = f.c + cbase;
+                const int32_t sl = s0 + 32 * u + lane;
+                const double zz = sed_drop(C, vv[u], zt[u], dt32);
+                const bool keep = x[u] > 0 && !dneg(zz);
+                const unsigned km = __ballot_sync(FULL, keep), wm = __ballot_sync(FULL, sl < hi) & ~km;
+                stay += (uint32_t)__popc(km);
+                if (keep) {
+                    zeta_new[sl] = zz;
+                } else if (sl < hi) {
+                    const uint32_t at = wait + (uint32_t)__popc(wm & lt);
+                    s_z[warp][at] = zz;
+                    s_slot[warp][at] = sl | (x[u] > 0 ? 0 : (int32_t)0x80000000);
+                }
+                wait += (uint32_t)__popc(wm);
+                if (wait >= 32u) {
+                    __syncwarp();
+                    follow(32u);
+                    __syncwarp();
+                    wait -= 32u;
+                    if (lane < (int)wait) { // the rest to the front
+                        s_z[warp][lane] = s_z[warp][32 + lane];
+                        s_slot[warp][lane] = s_slot[warp][32 + lane];
                     }
+                    __syncwarp();
                 }
-                // stayers +zn, the others (padding too) with the sign bit set
-                const bool keep = ng == g;
-                stay += (uint32_t)__popc(__ballot_sync(FULL, keep));
-                int32_t id = -1;
-                if (sl < hi) {
-                    zeta_new[sl] = keep ? zn : __hiloint2double(__double2hiint(zn) | (int)0x80000000, __double2loint(zn));
-                    if (!keep)
-                        id = id_of_slot[sl];
-                }
-                const unsigned mv = __ballot_sync(FULL, id >= 0);
-                if (mv == 0u)
-                    continue;
-                const unsigned out = __ballot_sync(FULL, id >= 0 && ng == n_cells);
-                uint32_t place = 0;
-                if (out && lane == __ffs(out) - 1) // one counter for all that leave the domain
-                    place = atomicAdd(&M.arr[n_cells], (uint32_t)__popc(out));
-                place = __shfl_sync(FULL, place, out ? __ffs(out) - 1 : 0) + (uint32_t)__popc(out & lt);
-                if (id >= 0) {
-                    if (ng != n_cells)
-                        place = atomicAdd(&M.arr[ng], 1u);
-                    const uint32_t at = (uint32_t)lo + left + (uint32_t)__popc(mv & lt);
-                    M.group[at] = (uint32_t)ng;
-                    M.id[at] = (uint32_t)id;
-                    M.slot[at] = (uint32_t)sl;
-                    M.place[at] = place;
-                    if (em >= 0)
-                        emig[id] = em;
-                }
-                left += (uint32_t)__popc(mv);
             }
         }
+        __syncwarp();
+        if (wait)
+            follow(wait);
+        __syncwarp();
         if (lane == 0) {
             M.stay[g] = stay;
             M.left[g] = left;
@@ -737,6 +787,7 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                 }
         }
         uint32_t done = 0; // stayers so far
+        uint32_t mine = 0;
         for (int32_t s0 = lo; s0 < hi; s0 += 32 * kSedRun) {
             int64_t x[kSedRun];
             double w[kSedRun], z[kSedRun];
@@ -757,7 +808,14 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                 const bool keep = !dneg(z[u]);
                 const unsigned km = __ballot_sync(FULL, keep);
                 uint32_t t = 0; // arrivals of lower id
-                if (A > 0 && sorted) {
+                if (A <= (uint32_t)kSedFew) {
+                    for (uint32_t k = 0; k < A; ++k) {
+                        const bool above = keep && (uint32_t)(key[k] >> 32) < (uint32_t)id[u];
+                        t += above ? 1u : 0u;
+                        const uint32_t c = (uint32_t)__popc(km & ~__ballot_sync(FULL, above));
+                        mine += lane == (int)k ? c : 0u; // lane k: stayers of lower id than arrival k
+                    }
+                } else if (sorted) {
                     uint32_t end = A;
                     while (t < end) { // first arrival above this id
                         const uint32_t mid = (t + end) >> 1;
@@ -772,7 +830,7 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                     if (keep && t < A && (same & lt) == 0u)
                         below[t] += (uint32_t)__popc(same);
                     __syncwarp();
-                } else if (A > 0 && keep) {
+                } else if (keep) {
                     for (uint32_t k = 0; k < A; ++k)
                         t += M.a_id[a0 + k] < (uint32_t)id[u] ? 1u : 0u;
                 }
@@ -785,7 +843,13 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
         for (uint32_t j0 = 0; j0 < A; j0 += 32) {
             const uint32_t j = j0 + lane;
             uint32_t slot = 0, id = 0, at = 0;
-            if (sorted) {
+            if (A <= (uint32_t)kSedFew) {
+                if (j < A) {
+                    id = (uint32_t)(key[j] >> 32);
+                    slot = (uint32_t)key[j];
+                    at = j + mine;
+                }
+            } else if (sorted) {
                 uint32_t c = j < A ? below[j] : 0u;
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) {
@@ -907,7 +971,6 @@ sdm_status sed_alloc(sdm_ctx *ctx)
     SedBuffers &b = *ctx->sed;
     const int64_t slots = ctx->n_slots_cap, cap = ctx->capacity_sd;
     const int32_t nc = ctx->cfg.n_cells;
-    const int64_t tiles = (cap + kRadixTile - 1) / kRadixTile;
     ctx->d_zeta = (double *)ctx->mem.get(sizeof(double) * slots);
     b.xi2 = sed_get<int64_t>(ctx, slots);
     b.v2 = sed_get<double>(ctx, slots);
@@ -924,7 +987,7 @@ sdm_status sed_alloc(sdm_ctx *ctx)
     b.counts = sed_get<uint32_t>(ctx, (size_t)nc + 1);
     b.ustart = sed_get<int32_t>(ctx, (size_t)nc + 2);
     b.precip = sed_get<double>(ctx, (size_t)kSedMaxBlocks + 1);
-    b.hist = sed_get<uint32_t>(ctx, (size_t)kRadixBuckets * tiles + kRadixBuckets);
+    b.hist = sed_get<uint32_t>(ctx, radix_hist_words(cap));
     b.flags = sed_get<uint32_t>(ctx, 4);
     b.moves = sed_get<uint32_t>(ctx, 4 * sed_stride(nc) + 2 * ((size_t)nc / 1024 + 1));
     b.emig = sed_get<int32_t>(ctx, cap);
@@ -947,7 +1010,7 @@ sdm_status sed_alloc(sdm_ctx *ctx)
         return fail(&ctx->error, SDM_ENOMEM, "sedimentation buffers: device allocation failed");
     }
     ctx->device_bytes += slots * (8 + 8 + 8 + 8 + 4 + 4 + 4 + 8 + 16) + cap * 4 + ((int64_t)nc + 2) * 32 +
-                         (int64_t)kRadixBuckets * (tiles + 1) * 4;
+                         (int64_t)radix_hist_words(cap) * 4;
     return SDM_OK;
 }
 
@@ -1156,8 +1219,11 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     CTX_CUDA(ctx, cudaMemcpyAsync(ctx->d_inst, &inst, sizeof inst, cudaMemcpyHostToDevice, s));
     const bool refreshed = refresh && !keep_plan && rc[kNumClass] == 0;
     if (refreshed)
-        for (int k = 0; k < kNumClass; ++k)
-            ctx->self_batch->plan.n_items[k] = (int)rc[k];
+        for (int k = 0; k < kNumClass; ++k) {
+            Plan &pl = ctx->self_batch->plan;
+            pl.n_items[k] = (int)rc[k];
+            pl.variant[k] = variant_of_class(k, pl.n_items[k], pl.tuning);
+        }
     if (ctx->self_batch && (keep_plan || refreshed))
         ctx->self_batch->versions[0] = ctx->layout_version;
     if (ctx->self_batch && !keep_plan && !refreshed) {
