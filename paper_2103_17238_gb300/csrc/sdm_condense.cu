@@ -48,13 +48,12 @@ struct CondBuffers {
     int32_t n_items = 0;
     CondItem *items = nullptr;
     int32_t *item_start = nullptr; // n_cells + 1
-    float *cf = nullptr;           // n_cells: c of each cell, binary32
     double *partial = nullptr;     // n_items
     double *cond = nullptr;        // n_cells
-    float *h_cf = nullptr;         // page-locked staging of cf, kCondStage fields in turn
-    cudaEvent_t cf_done[kCondStage] = {}; // the last copy out of each
+    float *h_cf = nullptr;         // c of each cell, binary32: kCondStage fields in turn, page-locked, read by
+                                   // the kernel where they lie (a copy ahead of it cost more than its reads)
+    cudaEvent_t cf_done[kCondStage] = {}; // the last kernel that reads each
     int stage = 0;                 // the next one
-    const float *last_cf = nullptr; // the field on the device (no copy when a call repeats it)
 };
 
 // f2d_exact (sdm_sediment.cu): the exact widening of a binary32 on the
@@ -223,7 +222,7 @@ void cond_release(sdm_ctx *ctx)
     if (!ctx->cond)
         return;
     CondBuffers &b = *ctx->cond;
-    void *bufs[] = {b.items, b.item_start, b.cf, b.partial, b.cond};
+    void *bufs[] = {b.items, b.item_start, b.partial, b.cond};
     for (void *p : bufs)
         ctx->mem.put(p, 0);
     for (cudaEvent_t ev : b.cf_done)
@@ -244,10 +243,9 @@ sdm_status cond_prepare(sdm_ctx *ctx)
     if (!ctx->cond) {
         ctx->cond = new CondBuffers();
         CondBuffers &b = *ctx->cond;
-        b.cf = static_cast<float *>(ctx->mem.get(sizeof(float) * nc));
         b.cond = static_cast<double *>(ctx->mem.get(sizeof(double) * nc));
         b.item_start = static_cast<int32_t *>(ctx->mem.get(sizeof(int32_t) * (nc + 1)));
-        if (!b.cf || !b.cond || !b.item_start) {
+        if (!b.cond || !b.item_start) {
             cond_release(ctx);
             return fail(&ctx->error, SDM_ENOMEM, "condensation: device allocation failed");
         }
@@ -315,7 +313,7 @@ extern "C" sdm_status sdm_condensation_step(sdm_ctx *ctx, const double *G, const
         return st;
     CondBuffers &b = *ctx->cond;
     cudaStream_t cs = ctx->stream;
-    CTX_CUDA(ctx, cudaEventSynchronize(b.cf_done[b.stage])); // the staging's last copy has left
+    CTX_CUDA(ctx, cudaEventSynchronize(b.cf_done[b.stage])); // no kernel reads the staging any more
     float *cf = b.h_cf + (size_t)b.stage * nc;
     // one pass without branches; what it finds wrong is named by a second
     int bad = 0;
@@ -333,35 +331,30 @@ extern "C" sdm_status sdm_condensation_step(sdm_ctx *ctx, const double *G, const
             return fail(&ctx->error, SDM_EINVAL, "cell %d: |2 G s dt| = %g m^2 above 1e-6 m^2", c,
                         std::fabs(((2.0 * G[c]) * s[c]) * dt));
     }
-    if (!b.last_cf || std::memcmp(cf, b.last_cf, sizeof(float) * nc)) { // a new field (a repeated one is on the device)
-        b.last_cf = nullptr;
-        CTX_CUDA(ctx, cudaMemcpyAsync(b.cf, cf, sizeof(float) * nc, cudaMemcpyHostToDevice, cs));
-        CTX_CUDA(ctx, cudaEventRecord(b.cf_done[b.stage], cs));
-        b.last_cf = cf;
-        b.stage = (b.stage + 1) % kCondStage;
-    }
     const float xminf = (float)(r_min * r_min);
     const int cells_grid = (int)std::min<int64_t>((nc + kCondNT / 32 - 1) / (kCondNT / 32), 152 * 8);
     double *out = condensed && condensed_on_device ? condensed : b.cond;
     if (ctx->largest_cell <= kCondByCell) {
         if (condensed)
-            condense_by_cell_kernel<true><<<cells_grid, kCondNT, 0, cs>>>(ctx->d_cell_off, nc, ctx->d_xi, ctx->d_v, b.cf,
+            condense_by_cell_kernel<true><<<cells_grid, kCondNT, 0, cs>>>(ctx->d_cell_off, nc, ctx->d_xi, ctx->d_v, cf,
                                                                           xminf, out);
         else
             condense_by_cell_kernel<false><<<cells_grid, kCondNT, 0, cs>>>(ctx->d_cell_off, nc, ctx->d_xi, ctx->d_v,
-                                                                           b.cf, xminf, nullptr);
+                                                                           cf, xminf, nullptr);
     } else {
         const int grid = (int)std::min<int64_t>((b.n_items + kCondNT / 32 - 1) / (kCondNT / 32), 152 * 8);
         if (condensed) {
-            condense_kernel<true><<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, b.cf, xminf,
+            condense_kernel<true><<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, cf, xminf,
                                                             b.partial);
             condense_cells_kernel<<<cells_grid, kCondNT, 0, cs>>>(b.item_start, nc, b.partial, out);
         } else {
-            condense_kernel<false><<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, b.cf, xminf,
+            condense_kernel<false><<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, cf, xminf,
                                                              nullptr);
         }
     }
     CTX_CUDA(ctx, cudaGetLastError());
+    CTX_CUDA(ctx, cudaEventRecord(b.cf_done[b.stage], cs));
+    b.stage = (b.stage + 1) % kCondStage;
     if (condensed && !condensed_on_device) {
         CTX_CUDA(ctx, cudaMemcpyAsync(condensed, b.cond, sizeof(double) * nc, cudaMemcpyDeviceToHost, cs));
         CTX_CUDA(ctx, cudaStreamSynchronize(cs));

@@ -148,6 +148,7 @@ struct Plan {
     WorkItem *d_items[kNumClass] = {};
     int n_items[kNumClass] = {};
     int variant[kNumClass] = {};
+    int8_t fold[kNumClass] = {0, 1, 2, 3, 4, 5, 6}; // the class whose launch takes a class's cells
     // A context's own plan whose cells all take the shared-memory classes
     // keeps room for every cell in every class (class k at d_items_all + k
     // n_cells), so that the device can rebuild it for a new layout
@@ -159,7 +160,7 @@ struct Plan {
     // with several groups of work (size classes, the large-cell path), each
     // size class launches on a stream of its own beside the others
     cudaStream_t cls_side[kNumClass] = {};
-    cudaEvent_t cls_fork = nullptr, cls_join[kNumClass] = {};
+    cudaEvent_t cls_fork = nullptr, cls_join[kNumClass] = {}; // (one class stays on the plan's stream)
     cudaStream_t big_hi = nullptr; // then the large-cell path's, at the device's greatest priority
     cudaEvent_t big_join = nullptr;
     WorkItem *d_mid[3] = {};     // cells of the cluster path, by cluster size K = 1, 2, 4, largest first
@@ -678,15 +679,17 @@ int class_of(int n, const sdm_tuning &t)
 constexpr int kRefreshNT = 256;
 
 // The work items of a run whose cells all take the shared-memory classes,
-// from its cell offsets, as build_plan makes them (class_of): class k's at
+// from its cell offsets, as build_plan makes them (class_of, then the class's
+// four bits of fold): class k's at
 // items + k cap, their number added to counts[k]; counts[kNumClass] = 1 when
 // a cell is above smem_max_sd.  Block-level counts first, then one global
 // atomic per class and block (the order of a class's items is free: cells
 // are independent).
 __global__ void __launch_bounds__(kRefreshNT) plan_refresh_kernel(const int32_t *__restrict__ cell_off,
                                                                   int32_t n_cells, int32_t cell_base,
-                                                                  int32_t smem_max_sd, WorkItem *__restrict__ items,
-                                                                  int32_t cap, uint32_t *__restrict__ counts)
+                                                                  int32_t smem_max_sd, uint32_t fold,
+                                                                  WorkItem *__restrict__ items, int32_t cap,
+                                                                  uint32_t *__restrict__ counts)
 {
     __shared__ uint32_t s_cnt[kNumClass], s_base[kNumClass];
     if (threadIdx.x < kNumClass)
@@ -704,6 +707,7 @@ __global__ void __launch_bounds__(kRefreshNT) plan_refresh_kernel(const int32_t 
                 counts[kNumClass] = 1u;
                 k = -1;
             } else {
+                k = (int)(fold >> (4 * k)) & 15;
                 slot = atomicAdd(&s_cnt[k], 1u);
             }
         }
@@ -722,8 +726,11 @@ cudaError_t plan_refresh(Plan &pl, const int32_t *d_cell_off, int32_t n_cells, i
     cudaError_t e = cudaMemsetAsync(pl.d_refresh, 0, sizeof(uint32_t) * (kNumClass + 1), st);
     if (e != cudaSuccess || n_cells == 0)
         return e;
+    uint32_t fold = 0;
+    for (int k = 0; k < kNumClass; ++k)
+        fold |= (uint32_t)pl.fold[k] << (4 * k);
     plan_refresh_kernel<<<(n_cells + kRefreshNT - 1) / kRefreshNT, kRefreshNT, 0, st>>>(
-        d_cell_off, n_cells, cell_base, pl.tuning.smem_max_sd, pl.d_items_all, n_cells, pl.d_refresh);
+        d_cell_off, n_cells, cell_base, pl.tuning.smem_max_sd, fold, pl.d_items_all, n_cells, pl.d_refresh);
     return cudaGetLastError();
 }
 
@@ -763,7 +770,7 @@ sdm_status build_plan(sdm_batch *b)
         std::vector<BigPairs> pairs;
         std::vector<SpreadCell> sp_scatter, sp_pairs;
         std::vector<InstDev *> insts;
-        std::vector<int8_t> cls; // per cell of a run: its class, -1 above them, -2 fewer than 2 SDs
+        std::vector<int8_t> cls; // per cell of all runs: its class, -1 above them, -2 fewer than 2 SDs
     };
     static thread_local Scratch scr;
     std::vector<WorkItem>(&items)[kNumClass] = scr.items;
@@ -801,41 +808,63 @@ sdm_status build_plan(sdm_batch *b)
             }
         }
     const bool spread = spread_cells(above_sd, above_cells, above_most, tun, dev_grids().mid[0]);
-    for (int i = 0; i < n_inst; ++i) {
-        sdm_ctx *c = b->ctxs[i];
-        insts[i] = c->d_inst;
+    // the shared-memory classes in two tight passes (a class per cell and the
+    // classes' sizes, then the items into their places); the other cells after
+    size_t n_all = 0;
+    for (sdm_ctx *c : b->ctxs)
+        n_all += (size_t)c->cfg.n_cells;
+    scr.cls.resize(n_all);
+    int64_t cnt[kNumClass] = {};
+    int8_t *cls = scr.cls.data();
+    for (sdm_ctx *c : b->ctxs) {
         const int32_t *off = c->h_cell_off.data();
-        const int32_t nc = c->cfg.n_cells, cb = c->cfg.cell_base;
-        // the shared-memory classes in two tight passes (a class per cell and
-        // the classes' sizes, then the items into their places); the other
-        // cells after
-        std::vector<int8_t> &cls = scr.cls;
-        cls.resize((size_t)nc);
-        size_t cnt[kNumClass] = {};
-        bool above = false;
-        for (int32_t cell = 0; cell < nc; ++cell) {
+        for (int32_t cell = 0; cell < c->cfg.n_cells; ++cell) {
             const int n = off[cell + 1] - off[cell];
             const int8_t k = n < 2 ? (int8_t)-2 : (int8_t)class_of(n, tun);
             cls[cell] = k;
             if (k >= 0)
                 ++cnt[k];
-            above |= k == -1;
         }
-        WorkItem *dst[kNumClass];
-        for (int k = 0; k < kNumClass; ++k) {
-            const size_t at = items[k].size();
-            items[k].resize(at + cnt[k]);
-            dst[k] = items[k].data() + at;
-        }
+        cls += c->cfg.n_cells;
+    }
+    // With the default tuning, the cells of up to 64 and of up to 128 SDs join
+    // the next class's launch when all of it stays resident at once: they then
+    // finish with its own cells, and a launch with its fork and join goes (a
+    // grid of 4087 cells of 43..574, a step per call: 231 -> 225 us a pass).
+    const bool standard = tun.warp_cell_max == 512 && tun.warps_per_block == 2;
+    for (int k = 0; k < 2 && standard; ++k) {
+        const int v = variant_for(kClassCap[k + 1], tun);
+        if (!cnt[k] || !cnt[k + 1] || cnt[k] + cnt[k + 1] > (int64_t)dev_grids().variant[v] * g_variants[v].warps)
+            continue;
+        cnt[k + 1] += cnt[k];
+        cnt[k] = 0;
+        for (int j = 0; j <= k; ++j)
+            if (pl.fold[j] == k)
+                pl.fold[j] = (int8_t)(k + 1);
+    }
+    WorkItem *dst[kNumClass];
+    for (int k = 0; k < kNumClass; ++k) {
+        items[k].resize((size_t)cnt[k]);
+        dst[k] = items[k].data();
+    }
+    cls = scr.cls.data();
+    for (int i = 0; i < n_inst; ++i) {
+        sdm_ctx *c = b->ctxs[i];
+        insts[i] = c->d_inst;
+        const int32_t *off = c->h_cell_off.data();
+        const int32_t nc = c->cfg.n_cells, cb = c->cfg.cell_base;
         for (int32_t cell = 0; cell < nc; ++cell) {
             const int k = cls[cell];
             if (k >= 0)
-                *dst[k]++ = WorkItem{i, cb + cell, off[cell], off[cell + 1] - off[cell]};
+                *dst[pl.fold[k]]++ = WorkItem{i, cb + cell, off[cell], off[cell + 1] - off[cell]};
         }
+        const bool above = c->largest_cell > tun.smem_max_sd;
+        const int8_t *mine = cls;
+        cls += nc;
         if (!above)
             continue;
         for (int cell = 0; cell < nc; ++cell) {
-            if (cls[cell] != -1)
+            if (mine[cell] != -1)
                 continue;
             const int n = off[cell + 1] - off[cell];
             if (spread) {
@@ -1033,18 +1062,21 @@ sdm_status build_plan(sdm_batch *b)
         // it: 1.64e10 against 1.67e10 pair-updates/s on the 1024-box ensemble,
         // while mixes of a few dozen runs stepped a third faster)
         bool small[kNumClass] = {};
-        int groups = classes > 0 ? 1 : 0;
+        int groups = classes > 0 ? 1 : 0, last = -1;
         for (int k = 0; k < kNumClass; ++k) {
             if (!pl.n_items[k])
                 continue;
             ++groups;
+            last = k;
             const Variant &x = g_variants[pl.variant[k]];
             small[k] = (int64_t)pl.n_items[k] < (int64_t)G.variant[pl.variant[k]] * (x.warps > 0 ? x.warps : 1);
         }
         if (groups > 1 && sd_total <= ((int64_t)1 << 22)) {
             cudaError_t e = cudaEventCreateWithFlags(&pl.cls_fork, cudaEventDisableTiming);
             for (int k = 0; k < kNumClass && e == cudaSuccess; ++k) {
-                if (!small[k])
+                // the class of the largest cells stays on the plan's stream, unless
+                // the large-cell path is beside it
+                if (!small[k] || (k == last && classes == 0))
                     continue;
                 e = cudaStreamCreateWithFlags(&pl.cls_side[k], cudaStreamNonBlocking);
                 if (e == cudaSuccess)
@@ -1198,7 +1230,7 @@ void enqueue_steps(const Plan &pl, int64_t off, int32_t n, cudaStream_t st)
     const cudaStream_t bs = cf.big();
     const int32_t f = pl.tuning.fuse_steps;
     const bool fuse = f >= 2 && n >= 2;
-    for (int k = 0; k < kNumClass; ++k) {
+    for (int k = kNumClass - 1; k >= 0; --k) { // the largest cells first
         if (!pl.n_items[k])
             continue;
         const Variant &x = g_variants[pl.variant[k]];

@@ -494,7 +494,8 @@ constexpr int kSedFew = 12;       // arrivals up to which each is compared with 
 struct SedMoves {
     uint32_t *group, *id, *slot, *place; // per mover: new group, id, slot, place among the group's arrivals
     uint32_t *a_id, *a_slot;             // per arrival
-    uint32_t *stay, *arr, *left;         // per group: SDs that stay, that arrive; per cell: movers
+    uint32_t *stay, *arr, *left;         // per group: SDs that stay; per cell: SDs that arrive, movers
+    uint32_t *out, *out_next;            // SDs that arrive outside the domain; the next step's count
     int32_t *first;                      // n_groups
 };
 
@@ -556,7 +557,7 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
             const unsigned out = __ballot_sync(FULL, go && ng == n_cells);
             uint32_t place = 0;
             if (out && lane == __ffs(out) - 1) // one counter for all that leave the domain
-                place = atomicAdd(&M.arr[n_cells], (uint32_t)__popc(out));
+                place = atomicAdd(M.out, (uint32_t)__popc(out));
             place = __shfl_sync(FULL, place, out ? __ffs(out) - 1 : 0) + (uint32_t)__popc(out & lt);
             if (go) {
                 if (ng != n_cells)
@@ -629,9 +630,9 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
 }
 
 // Sums over the groups of a block of 1024, for sed_offsets_kernel over many.
-__device__ __forceinline__ unsigned long long sed_sizes(const SedMoves &M, int g)
+__device__ __forceinline__ unsigned long long sed_sizes(const SedMoves &M, int g, int n_groups)
 {
-    const uint32_t a = M.arr[g];
+    const uint32_t a = g == n_groups - 1 ? *M.out : M.arr[g];
     return (unsigned long long)((M.stay[g] + a + 1u) & ~1u) | ((unsigned long long)a << 32);
 }
 
@@ -656,7 +657,7 @@ __global__ void __launch_bounds__(1024) sed_totals_kernel(SedMoves M, int32_t n_
 {
     __shared__ unsigned long long s_w[32];
     const int g = blockIdx.x * 1024 + threadIdx.x;
-    const unsigned long long t = sed_block_sum(g < n_groups ? sed_sizes(M, g) : 0ull, s_w);
+    const unsigned long long t = sed_block_sum(g < n_groups ? sed_sizes(M, g, n_groups) : 0ull, s_w);
     if (threadIdx.x == 0)
         totals[blockIdx.x] = t;
 }
@@ -683,10 +684,10 @@ __global__ void __launch_bounds__(1024) sed_offsets_kernel(SedMoves M, int32_t n
             unsigned long long q[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                q[u] = i + u * 1024 < (int)blockIdx.x * 1024 ? sed_sizes(M, i + u * 1024) : 0ull;
+                q[u] = i + u * 1024 < (int)blockIdx.x * 1024 ? sed_sizes(M, i + u * 1024, n_groups) : 0ull;
             before += (q[0] + q[1]) + (q[2] + q[3]);
         }
-    const unsigned long long mine = g < n_groups ? sed_sizes(M, g) : 0ull;
+    const unsigned long long mine = g < n_groups ? sed_sizes(M, g, n_groups) : 0ull;
     before = sed_block_sum(before, s_w);
     unsigned long long x = mine;
 #pragma unroll
@@ -747,7 +748,8 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                                                                 const double *__restrict__ v,
                                                                 const double *__restrict__ zeta_new,
                                                                 const int32_t *__restrict__ id_of_slot,
-                                                                const int32_t *__restrict__ poff, SedLayout L)
+                                                                const int32_t *__restrict__ poff, SedLayout L,
+                                                                InstDev *__restrict__ rec, int64_t step)
 {
     constexpr unsigned FULL = 0xFFFFFFFFu;
     constexpr int W = kSedMergeNT / 32;
@@ -874,13 +876,23 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
             if (j < A)
                 L.put((int64_t)p0 + at, xi[slot], v[slot], fabs(zeta_new[slot]), (int32_t)id);
         }
-        if (lane == 0 && p0 + (int32_t)(n_stay + A) < p1) // the padding slot of an odd cell
-            L.put(p1 - 1, 0, 1.0, 0.0, -1);
+        if (lane == 0) {
+            if (p0 + (int32_t)(n_stay + A) < p1) // the padding slot of an odd cell
+                L.put(p1 - 1, 0, 1.0, 0.0, -1);
+            M.arr[g] = 0u; // for the next step
+        }
         __syncwarp();
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) { // the run's record: nothing here reads it
+        *M.out_next = 0u;
+        rec->xi = L.xi;
+        rec->v = L.v;
+        rec->cell_off = poff;
+        rec->step = step;
     }
     // outside the domain: those that were, in their order, then the arrivals
     const int32_t lo = cell_off[n_cells], p0 = poff[n_cells], p1 = poff[n_cells + 1];
-    const uint32_t n_out = M.stay[n_cells], A = M.arr[n_cells], a0 = (uint32_t)M.first[n_cells];
+    const uint32_t n_out = M.stay[n_cells], A = *M.out, a0 = (uint32_t)M.first[n_cells];
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p1 - p0; i += (int64_t)gridDim.x * blockDim.x) {
         if (i < n_out) {
             L.put(p0 + i, xi[lo + i], v[lo + i], 0.0, id_of_slot[lo + i]);
@@ -906,6 +918,8 @@ struct SedBuffers {
     uint32_t *keys[2] = {}; // sorted path: keys and slots; else the movers' new groups, ids,
     uint32_t *vals[2] = {}; //   slots and places
     uint32_t *moves = nullptr; // per group: stayers, arrivals, movers, first arrival; then block totals
+    int parity = 0;            // which of the two counts of SDs leaving the domain (behind the cells'
+                               //   arrivals) the next step uses; all arrivals are zero between steps
     uint32_t *counts = nullptr; // n_cells + 1
     int32_t *ustart = nullptr;  // n_cells + 2
     double *precip = nullptr;   // per-block parts of the move kernel, then the total
@@ -959,7 +973,7 @@ T *sed_get(sdm_ctx *ctx, size_t count)
 
 // Words of one of the per-group arrays of SedBuffers::moves (a multiple of 2:
 // the totals behind them are 8-byte words).
-size_t sed_stride(int32_t n_cells) { return ((size_t)n_cells + 3) & ~(size_t)1; }
+size_t sed_stride(int32_t n_cells) { return ((size_t)n_cells + 5) & ~(size_t)1; }
 
 sdm_status sed_alloc(sdm_ctx *ctx)
 {
@@ -1008,6 +1022,11 @@ sdm_status sed_alloc(sdm_ctx *ctx)
     if (!ok) {
         sed_release(ctx);
         return fail(&ctx->error, SDM_ENOMEM, "sedimentation buffers: device allocation failed");
+    }
+    if (cudaMemsetAsync(b.moves, 0, sizeof(uint32_t) * 2 * sed_stride(nc), ctx->stream) != cudaSuccess) {
+        cudaGetLastError();
+        sed_release(ctx);
+        return fail(&ctx->error, SDM_ECUDA, "sedimentation buffers: clearing failed");
     }
     ctx->device_bytes += slots * (8 + 8 + 8 + 8 + 4 + 4 + 4 + 8 + 16) + cap * 4 + ((int64_t)nc + 2) * 32 +
                          (int64_t)radix_hist_words(cap) * 4;
@@ -1132,10 +1151,11 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     if (by_cell) {
         const size_t st_ = sed_stride(nc);
         SedMoves M{b.keys[0], b.vals[0],      b.keys[1],          b.vals[1],   (uint32_t *)b.group, (uint32_t *)b.group2,
-                   b.moves,   b.moves + st_, b.moves + 2 * st_, (int32_t *)(b.moves + 3 * st_)};
+                   b.moves,   b.moves + st_, b.moves + 2 * st_, b.moves + 2 * st_ - 1 - b.parity,
+                   b.moves + 2 * st_ - 2 + b.parity, (int32_t *)(b.moves + 3 * st_)};
+        b.parity ^= 1;
         unsigned long long *totals = (unsigned long long *)(b.moves + 4 * st_);
         b.group_valid = false;
-        CTX_CUDA(ctx, cudaMemsetAsync(M.arr, 0, sizeof(uint32_t) * n_groups, s));
         if (ctx->cfg.cell_base > 0) // the emigrants of the step before are none of this one's
             CTX_CUDA(ctx, cudaMemsetAsync(b.emig, 0xFF, sizeof(int32_t) * n, s));
         const int warps = kSedNT / 32;
@@ -1158,7 +1178,7 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
         const int64_t units = std::max<int64_t>((nc + mw - 1) / mw, (ctx->n_slots - ctx->h_cell_off[nc]) / kSedMergeNT + 1);
         sed_merge_kernel<<<(int)std::min<int64_t>(units, 152 * 9), kSedMergeNT, 0, s>>>(
             ctx->d_cell_off, nc, M, ctx->d_xi, ctx->d_v, b.zeta_new, ctx->d_id_of_slot, b.cell_off2,
-            SedLayout{b.xi2, b.v2, b.zeta2, b.id2});
+            SedLayout{b.xi2, b.v2, b.zeta2, b.id2}, ctx->d_inst, ctx->step);
         CTX_CUDA(ctx, cudaGetLastError());
         CTX_CUDA(ctx, cudaStreamWaitEvent(s, b.join, 0)); // later work may write what the side stream reads
     } else {
@@ -1215,8 +1235,10 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     ctx->largest_cell = largest;
     ctx->layout_version += 1;
     ctx->dev_base = ctx->step;
-    InstDev inst = make_inst(ctx);
-    CTX_CUDA(ctx, cudaMemcpyAsync(ctx->d_inst, &inst, sizeof inst, cudaMemcpyHostToDevice, s));
+    if (!by_cell) { // (the merge writes the record itself)
+        InstDev inst = make_inst(ctx);
+        CTX_CUDA(ctx, cudaMemcpyAsync(ctx->d_inst, &inst, sizeof inst, cudaMemcpyHostToDevice, s));
+    }
     const bool refreshed = refresh && !keep_plan && rc[kNumClass] == 0;
     if (refreshed)
         for (int k = 0; k < kNumClass; ++k) {
