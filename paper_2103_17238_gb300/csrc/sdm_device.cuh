@@ -36,6 +36,7 @@ struct InstDev {
     float pre_v[2];  // pre-filter: volumes of the regime bounds r1, r2 (rounded down)
     int32_t kernel, precision, n_cells;
     uint32_t status; // bit 0: a bounded device wait gave up (reported as SDM_ETIMEOUT)
+    uint32_t ticket; // blocks of a product's kernel that are done (0 between launches)
 };
 
 struct __align__(16) WorkItem {

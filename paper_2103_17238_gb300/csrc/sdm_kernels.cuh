@@ -1496,6 +1496,27 @@ __global__ void advance_steps_kernel(InstDev *const *insts, int32_t n_inst, int6
         insts[i]->step += delta ? delta[i] : n;
 }
 
+// Whether this is the last block of the grid to come here, after which it sees
+// what all of them wrote before (every thread calls it; the counter returns to 0).
+__device__ __forceinline__ bool last_block(uint32_t *ticket)
+{
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (s_last)
+            *ticket = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    return s_last;
+}
+
+// Products of up to this many blocks are finished by their last block, in one
+// launch; more by a launch of their own (wider than one block).
+constexpr int kLastBlockMax = 128;
+
 // ------------------------------------------------------------ diagnostics
 // Conservation sums of the SDs inside the domain (slots [0, n_in)): live
 // count, sum of xi (128-bit, exact) and sum of xi v: in fixed point over a
@@ -1544,6 +1565,7 @@ __device__ __forceinline__ DiagPart diag_block_reduce(DiagPart a)
         const DiagPart b = diag_shfl_down(a, d);
         diag_combine(a, b);
     }
+    __syncthreads(); // (a second reduction: the first one's sums are read)
     if (lane == 0)
         s_w[warp] = a;
     __syncthreads();
@@ -1553,8 +1575,20 @@ __device__ __forceinline__ DiagPart diag_block_reduce(DiagPart a)
     return a;
 }
 
-__global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(const InstDev *__restrict__ P, int64_t n_in,
-                                                               DiagPart *__restrict__ parts)
+__device__ __forceinline__ void diag_finish(const DiagPart *parts, int32_t n_parts, DiagPart *out)
+{
+    DiagPart a{0ull, 0ull, 0ull, 0.0};
+    for (int i = threadIdx.x; i < n_parts; i += kDiagNT) {
+        const volatile DiagPart *q = parts + i;
+        diag_combine(a, DiagPart{q->live, q->xi_lo, q->xi_hi, q->xv});
+    }
+    a = diag_block_reduce(a);
+    if (threadIdx.x == 0)
+        *out = a;
+}
+
+// out (null: parts only): the sums, from the last block (up to kLastBlockMax).
+__global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(InstDev *P, int64_t n_in, DiagPart *parts, DiagPart *out)
 {
     constexpr int Q = kDiagChunk / 64; // slot pairs per lane and round
     const int lane = threadIdx.x & 31;
@@ -1597,17 +1631,13 @@ __global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(const InstDev *__
     a = diag_block_reduce(a);
     if (threadIdx.x == 0)
         parts[blockIdx.x] = a;
+    if (out && last_block(&P->ticket))
+        diag_finish(parts, (int)gridDim.x, out);
 }
 
-__global__ void __launch_bounds__(kDiagNT) diag_final_kernel(const DiagPart *__restrict__ parts, int32_t n_parts,
-                                                             DiagPart *__restrict__ out)
+__global__ void __launch_bounds__(kDiagNT) diag_final_kernel(const DiagPart *parts, int32_t n_parts, DiagPart *out)
 {
-    DiagPart a{0ull, 0ull, 0ull, 0.0};
-    for (int i = threadIdx.x; i < n_parts; i += kDiagNT)
-        diag_combine(a, parts[i]);
-    a = diag_block_reduce(a);
-    if (threadIdx.x == 0)
-        *out = a;
+    diag_finish(parts, n_parts, out);
 }
 
 // -------------------------------------------------------------- spectrum
@@ -1878,11 +1908,35 @@ __device__ __forceinline__ double spec_divide(const SpecTab &T, int b, double x)
     return u64_to_double(__umul64hi((bits << 11) | (1ull << 63), T.recip[b]), true, w);
 }
 
+// out[b] = (sum over blocks of partial[b][block], fixed order) / den[b], by one
+// warp.
+__device__ __forceinline__ void spec_finish(const SpecTab &T, const double *partial, int32_t n_blocks, int b, double *out)
+{
+    const int lane = threadIdx.x & 31;
+    double sum = 0.0;
+    for (int j0 = lane; j0 < n_blocks; j0 += 8 * 32) { // eight loads in flight
+        double p[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            p[u] = j0 + 32 * u < n_blocks ? __ldcg(partial + (int64_t)b * n_blocks + j0 + 32 * u) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (j0 + 32 * u < n_blocks)
+                sum = __dadd_rn(sum, p[u]);
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1)
+        sum = __dadd_rn(sum, __shfl_down_sync(0xFFFFFFFFu, sum, d));
+    if (lane == 0)
+        out[b] = sum / T.den[b];
+}
+
 // Sums of every bin over all slots [0, n_slots) (padding and dead SDs hold
-// xi = 0): partial[bin][block].
-__global__ void __launch_bounds__(32 * kSpecWarps) spectrum_total_kernel(const InstDev *__restrict__ P, int64_t n_slots,
+// xi = 0): partial[bin][block]; with out, the spectrum itself from the last
+// block (up to kLastBlockMax), and the run's status word to *status.
+__global__ void __launch_bounds__(32 * kSpecWarps) spectrum_total_kernel(InstDev *P, int64_t n_slots,
                                                                          const __grid_constant__ SpecTab T,
-                                                                         double *__restrict__ partial)
+                                                                         double *partial, double *out, uint32_t *status)
 {
     __shared__ SpecSmem S;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1901,31 +1955,22 @@ __global__ void __launch_bounds__(32 * kSpecWarps) spectrum_total_kernel(const I
             sum = __dadd_rn(sum, S.part[w][lane]);
         partial[(int64_t)lane * gridDim.x + blockIdx.x] = sum;
     }
+    if (out && last_block(&P->ticket)) {
+        for (int b = warp; b < T.n_edges - 1; b += kSpecWarps)
+            spec_finish(T, partial, (int)gridDim.x, b, out);
+        if (status && threadIdx.x == 0)
+            *status = P->status;
+    }
 }
 
-// out[b] = (sum over blocks of partial[b][block], fixed order) / den[b]; one
-// warp (block) per bin.
-__global__ void spectrum_total_finalize_kernel(const double *__restrict__ partial, int32_t n_blocks,
-                                               const __grid_constant__ SpecTab T, double *__restrict__ out)
+// The spectrum from the partial sums of more blocks: one warp (block) per bin.
+__global__ void spectrum_total_finalize_kernel(const InstDev *__restrict__ P, const double *__restrict__ partial,
+                                               int32_t n_blocks, const __grid_constant__ SpecTab T,
+                                               double *__restrict__ out, uint32_t *status)
 {
-    const int b = blockIdx.x;
-    const int lane = threadIdx.x & 31;
-    double sum = 0.0;
-    for (int j0 = lane; j0 < n_blocks; j0 += 8 * 32) { // eight loads in flight
-        double p[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            p[u] = j0 + 32 * u < n_blocks ? partial[(int64_t)b * n_blocks + j0 + 32 * u] : 0.0;
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (j0 + 32 * u < n_blocks)
-                sum = __dadd_rn(sum, p[u]);
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1)
-        sum = __dadd_rn(sum, __shfl_down_sync(0xFFFFFFFFu, sum, d));
-    if (lane == 0)
-        out[b] = sum / T.den[b];
+    spec_finish(T, partial, n_blocks, blockIdx.x, out);
+    if (status && blockIdx.x == 0 && threadIdx.x == 0)
+        *status = P->status;
 }
 
 // dv/dlnr of every cell, cell-major.  One warp per cell, or (block_cells)
@@ -1988,7 +2033,7 @@ __device__ __forceinline__ bool volume_ok(double v)
 
 // Validation and per-group counts of set_attributes (groups: the cells, then
 // n_cells for the SDs outside the domain, cell id -1).  flags bit 0: an
-// invalid attribute (first bad SD index in *bad); bit 1: groups not sorted.
+// invalid attribute (*bad the complement of the first bad SD index; 0: none); bit 1: groups not sorted.
 // Each warp takes 128 consecutive SDs at a time, 32 by 32, and adds one count
 // per run of equal groups (one or two atomics per 32 for sorted input).
 __global__ void validate_count_kernel(int64_t lo, int64_t hi, const int64_t *__restrict__ xi,
@@ -2026,7 +2071,7 @@ __global__ void validate_count_kernel(int64_t lo, int64_t hi, const int64_t *__r
                     c = craw;
                 } else {
                     atomicOr(flags, 1u);
-                    atomicMin(bad, (unsigned long long)i);
+                    atomicMax(bad, ~(unsigned long long)i);
                 }
             }
             int32_t prev = __shfl_up_sync(FULL, craw, 1);
@@ -2110,23 +2155,35 @@ __global__ void place_sorted_kernel(int64_t n_sd, const uint32_t *__restrict__ g
     }
 }
 
-// Padding slots (the one slot after an odd group): dead, with a harmless
-// positive volume.
-__global__ void fill_padding_kernel(int32_t n_cells, const int32_t *__restrict__ poff, const int32_t *__restrict__ uoff,
-                                    int64_t *__restrict__ sxi, double *__restrict__ sv, int32_t *__restrict__ id_of_slot)
+// Padding slots (the one slot after an odd group): dead, with a
+// harmless positive volume; and the run's offsets and record from the block
+// that came up with poff and uoff.
+__global__ void fill_padding_kernel(int32_t n_groups, const int32_t *__restrict__ poff, const int32_t *__restrict__ uoff,
+                                    int64_t *__restrict__ sxi, double *__restrict__ sv, int32_t *__restrict__ id_of_slot,
+                                    int32_t *__restrict__ cell_off, const InstDev *__restrict__ rec_in,
+                                    InstDev *__restrict__ rec)
 {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n_cells; c += gridDim.x * blockDim.x) {
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n_groups; c += gridDim.x * blockDim.x) {
+        cell_off[c] = poff[c]; // the cells' and the end of the last one
         for (int32_t p = poff[c] + (uoff[c + 1] - uoff[c]); p < poff[c + 1]; ++p) {
             sxi[p] = 0;
             sv[p] = 1.0;
             id_of_slot[p] = -1;
         }
     }
+    constexpr int W = sizeof(InstDev) / 4;
+    static_assert(W <= 256 && sizeof(InstDev) % 4 == 0, "one block copies the record");
+    if (blockIdx.x == 0 && threadIdx.x < W)
+        reinterpret_cast<uint32_t *>(rec)[threadIdx.x] = reinterpret_cast<const uint32_t *>(rec_in)[threadIdx.x];
 }
 
+// The state in SD-id order; status (null: not wanted) receives the run's word.
 __global__ void gather_kernel(int64_t n_slots, const int64_t *__restrict__ sxi, const double *__restrict__ sv,
-                              const int32_t *__restrict__ id_of_slot, int64_t *__restrict__ xi, double *__restrict__ v)
+                              const int32_t *__restrict__ id_of_slot, int64_t *__restrict__ xi, double *__restrict__ v,
+                              const InstDev *__restrict__ P, uint32_t *status)
 {
+    if (status && blockIdx.x == 0 && threadIdx.x == 0)
+        *status = P->status;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_slots; p += (int64_t)gridDim.x * blockDim.x) {
         const int32_t id = id_of_slot[p];
         if (id < 0)

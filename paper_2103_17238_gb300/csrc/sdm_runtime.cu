@@ -227,9 +227,14 @@ struct sdm_ctx {
     // validation block in; offsets and the record out), kept between calls
     unsigned char *h_pin = nullptr;
     size_t h_pin_bytes = 0;
-    // page-locked staging of sdm_spectrum (edges and dln in, the status word
-    // back), used when the result goes to the host (the call synchronises)
+    // page-locked staging of sdm_spectrum and sdm_diagnostics (edges and dln in,
+    // results and the status word back), used when the result goes to the host
+    // (the calls synchronise)
     unsigned char *h_spec = nullptr;
+    // page-locked home of small states on their way in (sdm_set_attributes) and
+    // out (sdm_get_attributes), which the kernels read and write where they lie
+    unsigned char *h_small = nullptr;
+    cudaEvent_t small_ev = nullptr; // the last kernel that reads it
     // copies of host input run on their own stream, in kInChunks pieces, so
     // that each piece is validated while the next one is on its way
     cudaStream_t cstream = nullptr;
@@ -1515,6 +1520,8 @@ InstDev make_inst(const sdm_ctx *c)
     return d;
 }
 
+sdm_status status_result(sdm_ctx *ctx, uint32_t status);
+
 // Reads the run's device status word (after the stream has been synchronised).
 sdm_status check_device_status(sdm_ctx *ctx)
 {
@@ -1522,12 +1529,52 @@ sdm_status check_device_status(sdm_ctx *ctx)
     cudaError_t e = cudaMemcpy(&status, &ctx->d_inst->status, sizeof status, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "status read");
+    return status_result(ctx, status);
+}
+
+sdm_status status_result(sdm_ctx *ctx, uint32_t status)
+{
     if (status & 1u)
         return fail(&ctx->error, SDM_ETIMEOUT, "a device-side wait for a bulk copy gave up; results are incomplete");
     if (status & 2u)
         return fail(&ctx->error, SDM_ESTATE,
                     "a sort bucket of a large cell outgrew its room (its keys are far from uniform): that cell was not "
                     "stepped; results are incomplete");
+    return SDM_OK;
+}
+
+// States of up to kSmallSd SDs go between host arrays and the device through
+// h_small: copies of pageable memory cost their calls tens of us (a box of 4096:
+// twelve of them in, four out).
+constexpr int64_t kSmallSd = 16384;
+
+sdm_status small_staging(sdm_ctx *ctx)
+{
+    if (ctx->h_small)
+        return SDM_OK;
+    cudaError_t e = cudaHostAlloc((void **)&ctx->h_small, (size_t)kSmallSd * 20 + 64, cudaHostAllocDefault);
+    if (e == cudaSuccess)
+        e = cudaEventCreateWithFlags(&ctx->small_ev, cudaEventDisableTiming);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        if (ctx->h_small)
+            cudaFreeHost(ctx->h_small);
+        ctx->h_small = nullptr;
+        return fail(&ctx->error, SDM_ENOMEM, "page-locked host staging allocation failed");
+    }
+    return SDM_OK;
+}
+
+// h_spec: edges on their way in, or a product on its way out; then the status word.
+constexpr size_t kSpecPin = sizeof(double) * 2 * kMaxEdges + 64;
+
+sdm_status spec_staging(sdm_ctx *ctx)
+{
+    if (!ctx->h_spec && cudaHostAlloc((void **)&ctx->h_spec, kSpecPin, cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->h_spec = nullptr;
+        return fail(&ctx->error, SDM_ENOMEM, "page-locked host staging allocation failed");
+    }
     return SDM_OK;
 }
 
@@ -1642,12 +1689,25 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
     const double *dv = volume;
     const int32_t *dcell = cell_id;
     const size_t b_stage = b_xi + b_v + b_c;
-    // SD ranges of the pieces (one piece for device input)
-    const int n_in = on_device ? 1 : kInChunks;
+    // SD ranges of the pieces (one piece for device input and small states)
+    const bool small = !on_device && n_sd <= kSmallSd;
+    const int n_in = on_device || small ? 1 : kInChunks;
     int64_t piece[kInChunks + 1];
     for (int k = 0; k <= n_in; ++k)
         piece[k] = n_sd * k / n_in;
-    if (!on_device) {
+    if (small) {
+        st = small_staging(ctx);
+        if (st != SDM_OK)
+            return st;
+        CTX_CUDA(ctx, cudaEventSynchronize(ctx->small_ev)); // an earlier call's kernel has read its state
+        unsigned char *p = ctx->h_small;
+        std::memcpy(p, xi, b_xi);
+        std::memcpy(p + b_xi, volume, b_v);
+        std::memcpy(p + b_xi + b_v, cell_id, b_c);
+        dxi = (const int64_t *)p;
+        dv = (const double *)(p + b_xi);
+        dcell = (const int32_t *)(p + b_xi + b_v);
+    } else if (!on_device) {
         stage = mem.get(b_stage);
         if (!stage)
             return fail(&ctx->error, SDM_ENOMEM, "staging allocation failed");
@@ -1710,9 +1770,8 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
         ctx->h_pin_bytes = b_pin;
     }
     CTX_CUDA(ctx, cudaMemsetAsync(meta, 0, b_counts, s));
-    CTX_CUDA(ctx, cudaMemsetAsync(d_bad, 0xFF, sizeof(unsigned long long), s));
     for (int k = 0; k < n_in; ++k) { // piece k once it has landed (pieces land in order)
-        if (!on_device)
+        if (!on_device && !small)
             CTX_CUDA(ctx, cudaStreamWaitEvent(s, ctx->in_ev[k], 0));
         if (piece[k + 1] > piece[k])
             validate_count_kernel<<<(int)std::min<int64_t>((piece[k + 1] - piece[k] + 1023) / 1024, 1 << 20), 256, 0, s>>>(
@@ -1725,7 +1784,7 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
     const uint32_t *counts = (const uint32_t *)ctx->h_pin;
     const uint32_t flags = counts[n_groups];
     const unsigned long long bad =
-        *(const unsigned long long *)(ctx->h_pin + ((uintptr_t)d_bad - (uintptr_t)meta));
+        ~*(const unsigned long long *)(ctx->h_pin + ((uintptr_t)d_bad - (uintptr_t)meta));
     if (flags & 1u) {
         mem.put(meta, b_counts);
         mem.put(stage, b_stage);
@@ -1752,7 +1811,7 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
     // keep increasing id within a cell) and the layout gathered
     const bool unsorted = (flags & 2u) != 0;
     auto a256 = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t b_off = a256(sizeof(int32_t) * 2 * (n_groups + 1)), b_key = a256(sizeof(uint32_t) * n_sd);
+    const size_t b_off = a256(p_rec - p_off + sizeof(InstDev)), b_key = a256(sizeof(uint32_t) * n_sd);
     const size_t b_aux = b_off + (unsorted ? 2 * b_key + sizeof(uint32_t) * radix_hist_words(n_sd) : 0);
     void *aux = mem.get(b_aux);
     if (!aux) {
@@ -1762,8 +1821,6 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
     }
     int32_t *d_poff = (int32_t *)aux;
     int32_t *d_uoff = d_poff + (n_groups + 1);
-    // poff and uoff lie back to back in both buffers: one copy
-    CTX_CUDA(ctx, cudaMemcpyAsync(d_poff, poff, sizeof(int32_t) * 2 * (n_groups + 1), cudaMemcpyHostToDevice, s));
     // a context's own launch plan depends only on the padded layout and the
     // launch tuning: kept when both are unchanged
     std::vector<int32_t> cell_off(poff, poff + n_cells + 1);
@@ -1782,8 +1839,8 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
     // once; the next call writes that staging only after its own
     // synchronisation, which follows these copies on the stream.  The
     // scratch is released in stream order: nothing waits for the kernels.
-    CTX_CUDA(ctx, cudaMemcpyAsync(ctx->d_cell_off, poff, sizeof(int32_t) * (n_cells + 1), cudaMemcpyHostToDevice, s));
-    CTX_CUDA(ctx, cudaMemcpyAsync(ctx->d_inst, inst, sizeof *inst, cudaMemcpyHostToDevice, s));
+    // poff, uoff and the record lie alike in both buffers: one copy
+    CTX_CUDA(ctx, cudaMemcpyAsync(d_poff, poff, p_rec - p_off + sizeof *inst, cudaMemcpyHostToDevice, s));
     if (unsorted) {
         char *w = (char *)aux + b_off;
         const int bits = 32 - __builtin_clz((unsigned)n_cells | 1u);
@@ -1804,8 +1861,11 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
                                             ctx->d_id_of_slot);
     }
     // after the sort, whose other pair of arrays lies over the padding too
-    fill_padding_kernel<<<(n_groups + 255) / 256, 256, 0, s>>>(n_groups, d_poff, d_uoff, ctx->d_xi, ctx->d_v,
-                                                                ctx->d_id_of_slot);
+    fill_padding_kernel<<<(n_groups + 255) / 256, 256, 0, s>>>(
+        n_groups, d_poff, d_uoff, ctx->d_xi, ctx->d_v, ctx->d_id_of_slot, ctx->d_cell_off,
+        (const InstDev *)((char *)aux + (p_rec - p_off)), ctx->d_inst);
+    if (small)
+        CTX_CUDA(ctx, cudaEventRecord(ctx->small_ev, s));
     CTX_CUDA(ctx, cudaGetLastError());
     mem.put(aux, b_aux);
     mem.put(meta, b_counts);
@@ -1890,28 +1950,30 @@ sdm_status sdm_spectrum(sdm_ctx *ctx, const double *r_edges, int32_t n_edges, in
     }
     const size_t b_edges = sizeof(double) * host_e.size(), b_out = sizeof(double) * n_out;
     const size_t b_part = total ? sizeof(double) * (size_t)grid * kSpecMaxBins : (few ? 0 : b_out);
-    const size_t b_tmp = b_edges + b_part + (out_on_device ? 0 : b_out);
+    const bool direct = total && !out_on_device; // a total goes to the host from the kernel
+    const size_t b_tmp = b_edges + b_part + (out_on_device || direct ? 0 : b_out);
     // host result: the edges go out of, and the status word comes back into,
     // page-locked staging (the call synchronises before it returns, so the
     // next call finds the staging free)
-    constexpr size_t kSpecPin = sizeof(double) * 2 * kMaxEdges + 64;
-    if (!out_on_device && !ctx->h_spec) {
-        if (cudaHostAlloc((void **)&ctx->h_spec, kSpecPin, cudaHostAllocDefault) != cudaSuccess) {
-            cudaGetLastError();
-            ctx->h_spec = nullptr;
-            return fail(&ctx->error, SDM_ENOMEM, "page-locked host staging allocation failed");
-        }
+    if (!out_on_device) {
+        st = spec_staging(ctx);
+        if (st != SDM_OK)
+            return st;
     }
     char *tmp = (char *)ctx->mem.get(b_tmp);
     if (!tmp)
         return fail(&ctx->error, SDM_ENOMEM, "allocation failed");
     double *d_part = (double *)(tmp + b_edges);
-    double *d_out = out_on_device ? out : (double *)(tmp + b_edges + b_part);
+    uint32_t *h_status = out_on_device ? nullptr : (uint32_t *)(ctx->h_spec + sizeof(double) * 2 * kMaxEdges);
+    double *d_out = out_on_device ? out : (direct ? (double *)ctx->h_spec : (double *)(tmp + b_edges + b_part));
     if (few) {
         const SpecTab T = spec_table(r_edges, n_edges, vol);
         if (total) {
-            spectrum_total_kernel<<<grid, 32 * kSpecWarps, 0, s>>>(ctx->d_inst, n_in, T, d_part);
-            spectrum_total_finalize_kernel<<<nb, 32, 0, s>>>(d_part, grid, T, d_out);
+            const bool one = grid <= kLastBlockMax;
+            spectrum_total_kernel<<<grid, 32 * kSpecWarps, 0, s>>>(ctx->d_inst, n_in, T, d_part, one ? d_out : nullptr,
+                                                                   h_status);
+            if (!one)
+                spectrum_total_finalize_kernel<<<nb, 32, 0, s>>>(ctx->d_inst, d_part, grid, T, d_out, h_status);
         } else {
             // a block per cell where a warp alone would take many rounds
             const int block_cells = n_in / ctx->cfg.n_cells > 4 * kSpecChunk ? 1 : 0;
@@ -1934,10 +1996,13 @@ sdm_status sdm_spectrum(sdm_ctx *ctx, const double *r_edges, int32_t n_edges, in
     }
     CTX_CUDA(ctx, cudaGetLastError());
     if (!out_on_device) {
-        uint32_t *h_status = (uint32_t *)(ctx->h_spec + sizeof(double) * 2 * kMaxEdges);
-        CTX_CUDA(ctx, cudaMemcpyAsync(out, d_out, b_out, cudaMemcpyDeviceToHost, s));
-        CTX_CUDA(ctx, cudaMemcpyAsync(h_status, &ctx->d_inst->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        if (!direct) {
+            CTX_CUDA(ctx, cudaMemcpyAsync(out, d_out, b_out, cudaMemcpyDeviceToHost, s));
+            CTX_CUDA(ctx, cudaMemcpyAsync(h_status, &ctx->d_inst->status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        }
         CTX_CUDA(ctx, cudaStreamSynchronize(s));
+        if (direct)
+            std::memcpy(out, ctx->h_spec, b_out);
         ctx->mem.put(tmp, b_tmp);
         if (*h_status & 1u)
             return fail(&ctx->error, SDM_ETIMEOUT, "a device-side wait for a bulk copy gave up; results are incomplete");
@@ -1960,16 +2025,35 @@ sdm_status sdm_get_attributes(sdm_ctx *ctx, int64_t *xi, double *volume, int on_
     cudaStream_t s = ctx->stream;
     const int64_t n = ctx->n_sd;
     if (on_device) {
-        gather_kernel<<<grid_of(ctx->n_slots), 256, 0, s>>>(ctx->n_slots, ctx->d_xi, ctx->d_v, ctx->d_id_of_slot, xi, volume);
+        gather_kernel<<<grid_of(ctx->n_slots), 256, 0, s>>>(ctx->n_slots, ctx->d_xi, ctx->d_v, ctx->d_id_of_slot, xi,
+                                                            volume, ctx->d_inst, nullptr);
         CTX_CUDA(ctx, cudaGetLastError());
         return SDM_OK;
     }
     const size_t bx = sizeof(int64_t) * n, bv = sizeof(double) * n;
+    if (n <= kSmallSd) {
+        st = small_staging(ctx);
+        if (st != SDM_OK)
+            return st;
+        uint32_t *h_status = (uint32_t *)(ctx->h_small + (size_t)kSmallSd * 20);
+        // on the stream behind whatever still reads the staging
+        gather_kernel<<<grid_of(ctx->n_slots), 256, 0, s>>>(
+            ctx->n_slots, ctx->d_xi, ctx->d_v, ctx->d_id_of_slot, xi ? (int64_t *)ctx->h_small : nullptr,
+            volume ? (double *)(ctx->h_small + bx) : nullptr, ctx->d_inst, h_status);
+        CTX_CUDA(ctx, cudaGetLastError());
+        CTX_CUDA(ctx, cudaStreamSynchronize(s));
+        if (xi)
+            std::memcpy(xi, ctx->h_small, bx);
+        if (volume)
+            std::memcpy(volume, ctx->h_small + bx, bv);
+        return status_result(ctx, *h_status);
+    }
     char *tmp = (char *)ctx->mem.get(bx + bv);
     if (!tmp)
         return fail(&ctx->error, SDM_ENOMEM, "allocation failed");
     gather_kernel<<<grid_of(ctx->n_slots), 256, 0, s>>>(ctx->n_slots, ctx->d_xi, ctx->d_v, ctx->d_id_of_slot,
-                                       xi ? (int64_t *)tmp : nullptr, volume ? (double *)(tmp + bx) : nullptr);
+                                                        xi ? (int64_t *)tmp : nullptr,
+                                                        volume ? (double *)(tmp + bx) : nullptr, ctx->d_inst, nullptr);
     CTX_CUDA(ctx, cudaGetLastError());
     if (xi)
         CTX_CUDA(ctx, cudaMemcpyAsync(xi, tmp, bx, cudaMemcpyDeviceToHost, s));
@@ -2019,6 +2103,10 @@ sdm_status sdm_destroy(sdm_ctx *ctx)
         cudaFreeHost(ctx->h_pin);
     if (ctx->h_spec)
         cudaFreeHost(ctx->h_spec);
+    if (ctx->h_small)
+        cudaFreeHost(ctx->h_small);
+    if (ctx->small_ev)
+        cudaEventDestroy(ctx->small_ev);
     for (cudaEvent_t ev : ctx->in_ev)
         if (ev)
             cudaEventDestroy(ev);
@@ -2124,18 +2212,25 @@ sdm_status sdm_diagnostics(sdm_ctx *ctx, sdm_diag *out)
     const int64_t n_in = ctx->h_cell_off[ctx->cfg.n_cells]; // slots of the cells (not the SDs outside)
     // the grid depends on the size only: the same state gives the same bits
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(kDiagBlocks, (n_in + kDiagChunk * (kDiagNT / 32) - 1) / (kDiagChunk * (kDiagNT / 32))));
-    const size_t bytes = sizeof(DiagPart) * ((size_t)blocks + 1);
+    const size_t bytes = sizeof(DiagPart) * (size_t)blocks;
     DiagPart *d = (DiagPart *)ctx->mem.get(bytes);
     if (!d)
         return fail(&ctx->error, SDM_ENOMEM, "diagnostics scratch allocation failed");
     cudaStream_t s = ctx->stream;
-    diag_partial_kernel<<<blocks, kDiagNT, 0, s>>>(ctx->d_inst, n_in, d);
-    diag_final_kernel<<<1, kDiagNT, 0, s>>>(d, blocks, d + blocks);
-    DiagPart h{};
+    st = spec_staging(ctx);
+    if (st != SDM_OK) {
+        ctx->mem.put(d, bytes);
+        return st;
+    }
+    DiagPart *res = (DiagPart *)ctx->h_spec; // (both calls that use it wait for their result)
+    const bool one = blocks <= kLastBlockMax;
+    diag_partial_kernel<<<blocks, kDiagNT, 0, s>>>(ctx->d_inst, n_in, d, one ? res : nullptr);
+    if (!one)
+        diag_final_kernel<<<1, kDiagNT, 0, s>>>(d, blocks, res);
     CTX_CUDA(ctx, cudaGetLastError());
-    CTX_CUDA(ctx, cudaMemcpyAsync(&h, d + blocks, sizeof h, cudaMemcpyDeviceToHost, s));
     CTX_CUDA(ctx, cudaStreamSynchronize(s));
     ctx->mem.put(d, bytes);
+    const DiagPart h = *res;
     out->live_sd = (int64_t)h.live;
     out->sum_xi_lo = h.xi_lo;
     out->sum_xi_hi = h.xi_hi;

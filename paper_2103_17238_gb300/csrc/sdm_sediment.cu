@@ -51,7 +51,8 @@ constexpr int kSedNT = 256;
 // ------------------------------------------------------------------ kernels
 // zeta of every slot from z (SD-id order): z - (level) dz with level =
 // (cbase + c) / nx, which must lie in [0, dz) (zeta_in: z already holds
-// zeta); flags bit 0 and the first bad id on failure.  SDs outside the
+// zeta); flags bit 0 and the complement of the
+// first bad id on failure.  SDs outside the
 // domain and padding slots get zeta 0.  A warp takes 128 slots of a group at a
 // time, the ids and then the heights of all in flight together (43 us for
 // 4.19M SDs one by one).
@@ -92,7 +93,7 @@ __global__ void __launch_bounds__(kSedNT) sed_set_kernel(const int32_t *__restri
                     // in [0, dz): by the bit patterns (NaN and negative ones are above)
                     if ((unsigned long long)__double_as_longlong(zt) >= (unsigned long long)__double_as_longlong(dz)) {
                         atomicOr(flags, 1u);
-                        atomicMin(bad, (unsigned long long)id[u]);
+                        atomicMax(bad, ~(unsigned long long)id[u]);
                         zt = 0.0;
                     }
                 }
@@ -1073,19 +1074,18 @@ sdm_status set_positions_impl(sdm_ctx *ctx, const double *z, int32_t nx, double 
     }
     uint32_t *d_flags = ctx->sed->flags;
     unsigned long long *d_bad = (unsigned long long *)(d_flags + 2);
-    CTX_CUDA(ctx, cudaMemsetAsync(d_flags, 0, sizeof(uint32_t), s));
-    CTX_CUDA(ctx, cudaMemsetAsync(d_bad, 0xFF, sizeof(unsigned long long), s));
+    CTX_CUDA(ctx, cudaMemsetAsync(d_flags, 0, 16, s));
     sed_set_kernel<<<sed_grid(nc + 1), kSedNT, 0, s>>>(ctx->d_cell_off, nc, ctx->n_slots, ctx->d_id_of_slot, dz_arr,
                                                         nx, dz, ctx->cfg.cell_base, zeta_in, ctx->d_zeta, d_flags,
                                                         d_bad);
     ctx->sed->group_valid = false;
-    CTX_CUDA(ctx, cudaMemsetAsync(ctx->sed->emig, 0xFF, sizeof(int32_t) * ctx->n_sd, s));
-    uint32_t flags = 0;
-    unsigned long long bad = 0;
+    if (ctx->cfg.cell_base > 0) // only a piece of a grid has emigrants
+        CTX_CUDA(ctx, cudaMemsetAsync(ctx->sed->emig, 0xFF, sizeof(int32_t) * ctx->n_sd, s));
     CTX_CUDA(ctx, cudaGetLastError());
-    CTX_CUDA(ctx, cudaMemcpyAsync(&flags, d_flags, sizeof flags, cudaMemcpyDeviceToHost, s));
-    CTX_CUDA(ctx, cudaMemcpyAsync(&bad, d_bad, sizeof bad, cudaMemcpyDeviceToHost, s));
+    CTX_CUDA(ctx, cudaMemcpyAsync(ctx->sed->h_read, d_flags, 16, cudaMemcpyDeviceToHost, s));
     CTX_CUDA(ctx, cudaStreamSynchronize(s));
+    const uint32_t flags = *(const uint32_t *)ctx->sed->h_read;
+    const unsigned long long bad = ~((const unsigned long long *)ctx->sed->h_read)[1];
     ctx->mem.put(stage, bz);
     if (flags & 1u) {
         ctx->has_positions = false;
@@ -1312,7 +1312,7 @@ extern "C" sdm_status sdm_get_heights(sdm_ctx *ctx, double *zeta, int32_t *cell,
     cudaStream_t s = ctx->stream;
     const int32_t nc = ctx->cfg.n_cells;
     const int64_t n = ctx->n_sd;
-    const int32_t *emig = ctx->sed->emig;
+    const int32_t *emig = ctx->cfg.cell_base > 0 ? ctx->sed->emig : nullptr;
     if (on_device) {
         sed_get_kernel<<<sed_grid(nc + 1), kSedNT, 0, s>>>(ctx->d_cell_off, nc, ctx->n_slots, ctx->d_id_of_slot,
                                                             ctx->d_zeta, ctx->nx, ctx->dz, ctx->cfg.cell_base, emig,
