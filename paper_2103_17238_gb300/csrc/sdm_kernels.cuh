@@ -544,10 +544,12 @@ __global__ void __launch_bounds__(NT) one_cell_step_kernel(const __grid_constant
 // (every SD is in one pair per step, so nothing else in the launch reads or
 // writes it).  No queue of such pairs is kept: that leaves 10.5 KB of shared
 // memory per warp at 256 SDs, and 10 blocks of 2 warps per SM.
+constexpr int warp_buckets(int cap) { return 1 << ilog2_c(cap); } // 256 for 320 SDs
+
 template <int CAP, int STAGES>
 struct WarpSmem {
     // per warp: STAGES x (xi, v), sort word, bucket, perm
-    static constexpr size_t per_warp = (size_t)CAP * (16 * STAGES + 4 + 4 + 2);
+    static constexpr size_t per_warp = (size_t)CAP * (16 * STAGES + 4 + 2) + 4 * (size_t)warp_buckets(CAP);
 };
 
 __device__ __forceinline__ void cmp_swap(uint32_t &a, uint32_t &b)
@@ -557,8 +559,9 @@ __device__ __forceinline__ void cmp_swap(uint32_t &a, uint32_t &b)
     a = lo;
 }
 
-// Sorts E = 2, 4, 8 or 16 words held in registers (Batcher's odd-even merge
-// networks: 1, 5, 19 and 63 comparators).
+// Sorts E = 2, 4, 8, 10 or 16 words held in registers (Batcher's odd-even merge
+// networks: 1, 5, 19, 32 and 63 comparators; the one of 10 is that of 16 with the
+// comparators of the last six places left out).
 template <int E>
 __device__ __forceinline__ void sort_net(uint32_t (&v)[E])
 {
@@ -634,8 +637,41 @@ __device__ __forceinline__ void sort_net(uint32_t (&v)[E])
         cmp_swap(v[9], v[10]);
         cmp_swap(v[11], v[12]);
         cmp_swap(v[13], v[14]);
+    } else if constexpr (E == 10) {
+        cmp_swap(v[0], v[1]);
+        cmp_swap(v[2], v[3]);
+        cmp_swap(v[0], v[2]);
+        cmp_swap(v[1], v[3]);
+        cmp_swap(v[1], v[2]);
+        cmp_swap(v[4], v[5]);
+        cmp_swap(v[6], v[7]);
+        cmp_swap(v[4], v[6]);
+        cmp_swap(v[5], v[7]);
+        cmp_swap(v[5], v[6]);
+        cmp_swap(v[0], v[4]);
+        cmp_swap(v[2], v[6]);
+        cmp_swap(v[2], v[4]);
+        cmp_swap(v[1], v[5]);
+        cmp_swap(v[3], v[7]);
+        cmp_swap(v[3], v[5]);
+        cmp_swap(v[1], v[2]);
+        cmp_swap(v[3], v[4]);
+        cmp_swap(v[5], v[6]);
+        cmp_swap(v[8], v[9]);
+        cmp_swap(v[0], v[8]);
+        cmp_swap(v[4], v[8]);
+        cmp_swap(v[2], v[4]);
+        cmp_swap(v[6], v[8]);
+        cmp_swap(v[1], v[9]);
+        cmp_swap(v[5], v[9]);
+        cmp_swap(v[3], v[5]);
+        cmp_swap(v[7], v[9]);
+        cmp_swap(v[1], v[2]);
+        cmp_swap(v[3], v[4]);
+        cmp_swap(v[5], v[6]);
+        cmp_swap(v[7], v[8]);
     } else {
-        static_assert(E == 8, "sort_net: 2, 4, 8 or 16 words");
+        static_assert(E == 8, "sort_net: 2, 4, 8, 10 or 16 words");
         cmp_swap(v[0], v[1]);
         cmp_swap(v[2], v[3]);
         cmp_swap(v[4], v[5]);
@@ -671,19 +707,19 @@ constexpr int kMaxSwapRounds = 32;
 // the few spills (the one-step form went from 44.9 to 42.9 us per grid step
 // with L2 flushed, the fused form from 30.2 to 27.8).
 template <int CAP, int WARPS, int STAGES, bool FUSED = false>
-__global__ void __launch_bounds__(32 * WARPS, (CAP <= 256) ? 20 / WARPS : 0) warp_cell_step_kernel(const WorkItem *__restrict__ items, int32_t n_items,
+__global__ void __launch_bounds__(32 * WARPS, (CAP <= 256) ? 20 / WARPS : (CAP <= 320 ? 16 / WARPS : 0)) warp_cell_step_kernel(const WorkItem *__restrict__ items, int32_t n_items,
                                                                     InstDev *const *__restrict__ insts,
                                                                     int64_t step_offset, int32_t n_fused = 1)
 {
-    constexpr int NB = CAP;
-    constexpr int LB = ilog2_c(CAP);
-    constexpr int RP = CAP / 64 > 0 ? CAP / 64 : 1; // rank pairs per lane
+    constexpr int NB = warp_buckets(CAP);
+    constexpr int LB = ilog2_c(NB);
+    constexpr int RP = CAP / 64;                   // rank pairs per lane
     constexpr int BPL = NB / 32;                   // buckets per lane in the scan
-    static_assert((1 << LB) == CAP && CAP >= 64 && CAP <= 512, "warp kernel: CAP in 64..512");
+    static_assert(CAP == 64 || CAP == 128 || CAP == 256 || CAP == 320 || CAP == 512, "warp kernel: capacity");
     constexpr unsigned FULL = 0xFFFFFFFFu;
-    constexpr int RB = LB > 8 ? LB : 8;      // rank bits of a sort word
+    constexpr int RB = CAP <= 256 ? 8 : 9;   // rank bits of a sort word
     constexpr uint32_t RM = (1u << RB) - 1u; // rank mask
-    constexpr int KG = RP < 4 ? RP : 4;      // Philox blocks drawn at a time
+    constexpr int KG = RP < 4 || RP == 5 ? RP : 4; // Philox blocks drawn at a time
 
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -789,6 +825,7 @@ __global__ void __launch_bounds__(32 * WARPS, (CAP <= 256) ? 20 / WARPS : 0) war
         for (int rep = 0; rep < n_rep; ++rep) { // warp-uniform
         const int64_t s = s0 + rep;
 
+        static_assert(3 * (CAP / 2) <= CAP + NB, "room for every pair");
         if constexpr (BPL % 4 == 0) {
 #pragma unroll
             for (int i = 0; i < BPL / 4; ++i)
@@ -906,6 +943,13 @@ __global__ void __launch_bounds__(32 * WARPS, (CAP <= 256) ? 20 / WARPS : 0) war
                 const uint2 t = reinterpret_cast<const uint2 *>(s_word)[lane];
                 v[0] = t.x;
                 v[1] = t.y;
+            } else if constexpr (E % 4 != 0) {
+#pragma unroll
+                for (int i = 0; i < E; i += 2) {
+                    const uint2 t = reinterpret_cast<const uint2 *>(s_word + E * lane + i)[0];
+                    v[i] = t.x;
+                    v[i + 1] = t.y;
+                }
             } else {
 #pragma unroll
                 for (int i = 0; i < E; i += 4) {
@@ -956,6 +1000,10 @@ __global__ void __launch_bounds__(32 * WARPS, (CAP <= 256) ? 20 / WARPS : 0) war
                     reinterpret_cast<uint32_t *>(s_perm)[lane] = pk[0];
                 } else if constexpr (E == 4) {
                     reinterpret_cast<uint2 *>(s_perm)[lane] = make_uint2(pk[0], pk[1]);
+                } else if constexpr (E % 8 != 0) {
+#pragma unroll
+                    for (int i = 0; i < E / 2; ++i)
+                        reinterpret_cast<uint32_t *>(s_perm)[lane * (E / 2) + i] = pk[i];
                 } else {
 #pragma unroll
                     for (int i = 0; i < E / 8; ++i)
@@ -984,8 +1032,8 @@ __global__ void __launch_bounds__(32 * WARPS, (CAP <= 256) ? 20 / WARPS : 0) war
 
             // pairs (l = 2q, 2q + 1 share one Philox block).  A bound settles
             // most of them (gamma = 0); the rest are compacted into the sort
-            // arrays, dead by now (2 CAP words hold 2 CAP / 3 >= CAP / 2
-            // entries of 3 words: every pair fits), and go through the full
+            // arrays, dead by now (CAP + NB words hold CAP / 2 entries of 3
+            // words: every pair fits), and go through the full
             // filter one per lane: certain collisions are updated at once,
             // and so are undecided pairs, after their exact evaluation.
             const uint32_t n_pairs = n_c / 2;
@@ -998,7 +1046,7 @@ __global__ void __launch_bounds__(32 * WARPS, (CAP <= 256) ? 20 / WARPS : 0) war
             uint32_t n_todo = 0; // warp-uniform
             // QG Philox blocks per lane are drawn, and their pairs bounded,
             // before any compaction, so that the independent chains interleave.
-            constexpr int QG = CAP >= 256 ? 2 : 1;
+            constexpr int QG = CAP == 320 ? 3 : (CAP >= 256 ? 2 : 1);
             for (uint32_t q0 = 0; q0 < n_q; q0 += 32 * QG) { // warp-uniform trip count
                 uint4 w[QG];
 #pragma unroll
@@ -2034,8 +2082,8 @@ __device__ __forceinline__ bool volume_ok(double v)
 // Validation and per-group counts of set_attributes (groups: the cells, then
 // n_cells for the SDs outside the domain, cell id -1).  flags bit 0: an
 // invalid attribute (*bad the complement of the first bad SD index; 0: none); bit 1: groups not sorted.
-// Each warp takes 128 consecutive SDs at a time, 32 by 32, and adds one count
-// per run of equal groups (one or two atomics per 32 for sorted input).
+// Each warp takes 128 consecutive SDs at a time; a run of equal groups adds its
+// length by its two ends.
 __global__ void validate_count_kernel(int64_t lo, int64_t hi, const int64_t *__restrict__ xi,
                                       const double *__restrict__ v, const int32_t *__restrict__ cell, int32_t n_cells,
                                       uint32_t *__restrict__ counts, uint32_t *__restrict__ flags,
@@ -2059,36 +2107,38 @@ __global__ void validate_count_kernel(int64_t lo, int64_t hi, const int64_t *__r
             x[u] = in ? xi[i] : 0;
             vol[u] = in ? v[i] : 1.0;
         }
-        int32_t last = before == -1 ? n_cells : (before == -2 ? INT32_MIN : before); // lane 0: the SD before
+        // the groups, -1 behind the end; an invalid SD's cell stands for itself
+        int32_t c[U];
+        bool unsorted = false;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int64_t i = base + 32 * u + lane;
-            const bool in = i < hi;
-            const int32_t craw = c_in[u] == -1 ? n_cells : c_in[u]; // the group; outside sorts last
-            int32_t c = -1;                                           // counted group, -1: none
-            if (in) {
-                if (x[u] >= 0 && volume_ok(vol[u]) && c_in[u] >= -1 && c_in[u] < n_cells) {
-                    c = craw;
-                } else {
-                    atomicOr(flags, 1u);
-                    atomicMax(bad, ~(unsigned long long)i);
-                }
-            }
-            int32_t prev = __shfl_up_sync(FULL, craw, 1);
-            if (lane == 0)
-                prev = last;
-            if (__any_sync(FULL, in && prev > craw) && lane == 0)
-                atomicOr(flags, 2u);
-            last = __shfl_sync(FULL, craw, 31);
-            const int32_t next = __shfl_down_sync(FULL, c, 1);
-            const bool end = lane == 31 || next != c;
-            const unsigned ends = __ballot_sync(FULL, end);
-            if (end && c >= 0) {
-                const unsigned below = ends & ((1u << lane) - 1u);
-                const int start = below ? 32 - __clz(below) : 0;
-                atomicAdd(&counts[c], (uint32_t)(lane - start + 1));
+            c[u] = i < hi ? (c_in[u] == -1 ? n_cells : c_in[u]) : -1;
+            if (i < hi && !(x[u] >= 0 && volume_ok(vol[u]) && c_in[u] >= -1 && c_in[u] < n_cells)) {
+                atomicOr(flags, 1u);
+                atomicMax(bad, ~(unsigned long long)i);
             }
         }
+        int32_t prev = before == -1 ? n_cells : (before == -2 ? INT32_MIN : before); // lane 0: the SD before
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = base + 32 * u + lane;
+            int32_t up = __shfl_up_sync(FULL, c[u], 1), down = __shfl_down_sync(FULL, c[u], 1);
+            const int32_t next = u + 1 < U ? __shfl_sync(FULL, c[u + 1 < U ? u + 1 : u], 0) : INT32_MIN;
+            if (lane == 0)
+                up = prev;
+            if (lane == 31)
+                down = next;
+            prev = __shfl_sync(FULL, c[u], 31);
+            unsorted |= i < hi && up > c[u];
+            // a run of equal groups adds its length by its two ends (a warp's
+            // 128 SDs are cut off at either end)
+            const bool first = (u == 0 && lane == 0) || up != c[u], last = down != c[u];
+            if ((first || last) && (unsigned)c[u] <= (unsigned)n_cells)
+                atomicAdd(&counts[c[u]], (last ? (uint32_t)i + 1u : 0u) - (first ? (uint32_t)i : 0u));
+        }
+        if (__any_sync(FULL, unsorted) && lane == 0)
+            atomicOr(flags, 2u);
     }
 }
 

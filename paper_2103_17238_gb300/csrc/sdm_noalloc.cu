@@ -200,12 +200,12 @@ extern "C" sdm_status sdm_cell_step_noalloc(const sdm_config *cfg, int64_t step,
             constexpr int CAP = decltype(cap)::value, NT = decltype(nt)::value;
             one_cell_step_kernel<CAP, NT><<<1, NT, CellSmem<CAP, 1>::bytes, s>>>(inst, n, status);
         };
-        int cls = 0;
-        while (kClassCap[cls] < n)
-            ++cls;
-        switch (cls) {
+        int lg = 6;
+        while ((1 << lg) < n)
+            ++lg;
+        switch (lg) {
 #define X(CAP, NT, ST)                                                                                                 \
-    case ilog2_c(CAP) - 6:                                                                                             \
+    case ilog2_c(CAP):                                                                                                 \
         one(std::integral_constant<int, CAP>{}, std::integral_constant<int, NT>{});                                    \
         break;
             SDM_BLOCK_VARIANTS(X)

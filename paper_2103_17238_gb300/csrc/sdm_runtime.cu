@@ -138,8 +138,10 @@ struct Buf {
 
 constexpr int kInChunks = 4; // pieces of a host input copy (sdm_set_attributes)
 
-// Cell-size classes of the shared-memory path.
-constexpr int kClassCap[] = {64, 128, 256, 512, 1024, 2048, 4096};
+// Cell-size classes of the shared-memory path.  320 is for grids of 256 SDs per
+// cell on average whose SDs move between cells: half of the cells then hold a
+// few more, and paid for 512 (36 us a step beside 26 for the others, 24 now).
+constexpr int kClassCap[] = {64, 128, 256, 320, 512, 1024, 2048, 4096};
 constexpr int kNumClass = sizeof(kClassCap) / sizeof(kClassCap[0]);
 
 struct Plan {
@@ -148,7 +150,7 @@ struct Plan {
     WorkItem *d_items[kNumClass] = {};
     int n_items[kNumClass] = {};
     int variant[kNumClass] = {};
-    int8_t fold[kNumClass] = {0, 1, 2, 3, 4, 5, 6}; // the class whose launch takes a class's cells
+    int8_t fold[kNumClass] = {0, 1, 2, 3, 4, 5, 6, 7}; // the class whose launch takes a class's cells
     // A context's own plan whose cells all take the shared-memory classes
     // keeps room for every cell in every class (class k at d_items_all + k
     // n_cells), so that the device can rebuild it for a new layout
@@ -362,7 +364,8 @@ size_t big_hist_smem(int lb) { return (size_t)sizeof(uint32_t) << lb; }
 // tuning (sdm_set_tuning) picks one variant per size class when a plan is
 // built.
 #define SDM_WARP_VARIANTS(X)                                                                                           \
-    X(64, 1) X(64, 2) X(64, 4) X(128, 1) X(128, 2) X(128, 4) X(256, 1) X(256, 2) X(256, 4) X(512, 1) X(512, 2) X(512, 4)
+    X(64, 1) X(64, 2) X(64, 4) X(128, 1) X(128, 2) X(128, 4) X(256, 1) X(256, 2) X(256, 4)                             \
+    X(320, 1) X(320, 2) X(320, 4) X(512, 1) X(512, 2) X(512, 4)
 #define SDM_BLOCK_VARIANTS(X)                                                                                          \
     X(64, 32, 4) X(128, 64, 4) X(256, 128, 4) X(512, 256, 4) X(1024, 512, 3) X(2048, 1024, 2) X(4096, 1024, 2)
 
@@ -407,19 +410,21 @@ struct Variant {
     launch_fn launch;
 };
 
-// the fused kernels: warp per cell by size class (capacity 64 .. 512), and
-// block per cell for every class
+// the fused kernels: warp per cell by size class (capacity 64 .. 512), then
+// block per cell by SDM_BLOCK_VARIANTS
 struct FusedVariant {
+    int cap;
     int per_block; // cells of a block
     fused_fn launch;
 };
 const FusedVariant g_fused[] = {
-    {2, launch_warp_fused<64>}, {2, launch_warp_fused<128>}, {2, launch_warp_fused<256>}, {2, launch_warp_fused<512>},
-#define X(CAP, NT, ST) {1, launch_block_fused<CAP, NT>},
+    {64, 2, launch_warp_fused<64>},   {128, 2, launch_warp_fused<128>}, {256, 2, launch_warp_fused<256>},
+    {320, 2, launch_warp_fused<320>}, {512, 2, launch_warp_fused<512>},
+#define X(CAP, NT, ST) {CAP, 1, launch_block_fused<CAP, NT>},
     SDM_BLOCK_VARIANTS(X)
 #undef X
 };
-constexpr int kFusedWarp = 4; // then the block kernels by class
+constexpr int kFusedWarp = 5;
 
 const Variant g_variants[] = {
 #define X(CAP, WARPS) {CAP, WARPS, launch_warp<CAP, WARPS>},
@@ -474,14 +479,24 @@ sdm_tuning current_tuning()
 
 int variant_for(int cap, const sdm_tuning &t)
 {
+    const bool warp = cap <= t.warp_cell_max;
+    if (!warp && cap == 320) // blocks come in powers of two
+        cap = 512;
     for (int v = 0; v < kNumVariants; ++v) {
         const Variant &x = g_variants[v];
-        if (x.cap != cap)
-            continue;
-        if (cap <= t.warp_cell_max ? x.warps == t.warps_per_block : x.warps == 0)
+        if (x.cap == cap && (warp ? x.warps == t.warps_per_block : x.warps == 0))
             return v;
     }
     return -1;
+}
+
+// The fused kernel that goes with a variant.
+int fused_of(const Variant &x)
+{
+    int f = x.warps > 0 ? 0 : kFusedWarp;
+    while (g_fused[f].cap != x.cap)
+        ++f;
+    return f;
 }
 
 // The variant of class k for a plan's n cells of it.  With the default tuning,
@@ -494,8 +509,8 @@ int variant_of_class(int k, int n, const sdm_tuning &t)
     constexpr int kFew512 = 608, kFew256 = 304;
     const bool standard = t.warp_cell_max == 512 && t.warps_per_block == 2;
     sdm_tuning u = t;
-    if (standard && n <= (kClassCap[k] == 512 ? kFew512 : (kClassCap[k] == 256 ? kFew256 : 0)))
-        u.warp_cell_max = kClassCap[k] / 2;
+    if (standard && n <= (kClassCap[k] == 512 ? kFew512 : (kClassCap[k] == 256 || kClassCap[k] == 320 ? kFew256 : 0)))
+        u.warp_cell_max = 128;
     return variant_for(kClassCap[k], u);
 }
 
@@ -622,7 +637,7 @@ cudaError_t configure_kernels()
             e = r;                                                                                                     \
         G.fused[v++] = std::max(1, per_sm) * sms;                                                                      \
     }
-        X(64) X(128) X(256) X(512)
+        X(64) X(128) X(256) X(320) X(512)
 #undef X
 #define X(CAP, NT, ST)                                                                                                 \
     {                                                                                                                  \
@@ -672,14 +687,17 @@ void launch_variant(int v, int n, const WorkItem *items, InstDev *const *insts, 
 }
 
 // Size class of a cell of n >= 2 stored SDs under the tuning (the smallest
-// class capacity 64 2^c >= n); -1: the multi-pass path.
-int class_of(int n, const sdm_tuning &t)
+// class capacity >= n); -1: the paths of larger cells.
+__host__ __device__ inline int class_of(int n, int32_t smem_max_sd)
 {
-    const int c = n <= 64 ? 0 : 32 - __builtin_clz((unsigned)(n - 1)) - 6;
-    if (c >= kNumClass || kClassCap[c] > t.smem_max_sd)
+    if (n > smem_max_sd)
         return -1;
-    return c;
+    int lg = 6; // 64 2^(lg - 6) >= n
+    while ((1 << lg) < n)
+        ++lg;
+    return lg - 6 + (n > 320 ? 1 : 0); // 320 lies between 256 and 512
 }
+static_assert(kClassCap[3] == 320 && kClassCap[4] == 512 && kClassCap[kNumClass - 1] == 4096, "class_of");
 
 constexpr int kRefreshNT = 256;
 
@@ -707,10 +725,9 @@ __global__ void __launch_bounds__(kRefreshNT) plan_refresh_kernel(const int32_t 
         o = cell_off[c];
         n = cell_off[c + 1] - o;
         if (n >= 2) {
-            k = n <= 64 ? 0 : 32 - __clz(n - 1) - 6;
-            if (k >= kNumClass || (64 << k) > smem_max_sd) {
+            k = class_of(n, smem_max_sd);
+            if (k < 0) {
                 counts[kNumClass] = 1u;
-                k = -1;
             } else {
                 k = (int)(fold >> (4 * k)) & 15;
                 slot = atomicAdd(&s_cnt[k], 1u);
@@ -825,19 +842,21 @@ sdm_status build_plan(sdm_batch *b)
         const int32_t *off = c->h_cell_off.data();
         for (int32_t cell = 0; cell < c->cfg.n_cells; ++cell) {
             const int n = off[cell + 1] - off[cell];
-            const int8_t k = n < 2 ? (int8_t)-2 : (int8_t)class_of(n, tun);
+            const int8_t k = n < 2 ? (int8_t)-2 : (int8_t)class_of(n, tun.smem_max_sd);
             cls[cell] = k;
             if (k >= 0)
                 ++cnt[k];
         }
         cls += c->cfg.n_cells;
     }
-    // With the default tuning, the cells of up to 64 and of up to 128 SDs join
-    // the next class's launch when all of it stays resident at once: they then
+    // With the default tuning, the cells of up to 64, up to 128 and up to 320 SDs
+    // join the next class's launch when all of it stays resident at once: they then
     // finish with its own cells, and a launch with its fork and join goes (a
     // grid of 4087 cells of 43..574, a step per call: 231 -> 225 us a pass).
     const bool standard = tun.warp_cell_max == 512 && tun.warps_per_block == 2;
-    for (int k = 0; k < 2 && standard; ++k) {
+    for (int k = 0; k < 4 && standard; ++k) {
+        if (k == 2)
+            continue;
         const int v = variant_for(kClassCap[k + 1], tun);
         if (!cnt[k] || !cnt[k + 1] || cnt[k] + cnt[k + 1] > (int64_t)dev_grids().variant[v] * g_variants[v].warps)
             continue;
@@ -1240,7 +1259,7 @@ void enqueue_steps(const Plan &pl, int64_t off, int32_t n, cudaStream_t st)
             continue;
         const Variant &x = g_variants[pl.variant[k]];
         if (fuse) {
-            const int fi = x.warps > 0 ? k : kFusedWarp + k;
+            const int fi = fused_of(x);
             const FusedVariant &fv = g_fused[fi];
             const int grid = std::min((pl.n_items[k] + fv.per_block - 1) / fv.per_block, dev_grids().fused[fi]);
             for (int32_t i = 0; i < n; i += f)

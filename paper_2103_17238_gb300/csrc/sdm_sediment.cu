@@ -761,11 +761,36 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
     unsigned long long *key = s_key[warp];
     uint32_t *below = s_below[warp];
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    // a cell's numbers, one per lane, loaded a cell ahead
+    auto numbers = [&](int g) -> uint32_t {
+        if (g >= n_cells || lane > 6)
+            return 0u;
+        if (lane < 4)
+            return (uint32_t)(lane < 2 ? cell_off : poff)[g + (lane & 1)];
+        return lane == 4 ? M.arr[g] : (lane == 5 ? (uint32_t)M.first[g] : M.stay[g]);
+    };
+    uint32_t ahead = numbers(gw);
     for (int g = gw; g < n_cells; g += nw) { // uniform over the warp
-        const int32_t lo = cell_off[g], hi = cell_off[g + 1];
-        const int32_t p0 = poff[g], p1 = poff[g + 1];
-        const uint32_t A = M.arr[g], a0 = (uint32_t)M.first[g];
-        const uint32_t n_stay = M.stay[g];
+        const int32_t lo = __shfl_sync(FULL, ahead, 0), hi = __shfl_sync(FULL, ahead, 1);
+        const int32_t p0 = __shfl_sync(FULL, ahead, 2), p1 = __shfl_sync(FULL, ahead, 3);
+        const uint32_t A = __shfl_sync(FULL, ahead, 4), a0 = __shfl_sync(FULL, ahead, 5);
+        const uint32_t n_stay = __shfl_sync(FULL, ahead, 6);
+        ahead = numbers(g + nw);
+        int64_t x[kSedRun];
+        double w[kSedRun], z[kSedRun];
+        int32_t id[kSedRun];
+        auto fetch = [&](int32_t s0) { // 128 slots, every load together
+#pragma unroll
+            for (int u = 0; u < kSedRun; ++u) {
+                const int32_t sl = s0 + 32 * u + lane;
+                const bool in = sl < hi;
+                z[u] = in ? zeta_new[sl] : -1.0;
+                x[u] = in ? xi[sl] : 0;
+                w[u] = in ? v[sl] : 1.0;
+                id[u] = in ? id_of_slot[sl] : -1;
+            }
+        };
+        fetch(lo); // on its way while the arrivals are sorted
         const bool sorted = A <= (uint32_t)kSedArrive;
         if (A > 0 && sorted) {
             uint32_t P2 = 1;
@@ -792,18 +817,6 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
         uint32_t done = 0; // stayers so far
         uint32_t mine = 0;
         for (int32_t s0 = lo; s0 < hi; s0 += 32 * kSedRun) {
-            int64_t x[kSedRun];
-            double w[kSedRun], z[kSedRun];
-            int32_t id[kSedRun];
-#pragma unroll
-            for (int u = 0; u < kSedRun; ++u) { // every load first
-                const int32_t sl = s0 + 32 * u + lane;
-                const bool in = sl < hi;
-                z[u] = in ? zeta_new[sl] : -1.0;
-                x[u] = in ? xi[sl] : 0;
-                w[u] = in ? v[sl] : 1.0;
-                id[u] = in ? id_of_slot[sl] : -1;
-            }
 #pragma unroll
             for (int u = 0; u < kSedRun; ++u) {
                 if (s0 + 32 * u >= hi) // uniform over the warp
@@ -841,14 +854,16 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                     L.put((int64_t)p0 + done + (uint32_t)__popc(km & lt) + t, x[u], w[u], z[u], id[u]);
                 done += (uint32_t)__popc(km);
             }
+            if (s0 + 32 * kSedRun < hi)
+                fetch(s0 + 32 * kSedRun);
         }
         uint32_t carry = 0; // stayers before the arrivals of this round
         for (uint32_t j0 = 0; j0 < A; j0 += 32) {
             const uint32_t j = j0 + lane;
-            uint32_t slot = 0, id = 0, at = 0;
+            uint32_t slot = 0, id_a = 0, at = 0;
             if (A <= (uint32_t)kSedFew) {
                 if (j < A) {
-                    id = (uint32_t)(key[j] >> 32);
+                    id_a = (uint32_t)(key[j] >> 32);
                     slot = (uint32_t)key[j];
                     at = j + mine;
                 }
@@ -861,21 +876,21 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                         c += y;
                 }
                 if (j < A) {
-                    id = (uint32_t)(key[j] >> 32);
+                    id_a = (uint32_t)(key[j] >> 32);
                     slot = (uint32_t)key[j];
                     at = j + carry + c;
                 }
                 carry += __shfl_sync(FULL, c, 31);
             } else if (j < A) { // more arrivals than the sort takes: by counting
-                id = M.a_id[a0 + j];
+                id_a = M.a_id[a0 + j];
                 slot = M.a_slot[a0 + j];
                 for (uint32_t k = 0; k < A; ++k)
-                    at += M.a_id[a0 + k] < id ? 1u : 0u;
+                    at += M.a_id[a0 + k] < id_a ? 1u : 0u;
                 for (int32_t s = lo; s < hi; ++s)
-                    at += !dneg(zeta_new[s]) && (uint32_t)id_of_slot[s] < id ? 1u : 0u;
+                    at += !dneg(zeta_new[s]) && (uint32_t)id_of_slot[s] < id_a ? 1u : 0u;
             }
             if (j < A)
-                L.put((int64_t)p0 + at, xi[slot], v[slot], fabs(zeta_new[slot]), (int32_t)id);
+                L.put((int64_t)p0 + at, xi[slot], v[slot], fabs(zeta_new[slot]), (int32_t)id_a);
         }
         if (lane == 0) {
             if (p0 + (int32_t)(n_stay + A) < p1) // the padding slot of an odd cell
@@ -933,8 +948,8 @@ struct SedBuffers {
 };
 
 // Bytes of the pinned read-back buffer for n_cells cells: n_cells + 2
-// offsets, the precipitated total (8-byte aligned) and 8 class-count words.
-size_t sed_read_bytes(int32_t n_cells) { return (((size_t)n_cells + 2) * 4 + 7) / 8 * 8 + 8 + 32; }
+// offsets, the precipitated total (8-byte aligned) and the class-count words.
+size_t sed_read_bytes(int32_t n_cells) { return (((size_t)n_cells + 2) * 4 + 7) / 8 * 8 + 8 + sizeof(uint32_t) * (kNumClass + 1); }
 
 void sed_release(sdm_ctx *ctx)
 {
