@@ -21,11 +21,14 @@
 //   sed_deal_kernel      the movers to their group's arrivals;
 //   sed_merge_kernel     one warp per new cell: its arrivals sorted by id, its
 //                        stayers streamed through, each moved up by the
-//                        arrivals of lower id; the new layout with its padding.
+//                        arrivals of lower id; the new layout with its padding
+//                        (a cell with many arrivals: by the whole block).
 // 112 B per SD (xi, v, heights; heights out; the layout in and out).  The
 // refresh of the context's own launch plan and the read-back run on a side
 // stream beside the last two; the host waits for the read-back only.
-// Measured on the 4.19M-SD grid: SED_FIGURES
+// Measured on the 4.19M-SD grid (us): fall 36, offsets 11, deal 7, merge 40, where
+// the sort of all SDs took 210 in all.  When every SD moves (4096 cells of 200, 500, 800
+// SDs, one level per step) a step takes 53, 128, 196 us against 94, 147, 202 sorted.
 //
 // With larger cells (a warp would take too long), a stable sort of all SDs:
 //   sed_move_kernel      per slot (four per thread): the fall, the new group
@@ -485,7 +488,7 @@ __global__ void sed_pad_kernel(int32_t n_groups, const int32_t *__restrict__ ust
 // sets are freed through their current pointers) and the scratch.
 // ------------------------------------------------- cells of up to kSedByCell
 constexpr int kSedByCell = 1024;  // slots of the largest cell that a warp takes
-constexpr int kSedArrive = 512;   // arrivals of a cell sorted in shared memory
+constexpr int kSedArrive = 256;   // arrivals of a cell that a warp takes; more by its block
 constexpr int kSedMergeNT = 128;
 constexpr int kSedFew = 12;       // arrivals up to which each is compared with every stayer, by ballots
 
@@ -560,9 +563,17 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
             if (out && lane == __ffs(out) - 1) // one counter for all that leave the domain
                 place = atomicAdd(M.out, (uint32_t)__popc(out));
             place = __shfl_sync(FULL, place, out ? __ffs(out) - 1 : 0) + (uint32_t)__popc(out & lt);
+            // one addition per group among the lanes (in heavy rain all 32 enter the same cell)
+            const bool in = go && ng != n_cells;
+            const unsigned same = __match_any_sync(FULL, in ? ng : -1 - lane);
+            const int head = __ffs(same) - 1;
+            uint32_t first = 0;
+            if (in && lane == head)
+                first = atomicAdd(&M.arr[ng], (uint32_t)__popc(same));
+            first = __shfl_sync(FULL, first, head);
             if (go) {
-                if (ng != n_cells)
-                    place = atomicAdd(&M.arr[ng], 1u);
+                if (in)
+                    place = first + (uint32_t)__popc(same & lt);
                 const uint32_t at = (uint32_t)lo + left + (uint32_t)__popc(mv & lt);
                 M.group[at] = (uint32_t)ng;
                 M.id[at] = (uint32_t)id;
@@ -744,6 +755,129 @@ struct SedLayout {
     }
 };
 
+// First place in the n ascending numbers at or above x.
+template <typename F>
+__device__ __forceinline__ uint32_t sed_lower(uint32_t n, uint32_t x, F &&at)
+{
+    uint32_t lo = 0;
+    while (lo < n) {
+        const uint32_t mid = (lo + n) >> 1;
+        if (at(mid) < x)
+            lo = mid + 1;
+        else
+            n = mid;
+    }
+    return lo;
+}
+
+// A cell with more than kSedArrive arrivals, by the whole block: the arrivals
+// sorted in runs of kSedRunKeys (written back when there are several), the
+// stayers' ids and counts in shared memory, every SD's place by binary
+// searches.  (By one warp that counted: 2.5 ms for 4096 cells of 1000 SDs of
+// which 600 fall into the next cell, 0.10 here.)
+constexpr int kSedRunKeys = kSedArrive * (kSedMergeNT / 32);
+struct SedHeavy {
+    uint32_t id[kSedByCell];
+    uint16_t stay[kSedByCell + 2]; // stayers before a slot
+    uint32_t warp[kSedMergeNT / 32];
+};
+
+__device__ __noinline__ void sed_merge_heavy(int g, const int32_t *__restrict__ cell_off, SedMoves M,
+                                             const int64_t *__restrict__ xi, const double *__restrict__ v,
+                                             const double *__restrict__ zeta_new,
+                                             const int32_t *__restrict__ id_of_slot, const int32_t *__restrict__ poff,
+                                             SedLayout L, unsigned long long *key, SedHeavy &H)
+{
+    constexpr int E = kSedByCell / kSedMergeNT; // slots per thread
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int32_t lo = cell_off[g], p0 = poff[g], p1 = poff[g + 1];
+    const uint32_t n = (uint32_t)(cell_off[g + 1] - lo), A = M.arr[g], a0 = (uint32_t)M.first[g];
+    uint32_t keep = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t i = (uint32_t)(t * E + e);
+        H.id[i] = i < n ? (uint32_t)id_of_slot[lo + i] : 0xFFFFFFFFu; // (padding: -1, above all)
+        keep |= (i < n && !dneg(zeta_new[lo + i]) ? 1u : 0u) << e;
+    }
+    uint32_t incl = (uint32_t)__popc(keep);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= d)
+            incl += y;
+    }
+    if (lane == 31)
+        H.warp[warp] = incl;
+    __syncthreads();
+    uint32_t before = incl - (uint32_t)__popc(keep), n_stay = 0;
+    for (int w = 0; w < kSedMergeNT / 32; ++w) {
+        before += w < warp ? H.warp[w] : 0u;
+        n_stay += H.warp[w];
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        H.stay[t * E + e] = (uint16_t)(before + (uint32_t)__popc(keep & ((1u << e) - 1u)));
+    if (t == 0)
+        H.stay[kSedByCell] = (uint16_t)n_stay;
+    for (uint32_t c0 = 0; c0 < A; c0 += kSedRunKeys) {
+        const uint32_t m = min(A - c0, (uint32_t)kSedRunKeys);
+        uint32_t P2 = 1;
+        while (P2 < m)
+            P2 <<= 1;
+        for (uint32_t i = t; i < P2; i += kSedMergeNT)
+            key[i] = i < m ? ((unsigned long long)M.a_id[a0 + c0 + i] << 32) | M.a_slot[a0 + c0 + i] : ~0ull;
+        __syncthreads();
+        bool back = false; // those of one cell come in order
+        for (uint32_t i = t; i + 1 < m; i += kSedMergeNT)
+            back |= key[i] > key[i + 1];
+        for (uint32_t k = __syncthreads_or(back) ? 2u : 2u * P2; k <= P2; k <<= 1) // bitonic
+            for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+                for (uint32_t i = t; i < P2 / 2; i += kSedMergeNT) {
+                    const uint32_t a = 2 * i - (i & (j - 1)), b = a + j;
+                    const unsigned long long ka = key[a], kb = key[b];
+                    if ((ka > kb) == ((a & k) == 0)) {
+                        key[a] = kb;
+                        key[b] = ka;
+                    }
+                }
+                __syncthreads();
+            }
+        if (A > (uint32_t)kSedRunKeys) {
+            for (uint32_t i = t; i < m; i += kSedMergeNT) {
+                M.a_id[a0 + c0 + i] = (uint32_t)(key[i] >> 32);
+                M.a_slot[a0 + c0 + i] = (uint32_t)key[i];
+            }
+            __syncthreads();
+        }
+    }
+    const bool one = A <= (uint32_t)kSedRunKeys;
+    auto arrivals_below = [&](uint32_t id) {
+        if (one)
+            return sed_lower(A, id, [&](uint32_t i) { return (uint32_t)(key[i] >> 32); });
+        uint32_t r = 0;
+        for (uint32_t c0 = 0; c0 < A; c0 += kSedRunKeys)
+            r += sed_lower(min(A - c0, (uint32_t)kSedRunKeys), id, [&](uint32_t i) { return M.a_id[a0 + c0 + i]; });
+        return r;
+    };
+    for (uint32_t i = t; i < n; i += kSedMergeNT) {
+        const double z = zeta_new[lo + i];
+        if (!dneg(z))
+            L.put((int64_t)p0 + H.stay[i] + arrivals_below(H.id[i]), xi[lo + i], v[lo + i], z, (int32_t)H.id[i]);
+    }
+    for (uint32_t j = t; j < A; j += kSedMergeNT) {
+        const uint32_t id = one ? (uint32_t)(key[j] >> 32) : M.a_id[a0 + j];
+        const uint32_t slot = one ? (uint32_t)key[j] : M.a_slot[a0 + j];
+        const uint32_t at = (one ? j : arrivals_below(id)) + H.stay[sed_lower(n, id, [&](uint32_t i) { return H.id[i]; })];
+        L.put((int64_t)p0 + at, xi[slot], v[slot], fabs(zeta_new[slot]), (int32_t)id);
+    }
+    __syncthreads(); // the shared arrays and the count are read
+    if (t == 0) {
+        if (p0 + (int32_t)(n_stay + A) < p1) // the padding slot of an odd cell
+            L.put(p1 - 1, 0, 1.0, 0.0, -1);
+        M.arr[g] = 0u; // for the next step
+    }
+}
+
 __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *__restrict__ cell_off, int32_t n_cells,
                                                                 SedMoves M, const int64_t *__restrict__ xi,
                                                                 const double *__restrict__ v,
@@ -755,11 +889,15 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
     constexpr unsigned FULL = 0xFFFFFFFFu;
     constexpr int W = kSedMergeNT / 32;
     __shared__ unsigned long long s_key[W][kSedArrive]; // arrivals: id above slot, in order
-    __shared__ uint32_t s_below[W][kSedArrive];         // stayers that follow t arrivals and no more
+    __shared__ union {
+        uint32_t below[W][kSedArrive]; // stayers that follow t arrivals and no more
+        SedHeavy heavy;
+    } s_u;
+    static_assert(kSedByCell % kSedMergeNT == 0 && kSedRunKeys == W * kSedArrive, "the block's arrays");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     unsigned long long *key = s_key[warp];
-    uint32_t *below = s_below[warp];
+    uint32_t *below = s_u.below[warp];
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     // a cell's numbers, one per lane, loaded a cell ahead
     auto numbers = [&](int g) -> uint32_t {
@@ -770,12 +908,17 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
         return lane == 4 ? M.arr[g] : (lane == 5 ? (uint32_t)M.first[g] : M.stay[g]);
     };
     uint32_t ahead = numbers(gw);
+    int heavy = 0;
     for (int g = gw; g < n_cells; g += nw) { // uniform over the warp
         const int32_t lo = __shfl_sync(FULL, ahead, 0), hi = __shfl_sync(FULL, ahead, 1);
         const int32_t p0 = __shfl_sync(FULL, ahead, 2), p1 = __shfl_sync(FULL, ahead, 3);
         const uint32_t A = __shfl_sync(FULL, ahead, 4), a0 = __shfl_sync(FULL, ahead, 5);
         const uint32_t n_stay = __shfl_sync(FULL, ahead, 6);
         ahead = numbers(g + nw);
+        if (A > (uint32_t)kSedArrive) { // later, by the block
+            heavy = 1;
+            continue;
+        }
         int64_t x[kSedRun];
         double w[kSedRun], z[kSedRun];
         int32_t id[kSedRun];
@@ -791,8 +934,7 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
             }
         };
         fetch(lo); // on its way while the arrivals are sorted
-        const bool sorted = A <= (uint32_t)kSedArrive;
-        if (A > 0 && sorted) {
+        if (A > 0) {
             uint32_t P2 = 1;
             while (P2 < A)
                 P2 <<= 1;
@@ -801,7 +943,10 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                 below[i] = 0u;
             }
             __syncwarp();
-            for (uint32_t k = 2; k <= P2; k <<= 1) // bitonic
+            bool back = false; // those of one cell come in order
+            for (uint32_t i = lane; i + 1 < A; i += 32)
+                back |= key[i] > key[i + 1];
+            for (uint32_t k = __any_sync(FULL, back) ? 2u : 2u * P2; k <= P2; k <<= 1) // bitonic
                 for (uint32_t j = k >> 1; j > 0; j >>= 1) {
                     for (uint32_t i = lane; i < P2 / 2; i += 32) {
                         const uint32_t a = 2 * i - (i & (j - 1)), b = a + j;
@@ -831,7 +976,7 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                         const uint32_t c = (uint32_t)__popc(km & ~__ballot_sync(FULL, above));
                         mine += lane == (int)k ? c : 0u; // lane k: stayers of lower id than arrival k
                     }
-                } else if (sorted) {
+                } else {
                     uint32_t end = A;
                     while (t < end) { // first arrival above this id
                         const uint32_t mid = (t + end) >> 1;
@@ -846,9 +991,6 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                     if (keep && t < A && (same & lt) == 0u)
                         below[t] += (uint32_t)__popc(same);
                     __syncwarp();
-                } else if (keep) {
-                    for (uint32_t k = 0; k < A; ++k)
-                        t += M.a_id[a0 + k] < (uint32_t)id[u] ? 1u : 0u;
                 }
                 if (keep)
                     L.put((int64_t)p0 + done + (uint32_t)__popc(km & lt) + t, x[u], w[u], z[u], id[u]);
@@ -867,7 +1009,7 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                     slot = (uint32_t)key[j];
                     at = j + mine;
                 }
-            } else if (sorted) {
+            } else {
                 uint32_t c = j < A ? below[j] : 0u;
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) {
@@ -881,13 +1023,6 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
                     at = j + carry + c;
                 }
                 carry += __shfl_sync(FULL, c, 31);
-            } else if (j < A) { // more arrivals than the sort takes: by counting
-                id_a = M.a_id[a0 + j];
-                slot = M.a_slot[a0 + j];
-                for (uint32_t k = 0; k < A; ++k)
-                    at += M.a_id[a0 + k] < id_a ? 1u : 0u;
-                for (int32_t s = lo; s < hi; ++s)
-                    at += !dneg(zeta_new[s]) && (uint32_t)id_of_slot[s] < id_a ? 1u : 0u;
             }
             if (j < A)
                 L.put((int64_t)p0 + at, xi[slot], v[slot], fabs(zeta_new[slot]), (int32_t)id_a);
@@ -899,6 +1034,12 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
         }
         __syncwarp();
     }
+    if (__syncthreads_or(heavy)) // what is left of the block's cells
+        for (int g0 = blockIdx.x * W; g0 < n_cells; g0 += nw)
+            for (int g = g0; g < min(g0 + W, n_cells); ++g)
+                if (M.arr[g] > (uint32_t)kSedArrive) // uniform: cleared behind a barrier
+                    sed_merge_heavy(g, cell_off, M, xi, v, zeta_new, id_of_slot, poff, L, &s_key[0][0],
+                                    s_u.heavy);
     if (blockIdx.x == 0 && threadIdx.x == 0) { // the run's record: nothing here reads it
         *M.out_next = 0u;
         rec->xi = L.xi;

@@ -26,13 +26,16 @@ def env():
     return O, sdm, torch
 
 
-def _run(env, sizes, nx, dt, r_lo, r_hi, steps, seed):
+def _run(env, sizes, nx, dt, r_lo, r_hi, steps, seed, levels=None):
     O, sdm, torch = env
     rng = np.random.default_rng(seed)
     n_cells, dz = len(sizes), 10.0
     cell = np.repeat(np.arange(n_cells, dtype=np.int32), sizes)
     n = len(cell)
-    v = 4 / 3 * np.pi * np.exp(rng.uniform(np.log(r_lo), np.log(r_hi), n)) ** 3
+    r = np.exp(rng.uniform(np.log(r_lo), np.log(r_hi), n))
+    if levels is not None:  # every SD as many times larger as it shall fall levels
+        r *= np.maximum(levels[cell], 0.01)
+    v = 4 / 3 * np.pi * r**3
     xi = rng.integers(1, 10**6, n).astype(np.int64)
     xi[rng.random(n) < 0.02] = 0
     zeta = rng.uniform(0.0, dz, n)
@@ -73,3 +76,9 @@ def test_about_the_largest_cell(env, sizes):
 
 def test_many_cells(env):
     _run(env, list(np.random.default_rng(1).integers(0, 4, 70000)), 100, 5.0, 1e-5, 1e-3, 2, 9)
+
+
+@pytest.mark.parametrize("per", [300, 700, 1000])
+def test_cells_pile_up(env, per):
+    # four levels fall into the lowest: 4 per arrivals there (2048 are one run of the block's sort)
+    _run(env, [per, per, per - 1, per, per + 1], 1, 10.0, 1.24e-4, 1.26e-4, 2, per, levels=np.arange(5))
