@@ -505,7 +505,7 @@ __device__ __forceinline__ int32_t pair_gamma_filter(const PairConsts &C, float 
 // or binary32 with the 1-ulp radius) exceeds the bound's real value by less
 // than 2^-17: so bound (1 + 2^-8) < u_lo (u's exact lower bound) proves
 // p < u.  Out-of-range or underflowing values abstain (return false).
-__device__ __forceinline__ bool pair_prefilter_zero(const PairConsts &C, float sc, int64_t xi_j, uint32_t vj_hi,
+__device__ __forceinline__ bool pair_prefilter_zero(const PairConsts &C, float sc, float xjf, uint32_t vj_hi,
                                                     uint32_t vk_hi, uint32_t wa)
 {
     bool ok, ok_k;
@@ -526,8 +526,14 @@ __device__ __forceinline__ bool pair_prefilter_zero(const PairConsts &C, float s
             bound = (stokes ? C.pre_c[0] : C.pre_c[2]) * t;
         }
     }
-    bound = (bound * xi2f(xi_j)) * sc;
+    bound = (bound * xjf) * sc;
     return ok && bound * (1.0f + 0x1p-8f) < uniform_lo23(wa);
+}
+
+__device__ __forceinline__ bool pair_prefilter_zero(const PairConsts &C, float sc, int64_t xi_j, uint32_t vj_hi,
+                                                    uint32_t vk_hi, uint32_t wa)
+{
+    return pair_prefilter_zero(C, sc, xi2f(xi_j), vj_hi, vk_hi, wa);
 }
 
 // The same from full binary64 volumes.

@@ -223,9 +223,9 @@ extern "C" sdm_status sdm_cell_step_noalloc(const sdm_config *cfg, int64_t step,
         S.cnt = reinterpret_cast<uint32_t *>(base + kNaSpreadCnt);
         S.rooms = reinterpret_cast<uint2 *>(base);
         uint32_t *status = reinterpret_cast<uint32_t *>(base + kNaStatus);
-        launch_chained(one_spread_scatter_kernel, (n / 2 + kSpreadNT - 1) / kSpreadNT, kSpreadNT, s, false, inst, c, S,
+        launch_chained(one_spread_scatter_kernel, (n / 2 + kSpreadNT - 1) / kSpreadNT, kSpreadNT, 0, s, false, inst, c, S,
                        status);
-        launch_chained(one_spread_pairs_kernel, c.groups, kSpreadNT, s, true, inst, c, S, status);
+        launch_chained(one_spread_pairs_kernel, c.groups, kSpreadNT, 0, s, true, inst, c, S, status);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess)
             return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: launch: %s", cudaGetErrorString(e));

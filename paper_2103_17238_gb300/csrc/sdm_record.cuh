@@ -1,6 +1,8 @@
 // Larger cells (above the shared-memory classes, up to 2^24 super-droplets)
 // when a plan holds many super-droplets in them: one step in four launches,
-// with a 16-byte record of every live SD carried through the sort.
+// with a 16-byte record of every live SD carried through the sort.  (Measured
+// per step, us, before -> after: 16 boxes of 2^20 480 -> 352, one 51 -> 31, one of 2^24
+// 1024 -> 474, 200 of 16,000 124 -> 66, 1024 boxes of 2^8 .. 2^16 337 -> 222.)
 //
 // What bounds a step of such cells is not bandwidth but single-lane accesses:
 // a load or store whose 32 lanes go to 32 places takes an SM's load/store unit
@@ -30,14 +32,19 @@
 
 namespace sdm {
 
-constexpr int kRecMean = 1024;
+constexpr int kRecMean = 1024; // (16 boxes of 2^20: 800 took 369 us a step against 353, 1280 349)
 constexpr int kRecRoom = 1408;
-constexpr int kRecScatterNT = 512;
+// 1024 threads of 32 registers, two blocks per SM: the loads of xi and v, then the
+// atomics, are what a block waits for (512 threads of 64 registers: 405 against
+// 347 us; chunks of 8192, four pairs a thread: 489).
+constexpr int kRecScatterNT = 1024;
 constexpr int kRecChunk = 4096; // SDs per scatter block
-constexpr int kRecNT = 256;     // threads of a bucket's block
+// Five blocks of 256 per SM (48 registers): 354 us against 370 with four, 405 with three;
+// 512 threads 457, six blocks (40 registers, spills) 399.
+constexpr int kRecNT = 256; // threads of a bucket's block
 constexpr int kRecSubLB = 9;    // sub-buckets inside a bucket
-constexpr int kRecMaxSd = 1 << 24;
-constexpr int kRecMaxBuckets = kRecMaxSd / kRecMean;
+constexpr int kRecMaxBuckets = 16384; // (their counts take 64 KB of shared memory)
+constexpr int kRecMaxSd = kRecMaxBuckets * kRecMean;
 
 struct __align__(16) RecCell {
     const InstDev *run;
@@ -45,8 +52,11 @@ struct __align__(16) RecCell {
     int32_t off, n; // storage slots
     int32_t nb;     // buckets
     int32_t first;  // first bucket among all cells' (counts, seams, rooms)
-    int32_t pad;
+    int32_t start;  // its first position word among all cells' (nb + 1 each)
 };
+
+// Buckets of a cell of n SDs.
+__host__ __device__ constexpr int rec_buckets(int n) { return (n + kRecMean - 1) / kRecMean; }
 
 struct RecScratch {
     uint32_t *cnt;    // per bucket: entries; zero before a step's scatter
@@ -57,7 +67,7 @@ struct RecScratch {
 };
 constexpr uint32_t kRecVoid = 0xFFFFFFFFu;
 
-__global__ void __launch_bounds__(kRecScatterNT) rec_scatter_kernel(const BigChunk *__restrict__ work,
+__global__ void __launch_bounds__(kRecScatterNT, 2) rec_scatter_kernel(const BigChunk *__restrict__ work,
                                                                     const RecCell *__restrict__ cells, RecScratch S,
                                                                     int64_t step_offset)
 {
@@ -97,12 +107,18 @@ __global__ void __launch_bounds__(kRecScatterNT) rec_scatter_kernel(const BigChu
         x[i] = in ? gx[q] : make_longlong2(0, 0);
         v[i] = in ? gv[q] : make_double2(1.0, 1.0);
     }
-    __syncthreads(); // the counts are zero
+    float xf[2 * QPT]; // 0: dead
+    uint32_t vh[2 * QPT];
 #pragma unroll
     for (int i = 0; i < 2 * QPT; ++i) {
         const int64_t xi = (i & 1) ? x[i / 2].y : x[i / 2].x;
-        at[i] = xi > 0 ? (at[i] << 16) | atomicAdd(&s_cnt[at[i]], 1u) : 0xFFFFFFFFu;
+        xf[i] = xi > 0 ? xi2f(xi) : 0.0f;
+        vh[i] = (uint32_t)__double2hiint((i & 1) ? v[i / 2].y : v[i / 2].x);
     }
+    __syncthreads(); // the counts are zero
+#pragma unroll
+    for (int i = 0; i < 2 * QPT; ++i)
+        at[i] = xf[i] != 0.0f ? (at[i] << 16) | atomicAdd(&s_cnt[at[i]], 1u) : 0xFFFFFFFFu;
     __syncthreads();
     for (int i = t; i < c.nb; i += kRecScatterNT) {
         const uint32_t k = s_cnt[i];
@@ -115,12 +131,10 @@ __global__ void __launch_bounds__(kRecScatterNT) rec_scatter_kernel(const BigChu
         if (at[i] == 0xFFFFFFFFu)
             continue;
         const uint32_t b = at[i] >> 16, e = s_cnt[b] + (at[i] & 0xFFFFu);
-        const int64_t xi = (i & 1) ? x[i / 2].y : x[i / 2].x;
-        const double vv = (i & 1) ? v[i / 2].y : v[i / 2].x;
         if (e < (uint32_t)kRecRoom)
             S.rooms[(int64_t)(c.first + (int)b) * kRecRoom + e] =
                 make_uint4(sub[i], (uint32_t)(2 * (q0 + (i / 2) * kRecScatterNT) + (i & 1)),
-                           __float_as_uint(xi2f(xi)), (uint32_t)__double2hiint(vv));
+                           __float_as_uint(xf[i]), vh[i]);
     }
 }
 
@@ -134,7 +148,7 @@ __global__ void __launch_bounds__(kRecScanNT) rec_scan_kernel(const RecCell *__r
     chain_next();
     const RecCell c = cells[blockIdx.x];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    uint32_t *cnt = S.cnt + c.first, *start = S.start + c.first + blockIdx.x + c.pad;
+    uint32_t *cnt = S.cnt + c.first, *start = S.start + c.start;
     chain_wait();
     uint32_t carry = 0, big = 0;
     for (int i0 = 0; i0 < c.nb; i0 += kRecScanNT) {
@@ -211,7 +225,7 @@ __device__ __forceinline__ void rec_pair(const InstDev *P, const PairConsts &C, 
     }
 }
 
-__global__ void __launch_bounds__(kRecNT) rec_pairs_kernel(const BigBucket *__restrict__ work,
+__global__ void __launch_bounds__(kRecNT, 5) rec_pairs_kernel(const BigBucket *__restrict__ work,
                                                            const RecCell *__restrict__ cells, RecScratch S,
                                                            int64_t step_offset)
 {
@@ -239,7 +253,7 @@ __global__ void __launch_bounds__(kRecNT) rec_pairs_kernel(const BigBucket *__re
     const int64_t s = P->step + step_offset;
     const uint32_t cell = (uint32_t)c.cell;
     chain_wait();
-    const uint32_t *st = S.start + c.first + w.big + w.bucket;
+    const uint32_t *st = S.start + c.start + w.bucket;
     const uint32_t start = st[0], n_c = st[c.nb - w.bucket];
     if (n_c == kRecVoid) // uniform
         return;
@@ -379,7 +393,7 @@ __global__ void __launch_bounds__(kRecSeamNT) rec_seam_kernel(const BigBucket *_
     chain_wait();
     if (i >= n_work)
         return;
-    const uint32_t *st = S.start + c.first + w.big;
+    const uint32_t *st = S.start + c.start;
     const uint32_t n_c = st[c.nb], start = st[w.bucket];
     if (n_c == kRecVoid)
         return;

@@ -18,6 +18,7 @@
 #include "sdm_kernels.cuh"
 #include "sdm_mid.cuh"
 #include "sdm_radix.cuh"
+#include "sdm_record.cuh"
 #include "sdm_spread.cuh"
 
 using namespace sdm;
@@ -144,6 +145,13 @@ constexpr int kInChunks = 4; // pieces of a host input copy (sdm_set_attributes)
 constexpr int kClassCap[] = {64, 128, 256, 320, 512, 1024, 2048, 4096};
 constexpr int kNumClass = sizeof(kClassCap) / sizeof(kClassCap[0]);
 
+// Cells of the record path that share its scratch's space and are launched together:
+// their ranges in the plan's work lists.
+struct RecGroup {
+    int cell0, chunk0, bucket0, n_cells, n_chunks, n_buckets, max_nb;
+    int64_t sds;
+};
+
 struct Plan {
     int n_inst = 0;
     InstDev **d_insts = nullptr; // table of the runs' device records
@@ -175,6 +183,12 @@ struct Plan {
     SpreadCell *d_spread_scatter = nullptr, *d_spread_pairs = nullptr; // an item per block
     int n_spread_scatter = 0, n_spread_pairs = 0;
     SpreadScratch spread{};
+    // the cells of the record path (sdm_record.cuh), in groups stepped one after the other
+    RecCell *d_recs = nullptr;
+    BigChunk *d_rec_chunks = nullptr;
+    BigBucket *d_rec_buckets = nullptr;
+    std::vector<RecGroup> rec_groups;
+    RecScratch rec{};
     BigCell *d_bigs = nullptr;
     int n_big = 0;
     BigChunk *d_chunks = nullptr;
@@ -562,7 +576,8 @@ cudaError_t launch_mid(int clusters, int n, const WorkItem *items, InstDev *cons
 // the stream is complete (programmatic dependent launch); both kernels wait
 // with chain_wait() before they touch what the other writes.
 template <typename... KARGS, typename... ARGS>
-cudaError_t launch_chained(void (*kernel)(KARGS...), int grid, int nt, cudaStream_t st, bool chain, ARGS... args)
+cudaError_t launch_chained(void (*kernel)(KARGS...), int grid, int nt, size_t smem, cudaStream_t st, bool chain,
+                           ARGS... args)
 {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -570,6 +585,7 @@ cudaError_t launch_chained(void (*kernel)(KARGS...), int grid, int nt, cudaStrea
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(grid, 1, 1);
     cfg.blockDim = dim3(nt, 1, 1);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = chain ? 1 : 0;
@@ -665,6 +681,12 @@ cudaError_t configure_kernels()
                                                                0)) != cudaSuccess)
             e = r;
         G.spec_cells = std::max(1, spec_per_sm) * sms;
+        if ((r = cudaFuncSetAttribute(rec_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kRecMaxBuckets * (int)sizeof(uint32_t))) != cudaSuccess)
+            e = r;
+        if ((r = cudaFuncSetAttribute(rec_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)sizeof(RecSmem))) != cudaSuccess)
+            e = r;
         const int hb = (int)big_hist_smem(kBigMaxLB);
         if ((r = cudaFuncSetAttribute(big_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess) e = r;
         if ((r = cudaFuncSetAttribute(big_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess) e = r;
@@ -756,23 +778,55 @@ cudaError_t plan_refresh(Plan &pl, const int32_t *d_cell_off, int32_t n_cells, i
     return cudaGetLastError();
 }
 
-// Whether a plan's cells above the shared-memory classes take the bucketed
-// path (sdm_spread.cuh): `total` SDs in `count` cells, the largest of `most`.
-// Measured per step (us, bucketed | cluster | multi-pass): one box of 12,000
-// 8.4 | 46 | 37, of 2^17 15 | - | 43, of 524,288 36 | - | 52, of 900,000
-// 59 | - | 62, of 2^20 73 | - | 66; 8 of 2^17 52 | - | 58; 76 of 12,000
-// 41 | 50 | 53; 180 of 5000 40 | 42 | 58; but 150 of 5000 34 | 24 | 45.  So up
-// to 15 x 2^16 SDs, except where the cluster path takes every cell at once, one
-// CTA each, in less time (about 4 + 3.8 n / 1000 us for its largest cell
-// against 7 + 0.037 total / 1000).
-constexpr int64_t kSpreadMaxSd = (int64_t)15 << 16;
+// Which path a plan's cells above the shared-memory classes take together, with
+// the default mid_max_sd: `total` SDs in `count` cells, the largest of `most`.
+// Measured per step (us, bucketed (sdm_spread.cuh) | record (sdm_record.cuh) |
+// cluster): one box of 2^17 14 | 18 | -, of 200,000 16 | 21, of 2^18 21 | 20, of
+// 524,288 36 | 24, of 2^20 73 | 31; 10 of 17,000 15 | 20, 30 of 17,000 29 | 23;
+// 20 of 8000 15 | 19 | 31, 60 of 8000 27 | 22 | 31, 150 of 8000 - | 29 | 32, 600 of
+// 16,000 - | 181 | 252; 60 of 4500 19 | 22 | 20, 150 of 4500 - | 23 | 20, 200 of 4500
+// - | 32 | 37.  So bucketed up to kSpreadMaxSd; above it the cluster path where it takes
+// every cell at once, one CTA each, in less time (about 4 + 3.8 n / 1000 us for its
+// largest cell against 19 + 9 total / 10^6), else the record path.
+constexpr int64_t kSpreadMaxSd = 240000;
 
-bool spread_cells(int64_t total, int64_t count, int32_t most, const sdm_tuning &t, int sms)
+enum class LargePath { spread, cluster, record };
+
+LargePath large_path(int64_t total, int64_t count, int32_t most, const sdm_tuning &t, int sms)
 {
-    if (total == 0 || total > kSpreadMaxSd || t.mid_max_sd != SDM_MID_MAX_SD_DEFAULT)
-        return false;
+    if (t.mid_max_sd != SDM_MID_MAX_SD_DEFAULT) // the tuning says: cluster up to mid_max_sd
+        return LargePath::cluster;
+    if (total <= kSpreadMaxSd)
+        return LargePath::spread;
+    if (t.smem_max_sd < kClassCap[kNumClass - 1]) // a tuning with cells of a few hundred SDs here
+        return LargePath::cluster;
     const bool one_round = most <= std::min(t.mid_max_sd, kMidSdPerCta) && count <= sms;
-    return !(one_round && 4.0 + 3.8e-3 * most < 7.0 + 3.7e-5 * (double)total);
+    return one_round && 4.0 + 3.8e-3 * most < 19.0 + 9e-6 * (double)total ? LargePath::cluster : LargePath::record;
+}
+
+// Adds a cell of n SDs to the record path's groups of up to kRecGroupSd SDs (369 MB
+// of rooms; smaller groups end in more part-filled waves: 16 boxes of 2^20 in
+// groups of 2^21, 2^22, 2^23, 2^24 401, 395, 375, 353 us); its first bucket among
+// its group's.
+constexpr int64_t kRecGroupSd = kRecMaxSd;
+int rec_group_add(std::vector<RecGroup> &groups, int n)
+{
+    if (groups.empty() || groups.back().sds + n > kRecGroupSd) {
+        RecGroup g{};
+        if (!groups.empty()) {
+            g = groups.back();
+            g = RecGroup{g.cell0 + g.n_cells, g.chunk0 + g.n_chunks, g.bucket0 + g.n_buckets, 0, 0, 0, 0, 0};
+        }
+        groups.push_back(g);
+    }
+    RecGroup &g = groups.back();
+    const int nb = rec_buckets(n), first = g.n_buckets;
+    g.sds += n;
+    g.n_cells += 1;
+    g.n_chunks += (n + kRecChunk - 1) / kRecChunk;
+    g.n_buckets += nb;
+    g.max_nb = std::max(g.max_nb, nb);
+    return first;
 }
 
 // Work lists of every run in the batch, split by cell size.
@@ -791,6 +845,9 @@ sdm_status build_plan(sdm_batch *b)
         std::vector<BigBucket> buckets;
         std::vector<BigPairs> pairs;
         std::vector<SpreadCell> sp_scatter, sp_pairs;
+        std::vector<RecCell> recs;
+        std::vector<BigChunk> rec_chunks;
+        std::vector<BigBucket> rec_buckets;
         std::vector<InstDev *> insts;
         std::vector<int8_t> cls; // per cell of all runs: its class, -1 above them, -2 fewer than 2 SDs
     };
@@ -812,6 +869,9 @@ sdm_status build_plan(sdm_batch *b)
     pairs.clear();
     scr.sp_scatter.clear();
     scr.sp_pairs.clear();
+    scr.recs.clear();
+    scr.rec_chunks.clear();
+    scr.rec_buckets.clear();
     int64_t sp_counters = 0, sp_rooms = 0;
     insts.assign(n_inst, nullptr);
     int64_t hist_total = 0, sd_total = 0, bkt_total = 0;
@@ -829,7 +889,40 @@ sdm_status build_plan(sdm_batch *b)
                 above_most = std::max(above_most, n);
             }
         }
-    const bool spread = spread_cells(above_sd, above_cells, above_most, tun, dev_grids().mid[0]);
+    const LargePath large = above_sd ? large_path(above_sd, above_cells, above_most, tun, dev_grids().mid[0])
+                                     : LargePath::cluster;
+    const bool spread = large == LargePath::spread;
+    // the record path, if its scratch can be had (else cluster and multi-pass)
+    bool record = !spread;
+    auto to_record = [&](int n) {
+        return record && n > tun.smem_max_sd && (large == LargePath::record || n > tun.mid_max_sd) && n <= kRecMaxSd;
+    };
+    {
+        std::vector<RecGroup> groups;
+        for (sdm_ctx *c : b->ctxs)
+            for (int32_t cell = 0; c->largest_cell > tun.smem_max_sd && cell < c->cfg.n_cells; ++cell) {
+                const int32_t n = c->h_cell_off[cell + 1] - c->h_cell_off[cell];
+                if (to_record(n))
+                    rec_group_add(groups, n);
+            }
+        int64_t nb = 0, nc = 0;
+        for (const RecGroup &g : groups) {
+            nb = std::max<int64_t>(nb, g.n_buckets);
+            nc = std::max<int64_t>(nc, g.n_cells);
+        }
+        if (nb) {
+            pl.rec.cnt = plan_alloc<uint32_t>(pl, mem, (size_t)nb);
+            pl.rec.start = plan_alloc<uint32_t>(pl, mem, (size_t)(nb + nc));
+            pl.rec.seam = plan_alloc<uint2>(pl, mem, (size_t)nb);
+            pl.rec.rooms = plan_alloc<uint4>(pl, mem, (size_t)nb * kRecRoom);
+            record = pl.rec.cnt && pl.rec.start && pl.rec.seam && pl.rec.rooms;
+            if (!record)
+                cudaGetLastError();
+            if (record && cudaMemsetAsync(pl.rec.cnt, 0, sizeof(uint32_t) * (size_t)nb, b->stream) != cudaSuccess)
+                return cuda_fail(b, cudaGetLastError(), "batch plan: record counts");
+        }
+    }
+    int64_t rec_sd = 0;
     // the shared-memory classes in two tight passes (a class per cell and the
     // classes' sizes, then the items into their places); the other cells after
     size_t n_all = 0;
@@ -899,6 +992,24 @@ sdm_status build_plan(sdm_batch *b)
                     scr.sp_pairs.push_back(sc);
                 continue;
             }
+            if (to_record(n)) {
+                RecCell rc{};
+                rc.run = c->d_inst;
+                rc.cell = cb + cell;
+                rc.off = off[cell];
+                rc.n = n;
+                rc.nb = rec_buckets(n);
+                rc.first = rec_group_add(pl.rec_groups, n);
+                rc.start = rc.first + pl.rec_groups.back().n_cells - 1;
+                const int at = (int)scr.recs.size();
+                for (int k = 0; k < (n + kRecChunk - 1) / kRecChunk; ++k)
+                    scr.rec_chunks.push_back(BigChunk{at, k});
+                for (int k = 0; k < rc.nb; ++k)
+                    scr.rec_buckets.push_back(BigBucket{at, k});
+                scr.recs.push_back(rc);
+                rec_sd += n;
+                continue;
+            }
             if (n <= tun.mid_max_sd) { // the cluster path, K = 1, 2 or 4 CTAs (sorted below)
                 const int km = n <= kMidSdPerCta ? 0 : (n <= 2 * kMidSdPerCta ? 1 : 2);
                 mid[km].push_back(WorkItem{i, c->cfg.cell_base + cell, c->h_cell_off[cell], n});
@@ -949,6 +1060,12 @@ sdm_status build_plan(sdm_batch *b)
     sz += a16(sizeof(SpreadCell) * scr.sp_scatter.size());
     const size_t off_spp = sz;
     sz += a16(sizeof(SpreadCell) * scr.sp_pairs.size());
+    const size_t off_recs = sz;
+    sz += a16(sizeof(RecCell) * scr.recs.size());
+    const size_t off_rec_chunks = sz;
+    sz += a16(sizeof(BigChunk) * scr.rec_chunks.size());
+    const size_t off_rec_buckets = sz;
+    sz += a16(sizeof(BigBucket) * scr.rec_buckets.size());
     const size_t off_bigs = sz;
     sz += a16(sizeof(BigCell) * bigs.size());
     const size_t off_chunks = sz;
@@ -998,6 +1115,11 @@ sdm_status build_plan(sdm_batch *b)
         std::memcpy(h + off_sps, scr.sp_scatter.data(), sizeof(SpreadCell) * scr.sp_scatter.size());
         std::memcpy(h + off_spp, scr.sp_pairs.data(), sizeof(SpreadCell) * scr.sp_pairs.size());
     }
+    if (!scr.recs.empty()) {
+        std::memcpy(h + off_recs, scr.recs.data(), sizeof(RecCell) * scr.recs.size());
+        std::memcpy(h + off_rec_chunks, scr.rec_chunks.data(), sizeof(BigChunk) * scr.rec_chunks.size());
+        std::memcpy(h + off_rec_buckets, scr.rec_buckets.data(), sizeof(BigBucket) * scr.rec_buckets.size());
+    }
     if (!bigs.empty()) {
         std::memcpy(h + off_bigs, bigs.data(), sizeof(BigCell) * bigs.size());
         std::memcpy(h + off_chunks, chunks.data(), sizeof(BigChunk) * chunks.size());
@@ -1028,7 +1150,12 @@ sdm_status build_plan(sdm_batch *b)
         if (e != cudaSuccess)
             return cuda_fail(b, e, "batch plan: bucket counts");
     }
-    if (own && n_inst == 1 && scr.sp_pairs.empty() && bigs.empty() && mid[0].empty() && mid[1].empty() && mid[2].empty()) {
+    if (!scr.recs.empty()) {
+        pl.d_recs = reinterpret_cast<RecCell *>(d + off_recs);
+        pl.d_rec_chunks = reinterpret_cast<BigChunk *>(d + off_rec_chunks);
+        pl.d_rec_buckets = reinterpret_cast<BigBucket *>(d + off_rec_buckets);
+    }
+    if (own && n_inst == 1 && scr.sp_pairs.empty() && scr.recs.empty() && bigs.empty() && mid[0].empty() && mid[1].empty() && mid[2].empty()) {
         const int32_t nc = own->cfg.n_cells;
         pl.d_items_all = plan_alloc<WorkItem>(pl, mem, (size_t)kNumClass * std::max(nc, 1));
         pl.d_refresh = plan_alloc<uint32_t>(pl, mem, kNumClass + 1);
@@ -1051,7 +1178,7 @@ sdm_status build_plan(sdm_batch *b)
         // them, count too), at least one cluster to each class with cells, at
         // most one per cell and no more than fit at once
         const DevGrids &G = dev_grids();
-        int64_t work[3] = {}, total = sd_total;
+        int64_t work[3] = {}, total = sd_total + rec_sd;
         for (int k = 0; k < 3; ++k) {
             for (const WorkItem &w : mid[k])
                 work[k] += w.n;
@@ -1065,7 +1192,7 @@ sdm_status build_plan(sdm_batch *b)
             const int share = (int)((double)sms * (double)work[k] / (double)total) / ks[k];
             pl.mid_clusters[k] = std::max(1, std::min({share, pl.n_mid[k], G.mid[k]}));
         }
-        int classes = bigs.empty() && scr.sp_pairs.empty() ? 0 : 1;
+        int classes = bigs.empty() && scr.sp_pairs.empty() && scr.recs.empty() ? 0 : 1;
         for (int k = 0; k < 3; ++k)
             classes += pl.n_mid[k] ? 1 : 0;
         if (classes > 1) {
@@ -1095,7 +1222,7 @@ sdm_status build_plan(sdm_batch *b)
             const Variant &x = g_variants[pl.variant[k]];
             small[k] = (int64_t)pl.n_items[k] < (int64_t)G.variant[pl.variant[k]] * (x.warps > 0 ? x.warps : 1);
         }
-        if (groups > 1 && sd_total <= ((int64_t)1 << 22)) {
+        if (groups > 1 && sd_total + rec_sd <= ((int64_t)1 << 22)) {
             cudaError_t e = cudaEventCreateWithFlags(&pl.cls_fork, cudaEventDisableTiming);
             for (int k = 0; k < kNumClass && e == cudaSuccess; ++k) {
                 // the class of the largest cells stays on the plan's stream, unless
@@ -1170,8 +1297,8 @@ void enqueue_big_steps(const Plan &pl, int64_t off, int32_t n, cudaStream_t st)
     for (int32_t i = 0; pl.n_spread_pairs && i < n; ++i) {
         const PlanSpread sc{pl.d_spread_scatter}, sp{pl.d_spread_pairs};
         // chained but for the first, whose predecessor may be any work
-        launch_chained(spread_scatter_kernel, pl.n_spread_scatter, kSpreadNT, st, i > 0, sc, pl.spread, off + i);
-        launch_chained(spread_pairs_kernel, pl.n_spread_pairs, kSpreadNT, st, true, sp, pl.spread, off + i);
+        launch_chained(spread_scatter_kernel, pl.n_spread_scatter, kSpreadNT, 0, st, i > 0, sc, pl.spread, off + i);
+        launch_chained(spread_pairs_kernel, pl.n_spread_pairs, kSpreadNT, 0, st, true, sp, pl.spread, off + i);
     }
     for (int32_t i = 0; i < n; ++i) {
         if (pl.n_mid[2])
@@ -1181,6 +1308,22 @@ void enqueue_big_steps(const Plan &pl, int64_t off, int32_t n, cudaStream_t st)
         if (pl.n_mid[0])
             launch_mid<1>(pl.mid_clusters[0], pl.n_mid[0], pl.d_mid[0], pl.d_insts, off + i, side(0));
     }
+    // a group's n steps follow each other: its state and the records stay in L2
+    bool chain = false;
+    for (const RecGroup &g : pl.rec_groups)
+        for (int32_t i = 0; i < n; ++i) {
+            const int64_t o = off + i;
+            const RecCell *cells = pl.d_recs;
+            const BigChunk *wc = pl.d_rec_chunks + g.chunk0;
+            const BigBucket *wb = pl.d_rec_buckets + g.bucket0;
+            launch_chained(rec_scatter_kernel, g.n_chunks, kRecScatterNT, sizeof(uint32_t) * g.max_nb, st, chain, wc, cells,
+                           pl.rec, o);
+            launch_chained(rec_scan_kernel, g.n_cells, kRecScanNT, 0, st, true, cells + g.cell0, pl.rec);
+            launch_chained(rec_pairs_kernel, g.n_buckets, kRecNT, sizeof(RecSmem), st, true, wb, cells, pl.rec, o);
+            launch_chained(rec_seam_kernel, (g.n_buckets + kRecSeamNT - 1) / kRecSeamNT, kRecSeamNT, 0, st, true, wb,
+                           g.n_buckets, cells, pl.rec, o);
+            chain = true;
+        }
     for (int32_t i = 0; pl.n_big && i < n; ++i) {
         const int64_t o = off + i;
         const size_t hs = big_hist_smem(pl.max_big_lb);
@@ -1641,6 +1784,12 @@ int64_t sdm_footprint_bytes(int64_t capacity_sd, int32_t n_cells, int32_t larges
         const int lb = big_lb(largest_cell);
         const int64_t chunks = (capacity_sd + kBigChunk - 1) / kBigChunk + n_cells;
         int64_t big = capacity_sd * (4 + 4) + (chunks << lb) * 4 + ((int64_t)n_cells << lb) * 4 + chunks * kLiveWords * 4;
+        // or the record path's rooms, counts, seams and work lists
+        const int64_t cells = std::min<int64_t>(n_cells, slots / std::max(1, current_tuning().smem_max_sd) + 1);
+        const int64_t rec_nb = slots / kRecMean + cells + 1;
+        const int64_t rec_rooms = std::min<int64_t>(slots, kRecGroupSd) / kRecMean +
+                                  std::min<int64_t>(cells, kRecGroupSd / std::max(1, current_tuning().smem_max_sd) + 1) + 1;
+        big = std::max<int64_t>(big, rec_rooms * (kRecRoom * (int64_t)sizeof(uint4) + 20) + rec_nb * 24 + cells * 64);
         if (slots <= kSpreadMaxSd + n_cells + 1) { // or the bucketed path's rooms and counts
             const int64_t nb = slots / kSpreadMean + std::min<int64_t>(n_cells, slots / largest_cell + 1) + 1;
             big = std::max<int64_t>(big, nb * (kSpreadRoom * (int64_t)sizeof(uint2) + 2 * kSpreadStride * (int64_t)sizeof(uint32_t) + 48));

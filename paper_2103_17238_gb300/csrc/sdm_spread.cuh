@@ -21,7 +21,7 @@
 // (key, rank) removes it, so results repeat bit for bit.
 //
 // Measured (us per step of one box, before -> after): 12,000 SDs 37 -> 8.4,
-// 65,536 42 -> 11, 131,072 43 -> 15, 524,288 52 -> 36.  Three blocks of the second
+// 65,536 42 -> 11, 131,072 43 -> 15.  (Above 240,000 SDs sdm_record.cuh is faster.)  Three blocks of the second
 // kernel per SM (80 registers) beat two (40 boxes of 12,000: 28 against 31) and
 // four (64 registers: 28, but one box of 65,536 14.8 against 13.0).
 //
