@@ -1810,11 +1810,14 @@ constexpr int kSpecRep = 4;
 // above (.y: greater) the volume of edge i; one sentinel after the last.
 // start[k]: the last edge certainly below every v whose high word >> shift
 // is base + k (0: below all of the table; -1 as 255).
+struct SpecRecip { // 1 / x = m 2^w, m's top bit set (m = 0: x is 0 or infinite)
+    uint64_t m;
+    int32_t w;
+};
 struct SpecTab {
     double edge[kSpecMaxBins + 1];
-    double den[kSpecMaxBins];      // volume of air x width of the bin in ln r
-    uint64_t recip[kSpecMaxBins];  // 1 / den = recip 2^recip_w, recip's top bit set
-    int32_t recip_w[kSpecMaxBins];
+    double vol, dln[kSpecMaxBins]; // volume of air; width of each bin in ln r
+    SpecRecip vol_r, dln_r[kSpecMaxBins];
     uint2 key[kSpecMaxBins + 2];
     int32_t n_edges, shift, base, nt;
     uint8_t start[kSpecTabMax];
@@ -1946,18 +1949,20 @@ __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, cons
 
 // x / den by the 64-bit reciprocal (x >= 0): within 0.5 + 2^-9 ulp, where the
 // binary64 division would cost as much as everything else of a small cell.
-__device__ __forceinline__ double spec_divide(const SpecTab &T, int b, double x)
+__device__ __forceinline__ double spec_divide(double x, double den, const SpecRecip &r)
 {
     const uint64_t bits = (uint64_t)__double_as_longlong(x);
+    if (bits == 0 && r.m != 0)
+        return 0.0;
     const int e = (int)(bits >> 52);
-    const int w = e - 1075 + T.recip_w[b] + 53;
-    if (e == 0 || (unsigned)(w + 64 + 1000) > 2000u) // zero, or a result near the ends of the range
-        return x == 0.0 ? 0.0 : x / T.den[b];
-    return u64_to_double(__umul64hi((bits << 11) | (1ull << 63), T.recip[b]), true, w);
+    const int w = e - 1075 + r.w + 53;
+    if (r.m == 0 || e == 0 || e == 0x7FF || (unsigned)(w + 64 + 1000) > 2000u) // no reciprocal, the ends of the range
+        return x / den;
+    return u64_to_double(__umul64hi((bits << 11) | (1ull << 63), r.m), true, w);
 }
 
-// out[b] = (sum over blocks of partial[b][block], fixed order) / den[b], by one
-// warp.
+// out[b] = (sum over blocks of partial[b][block], fixed order) / vol / dln[b], by
+// one warp.
 __device__ __forceinline__ void spec_finish(const SpecTab &T, const double *partial, int32_t n_blocks, int b, double *out)
 {
     const int lane = threadIdx.x & 31;
@@ -1976,7 +1981,7 @@ __device__ __forceinline__ void spec_finish(const SpecTab &T, const double *part
     for (int d = 16; d > 0; d >>= 1)
         sum = __dadd_rn(sum, __shfl_down_sync(0xFFFFFFFFu, sum, d));
     if (lane == 0)
-        out[b] = sum / T.den[b];
+        out[b] = spec_divide(spec_divide(sum, T.vol, T.vol_r), T.dln[b], T.dln_r[b]);
 }
 
 // Sums of every bin over all slots [0, n_slots) (padding and dead SDs hold
@@ -2053,7 +2058,8 @@ __global__ void __launch_bounds__(32 * kSpecWarps) spectrum_cells_kernel(const I
                 continue;
         }
         if (lane < nb)
-            out[(int64_t)c * nb + lane] = spec_divide(T, lane, acc);
+            out[(int64_t)c * nb + lane] =
+                spec_divide(spec_divide(acc, T.vol, T.vol_r), T.dln[lane], T.dln_r[lane]);
     }
 }
 

@@ -11,8 +11,8 @@ namespace sdm {
 constexpr int kRadixNT = 256;
 // Keys per block and pass: 4096 (1,024 tiles of 4.19M keys make one wave; tiles
 // of 2048 or 8192 took 0.224 and 0.241 ms against 0.210 per sort there), or 1024
-// below 2^21 keys, where tiles of 4096 leave SMs with one or none (975,000 keys:
-// RADIX_FIGURES).
+// below 2^21 keys, where tiles of 4096 leave SMs with one or none (sdm_set_attributes of
+// 975,000 in no order 150 against 141 us).
 constexpr int kRadixRounds = 16, kRadixRoundsFew = 4;
 constexpr int64_t kRadixFew = (int64_t)1 << 21;
 constexpr int radix_rounds(int64_t n) { return n < kRadixFew ? kRadixRoundsFew : kRadixRounds; }

@@ -1608,6 +1608,18 @@ void set_prefilter(InstDev &d)
     d.pre_v[1] = down(4.0 / 3.0 * pi * d.r2 * d.r2 * d.r2);
 }
 
+SpecRecip spec_recip(double x)
+{
+    SpecRecip r{};
+    if (!finite_pos(x))
+        return r;
+    int w = 0;
+    const long double m = std::frexp(1.0L / (long double)x, &w); // in [1/2, 1)
+    r.m = (uint64_t)std::ldexp(m, 64);
+    r.w = w - 64;
+    return r;
+}
+
 // The edges of a spectrum of at most kSpecMaxBins bins as its kernels use
 // them (n_edges finite, increasing, > 0).
 SpecTab spec_table(const double *e, int32_t n_edges, double vol)
@@ -1626,13 +1638,11 @@ SpecTab spec_table(const double *e, int32_t n_edges, double vol)
         T.key[i] = make_uint2(lo, std::isfinite(v) ? high_word(v * (1.0 + 0x1p-17)) + 1u : 0xFFFFFFFFu);
     }
     T.key[n_edges] = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
+    T.vol = vol;
+    T.vol_r = spec_recip(vol);
     for (int32_t b = 0; b + 1 < n_edges; ++b) {
-        const double dln = std::log(e[b + 1]) - std::log(e[b]);
-        T.den[b] = vol * dln;
-        int w = 0;
-        const long double r = std::frexp(1.0L / ((long double)vol * (long double)dln), &w); // in [1/2, 1)
-        T.recip[b] = (uint64_t)std::ldexp(r, 64);
-        T.recip_w[b] = w - 64;
+        T.dln[b] = std::log(e[b + 1]) - std::log(e[b]);
+        T.dln_r[b] = spec_recip(T.dln[b]);
     }
     // entry 0 below the first edge, the last one above the last edge
     T.shift = 15;
