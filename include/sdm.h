@@ -310,18 +310,20 @@ typedef struct sdm_tuning {
     int32_t smem_max_sd;     /* largest cell sorted in shared memory: 512, 1024, 2048 or 4096 (default) */
     int32_t warp_cell_max;   /* largest cell run by one warp: 0, 64, 128, 256 or 512 (default), <= smem_max_sd */
     int32_t warps_per_block; /* warps per block of the warp-per-cell kernel: 1, 2 (default) or 4 */
-    int32_t fuse_steps;      /* 2..1024 (default SDM_FUSE_STEPS_DEFAULT): the warp-per-cell kernel
-                              * keeps each cell in shared memory for up to fuse_steps consecutive
-                              * steps of one sdm_batch_step / sdm_coalescence_step call (the same
+    int32_t fuse_steps;      /* 2..1024 (default SDM_FUSE_STEPS_DEFAULT): the kernels of cells up
+                              * to smem_max_sd keep each cell in shared memory for up to fuse_steps
+                              * consecutive steps of one sdm_batch_step / sdm_coalescence_step call (the same
                               * state, bit for bit: cells are independent, so a cell may take its
-                              * steps apart from the others); cells of other sizes still take one
-                              * launch per step, and a one-step call is one launch either way.
+                              * steps apart from the others); larger cells still take their
+                              * launches per step, and a one-step call is one launch either way.
                               * 0 or 1: one launch per step for every cell.  A graph captures the
                               * same launches. */
     int32_t mid_max_sd;      /* largest cell above smem_max_sd stepped by one thread-block cluster
                               * (1, 2 or 4 CTAs of up to 16384 SDs each, the whole step in shared
-                              * and distributed shared memory); larger cells take the multi-pass
-                              * global path.  0: no cluster path.  Default SDM_MID_MAX_SD_DEFAULT. */
+                              * and distributed shared memory); larger cells take passes over
+                              * global memory.  0: no cluster path.  Default SDM_MID_MAX_SD_DEFAULT:
+                              * the library chooses the path of all cells above smem_max_sd from
+                              * their number and sizes (up to this size the cluster may be it). */
 } sdm_tuning;
 
 #define SDM_FUSE_STEPS_DEFAULT 64

@@ -488,6 +488,7 @@ __global__ void sed_pad_kernel(int32_t n_groups, const int32_t *__restrict__ ust
 // sets are freed through their current pointers) and the scratch.
 // ------------------------------------------------- cells of up to kSedByCell
 constexpr int kSedByCell = 1024;  // slots of the largest cell that a warp takes
+constexpr int kSedFewCells = 608, kSedFewLargest = 800; // sdm_sedimentation_step's rule for few cells
 constexpr int kSedArrive = 256;   // arrivals of a cell that a warp takes; more by its block
 constexpr int kSedMergeNT = 128;
 constexpr int kSedFew = 12;       // arrivals up to which each is compared with every stayer, by ballots
@@ -722,6 +723,8 @@ __global__ void __launch_bounds__(1024) sed_offsets_kernel(SedMoves M, int32_t n
         if (g == n_groups - 1)
             poff[n_groups] = (int32_t)(uint32_t)(at + mine);
     }
+    if (g == n_groups - 1) // behind the total: how many SDs move
+        *reinterpret_cast<uint32_t *>(precip_total + 1) = (uint32_t)((at + mine) >> 32);
     if (blockIdx.x == 0)
         sed_precip_total(precip, n_parts, precip_total);
 }
@@ -1079,7 +1082,8 @@ struct SedBuffers {
                                //   arrivals) the next step uses; all arrivals are zero between steps
     uint32_t *counts = nullptr; // n_cells + 1
     int32_t *ustart = nullptr;  // n_cells + 2
-    double *precip = nullptr;   // per-block parts of the move kernel, then the total
+    double *precip = nullptr;   // per-block parts of the move kernel, the total, the movers' count
+    int sorted_left = 0;        // steps that take the sorted path before the movers are counted again
     uint32_t *hist = nullptr;   // 256 x tiles, then 256 digit totals
     uint32_t *flags = nullptr;  // flags, then the first bad id (8-byte aligned)
     int32_t *emig = nullptr;    // per SD id: its cell in another piece of the grid after the last step, or -1
@@ -1089,8 +1093,9 @@ struct SedBuffers {
 };
 
 // Bytes of the pinned read-back buffer for n_cells cells: n_cells + 2
-// offsets, the precipitated total (8-byte aligned) and the class-count words.
-size_t sed_read_bytes(int32_t n_cells) { return (((size_t)n_cells + 2) * 4 + 7) / 8 * 8 + 8 + sizeof(uint32_t) * (kNumClass + 1); }
+// offsets, the precipitated total (8-byte aligned) with the movers' count, and
+// the class-count words.
+size_t sed_read_bytes(int32_t n_cells) { return (((size_t)n_cells + 2) * 4 + 7) / 8 * 8 + 16 + sizeof(uint32_t) * (kNumClass + 1); }
 
 void sed_release(sdm_ctx *ctx)
 {
@@ -1157,7 +1162,7 @@ sdm_status sed_alloc(sdm_ctx *ctx)
     }
     b.counts = sed_get<uint32_t>(ctx, (size_t)nc + 1);
     b.ustart = sed_get<int32_t>(ctx, (size_t)nc + 2);
-    b.precip = sed_get<double>(ctx, (size_t)kSedMaxBlocks + 1);
+    b.precip = sed_get<double>(ctx, (size_t)kSedMaxBlocks + 2);
     b.hist = sed_get<uint32_t>(ctx, radix_hist_words(cap));
     b.flags = sed_get<uint32_t>(ctx, 4);
     b.moves = sed_get<uint32_t>(ctx, 4 * sed_stride(nc) + 2 * ((size_t)nc / 1024 + 1));
@@ -1235,6 +1240,7 @@ sdm_status set_positions_impl(sdm_ctx *ctx, const double *z, int32_t nx, double 
                                                         nx, dz, ctx->cfg.cell_base, zeta_in, ctx->d_zeta, d_flags,
                                                         d_bad);
     ctx->sed->group_valid = false;
+    ctx->sed->sorted_left = 0;
     if (ctx->cfg.cell_base > 0) // only a piece of a grid has emigrants
         CTX_CUDA(ctx, cudaMemsetAsync(ctx->sed->emig, 0xFF, sizeof(int32_t) * ctx->n_sd, s));
     CTX_CUDA(ctx, cudaGetLastError());
@@ -1286,7 +1292,7 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     unsigned char *hr = static_cast<unsigned char *>(b.h_read);
     const int32_t *off = reinterpret_cast<const int32_t *>(hr);
     const size_t at_pr = (((size_t)nc + 2) * 4 + 7) / 8 * 8;
-    const uint32_t *rc = reinterpret_cast<const uint32_t *>(hr + at_pr + 8);
+    const uint32_t *rc = reinterpret_cast<const uint32_t *>(hr + at_pr + 16);
     // on the side stream, beside what follows the new offsets: the refresh of
     // the context's own launch plan (when refreshable: rebuilt on the device for
     // the new layout) and the read-back into the pinned buffer (offsets,
@@ -1294,16 +1300,28 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     auto side_work = [&]() -> sdm_status {
         if (refresh) {
             CTX_CUDA(ctx, plan_refresh(sb->plan, b.cell_off2, nc, ctx->cfg.cell_base, b.side));
-            CTX_CUDA(ctx, cudaMemcpyAsync(hr + at_pr + 8, sb->plan.d_refresh, sizeof(uint32_t) * (kNumClass + 1),
+            CTX_CUDA(ctx, cudaMemcpyAsync(hr + at_pr + 16, sb->plan.d_refresh, sizeof(uint32_t) * (kNumClass + 1),
                                           cudaMemcpyDeviceToHost, b.side));
         }
         CTX_CUDA(ctx, cudaMemcpyAsync(hr, b.cell_off2, sizeof(int32_t) * (n_groups + 1), cudaMemcpyDeviceToHost, b.side));
-        CTX_CUDA(ctx, cudaMemcpyAsync(hr + at_pr, b.precip + kSedMaxBlocks, sizeof(double), cudaMemcpyDeviceToHost,
+        CTX_CUDA(ctx, cudaMemcpyAsync(hr + at_pr, b.precip + kSedMaxBlocks, 2 * sizeof(double), cudaMemcpyDeviceToHost,
                                       b.side));
         CTX_CUDA(ctx, cudaEventRecord(b.join, b.side));
         return SDM_OK;
     };
-    const bool by_cell = ctx->largest_cell <= kSedByCell;
+    // A few cells leave most of the chip idle while a warp follows a cell's movers
+    // and merges them one after the other (us a step, by cells | sorted: 16 to 128 cells of
+    // 1000, 5% moving 55 | 50, all moving 75 | 50; of 600 43 | 50 and 95 | 50; of
+    // 300 33 | 50 and 67 | 50; 512 cells of 1000 66 | 80 and 103 | 93; 4096 cells: by
+    // cells is faster for any share): sorted if the cells are large, or if over a third
+    // of the SDs moved a few steps ago.
+    const bool few = nc <= kSedFewCells;
+    if (!few)
+        b.sorted_left = 0;
+    const bool by_cell = ctx->largest_cell <= kSedByCell && !(2 * nc <= kSedFewCells && ctx->largest_cell > kSedFewLargest) &&
+                         b.sorted_left == 0;
+    if (b.sorted_left > 0)
+        --b.sorted_left;
     if (by_cell) {
         const size_t st_ = sed_stride(nc);
         SedMoves M{b.keys[0], b.vals[0],      b.keys[1],          b.vals[1],   (uint32_t *)b.group, (uint32_t *)b.group2,
@@ -1374,6 +1392,12 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     CTX_CUDA(ctx, cudaEventSynchronize(b.join));
     double precip = 0.0;
     std::memcpy(&precip, hr + at_pr, sizeof precip);
+    if (by_cell && few) {
+        uint32_t movers = 0;
+        std::memcpy(&movers, hr + at_pr + 8, sizeof movers);
+        if ((int64_t)movers * 3 > n)
+            b.sorted_left = 16;
+    }
     // the new layout becomes the state; the old one the next scratch
     std::swap(ctx->d_xi, b.xi2);
     std::swap(ctx->d_v, b.v2);

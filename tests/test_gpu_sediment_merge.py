@@ -1,7 +1,7 @@
 """The sedimentation step by cells (each new cell merged from its stayers and
 its arrivals) against the oracle, at the sizes where it can go wrong: every SD
 of a cell falling at once (up to, and beyond, the 512 arrivals sorted in shared
-memory), cells about 1024 slots (above it all SDs are sorted instead, and the
+memory; few cells go over to the sort then, many do not), cells about 1024 slots (above it all SDs are sorted instead, and the
 layout passes from one path to the other), over 65,536 cells (offsets over
 block totals), and a piece of a grid."""
 import numpy as np
@@ -82,3 +82,14 @@ def test_many_cells(env):
 def test_cells_pile_up(env, per):
     # four levels fall into the lowest: 4 per arrivals there (2048 are one run of the block's sort)
     _run(env, [per, per, per - 1, per, per + 1], 1, 10.0, 1.24e-4, 1.26e-4, 2, per, levels=np.arange(5))
+
+
+@pytest.mark.parametrize("per", [257, 500, 1000])
+def test_whole_cells_fall_among_many(env, per):
+    _run(env, [per] * 5 + [2] * 640, 1, 10.0, 1.2e-4, 1.24e-4, 4, per)
+
+
+@pytest.mark.parametrize("per", [200, 700])
+def test_cells_pile_up_among_many(env, per):
+    levels = np.concatenate([np.arange(5), np.zeros(640)])
+    _run(env, [per, per, per - 1, per, per + 1] + [2] * 640, 1, 10.0, 1.24e-4, 1.26e-4, 2, per, levels=levels)
