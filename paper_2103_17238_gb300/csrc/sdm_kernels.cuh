@@ -2016,14 +2016,41 @@ __global__ void __launch_bounds__(32 * kSpecWarps) spectrum_total_kernel(InstDev
     }
 }
 
-// The spectrum from the partial sums of more blocks: one warp (block) per bin.
-__global__ void spectrum_total_finalize_kernel(const InstDev *__restrict__ P, const double *__restrict__ partial,
-                                               int32_t n_blocks, const __grid_constant__ SpecTab T,
-                                               double *__restrict__ out, uint32_t *status)
+// The spectrum from the partial sums of more blocks: one block per bin, a load
+// or five per thread at once (7.6 us for 1064 partials by one warp each, 4.7 now).
+constexpr int kSpecFinalNT = 256;
+__global__ void __launch_bounds__(kSpecFinalNT) spectrum_total_finalize_kernel(const InstDev *__restrict__ P,
+                                                                               const double *__restrict__ partial,
+                                                                               int32_t n_blocks,
+                                                                               const __grid_constant__ SpecTab T,
+                                                                               double *__restrict__ out, uint32_t *status)
 {
-    spec_finish(T, partial, n_blocks, blockIdx.x, out);
-    if (status && blockIdx.x == 0 && threadIdx.x == 0)
-        *status = P->status;
+    constexpr int U = 5;
+    __shared__ double s_sum[kSpecFinalNT / 32];
+    const int t = threadIdx.x, b = blockIdx.x;
+    double sum = 0.0;
+    for (int j0 = t; j0 < n_blocks; j0 += U * kSpecFinalNT) {
+        double p[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            p[u] = j0 + u * kSpecFinalNT < n_blocks ? partial[(int64_t)b * n_blocks + j0 + u * kSpecFinalNT] : 0.0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            sum = __dadd_rn(sum, p[u]);
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1)
+        sum = __dadd_rn(sum, __shfl_down_sync(0xFFFFFFFFu, sum, d));
+    if ((t & 31) == 0)
+        s_sum[t >> 5] = sum;
+    __syncthreads();
+    if (t == 0) {
+        for (int w = 1; w < kSpecFinalNT / 32; ++w)
+            sum = __dadd_rn(sum, s_sum[w]);
+        out[b] = spec_divide(spec_divide(sum, T.vol, T.vol_r), T.dln[b], T.dln_r[b]);
+        if (status && b == 0)
+            *status = P->status;
+    }
 }
 
 // dv/dlnr of every cell, cell-major.  One warp per cell, or (block_cells)

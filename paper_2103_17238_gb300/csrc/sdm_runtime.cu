@@ -2151,7 +2151,7 @@ sdm_status sdm_spectrum(sdm_ctx *ctx, const double *r_edges, int32_t n_edges, in
             spectrum_total_kernel<<<grid, 32 * kSpecWarps, 0, s>>>(ctx->d_inst, n_in, T, d_part, one ? d_out : nullptr,
                                                                    h_status);
             if (!one)
-                spectrum_total_finalize_kernel<<<nb, 32, 0, s>>>(ctx->d_inst, d_part, grid, T, d_out, h_status);
+                spectrum_total_finalize_kernel<<<nb, kSpecFinalNT, 0, s>>>(ctx->d_inst, d_part, grid, T, d_out, h_status);
         } else {
             // a block per cell where a warp alone would take many rounds
             const int block_cells = n_in / ctx->cfg.n_cells > 4 * kSpecChunk ? 1 : 0;
