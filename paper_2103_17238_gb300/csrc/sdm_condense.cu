@@ -167,9 +167,23 @@ __global__ void __launch_bounds__(kCondNT) condense_by_cell_kernel(const int32_t
 {
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    // a cell's range and coefficient (page-locked memory) are loaded a cell ahead
+    // without the water (31.0 -> 30.3 us with a cold L2; with it 32.0 -> 33.0: not there)
+    int32_t next_lo = 0, next_hi = 0;
+    float next_c = 0.0f;
+    auto ahead = [&](int cell) {
+        if (cell < n_cells) {
+            next_lo = cell_off[cell];
+            next_hi = cell_off[cell + 1];
+            next_c = cf[cell];
+        }
+    };
+    ahead(gw);
     for (int cell = gw; cell < n_cells; cell += nw) {
-        const int32_t lo = cell_off[cell], hi = cell_off[cell + 1];
-        const float c = cf[cell];
+        const int32_t lo = next_lo, hi = next_hi;
+        const float c = next_c;
+        if constexpr (!WATER)
+            ahead(cell + nw);
         double acc = 0.0;
         for (int32_t at = lo; at < hi; at += kCondItem) {
             const double w = condense_round<WATER>(xi + at, v + at, min(kCondItem, hi - at), c, xminf);
@@ -177,6 +191,8 @@ __global__ void __launch_bounds__(kCondNT) condense_by_cell_kernel(const int32_t
         }
         if (WATER && lane == 0)
             out[cell] = c < 0.0f ? 0.0 - acc : acc;
+        if constexpr (WATER)
+            ahead(cell + nw);
     }
 }
 
