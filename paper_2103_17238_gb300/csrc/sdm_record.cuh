@@ -14,7 +14,8 @@
 //      piece of every bucket's room from one global atomic each; then
 //      one 16-byte store per live SD: 32 key bits below the bucket's, rank, xi
 //      truncated to binary32 and v's high word;
-//   2. rec_scan_kernel     first positions of the buckets;
+//   2. rec_scan_kernel     first positions of the buckets (above kRecSumSd; else
+//      each bucket's block adds up the counts);
 //   3. rec_pairs_kernel    one block per bucket: its records by one bulk copy,
 //      ordered by their key bits; the pairs' bound (pair_prefilter_zero needs no
 //      more than the record) on all of them, and only what it leaves
@@ -42,6 +43,11 @@ constexpr int kRecChunk = 4096; // SDs per scatter block
 // Five blocks of 256 per SM (48 registers): 354 us against 370 with four, 405 with three;
 // 512 threads 457, six blocks (40 registers, spills) 399.
 constexpr int kRecNT = 256; // threads of a bucket's block
+// Groups of up to this many SDs have no scan launch: every bucket's block adds up its
+// cell's counts (us, scan | sums: one box of 2^18 19.6 | 18.7, of 2^20 31.4 | 30.4, of 2^21
+// 51.6 | 51.1; 16 of 2^15 23.0 | 21.7; but 32 of 2^17 88.8 | 89.6, 16 of 2^20 349 | 356, one
+// of 2^24 462 | 512).
+constexpr int64_t kRecSumSd = (int64_t)1 << 21;
 constexpr int kRecSubLB = 9;    // sub-buckets inside a bucket
 constexpr int kRecMaxBuckets = 16384; // (their counts take 64 KB of shared memory)
 constexpr int kRecMaxSd = kRecMaxBuckets * kRecMean;
@@ -138,8 +144,7 @@ __global__ void __launch_bounds__(kRecScatterNT, 2) rec_scatter_kernel(const Big
     }
 }
 
-// One block per cell: the buckets' first positions, the counts cleared for the
-// next step.
+// One block per cell: the buckets' first positions.
 constexpr int kRecScanNT = 1024;
 __global__ void __launch_bounds__(kRecScanNT) rec_scan_kernel(const RecCell *__restrict__ cells, RecScratch S)
 {
@@ -148,14 +153,13 @@ __global__ void __launch_bounds__(kRecScanNT) rec_scan_kernel(const RecCell *__r
     chain_next();
     const RecCell c = cells[blockIdx.x];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    uint32_t *cnt = S.cnt + c.first, *start = S.start + c.start;
+    const uint32_t *cnt = S.cnt + c.first;
+    uint32_t *start = S.start + c.start;
     chain_wait();
     uint32_t carry = 0, big = 0;
     for (int i0 = 0; i0 < c.nb; i0 += kRecScanNT) {
         const int i = i0 + t;
         const uint32_t x = i < c.nb ? cnt[i] : 0u;
-        if (i < c.nb)
-            cnt[i] = 0u;
         big |= x > (uint32_t)kRecRoom ? 1u : 0u;
         uint32_t incl = x;
 #pragma unroll
@@ -187,7 +191,7 @@ struct RecSmem {
     uint32_t word[kRecRoom]; // 21 key bits above the record's place, in sub-buckets; then (16 bits each) the order
     uint32_t hist[(1 << kRecSubLB) + 4];
     uint16_t list[kRecRoom / 2 + 2]; // pairs the bound leaves
-    uint32_t warp[32];
+    uint32_t warp[32], sum[2][kRecNT / 32];
     uint64_t bar;
     uint32_t n_list;
 };
@@ -225,6 +229,9 @@ __device__ __forceinline__ void rec_pair(const InstDev *P, const PairConsts &C, 
     }
 }
 
+// SUM: a bucket's block adds up the counts itself and writes its first position
+// for the seam kernel; else rec_scan_kernel has.
+template <bool SUM>
 __global__ void __launch_bounds__(kRecNT, 5) rec_pairs_kernel(const BigBucket *__restrict__ work,
                                                            const RecCell *__restrict__ cells, RecScratch S,
                                                            int64_t step_offset)
@@ -253,14 +260,43 @@ __global__ void __launch_bounds__(kRecNT, 5) rec_pairs_kernel(const BigBucket *_
     const int64_t s = P->step + step_offset;
     const uint32_t cell = (uint32_t)c.cell;
     chain_wait();
-    const uint32_t *st = S.start + c.start + w.bucket;
-    const uint32_t start = st[0], n_c = st[c.nb - w.bucket];
-    if (n_c == kRecVoid) // uniform
-        return;
-    const uint32_t nk = (w.bucket + 1 < c.nb ? st[1] : n_c) - start;
-    if (nk == 0)
-        return;
     const uint4 *room = S.rooms + (int64_t)(c.first + w.bucket) * kRecRoom;
+    uint32_t *st = S.start + c.start + w.bucket;
+    uint32_t start, n_c, nk;
+    if constexpr (SUM) {
+        const uint32_t *cnt = S.cnt + c.first;
+        uint32_t before = 0, all = 0, big = 0;
+        for (int i = t; i < c.nb; i += kRecNT) {
+            const uint32_t x = cnt[i];
+            all += x;
+            before += i < w.bucket ? x : 0u;
+            big |= x > (uint32_t)kRecRoom ? 1u : 0u;
+        }
+        nk = cnt[w.bucket];
+        before = __reduce_add_sync(FULL, before);
+        all = __reduce_add_sync(FULL, all);
+        if (lane == 0) {
+            M.sum[0][warp] = before;
+            M.sum[1][warp] = all;
+        }
+        const int over = __syncthreads_or((int)big);
+        start = __reduce_add_sync(FULL, lane < NW ? M.sum[0][lane] : 0u);
+        n_c = over ? kRecVoid : __reduce_add_sync(FULL, lane < NW ? M.sum[1][lane] : 0u);
+        if (t == 0) {
+            st[0] = start;
+            if (w.bucket == 0) {
+                st[c.nb] = n_c;
+                if (over)
+                    atomicOr(&const_cast<InstDev *>(P)->status, 2u);
+            }
+        }
+    } else {
+        start = st[0];
+        n_c = st[c.nb - w.bucket];
+        nk = (w.bucket + 1 < c.nb ? st[1] : n_c) - start;
+    }
+    if (n_c == kRecVoid || nk == 0) // uniform
+        return;
     if (t == 0) {
         mbar_arrive_expect_tx(&M.bar, nk * 16u);
         bulk_g2s(M.rec, room, nk * 16u, &M.bar);
@@ -393,6 +429,7 @@ __global__ void __launch_bounds__(kRecSeamNT) rec_seam_kernel(const BigBucket *_
     chain_wait();
     if (i >= n_work)
         return;
+    S.cnt[c.first + w.bucket] = 0u; // for the next step
     const uint32_t *st = S.start + c.start;
     const uint32_t n_c = st[c.nb], start = st[w.bucket];
     if (n_c == kRecVoid)

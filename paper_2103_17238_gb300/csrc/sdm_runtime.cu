@@ -684,9 +684,10 @@ cudaError_t configure_kernels()
         if ((r = cudaFuncSetAttribute(rec_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       kRecMaxBuckets * (int)sizeof(uint32_t))) != cudaSuccess)
             e = r;
-        if ((r = cudaFuncSetAttribute(rec_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sizeof(RecSmem))) != cudaSuccess)
-            e = r;
+        for (auto k : {rec_pairs_kernel<false>, rec_pairs_kernel<true>})
+            if ((r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RecSmem))) !=
+                cudaSuccess)
+                e = r;
         const int hb = (int)big_hist_smem(kBigMaxLB);
         if ((r = cudaFuncSetAttribute(big_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess) e = r;
         if ((r = cudaFuncSetAttribute(big_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess) e = r;
@@ -1318,8 +1319,11 @@ void enqueue_big_steps(const Plan &pl, int64_t off, int32_t n, cudaStream_t st)
             const BigBucket *wb = pl.d_rec_buckets + g.bucket0;
             launch_chained(rec_scatter_kernel, g.n_chunks, kRecScatterNT, sizeof(uint32_t) * g.max_nb, st, chain, wc, cells,
                            pl.rec, o);
-            launch_chained(rec_scan_kernel, g.n_cells, kRecScanNT, 0, st, true, cells + g.cell0, pl.rec);
-            launch_chained(rec_pairs_kernel, g.n_buckets, kRecNT, sizeof(RecSmem), st, true, wb, cells, pl.rec, o);
+            const bool sum = g.sds <= kRecSumSd;
+            if (!sum)
+                launch_chained(rec_scan_kernel, g.n_cells, kRecScanNT, 0, st, true, cells + g.cell0, pl.rec);
+            launch_chained(sum ? rec_pairs_kernel<true> : rec_pairs_kernel<false>, g.n_buckets, kRecNT, sizeof(RecSmem), st,
+                           true, wb, cells, pl.rec, o);
             launch_chained(rec_seam_kernel, (g.n_buckets + kRecSeamNT - 1) / kRecSeamNT, kRecSeamNT, 0, st, true, wb,
                            g.n_buckets, cells, pl.rec, o);
             chain = true;
