@@ -387,8 +387,11 @@ typedef struct sdm_diag {
     int64_t live_sd;    /* SDs inside the domain (cell >= 0) with xi > 0 */
     uint64_t sum_xi_lo; /* sum of their xi, exact as a 128-bit integer: low 64 bits */
     uint64_t sum_xi_hi; /*   and high 64 bits */
-    double sum_xi_v;    /* sum of their xi v, m^3, in binary64: each product added with one
-                           rounding, in a fixed order, so repeated calls give the same bits */
+    double sum_xi_v;    /* sum of their xi v, m^3.  Rounds of 256 SDs in storage order are summed in
+                           fixed point (each product cut below 2^-61 of its round's greatest, no
+                           rounding between them), the rounds in binary64 in a fixed order, so
+                           repeated calls give the same bits; an SD whose volume evaporation left
+                           at or below zero is added in binary64, with its sign */
 } sdm_diag;
 
 /* The sums over the context's current state, computed on its stream; the

@@ -123,6 +123,11 @@ struct FixedSum {
     }
 };
 
+// Whether v may enter the fixed-point sums below: positive and normal.  (An
+// evaporating step's rounding can leave a volume at or below zero; such SDs are
+// added in binary64, with their sign.)
+__device__ __forceinline__ bool volume_plain(double v) { return __double2hiint(v) >= 0x00100000; }
+
 // xi v: floor(log2 xi) + floor(log2 v) with v's biased exponent, and the
 // product (its top 62 or 63 bits) in units of 2^(emax - 61 - 1023).
 __device__ __forceinline__ uint32_t xiv_exponent(uint64_t x, double v)
@@ -1641,7 +1646,7 @@ __global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(InstDev *P, int64
     constexpr int Q = kDiagChunk / 64; // slot pairs per lane and round
     const int lane = threadIdx.x & 31;
     DiagPart a{0ull, 0ull, 0ull, 0.0};
-    double xv = 0.0;
+    double xv = 0.0, other = 0.0; // other: a lane's SDs whose volume is not plain
     const int64_t gw = ((int64_t)blockIdx.x * kDiagNT + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * kDiagNT) >> 5;
     for (int64_t at = gw * kDiagChunk; at < n_in; at += nw * kDiagChunk) {
         const int n = (int)min((int64_t)kDiagChunk, n_in - at); // even: every group has an even number of slots
@@ -1659,10 +1664,14 @@ __global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(InstDev *P, int64
 #pragma unroll
         for (int i = 0; i < 2 * Q; ++i) {
             const int64_t x = (i & 1) ? xx[i / 2].y : xx[i / 2].x;
+            const double v = (i & 1) ? vv[i / 2].y : vv[i / 2].x;
             if (x > 0) {
                 a.live += 1ull;
                 add128(a.xi_lo, a.xi_hi, (unsigned long long)x, 0ull);
-                e = max(e, xiv_exponent((uint64_t)x, (i & 1) ? vv[i / 2].y : vv[i / 2].x));
+                if (volume_plain(v))
+                    e = max(e, xiv_exponent((uint64_t)x, v));
+                else
+                    other = __fma_rn(xi2d(x), v, other);
             }
         }
         e = __reduce_max_sync(0xFFFFFFFFu, e);
@@ -1670,12 +1679,13 @@ __global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(InstDev *P, int64
 #pragma unroll
         for (int i = 0; i < 2 * Q; ++i) {
             const int64_t x = (i & 1) ? xx[i / 2].y : xx[i / 2].x;
-            if (x > 0)
-                f.add(xiv_fixed((uint64_t)x, (i & 1) ? vv[i / 2].y : vv[i / 2].x, e));
+            const double v = (i & 1) ? vv[i / 2].y : vv[i / 2].x;
+            if (x > 0 && volume_plain(v))
+                f.add(xiv_fixed((uint64_t)x, v, e));
         }
         xv = __dadd_rn(xv, f.warp_sum((int)e - 61 - 1023));
     }
-    a.xv = lane == 0 ? xv : 0.0;
+    a.xv = lane == 0 ? __dadd_rn(xv, other) : other;
     a = diag_block_reduce(a);
     if (threadIdx.x == 0)
         parts[blockIdx.x] = a;
