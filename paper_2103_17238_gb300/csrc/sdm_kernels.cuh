@@ -1889,6 +1889,18 @@ __device__ __forceinline__ int spec_bin(const SpecSmem &S, const SpecTab &T, dou
     return lo;
 }
 
+// sum + the sum of bin `lane` over the SDs of slots [0, n) of volume at or below zero,
+// in slot order: xi v with its sign, in the bin of the radius of |v|.
+__device__ __noinline__ double spec_odd(const SpecSmem &S, const SpecTab &T, const int64_t *gxi, const double *gv, int n,
+                                        double sum)
+{
+    const int lane = threadIdx.x & 31;
+    for (int i = 0; i < n; ++i)
+        if (gxi[i] > 0 && !volume_plain(gv[i]) && spec_bin(S, T, fabs(gv[i])) == lane)
+            sum = __fma_rn(xi2d(gxi[i]), gv[i], sum);
+    return sum;
+}
+
 // Adds the SDs of slots [lo, lo + n), n <= kSpecChunk, lo even, and returns
 // the sum of bin `lane`.  Every lane of the warp calls it.
 __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, const int64_t *__restrict__ gxi,
@@ -1900,6 +1912,7 @@ __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, cons
     uint64_t x[2 * Q];
     double v[2 * Q];
     int bin[2 * Q];
+    bool odd = false; // an SD whose volume is not plain
 #pragma unroll
     for (int i = 0; i < Q; ++i) { // every load first
         const int q = lane + 32 * i;
@@ -1917,7 +1930,9 @@ __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, cons
 #pragma unroll
     for (int i = 0; i < 2 * Q; ++i) {
         bin[i] = -1;
-        if ((int64_t)x[i] > 0) {
+        if ((int64_t)x[i] > 0 && !volume_plain(v[i])) {
+            odd = true;
+        } else if ((int64_t)x[i] > 0) {
             const int b = spec_bin(S, T, v[i]);
             if ((unsigned)b < (unsigned)nb) {
                 bin[i] = b;
@@ -1952,9 +1967,10 @@ __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, cons
     __syncwarp();
     spec_clear(S, warp, lane);
     __syncwarp();
-    if (e == 0u)
-        return 0.0;
-    return fixed_to_double<42>(a2, ((uint64_t)a1 << 21) + a0, (int)e - 61 - 1023);
+    double sum = e == 0u ? 0.0 : fixed_to_double<42>(a2, ((uint64_t)a1 << 21) + a0, (int)e - 61 - 1023);
+    if (__any_sync(0xFFFFFFFFu, odd))
+        sum = spec_odd(S, T, gxi, gv, n, sum);
+    return sum;
 }
 
 // x / den by the 64-bit reciprocal (x >= 0): within 0.5 + 2^-9 ulp, where the
@@ -1996,8 +2012,9 @@ __device__ __forceinline__ void spec_finish(const SpecTab &T, const double *part
 
 // Sums of every bin over all slots [0, n_slots) (padding and dead SDs hold
 // xi = 0): partial[bin][block]; with out, the spectrum itself from the last
-// block (up to kLastBlockMax), and the run's status word to *status.
-__global__ void __launch_bounds__(32 * kSpecWarps) spectrum_total_kernel(InstDev *P, int64_t n_slots,
+// block (up to kLastBlockMax), and the run's status word to *status.  (Seven
+// blocks per SM: 72 registers.)
+__global__ void __launch_bounds__(32 * kSpecWarps, 7) spectrum_total_kernel(InstDev *P, int64_t n_slots,
                                                                          const __grid_constant__ SpecTab T,
                                                                          double *partial, double *out, uint32_t *status)
 {

@@ -67,3 +67,19 @@ def test_sum_of_water(env, sizes):
     assert d["live_sd"] == int((st.xi > 0).sum()) and d["sum_xi"] == sum(int(x) for x in st.xi)
     assert abs(Fraction(d["sum_xi_v"]) - want) <= len(t) * mag / 2**53
     run.close()
+
+
+@pytest.mark.parametrize("per_cell", [False, True])
+@pytest.mark.parametrize("bins", [1, 31, 40])
+@pytest.mark.parametrize("sizes", [[64, 1000, 3, 256], [9000, 1], [2500]])
+def test_spectrum(env, sizes, bins, per_cell):
+    O, sdm, torch = env
+    run, st, P = _evaporated(env, sizes)
+    edges = np.exp(np.linspace(np.log(1e-8), np.log(2e-6), bins + 1))
+    got = run.spectrum(edges, per_cell=per_cell)
+    want = O.spectrum(P, st, edges, per_cell=per_cell)
+    pos = O.State(st.xi, np.abs(st.v), st.cell, None, st.n_cells)
+    mag = O.spectrum(P, pos, edges, per_cell=per_cell)
+    assert mag.max() > 0 and ((want < 0).any() or bins == 1)
+    assert np.all(np.abs(got - want) <= 2 * (len(st.xi) + 4) * 2.0**-53 * mag)
+    run.close()
