@@ -187,7 +187,8 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
 
 // Bounded wait on an mbarrier phase: ~2^22 polls (each poll may suspend the
 // thread for a hardware-defined interval), then give up.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, uint32_t max_polls = 1u << 22)
+constexpr uint32_t kWaitPolls = 1u << 22;
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, uint32_t max_polls = kWaitPolls)
 {
     for (uint32_t it = 0; it < max_polls; ++it)
         if (mbar_try_wait(bar, parity))

@@ -68,10 +68,15 @@ struct RecScratch {
     uint32_t *cnt;    // per bucket: entries; zero before a step's scatter
     uint32_t *start;  // per bucket: first position; a cell's count of live SDs behind its last
                       // (kRecVoid: a room overflowed)
-    uint2 *seam;      // per bucket: ranks of its first and last SD
+    uint2 *seam;      // per bucket that holds any: ranks of its first and last SD (kRecVoid: its wait gave up)
     uint4 *rooms;     // kRecRoom records per bucket
 };
 constexpr uint32_t kRecVoid = 0xFFFFFFFFu;
+
+// Polls of a bucket's wait for its records (a test's build lets some give up at once).
+#ifndef SDM_REC_POLLS
+#define SDM_REC_POLLS(bucket) kWaitPolls
+#endif
 
 __global__ void __launch_bounds__(kRecScatterNT, 2) rec_scatter_kernel(const BigChunk *__restrict__ work,
                                                                     const RecCell *__restrict__ cells, RecScratch S,
@@ -302,10 +307,13 @@ __global__ void __launch_bounds__(kRecNT, 5) rec_pairs_kernel(const BigBucket *_
         bulk_g2s(M.rec, room, nk * 16u, &M.bar);
     }
     __syncthreads();
-    const bool arrived = mbar_wait_bounded(&M.bar, 0u);
-    if (!__syncthreads_and(arrived)) { // (waited for long enough: nothing else is in flight)
-        if (t == 0)
+    const bool arrived = mbar_wait_bounded(&M.bar, 0u, SDM_REC_POLLS(w.bucket));
+    if (!__syncthreads_and(arrived)) { // report, leave no ranks for the seams, wait (bounded) for the copy, leave
+        if (t == 0) {
             atomicOr(&const_cast<InstDev *>(P)->status, 1u);
+            S.seam[c.first + w.bucket] = make_uint2(kRecVoid, kRecVoid);
+            mbar_wait_bounded(&M.bar, 0u);
+        }
         return;
     }
     // ---- order of the bucket
@@ -440,11 +448,14 @@ __global__ void __launch_bounds__(kRecSeamNT) rec_seam_kernel(const BigBucket *_
     int b = w.bucket + 1;
     while ((b + 1 < c.nb ? st[b + 1] : n_c) == end) // (end < n_c: some bucket holds the next position)
         ++b;
+    const uint32_t ra = S.seam[c.first + w.bucket].y, rb = S.seam[c.first + b].x;
+    if (ra == kRecVoid || rb == kRecVoid) // a bucket whose wait gave up: its SDs stay as they are
+        return;
     const InstDev *__restrict__ P = c.run;
     const uint32_t l = end / 2u;
     const uint4 u = draw4(P->seed, l >> 1, (uint32_t)c.cell, P->step + step_offset, 1u);
     rec_pair(P, pair_consts(P), n_c, u32_to_f32_rn((n_c & 1u) ? n_c : n_c - 1u), P->xi + c.off, P->v + c.off,
-             S.seam[c.first + w.bucket].y, S.seam[c.first + b].x, (l & 1u) ? u.z : u.x, (l & 1u) ? u.w : u.y);
+             ra, rb, (l & 1u) ? u.z : u.x, (l & 1u) ? u.w : u.y);
 }
 
 } // namespace sdm

@@ -1,0 +1,85 @@
+"""What a step leaves behind when a device wait gives up, on a build of the
+library in which some waits give up at once (tests/give_up.cu: the copies they
+wait for still arrive, and the kernel waits for them before it leaves, so
+nothing is out of range and the device stays usable).
+
+Record path: the SDs of a bucket that gave up stay as they were, with the
+partners that a pair across its ends would have had; every other pair is
+stepped as the oracle steps it; the call that reads the state reports
+SDM_ETIMEOUT; and the next step finds its counts in order."""
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env(tmp_path_factory):
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from oracle import oracle as O
+    from paper_2103_17238_gb300 import build as B
+    from paper_2103_17238_gb300 import sdm
+
+    O.build()
+    path = str(tmp_path_factory.mktemp("give_up") / "libsdm_give_up.so")
+    here = os.path.dirname(os.path.abspath(__file__))
+    subprocess.run([B.nvcc(), *B.NVCC_FLAGS, os.path.join(here, "give_up.cu"), "-o", path], check=True)
+    torch.cuda.set_device(0)
+    before, sdm._lib = sdm._lib, None
+    sdm.load(path)
+    yield O, sdm, torch
+    sdm._lib = before
+
+
+def _buckets_that_gave_up(O, seed, cell, s, ranks, nb):
+    b = np.array([(O.sort_key(seed, int(r), cell, s) * nb) >> 64 for r in ranks])
+    assert np.all(np.diff(b) >= 0)
+    return b % 3 == 1
+
+
+# several cells and cells that share a launch without and with the launch that scans the counts
+@pytest.mark.parametrize("sizes,steps", [([200001, 3, 40002, 5000], 3), ([(1 << 21) + 4098], 1)])
+def test_record_path(env, sizes, steps):
+    O, sdm, torch = env
+    rng = np.random.default_rng(23)
+    nc, seed, dv = len(sizes), 11, 1e-1
+    cell = np.repeat(np.arange(nc, dtype=np.int32), sizes)
+    n = len(cell)
+    xi = rng.integers(1, 10**9, n).astype(np.int64)
+    xi[rng.random(n) < 0.05] = 0
+    v = 4 / 3 * np.pi * np.exp(rng.uniform(np.log(2e-6), np.log(2e-3), n)) ** 3
+    run = sdm.Run(sdm.make_config("golovin", dv=dv, n_cells=nc, seed=seed), n).set_attributes(xi, v, cell)
+    st = O.State(xi.copy(), v.copy(), cell.copy(), None, nc)
+    P = O.params("golovin", dv=dv, seed=seed)
+    dx = torch.empty(n, dtype=torch.int64, device="cuda")
+    dw = torch.empty(n, dtype=torch.float64, device="cuda")
+    for s in range(steps):
+        x0, v0 = st.xi.copy(), st.v.copy()
+        O.step(P, st, s)
+        stepped = (st.xi != x0) | (st.v != v0)
+        kept = np.zeros(n, bool)
+        for c, size in enumerate(sizes):
+            if size <= 4096:
+                continue
+            first = int(np.searchsorted(cell, c))
+            perm = O.permutation(seed, c, s, x0[first:first + size])
+            out = _buckets_that_gave_up(O, seed, c, s, perm, -(-size // 1024))
+            pairs = perm[:len(perm) // 2 * 2].reshape(-1, 2)
+            kept[first + pairs[out[:len(perm) // 2 * 2].reshape(-1, 2).any(axis=1)].ravel()] = True
+        st.xi[kept], st.v[kept] = x0[kept], v0[kept]
+        assert (stepped & kept).sum() > 1000 and (stepped & ~kept).sum() > 1000
+        run.step(1)
+        sdm.sdm_get_attributes(run.h, xi=dx, volume=dw)
+        torch.cuda.synchronize()
+        bad = np.nonzero((dx.cpu().numpy() != st.xi) | (dw.cpu().numpy() != st.v))[0]
+        assert bad.size == 0, f"step {s}: {bad.size} SDs differ, first {bad[:5]} (cells {cell[bad[:5]]})"
+    with pytest.raises(sdm.SdmError) as e:
+        run.attributes()
+    assert e.value.status == sdm.SDM_ETIMEOUT
+    run.close()
