@@ -369,7 +369,8 @@ sdm_status sdm_get_tuning(sdm_tuning *out);
  * first call before any stream capture.  Every call shares the one array and
  * leaves its contents behind, so calls whose work overlaps on the GPU (two
  * streams, two host threads, two devices' calls aimed at one device) race:
- * order them on one stream.  Errors: SDM_EINVAL, SDM_ECUDA (also when a
+ * order them on one stream.  (They spoil one another; a later call takes
+ * nothing from what they left.)  Errors: SDM_EINVAL, SDM_ECUDA (also when a
  * CUDA error from earlier work is pending on the calling thread: it is
  * reported, not cleared, and nothing is launched; message from
  * sdm_last_error(NULL)). */

@@ -10,7 +10,9 @@
 // together with their work lists and run record live in one fixed-size,
 // file-scope device array, set up once per device.  A cell of up to 4096 SDs
 // needs none of it: one block steps it in one launch, its record a kernel
-// argument.  Up to 2^18 SDs take two launches (sdm_spread.cuh).
+// argument.  Up to 2^18 SDs take three launches (sdm_spread.cuh, its counters
+// cleared first).  No call relies on what another has left in the array: calls
+// that overlap spoil one another, never a later one.
 //
 // Compiled as part of the library's single translation unit (included at the
 // end of sdm_runtime.cu), after the kernels it launches.
@@ -43,8 +45,7 @@ constexpr size_t kNaInst = na_align(kNaPairs + sizeof(BigPairs) * (size_t)kNaMax
 constexpr size_t kNaInsts = na_align(kNaInst + sizeof(InstDev));
 constexpr size_t kNaCellOff = na_align(kNaInsts + sizeof(InstDev *));
 constexpr size_t kNaStatus = na_align(kNaCellOff + 2 * sizeof(int32_t));
-// the bucketed path's counts (zero between calls; its rooms lie over the
-// multi-pass path's arrays)
+// the bucketed path's counts (its rooms lie over the multi-pass path's arrays)
 constexpr int kNaSpreadMax = 1 << 18;
 constexpr size_t kNaSpreadCnt = na_align(kNaStatus + sizeof(uint32_t));
 constexpr size_t kNaBytes = na_align(kNaSpreadCnt + sizeof(uint32_t) * (spread_words(kNaSpreadMax / kSpreadMean + 1) + 4));
@@ -216,14 +217,15 @@ extern "C" sdm_status sdm_cell_step_noalloc(const sdm_config *cfg, int64_t step,
             return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: launch: %s", cudaGetErrorString(e));
         return SDM_OK;
     }
-    if (n <= kNaSpreadMax) { // the bucketed path: two launches
+    if (n <= kNaSpreadMax) { // the bucketed path
         int64_t counters = 0, rooms = 0;
         const SpreadCell c = spread_cell(nullptr, 0, 0, n, counters, rooms);
         SpreadScratch S;
         S.cnt = reinterpret_cast<uint32_t *>(base + kNaSpreadCnt);
         S.rooms = reinterpret_cast<uint2 *>(base);
         uint32_t *status = reinterpret_cast<uint32_t *>(base + kNaStatus);
-        launch_chained(one_spread_scatter_kernel, (n / 2 + kSpreadNT - 1) / kSpreadNT, kSpreadNT, 0, s, false, inst, c, S,
+        launch_chained(one_spread_clear_kernel, (c.nb + kSpreadNT - 1) / kSpreadNT, kSpreadNT, 0, s, false, c, S);
+        launch_chained(one_spread_scatter_kernel, (n / 2 + kSpreadNT - 1) / kSpreadNT, kSpreadNT, 0, s, true, inst, c, S,
                        status);
         launch_chained(one_spread_pairs_kernel, c.groups, kSpreadNT, 0, s, true, inst, c, S, status);
         const cudaError_t e = cudaGetLastError();

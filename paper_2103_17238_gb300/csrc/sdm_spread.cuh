@@ -16,7 +16,8 @@
 //      and its pairs: gathers, bound, certified filter, exact evaluation and
 //      update as in the warp kernel.  A pair that crosses into the next bucket
 //      takes that bucket's least entry.  The last CTA of a cell to have read
-//      the counts clears them for the next step.
+//      the counts clears them for the next step (the allocation-free step, whose
+//      counts outlive a call, clears them ahead of its scatter instead).
 // The order of entries within a room is left to the atomics; sorting by
 // (key, rank) removes it, so results repeat bit for bit.
 //
@@ -61,13 +62,14 @@ struct __align__(16) SpreadCell {
 };
 
 struct SpreadScratch {
-    uint32_t *cnt; // zero before a step, and again after it
+    uint32_t *cnt; // zero before a step, and in a plan again after it
     uint2 *rooms;  // kSpreadRoom entries per bucket
 };
 
 // A block's item in device memory (everything of its cell beside its place
 // in it: one load to the run's record), or one cell as an argument.
 struct PlanSpread {
+    static constexpr bool kClears = true; // the counts, behind the step
     const SpreadCell *items;
     __device__ __forceinline__ SpreadCell cell(int &first) const
     {
@@ -84,6 +86,7 @@ struct PlanSpread {
 
 template <int PER_BLOCK>
 struct OneSpread {
+    static constexpr bool kClears = false;
     const InstDev *P;
     SpreadCell c;
     uint32_t *status;
@@ -339,8 +342,10 @@ __device__ __forceinline__ void spread_pairs(const SRC src, const SpreadScratch 
         bad |= M.big[w];
     }
     if (t == 0) { // every thread's reads of the counts are done
-        __threadfence();
-        M.last = atomicAdd(S.cnt + c.cnt + spread_words(c.nb), 1u) == (uint32_t)c.groups - 1u ? 1u : 0u;
+        if constexpr (SRC::kClears) {
+            __threadfence();
+            M.last = atomicAdd(S.cnt + c.cnt + spread_words(c.nb), 1u) == (uint32_t)c.groups - 1u ? 1u : 0u;
+        }
         if (bad && b0 == 0)
             src.overflow(c);
     }
@@ -392,10 +397,12 @@ __device__ __forceinline__ void spread_pairs(const SRC src, const SpreadScratch 
             }
         }
     }
-    __syncthreads();
-    if (M.last) // the counts and the arrivals are zero again for the next step
-        for (int i = t; i <= spread_words(c.nb); i += kSpreadNT)
-            S.cnt[c.cnt + i] = 0u;
+    if constexpr (SRC::kClears) {
+        __syncthreads();
+        if (M.last) // the counts and the arrivals are zero again for the next step
+            for (int i = t; i <= spread_words(c.nb); i += kSpreadNT)
+                S.cnt[c.cnt + i] = 0u;
+    }
 }
 
 __global__ void __launch_bounds__(kSpreadNT) spread_scatter_kernel(PlanSpread src, SpreadScratch S, int64_t step_offset)
@@ -407,6 +414,15 @@ __global__ void __launch_bounds__(kSpreadNT, 3) spread_pairs_kernel(PlanSpread s
 {
     __shared__ __align__(16) SpreadSmem M;
     spread_pairs(src, S, step_offset, M);
+}
+
+// The counters of one cell to zero, ahead of its scatter.
+__global__ void __launch_bounds__(kSpreadNT) one_spread_clear_kernel(SpreadCell c, SpreadScratch S)
+{
+    chain_next();
+    const int b = (int)blockIdx.x * kSpreadNT + (int)threadIdx.x;
+    if (b < c.nb)
+        S.cnt[c.cnt + b * kSpreadStride] = 0u;
 }
 
 __global__ void __launch_bounds__(kSpreadNT) one_spread_scatter_kernel(const __grid_constant__ InstDev P, SpreadCell c,

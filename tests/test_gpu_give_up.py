@@ -6,7 +6,10 @@ nothing is out of range and the device stays usable).
 Record path: the SDs of a bucket that gave up stay as they were, with the
 partners that a pair across its ends would have had; every other pair is
 stepped as the oracle steps it; the call that reads the state reports
-SDM_ETIMEOUT; and the next step finds its counts in order."""
+SDM_ETIMEOUT; and the next step finds its counts in order.
+
+Allocation-free step: a call takes nothing from what its array held before, so
+calls that went wrong (overlapping ones, a launch that failed) spoil no later one."""
 import os
 import subprocess
 
@@ -83,3 +86,28 @@ def test_record_path(env, sizes, steps):
         run.attributes()
     assert e.value.status == sdm.SDM_ETIMEOUT
     run.close()
+
+
+@pytest.mark.parametrize("fill", [0xFF, 0x01])
+@pytest.mark.parametrize("n", [4096, 4098, 20000, 131072, 1 << 18, (1 << 18) + 2])
+def test_noalloc_takes_nothing_from_before(env, n, fill):
+    O, sdm, torch = env
+    rng = np.random.default_rng(n)
+    xi = rng.integers(1, 10**9, n).astype(np.int64)
+    xi[rng.random(n) < 0.05] = 0
+    v = 4 / 3 * np.pi * np.exp(rng.uniform(np.log(2e-6), np.log(2e-3), n)) ** 3
+    dx, dw = torch.from_numpy(xi).cuda(), torch.from_numpy(v).cuda()
+    cfg = sdm.make_config("golovin", dv=1e-1, n_cells=1, seed=3)
+    stream = sdm.current_stream_handle()
+    warm = torch.ones(64, dtype=torch.int64, device="cuda"), torch.full((64,), 1e-15, dtype=torch.float64, device="cuda")
+    sdm.sdm_cell_step_noalloc(cfg, 0, *warm, stream)
+    torch.cuda.synchronize()
+    st = O.State(xi.copy(), v.copy(), np.zeros(n, np.int32), None, 1)
+    P = O.params("golovin", dv=1e-1, seed=3)
+    for s in range(2):
+        assert sdm.load().give_up_fill_noalloc(fill) == 0
+        sdm.sdm_cell_step_noalloc(cfg, s, dx, dw, stream)
+        torch.cuda.synchronize()
+        O.step(P, st, s)
+        assert np.array_equal(dx.cpu().numpy(), st.xi) and np.array_equal(dw.cpu().numpy(), st.v)
+    assert int((st.xi != xi).sum()) > 0
