@@ -373,7 +373,10 @@ sdm_status sdm_get_tuning(sdm_tuning *out);
  * nothing from what they left.)  Errors: SDM_EINVAL, SDM_ECUDA (also when a
  * CUDA error from earlier work is pending on the calling thread: it is
  * reported, not cleared, and nothing is launched; message from
- * sdm_last_error(NULL)). */
+ * sdm_last_error(NULL)).  The call returns before its work is done, so what
+ * goes wrong on the device is reported, once, by the next call there, which
+ * does nothing else: SDM_ETIMEOUT (a bounded wait gave up) or SDM_ESTATE (a
+ * sort bucket outgrew its room), the earlier call's cell left as it was. */
 #define SDM_NOALLOC_MAX_SD 1048576
 
 sdm_status sdm_cell_step_noalloc(const sdm_config *cfg, int64_t step, int64_t *xi, double *volume, int64_t n_sd,

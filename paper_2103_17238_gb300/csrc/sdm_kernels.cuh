@@ -223,13 +223,18 @@ struct PlanCells {
     __device__ __forceinline__ void give_up(int inst) const { atomicOr(&insts[inst]->status, 1u); }
 };
 
+// The allocation-free step's words for a call's failures (host memory; each
+// written on its own, so that no atomic operation is needed there).
+constexpr int kWrongWait = 0, kWrongRoom = 1, kWrongWords = 2;
+__device__ __forceinline__ void set_wrong(uint32_t *words, int which) { *(volatile uint32_t *)(words + which) = 1u; }
+
 struct OneCell {
     const InstDev *P;
     int32_t n, n_items;
     uint32_t *status;
     __device__ __forceinline__ WorkItem item(int) const { return WorkItem{0, 0, 0, n}; }
     __device__ __forceinline__ const InstDev *record(int) const { return P; }
-    __device__ __forceinline__ void give_up(int) const { atomicOr(status, 1u); }
+    __device__ __forceinline__ void give_up(int) const { set_wrong(status, kWrongWait); }
 };
 
 template <int CAP, int STAGES>

@@ -44,10 +44,9 @@ constexpr size_t kNaPairs = na_align(kNaBuckets + sizeof(BigBucket) * ((size_t)1
 constexpr size_t kNaInst = na_align(kNaPairs + sizeof(BigPairs) * (size_t)kNaMaxPairBlocks);
 constexpr size_t kNaInsts = na_align(kNaInst + sizeof(InstDev));
 constexpr size_t kNaCellOff = na_align(kNaInsts + sizeof(InstDev *));
-constexpr size_t kNaStatus = na_align(kNaCellOff + 2 * sizeof(int32_t));
 // the bucketed path's counts (its rooms lie over the multi-pass path's arrays)
 constexpr int kNaSpreadMax = 1 << 18;
-constexpr size_t kNaSpreadCnt = na_align(kNaStatus + sizeof(uint32_t));
+constexpr size_t kNaSpreadCnt = na_align(kNaCellOff + 2 * sizeof(int32_t));
 constexpr size_t kNaBytes = na_align(kNaSpreadCnt + sizeof(uint32_t) * (spread_words(kNaSpreadMax / kSpreadMean + 1) + 4));
 static_assert((size_t)(kNaSpreadMax / kSpreadMean + 1) * kSpreadRoom * sizeof(uint2) <= kNaBstart, "rooms");
 
@@ -93,10 +92,19 @@ __global__ void noalloc_setup_kernel(unsigned char *base, InstDev inst, int32_t 
 std::mutex g_na_mutex;
 unsigned char *g_na_base[64] = {};
 
+// What went wrong in a call, by device: kWrongWait, kWrongRoom (sdm_kernels.cuh).
+// A call returns before its kernels run and must not wait for them, so they set
+// a word here, in the library's own host memory (registered once, page by page:
+// nothing is allocated), and the next call on the device reports it.
+alignas(65536) uint32_t g_na_wrong[65536 / sizeof(uint32_t)];
+bool g_na_registered = false;
+uint32_t *g_na_wrong_dev[64] = {};
+
 // Per-device set-up, with that device current: the array's device address
-// (host code only sees a stand-in symbol) and the kernels' shared-memory
-// limits.  Done by the first call on each device.
-sdm_status noalloc_base(unsigned char **out)
+// (host code only sees a stand-in symbol), the kernels' shared-memory limits
+// and the device's address of its words of g_na_wrong.  Done by the first call
+// on each device.
+sdm_status noalloc_base(unsigned char **out, int *device)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -112,9 +120,21 @@ sdm_status noalloc_base(unsigned char **out)
             return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: cudaGetSymbolAddress: %s", cudaGetErrorString(e));
         if ((e = configure_kernels()) != cudaSuccess)
             return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: kernel set-up: %s", cudaGetErrorString(e));
+        void *w = nullptr;
+        if (!g_na_registered)
+            e = cudaHostRegister(g_na_wrong, sizeof g_na_wrong, cudaHostRegisterPortable | cudaHostRegisterMapped);
+        g_na_registered |= e == cudaSuccess;
+        if (e == cudaSuccess)
+            e = cudaHostGetDevicePointer(&w, g_na_wrong, 0);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: status words: %s", cudaGetErrorString(e));
+        }
+        g_na_wrong_dev[dev] = static_cast<uint32_t *>(w) + dev * kWrongWords;
         g_na_base[dev] = static_cast<unsigned char *>(p);
     }
     *out = g_na_base[dev];
+    *device = dev;
     return SDM_OK;
 }
 
@@ -148,14 +168,13 @@ extern "C" sdm_status sdm_cell_step_noalloc(const sdm_config *cfg, int64_t step,
         return fail(nullptr, SDM_ECUDA, "sdm_cell_step_noalloc: a CUDA error from earlier work is pending: %s",
                     cudaGetErrorString(pending));
     unsigned char *base = nullptr;
-    st = noalloc_base(&base);
+    int cur = 0;
+    st = noalloc_base(&base, &cur);
     if (st != SDM_OK)
         return st;
     // both arrays must be memory of the current device (a host pointer or
     // another device's buffer would fault inside the kernels); the query
     // allocates nothing
-    int cur = 0;
-    cudaGetDevice(&cur);
     for (const void *ptr : {(const void *)xi, (const void *)volume}) {
         cudaPointerAttributes a{};
         const cudaError_t pe = cudaPointerGetAttributes(&a, ptr);
@@ -170,6 +189,18 @@ extern "C" sdm_status sdm_cell_step_noalloc(const sdm_config *cfg, int64_t step,
                         "device %d",
                         cur);
     }
+    uint32_t *wrong = g_na_wrong + cur * kWrongWords;
+    const bool wait = __atomic_exchange_n(wrong + kWrongWait, 0u, __ATOMIC_RELAXED) != 0u;
+    const bool room = __atomic_exchange_n(wrong + kWrongRoom, 0u, __ATOMIC_RELAXED) != 0u;
+    if (wait)
+        return fail(nullptr, SDM_ETIMEOUT,
+                    "sdm_cell_step_noalloc: in an earlier call on this device a wait for a bulk copy gave up, and that "
+                    "call's cell was not stepped; this call has done nothing");
+    if (room)
+        return fail(nullptr, SDM_ESTATE,
+                    "sdm_cell_step_noalloc: in an earlier call on this device a sort bucket outgrew its room (its keys "
+                    "are far from uniform), and that call's cell was not stepped; this call has done nothing");
+    uint32_t *status = g_na_wrong_dev[cur];
     cudaStream_t s = (cudaStream_t)cuda_stream;
     InstDev inst{};
     inst.xi = xi;
@@ -196,7 +227,6 @@ extern "C" sdm_status sdm_cell_step_noalloc(const sdm_config *cfg, int64_t step,
     inst.n_cells = 1;
     const int n = (int)n_sd;
     if (n <= 4096) { // one block, one launch, the record as an argument
-        uint32_t *status = reinterpret_cast<uint32_t *>(base + kNaStatus);
         auto one = [&](auto cap, auto nt) {
             constexpr int CAP = decltype(cap)::value, NT = decltype(nt)::value;
             one_cell_step_kernel<CAP, NT><<<1, NT, CellSmem<CAP, 1>::bytes, s>>>(inst, n, status);
@@ -223,7 +253,6 @@ extern "C" sdm_status sdm_cell_step_noalloc(const sdm_config *cfg, int64_t step,
         SpreadScratch S;
         S.cnt = reinterpret_cast<uint32_t *>(base + kNaSpreadCnt);
         S.rooms = reinterpret_cast<uint2 *>(base);
-        uint32_t *status = reinterpret_cast<uint32_t *>(base + kNaStatus);
         launch_chained(one_spread_clear_kernel, (c.nb + kSpreadNT - 1) / kSpreadNT, kSpreadNT, 0, s, false, c, S);
         launch_chained(one_spread_scatter_kernel, (n / 2 + kSpreadNT - 1) / kSpreadNT, kSpreadNT, 0, s, true, inst, c, S,
                        status);

@@ -96,7 +96,7 @@ struct OneSpread {
         return c;
     }
     __device__ __forceinline__ const InstDev *record(const SpreadCell &) const { return P; }
-    __device__ __forceinline__ void overflow(const SpreadCell &) const { atomicOr(status, 2u); }
+    __device__ __forceinline__ void overflow(const SpreadCell &) const { set_wrong(status, kWrongRoom); }
 };
 
 // Programmatic dependent launch: the next kernel of the chain may become

@@ -13,3 +13,21 @@ extern "C" int give_up_fill_noalloc(int value)
         return 1;
     return cudaDeviceSynchronize() == cudaSuccess ? 0 : 1;
 }
+
+static __global__ void report_kernel(uint32_t *status, int which)
+{
+    if (which)
+        OneSpread<1>{nullptr, SpreadCell{}, status}.overflow(SpreadCell{});
+    else
+        OneCell{nullptr, 0, 0, status}.give_up(0);
+}
+
+// As a kernel of that step reports a wait that gave up (0) or a full room (1).
+extern "C" int give_up_report(int which)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64 || !g_na_wrong_dev[dev])
+        return 1;
+    report_kernel<<<1, 1>>>(g_na_wrong_dev[dev], which);
+    return cudaDeviceSynchronize() == cudaSuccess ? 0 : 1;
+}

@@ -9,7 +9,8 @@ stepped as the oracle steps it; the call that reads the state reports
 SDM_ETIMEOUT; and the next step finds its counts in order.
 
 Allocation-free step: a call takes nothing from what its array held before, so
-calls that went wrong (overlapping ones, a launch that failed) spoil no later one."""
+calls that went wrong (overlapping ones, a launch that failed) spoil no later one;
+and what a kernel reports, the next call says, once."""
 import os
 import subprocess
 
@@ -111,3 +112,26 @@ def test_noalloc_takes_nothing_from_before(env, n, fill):
         O.step(P, st, s)
         assert np.array_equal(dx.cpu().numpy(), st.xi) and np.array_equal(dw.cpu().numpy(), st.v)
     assert int((st.xi != xi).sum()) > 0
+
+
+@pytest.mark.parametrize("n", [64, 5000, 1 << 19])
+@pytest.mark.parametrize("which,name", [(0, "SDM_ETIMEOUT"), (1, "SDM_ESTATE")])
+def test_noalloc_reports(env, which, name, n):
+    O, sdm, torch = env
+    dx = torch.full((n,), 1000, dtype=torch.int64, device="cuda")
+    dw = torch.full((n,), 1e-9, dtype=torch.float64, device="cuda")
+    cfg = sdm.make_config("golovin", dv=1e-3, n_cells=1, seed=3)
+    stream = sdm.current_stream_handle()
+    sdm.sdm_cell_step_noalloc(cfg, 0, dx, dw, stream)
+    torch.cuda.synchronize()
+    x0, w0 = dx.clone(), dw.clone()
+    assert sdm.load().give_up_report(which) == 0
+    with pytest.raises(sdm.SdmError) as e:
+        sdm.sdm_cell_step_noalloc(cfg, 1, dx, dw, stream)
+    assert e.value.status == getattr(sdm, name) and "earlier call" in str(e.value)
+    torch.cuda.synchronize()
+    assert torch.equal(dx, x0) and torch.equal(dw, w0)
+    sdm.sdm_cell_step_noalloc(cfg, 1, dx, dw, stream)
+    sdm.sdm_cell_step_noalloc(cfg, 2, dx, dw, stream)
+    torch.cuda.synchronize()
+    assert not torch.equal(dx, x0)
