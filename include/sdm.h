@@ -150,7 +150,9 @@ sdm_status sdm_coalescence_step(sdm_ctx *ctx, int32_t n_steps);
  *   per_cell = 1: out[n_cells * (n_edges - 1)], cell-major, divided by dv.
  * r_edges: host array, n_edges >= 2, strictly increasing, > 0.  out: caller
  * buffer, host (out_on_device = 0; the call synchronises the stream) or
- * device (ordered on the stream).  Errors: SDM_EINVAL, SDM_ESTATE, SDM_ECUDA. */
+ * device (ordered on the stream).  Errors: SDM_EINVAL, SDM_ESTATE, SDM_ECUDA;
+ * with a host result also SDM_ETIMEOUT (a bounded device wait of an earlier
+ * step gave up) and SDM_ESTATE (an earlier step left a cell unstepped). */
 sdm_status sdm_spectrum(sdm_ctx *ctx, const double *r_edges, int32_t n_edges, int per_cell, double *out,
                         int out_on_device);
 
@@ -158,7 +160,8 @@ sdm_status sdm_spectrum(sdm_ctx *ctx, const double *r_edges, int32_t n_edges, in
  * order (dead SDs included, with xi = 0), into caller buffers xi[n_sd] and
  * volume[n_sd] (either may be NULL).  Host buffers: synchronises the stream.
  * With sdm_set_attributes and sdm_config.step0 this checkpoints and resumes a
- * run bit for bit.  Errors: SDM_ESTATE, SDM_ECUDA. */
+ * run bit for bit.  Errors: SDM_ESTATE, SDM_ECUDA; host buffers also
+ * SDM_ETIMEOUT and SDM_ESTATE as sdm_spectrum. */
 sdm_status sdm_get_attributes(sdm_ctx *ctx, int64_t *xi, double *volume, int on_device);
 
 typedef struct sdm_info {
@@ -400,7 +403,9 @@ typedef struct sdm_diag {
 
 /* The sums over the context's current state, computed on its stream; the
  * call waits for them.  Errors: SDM_EINVAL (NULL out), SDM_ESTATE (no
- * attributes yet, or an unusable context), SDM_ENOMEM, SDM_ECUDA. */
+ * attributes yet, or an unusable context), SDM_ENOMEM, SDM_ECUDA, and
+ * SDM_ETIMEOUT and SDM_ESTATE as sdm_spectrum (the sums are written all the
+ * same). */
 sdm_status sdm_diagnostics(sdm_ctx *ctx, sdm_diag *out);
 
 /* Self-test of failure detection on the device, without a fault.  Every

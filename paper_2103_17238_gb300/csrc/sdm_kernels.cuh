@@ -1634,7 +1634,8 @@ __device__ __forceinline__ DiagPart diag_block_reduce(DiagPart a)
     return a;
 }
 
-__device__ __forceinline__ void diag_finish(const DiagPart *parts, int32_t n_parts, DiagPart *out)
+__device__ __forceinline__ void diag_finish(const InstDev *P, const DiagPart *parts, int32_t n_parts, DiagPart *out,
+                                            uint32_t *status)
 {
     DiagPart a{0ull, 0ull, 0ull, 0.0};
     for (int i = threadIdx.x; i < n_parts; i += kDiagNT) {
@@ -1642,12 +1643,16 @@ __device__ __forceinline__ void diag_finish(const DiagPart *parts, int32_t n_par
         diag_combine(a, DiagPart{q->live, q->xi_lo, q->xi_hi, q->xv});
     }
     a = diag_block_reduce(a);
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
         *out = a;
+        *status = P->status;
+    }
 }
 
-// out (null: parts only): the sums, from the last block (up to kLastBlockMax).
-__global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(InstDev *P, int64_t n_in, DiagPart *parts, DiagPart *out)
+// out (null: parts only): the sums, from the last block (up to kLastBlockMax), and
+// the run's status word to *status.
+__global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(InstDev *P, int64_t n_in, DiagPart *parts, DiagPart *out,
+                                                               uint32_t *status)
 {
     constexpr int Q = kDiagChunk / 64; // slot pairs per lane and round
     const int lane = threadIdx.x & 31;
@@ -1696,12 +1701,13 @@ __global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(InstDev *P, int64
     if (threadIdx.x == 0)
         parts[blockIdx.x] = a;
     if (out && last_block(&P->ticket))
-        diag_finish(parts, (int)gridDim.x, out);
+        diag_finish(P, parts, (int)gridDim.x, out, status);
 }
 
-__global__ void __launch_bounds__(kDiagNT) diag_final_kernel(const DiagPart *parts, int32_t n_parts, DiagPart *out)
+__global__ void __launch_bounds__(kDiagNT) diag_final_kernel(const InstDev *P, const DiagPart *parts, int32_t n_parts,
+                                                             DiagPart *out, uint32_t *status)
 {
-    diag_finish(parts, n_parts, out);
+    diag_finish(P, parts, n_parts, out, status);
 }
 
 // -------------------------------------------------------------- spectrum

@@ -2186,9 +2186,7 @@ sdm_status sdm_spectrum(sdm_ctx *ctx, const double *r_edges, int32_t n_edges, in
         if (direct)
             std::memcpy(out, ctx->h_spec, b_out);
         ctx->mem.put(tmp, b_tmp);
-        if (*h_status & 1u)
-            return fail(&ctx->error, SDM_ETIMEOUT, "a device-side wait for a bulk copy gave up; results are incomplete");
-        return SDM_OK;
+        return status_result(ctx, *h_status);
     }
     ctx->mem.put(tmp, b_tmp);
     return SDM_OK;
@@ -2405,10 +2403,11 @@ sdm_status sdm_diagnostics(sdm_ctx *ctx, sdm_diag *out)
         return st;
     }
     DiagPart *res = (DiagPart *)ctx->h_spec; // (both calls that use it wait for their result)
+    uint32_t *h_status = (uint32_t *)(ctx->h_spec + sizeof(double) * 2 * kMaxEdges);
     const bool one = blocks <= kLastBlockMax;
-    diag_partial_kernel<<<blocks, kDiagNT, 0, s>>>(ctx->d_inst, n_in, d, one ? res : nullptr);
+    diag_partial_kernel<<<blocks, kDiagNT, 0, s>>>(ctx->d_inst, n_in, d, one ? res : nullptr, h_status);
     if (!one)
-        diag_final_kernel<<<1, kDiagNT, 0, s>>>(d, blocks, res);
+        diag_final_kernel<<<1, kDiagNT, 0, s>>>(ctx->d_inst, d, blocks, res, h_status);
     CTX_CUDA(ctx, cudaGetLastError());
     CTX_CUDA(ctx, cudaStreamSynchronize(s));
     ctx->mem.put(d, bytes);
@@ -2417,7 +2416,7 @@ sdm_status sdm_diagnostics(sdm_ctx *ctx, sdm_diag *out)
     out->sum_xi_lo = h.xi_lo;
     out->sum_xi_hi = h.xi_hi;
     out->sum_xi_v = h.xv;
-    return SDM_OK;
+    return status_result(ctx, *h_status);
 }
 
 sdm_status sdm_selftest_bounded_wait(void *cuda_stream, int64_t max_polls)
