@@ -119,7 +119,7 @@ class Server:
                 took += 1
                 s = pending.pop(0)
                 with torch.cuda.stream(admit_stream):
-                    s.run = make_run(s.req.inst)  # returns after its upload has landed
+                    s.run = make_run(s.req.inst)  # its layout and record go on behind this call
                 s.admitted_at = time.perf_counter() - t0
                 used += s.footprint
                 joining.append(s)
@@ -138,6 +138,7 @@ class Server:
             if batch is None or members != [id(s) for s in active]:
                 if batch is not None:
                     batch.close()
+                main.wait_stream(admit_stream)  # the joined runs' layouts and records are written there
                 batch = self._batch([s.run for s in active])
                 members = [id(s) for s in active]
             max_active = max(max_active, len(active))
