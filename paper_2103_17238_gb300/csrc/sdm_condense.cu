@@ -33,7 +33,7 @@ namespace {
 constexpr int kCondItem = 256; // slots per work item (a multiple of 2: cells start at even slots)
 constexpr int kCondNT = 256;
 constexpr int kCondByCell = 1024; // largest cell that one warp takes (4 rounds)
-constexpr int kCondStage = 4;     // calls whose fields may be on their way at once
+constexpr int kCondStage = 4;     // fields in page-locked memory: the next call's, and those on their way
 constexpr float kR3ToVolF = (float)(4.0 * kPi / 3.0); // 4 pi / 3 (binary64 pi) rounded to binary32
 
 struct __align__(16) CondItem {
@@ -50,10 +50,15 @@ struct CondBuffers {
     int32_t *item_start = nullptr; // n_cells + 1
     double *partial = nullptr;     // n_items
     double *cond = nullptr;        // n_cells
-    float *h_cf = nullptr;         // c of each cell, binary32: kCondStage fields in turn, page-locked, read by
-                                   // the kernel where they lie (a copy ahead of it cost more than its reads)
+    // c of each cell, binary32.  A field other than the last is read by the kernel
+    // where it lies in page-locked memory (a copy ahead of it cost more than its
+    // reads), which leaves it in cf for the calls that repeat it: those are a
+    // launch and nothing else, in a captured graph too.
+    float *cf = nullptr;   // n_cells
+    float *h_cf = nullptr; // kCondStage fields
     cudaEvent_t cf_done[kCondStage] = {}; // the last kernel that reads each
-    int stage = 0;                 // the next one
+    int stage = 0;         // the next call's: no kernel reads it
+    int last = -1;         // the one that is in cf (-1: none)
 };
 
 // f2d_exact (sdm_sediment.cu): the exact widening of a binary32 on the
@@ -158,12 +163,14 @@ __device__ __forceinline__ double condense_round(const int64_t *__restrict__ xi,
 
 // Every cell by one warp: no work list, nothing to rebuild when the layout
 // changes, no second pass.  56 + 10 us per call of the 4.19M-SD grid as two
-// kernels with binary64 sums (the binary64 pipe 68% busy).
-template <bool WATER>
+// kernels with binary64 sums (the binary64 pipe 68% busy).  KEEP: the field is
+// left in `keep`.
+template <bool WATER, bool KEEP>
 __global__ void __launch_bounds__(kCondNT) condense_by_cell_kernel(const int32_t *__restrict__ cell_off, int32_t n_cells,
                                                                    const int64_t *__restrict__ xi,
                                                                    double *__restrict__ v, const float *__restrict__ cf,
-                                                                   float xminf, double *__restrict__ out)
+                                                                   float *__restrict__ keep, float xminf,
+                                                                   double *__restrict__ out)
 {
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
@@ -191,6 +198,8 @@ __global__ void __launch_bounds__(kCondNT) condense_by_cell_kernel(const int32_t
         }
         if (WATER && lane == 0)
             out[cell] = c < 0.0f ? 0.0 - acc : acc;
+        if (KEEP && lane == 0)
+            keep[cell] = c;
         if constexpr (WATER)
             ahead(cell + nw);
     }
@@ -200,11 +209,14 @@ __global__ void __launch_bounds__(kCondNT) condense_by_cell_kernel(const int32_t
 template <bool WATER>
 __global__ void __launch_bounds__(kCondNT) condense_kernel(const CondItem *__restrict__ items, int32_t n_items,
                                                            const int64_t *__restrict__ xi, double *__restrict__ v,
-                                                           const float *__restrict__ cf, float xminf,
-                                                           double *__restrict__ partial)
+                                                           const float *__restrict__ cf, float *__restrict__ keep,
+                                                           int32_t n_cells, float xminf, double *__restrict__ partial)
 {
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    if (keep) // (null: not wanted) cells without an item too
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_cells; i += gridDim.x * blockDim.x)
+            keep[i] = cf[i];
     for (int it = gw; it < n_items; it += nw) {
         const CondItem I = items[it];
         const float c = cf[I.cell];
@@ -238,7 +250,7 @@ void cond_release(sdm_ctx *ctx)
     if (!ctx->cond)
         return;
     CondBuffers &b = *ctx->cond;
-    void *bufs[] = {b.items, b.item_start, b.partial, b.cond};
+    void *bufs[] = {b.items, b.partial, b.cond}; // (item_start and cf lie behind cond)
     for (void *p : bufs)
         ctx->mem.put(p, 0);
     for (cudaEvent_t ev : b.cf_done)
@@ -259,9 +271,10 @@ sdm_status cond_prepare(sdm_ctx *ctx)
     if (!ctx->cond) {
         ctx->cond = new CondBuffers();
         CondBuffers &b = *ctx->cond;
-        b.cond = static_cast<double *>(ctx->mem.get(sizeof(double) * nc));
-        b.item_start = static_cast<int32_t *>(ctx->mem.get(sizeof(int32_t) * (nc + 1)));
-        if (!b.cond || !b.item_start) {
+        b.cond = static_cast<double *>(ctx->mem.get(sizeof(double) * nc + sizeof(int32_t) * (nc + 1) + sizeof(float) * nc));
+        b.item_start = reinterpret_cast<int32_t *>(b.cond + nc);
+        b.cf = reinterpret_cast<float *>(b.item_start + nc + 1);
+        if (!b.cond) {
             cond_release(ctx);
             return fail(&ctx->error, SDM_ENOMEM, "condensation: device allocation failed");
         }
@@ -329,15 +342,14 @@ extern "C" sdm_status sdm_condensation_step(sdm_ctx *ctx, const double *G, const
         return st;
     CondBuffers &b = *ctx->cond;
     cudaStream_t cs = ctx->stream;
-    CTX_CUDA(ctx, cudaEventSynchronize(b.cf_done[b.stage])); // no kernel reads the staging any more
-    float *cf = b.h_cf + (size_t)b.stage * nc;
+    float *field = b.h_cf + (size_t)b.stage * nc;
     // one pass without branches; what it finds wrong is named by a second
     int bad = 0;
     for (int32_t c = 0; c < nc; ++c) {
         const double g = ((2.0 * G[c]) * s[c]) * dt;
         bad |= (int)!(G[c] >= 0.0) | (int)!(s[c] >= -1.0) | (int)!(s[c] <= 1.0) | (int)!(std::fabs(g) <= 1e-6) |
                (int)!(G[c] <= 1.7976931348623157e308);
-        cf[c] = (float)g;
+        field[c] = (float)g;
     }
     for (int32_t c = 0; bad && c < nc; ++c) {
         if (!(std::isfinite(G[c]) && G[c] >= 0.0) || !(std::isfinite(s[c]) && s[c] >= -1.0 && s[c] <= 1.0))
@@ -347,30 +359,35 @@ extern "C" sdm_status sdm_condensation_step(sdm_ctx *ctx, const double *G, const
             return fail(&ctx->error, SDM_EINVAL, "cell %d: |2 G s dt| = %g m^2 above 1e-6 m^2", c,
                         std::fabs(((2.0 * G[c]) * s[c]) * dt));
     }
+    const bool changed = b.last < 0 || std::memcmp(field, b.h_cf + (size_t)b.last * nc, sizeof(float) * nc) != 0;
+    const float *cf = changed ? field : b.cf;
+    float *keep = changed ? b.cf : nullptr;
     const float xminf = (float)(r_min * r_min);
     const int cells_grid = (int)std::min<int64_t>((nc + kCondNT / 32 - 1) / (kCondNT / 32), 152 * 8);
     double *out = condensed && condensed_on_device ? condensed : b.cond;
     if (ctx->largest_cell <= kCondByCell) {
-        if (condensed)
-            condense_by_cell_kernel<true><<<cells_grid, kCondNT, 0, cs>>>(ctx->d_cell_off, nc, ctx->d_xi, ctx->d_v, cf,
-                                                                          xminf, out);
-        else
-            condense_by_cell_kernel<false><<<cells_grid, kCondNT, 0, cs>>>(ctx->d_cell_off, nc, ctx->d_xi, ctx->d_v,
-                                                                           cf, xminf, nullptr);
+        const auto kernel = condensed ? (changed ? condense_by_cell_kernel<true, true> : condense_by_cell_kernel<true, false>)
+                                      : (changed ? condense_by_cell_kernel<false, true>
+                                                 : condense_by_cell_kernel<false, false>);
+        kernel<<<cells_grid, kCondNT, 0, cs>>>(ctx->d_cell_off, nc, ctx->d_xi, ctx->d_v, cf, keep, xminf, out);
     } else {
         const int grid = (int)std::min<int64_t>((b.n_items + kCondNT / 32 - 1) / (kCondNT / 32), 152 * 8);
         if (condensed) {
-            condense_kernel<true><<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, cf, xminf,
-                                                            b.partial);
+            condense_kernel<true><<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, cf, keep, nc,
+                                                            xminf, b.partial);
             condense_cells_kernel<<<cells_grid, kCondNT, 0, cs>>>(b.item_start, nc, b.partial, out);
         } else {
-            condense_kernel<false><<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, cf, xminf,
-                                                             nullptr);
+            condense_kernel<false><<<grid, kCondNT, 0, cs>>>(b.items, b.n_items, ctx->d_xi, ctx->d_v, cf, keep, nc,
+                                                             xminf, nullptr);
         }
     }
     CTX_CUDA(ctx, cudaGetLastError());
-    CTX_CUDA(ctx, cudaEventRecord(b.cf_done[b.stage], cs));
-    b.stage = (b.stage + 1) % kCondStage;
+    if (changed) {
+        CTX_CUDA(ctx, cudaEventRecord(b.cf_done[b.stage], cs));
+        b.last = b.stage;
+        b.stage = (b.stage + 1) % kCondStage;
+        CTX_CUDA(ctx, cudaEventSynchronize(b.cf_done[b.stage])); // its kernel, three fields ago
+    }
     if (condensed && !condensed_on_device) {
         CTX_CUDA(ctx, cudaMemcpyAsync(condensed, b.cond, sizeof(double) * nc, cudaMemcpyDeviceToHost, cs));
         CTX_CUDA(ctx, cudaStreamSynchronize(cs));
