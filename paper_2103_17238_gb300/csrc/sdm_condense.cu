@@ -364,7 +364,9 @@ extern "C" sdm_status sdm_condensation_step(sdm_ctx *ctx, const double *G, const
     float *keep = changed ? b.cf : nullptr;
     const float xminf = (float)(r_min * r_min);
     const int cells_grid = (int)std::min<int64_t>((nc + kCondNT / 32 - 1) / (kCondNT / 32), 152 * 8);
-    double *out = condensed && condensed_on_device ? condensed : b.cond;
+    // the kernels write a device buffer themselves if it lies on eight bytes, else a copy does
+    const bool direct = condensed && condensed_on_device && ((uintptr_t)condensed & 7) == 0;
+    double *out = direct ? condensed : b.cond;
     if (ctx->largest_cell <= kCondByCell) {
         const auto kernel = condensed ? (changed ? condense_by_cell_kernel<true, true> : condense_by_cell_kernel<true, false>)
                                       : (changed ? condense_by_cell_kernel<false, true>
@@ -388,6 +390,8 @@ extern "C" sdm_status sdm_condensation_step(sdm_ctx *ctx, const double *G, const
         b.stage = (b.stage + 1) % kCondStage;
         CTX_CUDA(ctx, cudaEventSynchronize(b.cf_done[b.stage])); // its kernel, three fields ago
     }
+    if (condensed && condensed_on_device && !direct)
+        CTX_CUDA(ctx, cudaMemcpyAsync(condensed, b.cond, sizeof(double) * nc, cudaMemcpyDeviceToDevice, cs));
     if (condensed && !condensed_on_device) {
         CTX_CUDA(ctx, cudaMemcpyAsync(condensed, b.cond, sizeof(double) * nc, cudaMemcpyDeviceToHost, cs));
         CTX_CUDA(ctx, cudaStreamSynchronize(cs));
