@@ -22,7 +22,9 @@
 //   sed_merge_kernel     one warp per new cell: its arrivals sorted by id, its
 //                        stayers streamed through, each moved up by the
 //                        arrivals of lower id; the new layout with its padding
-//                        (a cell with many arrivals: by the whole block).
+//                        (a cell with many arrivals: by the whole block; with
+//                        over kSedRunKeys of them in one cell it leaves all as
+//                        it was, and the step is taken again by the sort).
 // 112 B per SD (xi, v, heights; heights out; the layout in and out).  The
 // refresh of the context's own launch plan and the read-back run on a side
 // stream beside the last two; the host waits for the read-back only.
@@ -491,6 +493,7 @@ constexpr int kSedByCell = 1024;  // slots of the largest cell that a warp takes
 constexpr int kSedFewCells = 608, kSedFewLargest = 800; // sdm_sedimentation_step's rule for few cells
 constexpr int kSedArrive = 256;   // arrivals of a cell that a warp takes; more by its block
 constexpr int kSedMergeNT = 128;
+constexpr int kSedRunKeys = kSedArrive * (kSedMergeNT / 32); // arrivals of a cell that a block takes
 constexpr int kSedFew = 12;       // arrivals up to which each is compared with every stayer, by ballots
 
 // What the movers of the cells and the arrivals of the groups are kept in.
@@ -502,6 +505,7 @@ struct SedMoves {
     uint32_t *stay, *arr, *left;         // per group: SDs that stay; per cell: SDs that arrive, movers
     uint32_t *out, *out_next;            // SDs that arrive outside the domain; the next step's count
     int32_t *first;                      // n_groups
+    uint32_t *moved, *piled; // how many SDs move; whether a cell receives more than kSedRunKeys
 };
 
 // A warp first takes every SD's height down; the few that leave their cell (or
@@ -636,6 +640,7 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
         }
     }
     if (gw == 0 && lane == 0) { // those outside stay there (their last slot may be padding)
+        *M.piled = 0u;
         const int32_t lo = cell_off[n_cells];
         M.stay[n_cells] = (uint32_t)(n_slots - lo) - (n_slots > lo && id_of_slot[n_slots - 1] < 0 ? 1u : 0u);
     }
@@ -723,8 +728,10 @@ __global__ void __launch_bounds__(1024) sed_offsets_kernel(SedMoves M, int32_t n
         if (g == n_groups - 1)
             poff[n_groups] = (int32_t)(uint32_t)(at + mine);
     }
-    if (g == n_groups - 1) // behind the total: how many SDs move
-        *reinterpret_cast<uint32_t *>(precip_total + 1) = (uint32_t)((at + mine) >> 32);
+    if (g < n_groups - 1 && M.arr[g] > (uint32_t)kSedRunKeys)
+        *M.piled = 1u;
+    if (g == n_groups - 1)
+        *M.moved = (uint32_t)((at + mine) >> 32);
     if (blockIdx.x == 0)
         sed_precip_total(precip, n_parts, precip_total);
 }
@@ -774,11 +781,9 @@ __device__ __forceinline__ uint32_t sed_lower(uint32_t n, uint32_t x, F &&at)
 }
 
 // A cell with more than kSedArrive arrivals, by the whole block: the arrivals
-// sorted in runs of kSedRunKeys (written back when there are several), the
-// stayers' ids and counts in shared memory, every SD's place by binary
-// searches.  (By one warp that counted: 2.5 ms for 4096 cells of 1000 SDs of
-// which 600 fall into the next cell, 0.10 here.)
-constexpr int kSedRunKeys = kSedArrive * (kSedMergeNT / 32);
+// sorted, the stayers' ids and counts in shared memory, every SD's place by
+// binary searches.  (By one warp that counted: 2.5 ms for 4096 cells of 1000 SDs
+// of which 600 fall into the next cell, 0.10 here.)
 struct SedHeavy {
     uint32_t id[kSedByCell];
     uint16_t stay[kSedByCell + 2]; // stayers before a slot
@@ -822,45 +827,29 @@ __device__ __noinline__ void sed_merge_heavy(int g, const int32_t *__restrict__ 
         H.stay[t * E + e] = (uint16_t)(before + (uint32_t)__popc(keep & ((1u << e) - 1u)));
     if (t == 0)
         H.stay[kSedByCell] = (uint16_t)n_stay;
-    for (uint32_t c0 = 0; c0 < A; c0 += kSedRunKeys) {
-        const uint32_t m = min(A - c0, (uint32_t)kSedRunKeys);
-        uint32_t P2 = 1;
-        while (P2 < m)
-            P2 <<= 1;
-        for (uint32_t i = t; i < P2; i += kSedMergeNT)
-            key[i] = i < m ? ((unsigned long long)M.a_id[a0 + c0 + i] << 32) | M.a_slot[a0 + c0 + i] : ~0ull;
-        __syncthreads();
-        bool back = false; // those of one cell come in order
-        for (uint32_t i = t; i + 1 < m; i += kSedMergeNT)
-            back |= key[i] > key[i + 1];
-        for (uint32_t k = __syncthreads_or(back) ? 2u : 2u * P2; k <= P2; k <<= 1) // bitonic
-            for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-                for (uint32_t i = t; i < P2 / 2; i += kSedMergeNT) {
-                    const uint32_t a = 2 * i - (i & (j - 1)), b = a + j;
-                    const unsigned long long ka = key[a], kb = key[b];
-                    if ((ka > kb) == ((a & k) == 0)) {
-                        key[a] = kb;
-                        key[b] = ka;
-                    }
+    uint32_t P2 = 1;
+    while (P2 < A)
+        P2 <<= 1;
+    for (uint32_t i = t; i < P2; i += kSedMergeNT)
+        key[i] = i < A ? ((unsigned long long)M.a_id[a0 + i] << 32) | M.a_slot[a0 + i] : ~0ull;
+    __syncthreads();
+    bool back = false; // those of one cell come in order
+    for (uint32_t i = t; i + 1 < A; i += kSedMergeNT)
+        back |= key[i] > key[i + 1];
+    for (uint32_t k = __syncthreads_or(back) ? 2u : 2u * P2; k <= P2; k <<= 1) // bitonic
+        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+            for (uint32_t i = t; i < P2 / 2; i += kSedMergeNT) {
+                const uint32_t a = 2 * i - (i & (j - 1)), b = a + j;
+                const unsigned long long ka = key[a], kb = key[b];
+                if ((ka > kb) == ((a & k) == 0)) {
+                    key[a] = kb;
+                    key[b] = ka;
                 }
-                __syncthreads();
-            }
-        if (A > (uint32_t)kSedRunKeys) {
-            for (uint32_t i = t; i < m; i += kSedMergeNT) {
-                M.a_id[a0 + c0 + i] = (uint32_t)(key[i] >> 32);
-                M.a_slot[a0 + c0 + i] = (uint32_t)key[i];
             }
             __syncthreads();
         }
-    }
-    const bool one = A <= (uint32_t)kSedRunKeys;
     auto arrivals_below = [&](uint32_t id) {
-        if (one)
-            return sed_lower(A, id, [&](uint32_t i) { return (uint32_t)(key[i] >> 32); });
-        uint32_t r = 0;
-        for (uint32_t c0 = 0; c0 < A; c0 += kSedRunKeys)
-            r += sed_lower(min(A - c0, (uint32_t)kSedRunKeys), id, [&](uint32_t i) { return M.a_id[a0 + c0 + i]; });
-        return r;
+        return sed_lower(A, id, [&](uint32_t i) { return (uint32_t)(key[i] >> 32); });
     };
     for (uint32_t i = t; i < n; i += kSedMergeNT) {
         const double z = zeta_new[lo + i];
@@ -868,9 +857,8 @@ __device__ __noinline__ void sed_merge_heavy(int g, const int32_t *__restrict__ 
             L.put((int64_t)p0 + H.stay[i] + arrivals_below(H.id[i]), xi[lo + i], v[lo + i], z, (int32_t)H.id[i]);
     }
     for (uint32_t j = t; j < A; j += kSedMergeNT) {
-        const uint32_t id = one ? (uint32_t)(key[j] >> 32) : M.a_id[a0 + j];
-        const uint32_t slot = one ? (uint32_t)key[j] : M.a_slot[a0 + j];
-        const uint32_t at = (one ? j : arrivals_below(id)) + H.stay[sed_lower(n, id, [&](uint32_t i) { return H.id[i]; })];
+        const uint32_t id = (uint32_t)(key[j] >> 32), slot = (uint32_t)key[j];
+        const uint32_t at = j + H.stay[sed_lower(n, id, [&](uint32_t i) { return H.id[i]; })];
         L.put((int64_t)p0 + at, xi[slot], v[slot], fabs(zeta_new[slot]), (int32_t)id);
     }
     __syncthreads(); // the shared arrays and the count are read
@@ -881,7 +869,9 @@ __device__ __noinline__ void sed_merge_heavy(int g, const int32_t *__restrict__ 
     }
 }
 
-__global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *__restrict__ cell_off, int32_t n_cells,
+// Nine blocks per SM (56 registers): with eight (64) a step of the 4.19M-SD grid takes
+// 4.7 us more.
+__global__ void __launch_bounds__(kSedMergeNT, 9) sed_merge_kernel(const int32_t *__restrict__ cell_off, int32_t n_cells,
                                                                 SedMoves M, const int64_t *__restrict__ xi,
                                                                 const double *__restrict__ v,
                                                                 const double *__restrict__ zeta_new,
@@ -904,6 +894,8 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
     // a cell's numbers, one per lane, loaded a cell ahead
     auto numbers = [&](int g) -> uint32_t {
+        if (lane == 7) // (the same for every cell)
+            return *M.piled;
         if (g >= n_cells || lane > 6)
             return 0u;
         if (lane < 4)
@@ -911,6 +903,14 @@ __global__ void __launch_bounds__(kSedMergeNT) sed_merge_kernel(const int32_t *_
         return lane == 4 ? M.arr[g] : (lane == 5 ? (uint32_t)M.first[g] : M.stay[g]);
     };
     uint32_t ahead = numbers(gw);
+    if (__syncthreads_or(lane == 7 && ahead != 0u)) { // taken again by the sort: the counts are made ready, no more
+        for (int g = gw; g < n_cells; g += nw)
+            if (lane == 0)
+                M.arr[g] = 0u;
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            *M.out_next = 0u;
+        return;
+    }
     int heavy = 0;
     for (int g = gw; g < n_cells; g += nw) { // uniform over the warp
         const int32_t lo = __shfl_sync(FULL, ahead, 0), hi = __shfl_sync(FULL, ahead, 1);
@@ -1082,7 +1082,7 @@ struct SedBuffers {
                                //   arrivals) the next step uses; all arrivals are zero between steps
     uint32_t *counts = nullptr; // n_cells + 1
     int32_t *ustart = nullptr;  // n_cells + 2
-    double *precip = nullptr;   // per-block parts of the move kernel, the total, the movers' count
+    double *precip = nullptr;   // per-block parts of the move kernel, the total, the movers' count and the mark
     int sorted_left = 0;        // steps that take the sorted path before the movers are counted again
     uint32_t *hist = nullptr;   // 256 x tiles, then 256 digit totals
     uint32_t *flags = nullptr;  // flags, then the first bad id (8-byte aligned)
@@ -1093,8 +1093,8 @@ struct SedBuffers {
 };
 
 // Bytes of the pinned read-back buffer for n_cells cells: n_cells + 2
-// offsets, the precipitated total (8-byte aligned) with the movers' count, and
-// the class-count words.
+// offsets, the precipitated total (8-byte aligned) with the movers' count and the
+// mark of a pile, and the class-count words.
 size_t sed_read_bytes(int32_t n_cells) { return (((size_t)n_cells + 2) * 4 + 7) / 8 * 8 + 16 + sizeof(uint32_t) * (kNumClass + 1); }
 
 void sed_release(sdm_ctx *ctx)
@@ -1314,19 +1314,56 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     // 1000, 5% moving 55 | 50, all moving 75 | 50; of 600 43 | 50 and 95 | 50; of
     // 300 33 | 50 and 67 | 50; 512 cells of 1000 66 | 80 and 103 | 93; 4096 cells: by
     // cells is faster for any share): sorted if the cells are large, or if over a third
-    // of the SDs moved a few steps ago.
+    // of the SDs moved a few steps ago.  Any number of cells: sorted for as long when
+    // one of them received more than kSedRunKeys SDs (a block that merges a pile works
+    // alone: 640 columns of 3 cells of 1000 that all fall into the lowest one 473 us
+    // merged in runs, 183 sorted; 10 columns of 64, 120 ms and 0.15).  The step that
+    // finds that out is taken twice (257 and 328 us).
     const bool few = nc <= kSedFewCells;
-    if (!few)
-        b.sorted_left = 0;
-    const bool by_cell = ctx->largest_cell <= kSedByCell && !(2 * nc <= kSedFewCells && ctx->largest_cell > kSedFewLargest) &&
+    bool by_cell = ctx->largest_cell <= kSedByCell && !(2 * nc <= kSedFewCells && ctx->largest_cell > kSedFewLargest) &&
                          b.sorted_left == 0;
+    auto sorted_step = [&]() -> sdm_status {
+        if (!b.group_valid)
+            sed_group_kernel<<<sed_grid(n_groups), kSedNT, 0, s>>>(ctx->d_cell_off, nc, ctx->n_slots, b.group);
+        CTX_CUDA(ctx, cudaMemsetAsync(b.counts, 0, sizeof(uint32_t) * n_groups, s));
+        const int move_blocks = (int)std::max<int64_t>(
+            1,
+            std::min<int64_t>(kSedMaxBlocks, (ctx->n_slots + (int64_t)kSedNT * kSedU - 1) / ((int64_t)kSedNT * kSedU)));
+        sed_move_kernel<<<move_blocks, kSedNT, 0, s>>>(ctx->d_inst, nc, ctx->n_slots, ctx->nx, ctx->dz,
+                                                       (float)ctx->cfg.dt, ctx->d_zeta, b.group, ctx->d_id_of_slot,
+                                                       b.keys[0], b.vals[0], b.zeta_new, b.counts, b.precip,
+                                                       ctx->cfg.cell_base, b.emig);
+        // the offset scan, the padding and the rest of the side stream's work
+        // beside the radix sort, which needs none of them
+        CTX_CUDA(ctx, cudaEventRecord(b.fork, s));
+        CTX_CUDA(ctx, cudaStreamWaitEvent(b.side, b.fork, 0));
+        sed_scan_kernel<<<1, 1024, 0, b.side>>>(b.counts, n_groups, b.ustart, b.cell_off2, b.precip, move_blocks,
+                                                b.precip + kSedMaxBlocks);
+        // the new layout's padding slots (the gather writes only the others)
+        sed_pad_kernel<<<(n_groups + 255) / 256, 256, 0, b.side>>>(n_groups, b.ustart, b.cell_off2, b.xi2, b.v2,
+                                                                    b.zeta2, b.id2, b.group2);
+        const sdm_status sw = side_work();
+        if (sw != SDM_OK)
+            return sw;
+        // stable sort of the new groups, SD-id order in
+        const int bits = 32 - __builtin_clz((unsigned)nc | 1u);
+        const int cur = radix_sort(b.keys, b.vals, false, n, bits, b.hist, s);
+        CTX_CUDA(ctx, cudaStreamWaitEvent(s, b.join, 0));
+        sed_gather_kernel<<<1216, 256, 0, s>>>(n, b.keys[cur], b.vals[cur], b.ustart, b.cell_off2, ctx->d_xi, ctx->d_v,
+                                               b.zeta_new, ctx->d_id_of_slot, b.xi2, b.v2, b.zeta2, b.id2, b.group2);
+        CTX_CUDA(ctx, cudaGetLastError());
+        std::swap(b.group, b.group2);
+        b.group_valid = true;
+        return SDM_OK;
+    };
     if (b.sorted_left > 0)
         --b.sorted_left;
     if (by_cell) {
         const size_t st_ = sed_stride(nc);
         SedMoves M{b.keys[0], b.vals[0],      b.keys[1],          b.vals[1],   (uint32_t *)b.group, (uint32_t *)b.group2,
                    b.moves,   b.moves + st_, b.moves + 2 * st_, b.moves + 2 * st_ - 1 - b.parity,
-                   b.moves + 2 * st_ - 2 + b.parity, (int32_t *)(b.moves + 3 * st_)};
+                   b.moves + 2 * st_ - 2 + b.parity, (int32_t *)(b.moves + 3 * st_),
+                   (uint32_t *)(b.precip + kSedMaxBlocks + 1), (uint32_t *)(b.precip + kSedMaxBlocks + 1) + 1};
         b.parity ^= 1;
         unsigned long long *totals = (unsigned long long *)(b.moves + 4 * st_);
         b.group_valid = false;
@@ -1355,49 +1392,22 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
             SedLayout{b.xi2, b.v2, b.zeta2, b.id2}, ctx->d_inst, ctx->step);
         CTX_CUDA(ctx, cudaGetLastError());
         CTX_CUDA(ctx, cudaStreamWaitEvent(s, b.join, 0)); // later work may write what the side stream reads
-    } else {
-        if (!b.group_valid)
-            sed_group_kernel<<<sed_grid(n_groups), kSedNT, 0, s>>>(ctx->d_cell_off, nc, ctx->n_slots, b.group);
-        CTX_CUDA(ctx, cudaMemsetAsync(b.counts, 0, sizeof(uint32_t) * n_groups, s));
-        const int move_blocks = (int)std::max<int64_t>(
-            1,
-            std::min<int64_t>(kSedMaxBlocks, (ctx->n_slots + (int64_t)kSedNT * kSedU - 1) / ((int64_t)kSedNT * kSedU)));
-        sed_move_kernel<<<move_blocks, kSedNT, 0, s>>>(ctx->d_inst, nc, ctx->n_slots, ctx->nx, ctx->dz,
-                                                       (float)ctx->cfg.dt, ctx->d_zeta, b.group, ctx->d_id_of_slot,
-                                                       b.keys[0], b.vals[0], b.zeta_new, b.counts, b.precip,
-                                                       ctx->cfg.cell_base, b.emig);
-        // the offset scan, the padding and the rest of the side stream's work
-        // beside the radix sort, which needs none of them
-        CTX_CUDA(ctx, cudaEventRecord(b.fork, s));
-        CTX_CUDA(ctx, cudaStreamWaitEvent(b.side, b.fork, 0));
-        sed_scan_kernel<<<1, 1024, 0, b.side>>>(b.counts, n_groups, b.ustart, b.cell_off2, b.precip, move_blocks,
-                                                b.precip + kSedMaxBlocks);
-        // the new layout's padding slots (the gather writes only the others)
-        sed_pad_kernel<<<(n_groups + 255) / 256, 256, 0, b.side>>>(n_groups, b.ustart, b.cell_off2, b.xi2, b.v2,
-                                                                    b.zeta2, b.id2, b.group2);
-        st = side_work();
+        // the read-back only: what writes the new layout goes on behind it
+        CTX_CUDA(ctx, cudaEventSynchronize(b.join));
+        uint32_t moved[2]; // movers, whether a cell receives too many
+        std::memcpy(moved, hr + at_pr + 8, sizeof moved);
+        if (moved[1] || (few && (int64_t)moved[0] * 3 > n))
+            b.sorted_left = 16;
+        by_cell = moved[1] == 0;
+    }
+    if (!by_cell) {
+        st = sorted_step();
         if (st != SDM_OK)
             return st;
-        // stable sort of the new groups, SD-id order in
-        const int bits = 32 - __builtin_clz((unsigned)nc | 1u);
-        const int cur = radix_sort(b.keys, b.vals, false, n, bits, b.hist, s);
-        CTX_CUDA(ctx, cudaStreamWaitEvent(s, b.join, 0));
-        sed_gather_kernel<<<1216, 256, 0, s>>>(n, b.keys[cur], b.vals[cur], b.ustart, b.cell_off2, ctx->d_xi, ctx->d_v,
-                                               b.zeta_new, ctx->d_id_of_slot, b.xi2, b.v2, b.zeta2, b.id2, b.group2);
-        CTX_CUDA(ctx, cudaGetLastError());
-        std::swap(b.group, b.group2);
-        b.group_valid = true;
+        CTX_CUDA(ctx, cudaEventSynchronize(b.join));
     }
-    // the read-back only: what writes the new layout goes on behind it
-    CTX_CUDA(ctx, cudaEventSynchronize(b.join));
     double precip = 0.0;
     std::memcpy(&precip, hr + at_pr, sizeof precip);
-    if (by_cell && few) {
-        uint32_t movers = 0;
-        std::memcpy(&movers, hr + at_pr + 8, sizeof movers);
-        if ((int64_t)movers * 3 > n)
-            b.sorted_left = 16;
-    }
     // the new layout becomes the state; the old one the next scratch
     std::swap(ctx->d_xi, b.xi2);
     std::swap(ctx->d_v, b.v2);
