@@ -243,7 +243,9 @@ sdm_status sdm_set_positions(sdm_ctx *ctx, const double *z, int32_t nx, double d
 /* One sedimentation step (asynchronous up to one host read of the new cell
  * offsets; stream-ordered with the coalescence steps).  precipitated
  * (nullable host pointer) receives sum(xi v), m^3, of the SDs that fell
- * through the bottom in this step.  A batch (sdm_batch_create) holding the
+ * through the bottom in this step: the exact sum rounded to nearest, so it
+ * depends on those SDs only, not on the steps before (a run resumed from a
+ * checkpoint gives the same bits).  A batch (sdm_batch_create) holding the
  * context must be created again afterwards: its next step fails with
  * SDM_ESTATE.  Errors: SDM_ESTATE (no positions), SDM_ENOMEM, SDM_ECUDA. */
 sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated);

@@ -17,7 +17,7 @@
 //                        (new group, id, slot, place among the group's
 //                        arrivals), the water that leaves through the bottom;
 //   sed_offsets_kernel   the new cells' offsets (even) and their arrivals', the
-//                        precipitated total in a fixed order;
+//                        precipitated total, rounded from an exact sum;
 //   sed_deal_kernel      the movers to their group's arrivals;
 //   sed_merge_kernel     one warp per new cell: its arrivals sorted by id, its
 //                        stayers streamed through, each moved up by the
@@ -38,7 +38,7 @@
 //                        domain) as a key in SD-id order, counts per new
 //                        group, the water that leaves through the bottom;
 //   sed_scan_kernel      new group offsets (unpadded and padded to even
-//                        slots) and the precipitated total, in fixed order;
+//                        slots) and the precipitated total, as above;
 //   radix_sort           (sdm_radix.cuh) of the keys: per-tile digit counts, a
 //                        scan of each digit's row, a scan of the digit totals,
 //                        a ranked scatter;
@@ -169,8 +169,8 @@ __global__ void __launch_bounds__(kSedNT) sed_get_kernel(const int32_t *__restri
 // issued before use).  key[id] = its new group (n_cells: outside), val[id]
 // = its slot, zeta_new[slot] = its new height; counts[new group] (one
 // atomic per run of equal groups among a warp's 32 consecutive slots);
-// precip_part[block] = sum of xi v of the SDs that fell through the bottom
-// of the grid (thread order fixed, then a fixed tree over the block).
+// precip: the exact sum of xi v of the SDs that fell through the bottom of
+// the grid.
 // Levels are counted from the grid's bottom (cell cbase + c): an SD that
 // leaves this piece's lowest level into a level of another piece becomes
 // outside here, with emig[id] = its new cell there and zeta_new its height
@@ -239,22 +239,121 @@ __device__ __forceinline__ Fall sed_fall(const PairConsts &C, double v, double z
     return sed_levels(sed_drop(C, v, zt, dt32), g, nx, dz, cbase);
 }
 
-// precip_part[block] = the block's sum of pr (lanes, then warps, in a fixed tree).
-__device__ __forceinline__ void sed_precip(double pr, double *precip_part)
+// The precipitated water: an exact sum, so that it depends neither on the order
+// of its terms nor on the path that takes the step.  A term xi v is an integer
+// in units of 2^-1074, added as digits of 32 bits to signed 64-bit bins (bin i
+// weighs 2^(32 i - 1074); 2^31 terms fit), and the sum of all is rounded once.
+// (In binary64, as it was, a term took the narrow pipe's additions: a step in
+// which all of 16,384 cells of 256 fall out 254 us, 237 now.)
+constexpr int kExactBins = 72;
+typedef unsigned long long ExactBin; // two's complement
+
+// Adds xi v of the lanes with `on` (all lanes of the warp call it).  Lanes whose
+// digits lie in the same bins, with the same sign, share their additions.
+__device__ __noinline__ void exact_add(ExactBin *bins, bool on, int64_t xi, double v)
 {
-    __shared__ double s_pr[kSedNT / 32];
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    const uint64_t bits = (uint64_t)__double_as_longlong(v);
+    const uint32_t e = (uint32_t)(bits >> 52) & 0x7FFu;
+    const uint64_t m = (bits & 0xFFFFFFFFFFFFFull) | (e ? 1ull << 52 : 0ull);
+    const uint32_t at = e ? e - 1u : 0u, sh = at & 31u; // the last place of v weighs 2^(at - 1074)
+    const uint64_t lo = (uint64_t)xi * m, hi = __umul64hi((uint64_t)xi, m);
+    const uint64_t w0 = lo << sh, w1 = (hi << sh) | (sh ? lo >> (64u - sh) : 0ull), w2 = sh ? hi >> (64u - sh) : 0ull;
+    const uint32_t digit[5] = {(uint32_t)w0, (uint32_t)(w0 >> 32), (uint32_t)w1, (uint32_t)(w1 >> 32), (uint32_t)w2};
+    const uint32_t group = (at >> 5) | (uint32_t)(bits >> 63) << 8;
+    for (unsigned todo = __ballot_sync(FULL, on); todo;) {
+        const uint32_t g = __shfl_sync(FULL, group, __ffs(todo) - 1);
+        const bool mine = on && group == g;
+        ExactBin sum = 0;
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1)
-        pr = __dadd_rn(pr, __shfl_down_sync(0xFFFFFFFFu, pr, d));
-    if ((threadIdx.x & 31) == 0)
-        s_pr[threadIdx.x >> 5] = pr;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kSedNT / 32; ++w)
-            t = __dadd_rn(t, s_pr[w]);
-        precip_part[blockIdx.x] = t;
+        for (int k = 0; k < 5; ++k) {
+            const uint32_t d = mine ? digit[k] : 0u;
+            const uint32_t low = __reduce_add_sync(FULL, d & 0xFFFFu), high = __reduce_add_sync(FULL, d >> 16);
+            if (lane == k)
+                sum = ((ExactBin)high << 16) + low;
+        }
+        if (lane < 5 && sum)
+            atomicAdd(&bins[(g & 0xFFu) + lane], g >> 8 ? 0ull - sum : sum);
+        todo &= ~__ballot_sync(FULL, mine);
     }
+}
+
+// The block's bins, zero before use (a barrier between), and into the sum of all blocks.
+__device__ __forceinline__ void exact_clear(ExactBin *bins)
+{
+    for (int i = threadIdx.x; i < kExactBins; i += blockDim.x)
+        bins[i] = 0ull;
+}
+
+__device__ __forceinline__ void exact_flush(const ExactBin *bins, ExactBin *total)
+{
+    __syncthreads();
+    for (int i = threadIdx.x; i < kExactBins; i += blockDim.x)
+        if (bins[i])
+            atomicAdd(&total[i], bins[i]);
+}
+
+// *out = the sum rounded to nearest even; total is zero again (one warp).
+__device__ __forceinline__ void exact_round(ExactBin *total, double *out)
+{
+    __shared__ uint32_t s_digit[kExactBins];
+    __shared__ long long s_bin[kExactBins];
+    const int lane = threadIdx.x & 31;
+    int first = kExactBins, last = -1;
+    for (int i = lane; i < kExactBins; i += 32) {
+        const ExactBin b = total[i];
+        s_bin[i] = (long long)b;
+        s_digit[i] = 0u;
+        if (b) {
+            total[i] = 0ull;
+            first = min(first, i);
+            last = i;
+        }
+    }
+    first = __reduce_min_sync(0xFFFFFFFFu, first);
+    last = __reduce_max_sync(0xFFFFFFFFu, last);
+    __syncwarp();
+    if (lane != 0)
+        return;
+    bool minus = false;
+    long long carry = 0;
+    int end = kExactBins;
+    for (int pass = 0; pass < 2; ++pass) { // a negative sum's digits in the second, of its negative
+        carry = 0;
+        for (int i = first; i < kExactBins && (i <= last || carry != 0); ++i) {
+            carry += minus ? -s_bin[i] : s_bin[i];
+            s_digit[i] = (uint32_t)carry;
+            carry >>= 32;
+            end = i + 1;
+            if (i > last && carry == -1 && s_digit[i] == 0xFFFFFFFFu)
+                break; // the sign, from here up
+        }
+        if (carry >= 0)
+            break;
+        minus = true;
+    }
+    int t = end - 1;
+    while (t >= first && s_digit[t] == 0u)
+        --t;
+    if (t < first) {
+        *out = 0.0;
+        return;
+    }
+    const uint32_t d2 = s_digit[t], d1 = t > 0 ? s_digit[t - 1] : 0u, d0 = t > 1 ? s_digit[t - 2] : 0u;
+    const int lz = __clz((int)d2);
+    uint64_t n = (uint64_t)d2 << 32 | d1;
+    n = lz ? (n << lz) | (d0 >> (32 - lz)) : n;
+    bool below = (lz ? d0 << lz : d0) != 0u;
+    for (int i = first; i < t - 2; ++i)
+        below |= s_digit[i] != 0u;
+    const int w = 32 * (t - 1) - lz - 1074; // the sum is n 2^w and a little
+    double r;
+    if (w + 1085 >= 1 && w + 1085 <= 2045)
+        r = u64_to_double(n, below, w);
+    else // the ends of the range, which no volume of water comes near
+        r = ldexp(__ull2double_rn(n), w);
+    *out = minus ? -r : r;
 }
 
 __global__ void __launch_bounds__(kSedNT) sed_move_kernel(const InstDev *__restrict__ P, int32_t n_cells, int64_t n_slots,
@@ -264,16 +363,18 @@ __global__ void __launch_bounds__(kSedNT) sed_move_kernel(const InstDev *__restr
                                                           const int32_t *__restrict__ id_of_slot,
                                                           uint32_t *__restrict__ key, uint32_t *__restrict__ val,
                                                           double *__restrict__ zeta_new, uint32_t *__restrict__ counts,
-                                                          double *__restrict__ precip_part, int32_t cbase,
+                                                          ExactBin *__restrict__ precip, int32_t cbase,
                                                           int32_t *__restrict__ emig)
 {
     constexpr unsigned FULL = 0xFFFFFFFFu;
+    __shared__ ExactBin s_precip[kExactBins];
+    exact_clear(s_precip);
+    __syncthreads();
     const PairConsts C = pair_consts(P);
     const int lane = threadIdx.x & 31;
     const int64_t *__restrict__ gxi = P->xi;
     const double *__restrict__ gv = P->v;
     const int64_t stride = (int64_t)gridDim.x * kSedNT;
-    double pr = 0.0;
     // warp-uniform trip count: every lane runs every round (shuffles, ballots)
     for (int64_t w0 = ((int64_t)blockIdx.x * kSedNT + (threadIdx.x & ~31)); w0 < n_slots; w0 += kSedU * stride) {
         int32_t id[kSedU], g[kSedU];
@@ -293,6 +394,7 @@ __global__ void __launch_bounds__(kSedNT) sed_move_kernel(const InstDev *__restr
         for (int u = 0; u < kSedU; ++u) {
             const int64_t sl = w0 + u * stride + lane;
             int32_t ng = -1; // -1: no SD in this slot
+            bool fell = false;
             if (id[u] >= 0) {
                 double zn = 0.0;
                 int32_t em = -1;
@@ -300,7 +402,7 @@ __global__ void __launch_bounds__(kSedNT) sed_move_kernel(const InstDev *__restr
                 if (g[u] < n_cells && x[u] > 0) {
                     const Fall f = sed_fall(C, vv[u], zt[u], dt32, g[u], nx, dz, cbase);
                     if (f.c + cbase < 0) {
-                        pr = __dadd_rn(pr, __dmul_rn(xi2d(x[u]), vv[u]));
+                        fell = true;
                     } else {
                         zn = f.z;
                         if (f.c >= 0)
@@ -314,6 +416,8 @@ __global__ void __launch_bounds__(kSedNT) sed_move_kernel(const InstDev *__restr
                 zeta_new[sl] = zn;
                 emig[id[u]] = em;
             }
+            if (__any_sync(FULL, fell))
+                exact_add(s_precip, fell, x[u], vv[u]);
             const int32_t nxt = __shfl_down_sync(FULL, ng, 1);
             const bool end = lane == 31 || nxt != ng;
             const unsigned ends = __ballot_sync(FULL, end);
@@ -324,53 +428,17 @@ __global__ void __launch_bounds__(kSedNT) sed_move_kernel(const InstDev *__restr
             }
         }
     }
-    sed_precip(pr, precip_part);
-}
-
-// *precip_total = the sum of precip[0 .. n_parts), by one block of 1024:
-// thread t sums parts t, t + 1024, ... in order, then a fixed tree over the
-// threads (the loads of four parts in flight at once, the sums in the same
-// order).
-__device__ __forceinline__ void sed_precip_total(const double *__restrict__ precip, int32_t n_parts,
-                                                 double *__restrict__ precip_total)
-{
-    __shared__ double s_pr[32];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    double pr = 0.0;
-    for (int i0 = t; i0 < n_parts; i0 += 4 * 1024) {
-        double q[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            q[u] = i0 + u * 1024 < n_parts ? precip[i0 + u * 1024] : 0.0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (i0 + u * 1024 < n_parts)
-                pr = __dadd_rn(pr, q[u]);
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1)
-        pr = __dadd_rn(pr, __shfl_down_sync(0xFFFFFFFFu, pr, d));
-    if (lane == 0)
-        s_pr[warp] = pr;
-    __syncthreads();
-    if (warp == 0) {
-        pr = s_pr[lane];
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1)
-            pr = __dadd_rn(pr, __shfl_down_sync(0xFFFFFFFFu, pr, d));
-        if (lane == 0)
-            *precip_total = pr;
-    }
+    exact_flush(s_precip, precip);
 }
 
 // One block: ustart = exclusive scan of counts[0 .. n_groups) (total at
 // ustart[n_groups]); poff the same with every count rounded up to even;
-// *precip_total = sum of precip[0 .. n_parts) in a fixed order.  Both scans
+// *precip_total = the rounded sum of the bins.  Both scans
 // run at once on packed 64-bit sums (unpadded below, padded above: neither
 // exceeds 2^31), 8 consecutive groups per thread, tiles of 8192 groups.
 __global__ void __launch_bounds__(1024) sed_scan_kernel(const uint32_t *__restrict__ counts, int32_t n_groups,
                                                         int32_t *__restrict__ ustart, int32_t *__restrict__ poff,
-                                                        const double *__restrict__ precip, int32_t n_parts,
+                                                        ExactBin *__restrict__ precip,
                                                         double *__restrict__ precip_total)
 {
     constexpr int E = 8, TILE = 1024 * E;
@@ -446,7 +514,8 @@ __global__ void __launch_bounds__(1024) sed_scan_kernel(const uint32_t *__restri
         ustart[n_groups] = (int32_t)(uint32_t)carry;
         poff[n_groups] = (int32_t)(uint32_t)(carry >> 32);
     }
-    sed_precip_total(precip, n_parts, precip_total);
+    if (warp == 0)
+        exact_round(precip, precip_total);
 }
 
 // The new layout: the j-th SD in (group, id) order goes to slot
@@ -520,10 +589,13 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
                                                           const double *__restrict__ zeta,
                                                           const int32_t *__restrict__ id_of_slot,
                                                           double *__restrict__ zeta_new, SedMoves M,
-                                                          double *__restrict__ precip_part, int32_t cbase,
+                                                          ExactBin *__restrict__ precip, int32_t cbase,
                                                           int32_t *__restrict__ emig)
 {
     constexpr unsigned FULL = 0xFFFFFFFFu;
+    __shared__ ExactBin s_precip[kExactBins];
+    exact_clear(s_precip);
+    __syncthreads();
     __shared__ double s_z[kSedNT / 32][kSedWait];
     __shared__ int32_t s_slot[kSedNT / 32][kSedWait]; // with the sign bit for an SD that does not fall (dead, padding)
     const PairConsts C = pair_consts(P);
@@ -532,13 +604,13 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
     const int64_t *__restrict__ gxi = P->xi;
     const double *__restrict__ gv = P->v;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-    double pr = 0.0;
     for (int g = gw; g < n_cells; g += nw) { // uniform over the warp
         const int32_t lo = cell_off[g], hi = cell_off[g + 1];
         uint32_t stay = 0, left = 0, wait = 0; // uniform
         auto follow = [&](uint32_t n) {        // the first n <= 32 waiting entries
             int32_t ng = n_cells, em = -1, id = -1, sl = 0;
             double zn = 0.0;
+            bool fell = false;
             if (lane < (int)n) {
                 const int32_t e = s_slot[warp][lane];
                 sl = e & 0x7FFFFFFF;
@@ -546,7 +618,7 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
                 if (e >= 0) {
                     const Fall f = sed_levels(s_z[warp][lane], g, nx, dz, cbase);
                     if (f.c + cbase < 0) {
-                        pr = __dadd_rn(pr, __dmul_rn(xi2d(gxi[sl]), gv[sl]));
+                        fell = true;
                     } else {
                         zn = f.z;
                         if (f.c >= 0)
@@ -556,6 +628,8 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
                     }
                 }
             }
+            if (__any_sync(FULL, fell))
+                exact_add(s_precip, fell, fell ? gxi[sl] : 0, fell ? gv[sl] : 0.0);
             // (level 0 dz above: zeta + dz rounded up to dz, so it stays after all)
             const bool keep = lane < (int)n && ng == g;
             stay += (uint32_t)__popc(__ballot_sync(FULL, keep));
@@ -644,7 +718,7 @@ __global__ void __launch_bounds__(kSedNT) sed_fall_kernel(const InstDev *__restr
         const int32_t lo = cell_off[n_cells];
         M.stay[n_cells] = (uint32_t)(n_slots - lo) - (n_slots > lo && id_of_slot[n_slots - 1] < 0 ? 1u : 0u);
     }
-    sed_precip(pr, precip_part);
+    exact_flush(s_precip, precip);
 }
 
 // Sums over the groups of a block of 1024, for sed_offsets_kernel over many.
@@ -681,13 +755,13 @@ __global__ void __launch_bounds__(1024) sed_totals_kernel(SedMoves M, int32_t n_
 }
 
 // poff[g] = first slot of group g (every group an even number), M.first[g] =
-// its first arrival; block 0 also sums the precipitated water.  The groups
+// its first arrival; block 0 also rounds the precipitated water.  The groups
 // before a block are summed by the block itself (up to 64 blocks: totals
 // null), or their blocks' totals.
 __global__ void __launch_bounds__(1024) sed_offsets_kernel(SedMoves M, int32_t n_groups,
                                                            const unsigned long long *__restrict__ totals,
                                                            int32_t *__restrict__ poff,
-                                                           const double *__restrict__ precip, int32_t n_parts,
+                                                           ExactBin *__restrict__ precip,
                                                            double *__restrict__ precip_total)
 {
     __shared__ unsigned long long s_w[32];
@@ -732,8 +806,8 @@ __global__ void __launch_bounds__(1024) sed_offsets_kernel(SedMoves M, int32_t n
         *M.piled = 1u;
     if (g == n_groups - 1)
         *M.moved = (uint32_t)((at + mine) >> 32);
-    if (blockIdx.x == 0)
-        sed_precip_total(precip, n_parts, precip_total);
+    if (blockIdx.x == 0 && warp == 0)
+        exact_round(precip, precip_total);
 }
 
 __global__ void __launch_bounds__(kSedNT) sed_deal_kernel(const int32_t *__restrict__ cell_off, int32_t n_cells,
@@ -1082,7 +1156,8 @@ struct SedBuffers {
                                //   arrivals) the next step uses; all arrivals are zero between steps
     uint32_t *counts = nullptr; // n_cells + 1
     int32_t *ustart = nullptr;  // n_cells + 2
-    double *precip = nullptr;   // per-block parts of the move kernel, the total, the movers' count and the mark
+    ExactBin *precip = nullptr; // the precipitated water's bins (zero between steps), then its sum, the
+                                //   movers' count and the mark of a pile
     int sorted_left = 0;        // steps that take the sorted path before the movers are counted again
     uint32_t *hist = nullptr;   // 256 x tiles, then 256 digit totals
     uint32_t *flags = nullptr;  // flags, then the first bad id (8-byte aligned)
@@ -1162,7 +1237,7 @@ sdm_status sed_alloc(sdm_ctx *ctx)
     }
     b.counts = sed_get<uint32_t>(ctx, (size_t)nc + 1);
     b.ustart = sed_get<int32_t>(ctx, (size_t)nc + 2);
-    b.precip = sed_get<double>(ctx, (size_t)kSedMaxBlocks + 2);
+    b.precip = sed_get<ExactBin>(ctx, (size_t)kExactBins + 2);
     b.hist = sed_get<uint32_t>(ctx, radix_hist_words(cap));
     b.flags = sed_get<uint32_t>(ctx, 4);
     b.moves = sed_get<uint32_t>(ctx, 4 * sed_stride(nc) + 2 * ((size_t)nc / 1024 + 1));
@@ -1185,7 +1260,8 @@ sdm_status sed_alloc(sdm_ctx *ctx)
         sed_release(ctx);
         return fail(&ctx->error, SDM_ENOMEM, "sedimentation buffers: device allocation failed");
     }
-    if (cudaMemsetAsync(b.moves, 0, sizeof(uint32_t) * 2 * sed_stride(nc), ctx->stream) != cudaSuccess) {
+    if (cudaMemsetAsync(b.moves, 0, sizeof(uint32_t) * 2 * sed_stride(nc), ctx->stream) != cudaSuccess ||
+        cudaMemsetAsync(b.precip, 0, sizeof(ExactBin) * kExactBins, ctx->stream) != cudaSuccess) {
         cudaGetLastError();
         sed_release(ctx);
         return fail(&ctx->error, SDM_ECUDA, "sedimentation buffers: clearing failed");
@@ -1289,6 +1365,7 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
     const int64_t n = ctx->n_sd;
     sdm_batch *sb = ctx->self_batch;
     const bool refresh = sb && sb->plan.refreshable && same_tuning(sb->plan.tuning, current_tuning());
+    double *precip_sum = reinterpret_cast<double *>(b.precip + kExactBins);
     unsigned char *hr = static_cast<unsigned char *>(b.h_read);
     const int32_t *off = reinterpret_cast<const int32_t *>(hr);
     const size_t at_pr = (((size_t)nc + 2) * 4 + 7) / 8 * 8;
@@ -1304,7 +1381,7 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
                                           cudaMemcpyDeviceToHost, b.side));
         }
         CTX_CUDA(ctx, cudaMemcpyAsync(hr, b.cell_off2, sizeof(int32_t) * (n_groups + 1), cudaMemcpyDeviceToHost, b.side));
-        CTX_CUDA(ctx, cudaMemcpyAsync(hr + at_pr, b.precip + kSedMaxBlocks, 2 * sizeof(double), cudaMemcpyDeviceToHost,
+        CTX_CUDA(ctx, cudaMemcpyAsync(hr + at_pr, b.precip + kExactBins, 2 * sizeof(double), cudaMemcpyDeviceToHost,
                                       b.side));
         CTX_CUDA(ctx, cudaEventRecord(b.join, b.side));
         return SDM_OK;
@@ -1337,8 +1414,7 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
         // beside the radix sort, which needs none of them
         CTX_CUDA(ctx, cudaEventRecord(b.fork, s));
         CTX_CUDA(ctx, cudaStreamWaitEvent(b.side, b.fork, 0));
-        sed_scan_kernel<<<1, 1024, 0, b.side>>>(b.counts, n_groups, b.ustart, b.cell_off2, b.precip, move_blocks,
-                                                b.precip + kSedMaxBlocks);
+        sed_scan_kernel<<<1, 1024, 0, b.side>>>(b.counts, n_groups, b.ustart, b.cell_off2, b.precip, precip_sum);
         // the new layout's padding slots (the gather writes only the others)
         sed_pad_kernel<<<(n_groups + 255) / 256, 256, 0, b.side>>>(n_groups, b.ustart, b.cell_off2, b.xi2, b.v2,
                                                                     b.zeta2, b.id2, b.group2);
@@ -1363,7 +1439,7 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
         SedMoves M{b.keys[0], b.vals[0],      b.keys[1],          b.vals[1],   (uint32_t *)b.group, (uint32_t *)b.group2,
                    b.moves,   b.moves + st_, b.moves + 2 * st_, b.moves + 2 * st_ - 1 - b.parity,
                    b.moves + 2 * st_ - 2 + b.parity, (int32_t *)(b.moves + 3 * st_),
-                   (uint32_t *)(b.precip + kSedMaxBlocks + 1), (uint32_t *)(b.precip + kSedMaxBlocks + 1) + 1};
+                   (uint32_t *)(b.precip + kExactBins + 1), (uint32_t *)(b.precip + kExactBins + 1) + 1};
         b.parity ^= 1;
         unsigned long long *totals = (unsigned long long *)(b.moves + 4 * st_);
         b.group_valid = false;
@@ -1378,7 +1454,7 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
         if (blocks > 64)
             sed_totals_kernel<<<blocks, 1024, 0, s>>>(M, n_groups, totals);
         sed_offsets_kernel<<<blocks, 1024, 0, s>>>(M, n_groups, blocks > 64 ? totals : nullptr, b.cell_off2, b.precip,
-                                                   fall_blocks, b.precip + kSedMaxBlocks);
+                                                   precip_sum);
         CTX_CUDA(ctx, cudaEventRecord(b.fork, s));
         CTX_CUDA(ctx, cudaStreamWaitEvent(b.side, b.fork, 0));
         st = side_work();
