@@ -1798,16 +1798,17 @@ int64_t sdm_footprint_bytes(int64_t capacity_sd, int32_t n_cells, int32_t larges
         const int lb = big_lb(largest_cell);
         const int64_t chunks = (capacity_sd + kBigChunk - 1) / kBigChunk + n_cells;
         int64_t big = capacity_sd * (4 + 4) + (chunks << lb) * 4 + ((int64_t)n_cells << lb) * 4 + chunks * kLiveWords * 4;
-        // or the record path's rooms, counts, seams and work lists
+        // the record path's rooms, counts, seams and work lists
         const int64_t cells = std::min<int64_t>(n_cells, slots / std::max(1, current_tuning().smem_max_sd) + 1);
         const int64_t rec_nb = slots / kRecMean + cells + 1;
         const int64_t rec_rooms = std::min<int64_t>(slots, kRecGroupSd) / kRecMean +
                                   std::min<int64_t>(cells, kRecGroupSd / std::max(1, current_tuning().smem_max_sd) + 1) + 1;
-        big = std::max<int64_t>(big, rec_rooms * (kRecRoom * (int64_t)sizeof(uint4) + 20) + rec_nb * 24 + cells * 64);
-        if (slots <= kSpreadMaxSd + n_cells + 1) { // or the bucketed path's rooms and counts
-            const int64_t nb = slots / kSpreadMean + std::min<int64_t>(n_cells, slots / largest_cell + 1) + 1;
-            big = std::max<int64_t>(big, nb * (kSpreadRoom * (int64_t)sizeof(uint2) + 2 * kSpreadStride * (int64_t)sizeof(uint32_t) + 48));
-        }
+        const int64_t rec = rec_rooms * (kRecRoom * (int64_t)sizeof(uint4) + 20) + rec_nb * 24 + cells * 64;
+        // (cells above the record path's largest take the multi-pass path beside it)
+        big = largest_cell > kRecMaxSd ? big + rec : std::max(big, rec);
+        // or the bucketed path's rooms and counts
+        const int64_t nb = std::min(slots, kSpreadMaxSd) / kSpreadMean + cells + 1;
+        big = std::max<int64_t>(big, nb * (kSpreadRoom * (int64_t)sizeof(uint2) + 2 * kSpreadStride * (int64_t)sizeof(uint32_t) + 48));
         bytes += big;
     }
     return bytes;
