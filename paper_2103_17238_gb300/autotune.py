@@ -1,14 +1,15 @@
 """Autotuner of the launch shape: which cells go through the shared-memory
-sort, which through the cluster path and which through the multi-pass global
-path, which cells run one warp per cell, how many warps share a block, and
-how many steps the warp-per-cell kernel fuses per launch.
+sort, which through the cluster path and which through passes over global
+memory, which cells run one warp per cell, how many warps share a block, and
+how many steps the shared-memory kernels fuse per launch.
 
 The tuning never changes results: every candidate computes the same state bit
 for bit.  The tuner times each candidate on the caller's own runs (one fused
 batch, CUDA events, a few steps after a warm-up step) and keeps the fastest.
-Results are cached in a JSON file keyed by the GPU name and a signature of
-the workload (the histogram of stored cell sizes per kernel), so a second
-batch of the same shape on the same GPU does not re-time.
+Results are cached in a JSON file keyed by the GPU name, the version of the
+library's paths (PATHS_VERSION) and a signature of the workload (the histogram
+of stored cell sizes per kernel), so a second batch of the same shape on the
+same GPU does not re-time.
 """
 from __future__ import annotations
 
@@ -19,6 +20,13 @@ import time
 import numpy as np
 
 from . import sdm
+
+# Raised whenever a tuning selects other kernels than before: what an entry timed
+# is then no longer what it would choose.  (1, without a number in the key: cells
+# above mid_max_sd took the multi-pass path.  2: they take the record path, and a
+# mid_max_sd other than the default pins cells to the cluster path: 36 boxes of
+# 60,000 107 us a step there, 49 with the default.)
+PATHS_VERSION = 2
 
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "sdm_gb300", "autotune.json")
 
@@ -97,7 +105,7 @@ def tune(runs, steps: int = 4, cache_path: str | None = DEFAULT_CACHE, candidate
     then the fused steps with the best of both."""
     import torch
 
-    key = f"{torch.cuda.get_device_name()}|{signature(runs)}"
+    key = f"{torch.cuda.get_device_name()}|paths {PATHS_VERSION}|{signature(runs)}"
     cache = _load(cache_path) if cache_path else {}
     if not force and key in cache:
         best = cache[key]["best"]
