@@ -200,6 +200,7 @@ struct Plan {
     BigScratch scratch{};
     int max_big_lb = 0;
     std::vector<Buf> bufs;
+    Buf rooms{}; // the bucketed or the record path's rooms (in bufs)
     int64_t bytes = 0;
     sdm_tuning tuning{}; // the launch tuning the plan was built with
     std::vector<unsigned char> host_pack; // the tables uploaded in one copy
@@ -257,6 +258,11 @@ struct sdm_ctx {
     cudaEvent_t in_ev[kInChunks + 1] = {};
     int64_t device_bytes = 0;
     sdm_batch *self_batch = nullptr;
+    // the rooms of the own plan before, for the next one: sedimentation makes a plan
+    // of larger cells anew at every step, and the library's own pool gives freed
+    // memory back at every synchronisation (300,001 SDs, step and sedimentation 188
+    // us with rooms allocated each time)
+    Buf spare_rooms{};
     // pinned host copy of the own batch's launch plan: uploaded from here,
     // written again only after the event shows the last upload done
     void *h_plan = nullptr;
@@ -333,6 +339,30 @@ T *plan_alloc(Plan &pl, DevMem &mem, size_t count)
     pl.bufs.push_back(b);
     pl.bytes += (int64_t)b.bytes;
     return static_cast<T *>(b.p);
+}
+
+// A plan's rooms: the context's spare ones when they do (own: the plan's context, if
+// it is one's own), else new ones.
+template <typename T>
+T *plan_rooms(Plan &pl, DevMem &mem, sdm_ctx *own, size_t count)
+{
+    if (own && own->spare_rooms.p) {
+        const Buf b = own->spare_rooms;
+        own->spare_rooms = Buf{};
+        if (b.bytes >= count * sizeof(T) && b.bytes / 2 <= count * sizeof(T)) {
+            pl.bufs.push_back(b);
+            pl.bytes += (int64_t)b.bytes;
+            pl.rooms = b;
+            return static_cast<T *>(b.p);
+        }
+        own->mem.put(b.p, b.bytes);
+        if (b.bytes < count * sizeof(T)) // a layout that changes: a sixteenth more, for the next ones
+            count += count / 16 + 8;
+    }
+    T *p = plan_alloc<T>(pl, mem, count);
+    if (p)
+        pl.rooms = pl.bufs.back();
+    return p;
 }
 
 void plan_free(Plan &pl, DevMem &mem)
@@ -915,8 +945,10 @@ sdm_status build_plan(sdm_batch *b)
             pl.rec.cnt = plan_alloc<uint32_t>(pl, mem, (size_t)nb);
             pl.rec.start = plan_alloc<uint32_t>(pl, mem, (size_t)(nb + nc));
             pl.rec.seam = plan_alloc<uint2>(pl, mem, (size_t)nb);
-            pl.rec.rooms = plan_alloc<uint4>(pl, mem, (size_t)nb * kRecRoom);
-            record = pl.rec.cnt && pl.rec.start && pl.rec.seam && pl.rec.rooms;
+            record = pl.rec.cnt && pl.rec.start && pl.rec.seam;
+            if (record)
+                pl.rec.rooms = plan_rooms<uint4>(pl, mem, b->own, (size_t)nb * kRecRoom);
+            record = record && pl.rec.rooms;
             if (!record)
                 cudaGetLastError();
             if (record && cudaMemsetAsync(pl.rec.cnt, 0, sizeof(uint32_t) * (size_t)nb, b->stream) != cudaSuccess)
@@ -1144,7 +1176,7 @@ sdm_status build_plan(sdm_batch *b)
         pl.n_spread_scatter = (int)scr.sp_scatter.size();
         pl.n_spread_pairs = (int)scr.sp_pairs.size();
         pl.spread.cnt = plan_alloc<uint32_t>(pl, mem, (size_t)sp_counters);
-        pl.spread.rooms = plan_alloc<uint2>(pl, mem, (size_t)sp_rooms * kSpreadRoom);
+        pl.spread.rooms = plan_rooms<uint2>(pl, mem, own, (size_t)sp_rooms * kSpreadRoom);
         if (!pl.spread.cnt || !pl.spread.rooms)
             return fail(&b->error, SDM_ENOMEM, "batch plan: bucket scratch allocation failed");
         const cudaError_t e = cudaMemsetAsync(pl.spread.cnt, 0, sizeof(uint32_t) * (size_t)sp_counters, b->stream);
@@ -1267,6 +1299,10 @@ sdm_status build_plan(sdm_batch *b)
         if (!pl.scratch.hist || !pl.scratch.bstart || !pl.scratch.rank || !pl.scratch.perm ||
             !pl.scratch.scale || !pl.scratch.scale_f || !pl.scratch.live)
             return fail(&b->error, SDM_ENOMEM, "batch plan: big-cell scratch allocation failed");
+    }
+    if (own && own->spare_rooms.p) { // this plan has no use for them
+        own->mem.put(own->spare_rooms.p, own->spare_rooms.bytes);
+        own->spare_rooms = Buf{};
     }
     // the host copy lives as long as the plan (or, pinned, until the event
     // below has passed): no wait for the upload
@@ -1488,6 +1524,25 @@ void batch_release(sdm_batch *b)
     b->capture_stream = nullptr;
     plan_free(b->plan, b->mem);
     b->mem.release_kept();
+}
+
+// Drops a context's own plan; its rooms stay for the next one.
+void drop_own_plan(sdm_ctx *ctx)
+{
+    sdm_batch *b = ctx->self_batch;
+    if (!b)
+        return;
+    Plan &pl = b->plan;
+    if (pl.rooms.bytes > DevMem::kKeepMax) // (smaller blocks are the batch's own, see DevMem)
+        for (size_t i = 0; i < pl.bufs.size(); ++i)
+            if (pl.bufs[i].p == pl.rooms.p) {
+                ctx->spare_rooms = pl.rooms;
+                pl.bufs.erase(pl.bufs.begin() + (std::ptrdiff_t)i);
+                break;
+            }
+    batch_release(b);
+    delete b;
+    ctx->self_batch = nullptr;
 }
 
 sdm_status batch_step(sdm_batch *b, int32_t n_steps)
@@ -2056,11 +2111,8 @@ sdm_status sdm_set_attributes(sdm_ctx *ctx, int64_t n_sd, const int64_t *xi, con
     ctx->has_attributes = true;
     if (ctx->self_batch && keep_plan)
         ctx->self_batch->versions[0] = ctx->layout_version;
-    if (ctx->self_batch && !keep_plan) {
-        batch_release(ctx->self_batch);
-        delete ctx->self_batch;
-        ctx->self_batch = nullptr;
-    }
+    if (!keep_plan)
+        drop_own_plan(ctx);
     return SDM_OK;
 }
 
@@ -2252,7 +2304,8 @@ sdm_status sdm_get_info(const sdm_ctx *ctx, sdm_info *out)
     out->n_sd = ctx->n_sd;
     out->capacity_sd = ctx->capacity_sd;
     out->step = ctx->step;
-    out->device_bytes = ctx->device_bytes + (ctx->self_batch ? ctx->self_batch->plan.bytes : 0);
+    out->device_bytes = ctx->device_bytes + (ctx->self_batch ? ctx->self_batch->plan.bytes : 0) +
+                        (int64_t)ctx->spare_rooms.bytes;
     out->n_cells = ctx->cfg.n_cells;
     out->largest_cell = ctx->largest_cell;
     return SDM_OK;
@@ -2263,10 +2316,8 @@ sdm_status sdm_destroy(sdm_ctx *ctx)
     NvtxRange nvtx_range("sdm_destroy");
     if (!ctx)
         return SDM_OK;
-    if (ctx->self_batch) {
-        batch_release(ctx->self_batch);
-        delete ctx->self_batch;
-    }
+    drop_own_plan(ctx);
+    ctx->mem.put(ctx->spare_rooms.p, ctx->spare_rooms.bytes);
     ctx->mem.put(ctx->d_xi, 0);
     ctx->mem.put(ctx->d_v, 0);
     ctx->mem.put(ctx->d_id_of_slot, 0);

@@ -1534,11 +1534,8 @@ extern "C" sdm_status sdm_sedimentation_step(sdm_ctx *ctx, double *precipitated)
         }
     if (ctx->self_batch && (keep_plan || refreshed))
         ctx->self_batch->versions[0] = ctx->layout_version;
-    if (ctx->self_batch && !keep_plan && !refreshed) {
-        batch_release(ctx->self_batch);
-        delete ctx->self_batch;
-        ctx->self_batch = nullptr;
-    }
+    if (!keep_plan && !refreshed)
+        drop_own_plan(ctx);
     if (precipitated)
         *precipitated = precip;
     return SDM_OK;
