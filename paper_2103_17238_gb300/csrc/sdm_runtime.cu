@@ -1796,6 +1796,10 @@ sdm_status small_staging(sdm_ctx *ctx)
     return SDM_OK;
 }
 
+// Largest cell whose spectrum, alone in its run, a block takes by itself (device
+// buffer; us a call, block | total: 300 SDs 26 | 36, 1000 27 | 37, 4096 34 | 36).
+constexpr int kSpecOneCell = 4096;
+
 // h_spec: edges on their way in, or a product on its way out; then the status word.
 constexpr size_t kSpecPin = sizeof(double) * 2 * kMaxEdges + 64;
 
@@ -2168,9 +2172,10 @@ sdm_status sdm_spectrum(sdm_ctx *ctx, const double *r_edges, int32_t n_edges, in
     // up to 32 bins: the warp kernels, the edges passed by value; more: one
     // block per cell with shared-memory atomics, the edges copied to the device
     const bool few = nb <= kSpecMaxBins;
-    // one cell's spectrum is the total's
-    const bool total = few && (!per_cell || ctx->cfg.n_cells == 1);
     const int64_t n_in = ctx->h_cell_off[ctx->cfg.n_cells];
+    // one cell's spectrum is the total's, but for a small one's into a device buffer,
+    // which a block finishes by itself
+    const bool total = few && (!per_cell || (ctx->cfg.n_cells == 1 && (!out_on_device || n_in > kSpecOneCell)));
     const double vol = per_cell ? ctx->cfg.dv : ctx->cfg.dv * (double)ctx->cfg.n_cells;
     const int grid = total ? (int)std::max<int64_t>(1, std::min<int64_t>(dev_grids().spec,
                                                                          (n_in + kSpecWarps * kSpecChunk - 1) /
@@ -2210,8 +2215,13 @@ sdm_status sdm_spectrum(sdm_ctx *ctx, const double *r_edges, int32_t n_edges, in
             if (!one)
                 spectrum_total_finalize_kernel<<<nb, kSpecFinalNT, 0, s>>>(ctx->d_inst, d_part, grid, T, d_out, h_status);
         } else {
-            // a block per cell where a warp alone would take many rounds
-            const int block_cells = n_in / ctx->cfg.n_cells > 4 * kSpecChunk ? 1 : 0;
+            // a block per cell where a warp alone would take many rounds, for the cells on
+            // average or for the largest one: it then waits for that warp, about 10 us per
+            // 1000 SDs, or with blocks for a quarter of that and for the turns of blocks of
+            // mostly small cells, 3 us per 1000 cells; blocks if that is less by half
+            const int64_t largest = ctx->largest_cell, cells = ctx->cfg.n_cells;
+            const bool one_large = largest > 8 * kSpecChunk && 3 * largest > 4 * cells;
+            const int block_cells = n_in / cells > 4 * kSpecChunk || one_large || cells == 1 ? 1 : 0;
             const int units = block_cells ? ctx->cfg.n_cells : (ctx->cfg.n_cells + kSpecWarps - 1) / kSpecWarps;
             spectrum_cells_kernel<<<std::min(units, dev_grids().spec_cells), 32 * kSpecWarps, 0, s>>>(
                 ctx->d_inst, ctx->cfg.n_cells, T, block_cells, d_out);
