@@ -1245,7 +1245,7 @@ sdm_status build_plan(sdm_batch *b)
         // fills the device by itself, and the classes beside it only slowed
         // it: 1.64e10 against 1.67e10 pair-updates/s on the 1024-box ensemble,
         // while mixes of a few dozen runs stepped a third faster)
-        bool small[kNumClass] = {};
+        bool small[kNumClass] = {}, full = false;
         int groups = classes > 0 ? 1 : 0, last = -1;
         for (int k = 0; k < kNumClass; ++k) {
             if (!pl.n_items[k])
@@ -1254,13 +1254,16 @@ sdm_status build_plan(sdm_batch *b)
             last = k;
             const Variant &x = g_variants[pl.variant[k]];
             small[k] = (int64_t)pl.n_items[k] < (int64_t)G.variant[pl.variant[k]] * (x.warps > 0 ? x.warps : 1);
+            full |= !small[k];
         }
         if (groups > 1 && sd_total + rec_sd <= ((int64_t)1 << 22)) {
             cudaError_t e = cudaEventCreateWithFlags(&pl.cls_fork, cudaEventDisableTiming);
             for (int k = 0; k < kNumClass && e == cudaSuccess; ++k) {
-                // the class of the largest cells stays on the plan's stream, unless
-                // the large-cell path is beside it
-                if (!small[k] || (k == last && classes == 0))
+                // the class of the largest cells stays on the plan's stream if nothing
+                // else does: the large-cell path, or a class that fills the device
+                // (beside one that did, a cell of 1000 waited for 4096 of 30: 16.2 us a
+                // step, 8.4 forked)
+                if (!small[k] || (k == last && classes == 0 && !full))
                     continue;
                 e = cudaStreamCreateWithFlags(&pl.cls_side[k], cudaStreamNonBlocking);
                 if (e == cudaSuccess)
