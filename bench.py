@@ -639,8 +639,8 @@ def measure_mid_cells(sdm, torch, steps=10):
     """Mid-size cells, one cluster size at a time, filling the GPU once: 152
     Golovin boxes of 12,000 SDs (one CTA each), 72 of 24,000 (clusters of
     2), 36 of 60,000 (clusters of 4; 36 such clusters fit at once), each
-    through the cluster path and through the multi-pass global path
-    (tuning mid_max_sd 65536 and 0, one launch per step).  The states of the
+    through the cluster path and through the record path over global memory
+    (tuning mid_max_sd 65536 and 0, one call per step).  The states of the
     two paths are compared bit for bit."""
     out = {"workload": "Golovin boxes (b=1500 s^-1, dV=1e6 m^3), one cell each, seeds 0.., one launch per step",
            "steps": steps}
@@ -648,7 +648,7 @@ def measure_mid_cells(sdm, torch, steps=10):
     try:
         for n_sd, cells, k in ((12000, 152, 1), (24000, 72, 2), (60000, 36, 4)):
             res, states = {}, []
-            for name, mid in (("cluster", 65536), ("multi_pass", 0)):
+            for name, mid in (("cluster", 65536), ("record", 0)):
                 sdm.sdm_set_tuning({**base, "mid_max_sd": mid})
                 runs = [sdm.Run(sdm.make_config("golovin", dv=I.DV_BOX, seed=c), n_sd).set_attributes(
                     *(lambda t: (t.xi, t.v, t.cell))(I.box_golovin(n_sd, seed=c))) for c in range(cells)]

@@ -304,13 +304,13 @@ sdm_status sdm_condensation_step(sdm_ctx *ctx, const double *G, const double *s,
                                  int condensed_on_device);
 
 /* ---- launch tuning.  Which cells are sorted in shared memory (the rest take
- * the multi-pass global path), which run one warp per cell, and how many
- * warps share a block.  Results never depend on it: every setting gives the
- * same state bit for bit.  Process-wide; applies to contexts and batches
- * whose launch plans are built after the call (a context builds its plan at
- * its first sdm_coalescence_step after sdm_set_attributes, a batch at
- * sdm_batch_create).  paper_2103_17238_gb300/autotune.py times candidates
- * and sets the fastest. */
+ * a thread-block cluster each, or passes over global memory), which run one
+ * warp per cell, and how many warps share a block.  Results never depend on
+ * it: every setting gives the same state bit for bit.  Process-wide; applies
+ * to contexts and batches whose launch plans are built after the call (a
+ * context builds its plan at its first sdm_coalescence_step after
+ * sdm_set_attributes, a batch at sdm_batch_create).
+ * paper_2103_17238_gb300/autotune.py times candidates and sets the fastest. */
 typedef struct sdm_tuning {
     int32_t smem_max_sd;     /* largest cell sorted in shared memory: 512, 1024, 2048 or 4096 (default) */
     int32_t warp_cell_max;   /* largest cell run by one warp: 0, 64, 128, 256 or 512 (default), <= smem_max_sd */

@@ -836,7 +836,7 @@ LargePath large_path(int64_t total, int64_t count, int32_t most, const sdm_tunin
 }
 
 // Adds a cell of n SDs to the record path's groups of up to kRecGroupSd SDs (369 MB
-// of rooms; smaller groups end in more part-filled waves: 16 boxes of 2^20 in
+// of rooms, up to 461 where cells just above 4096 leave their last room empty; smaller groups end in more part-filled waves: 16 boxes of 2^20 in
 // groups of 2^21, 2^22, 2^23, 2^24 401, 395, 375, 353 us); its first bucket among
 // its group's.
 constexpr int64_t kRecGroupSd = kRecMaxSd;
@@ -1207,7 +1207,7 @@ sdm_status build_plan(sdm_batch *b)
     }
     {
         // the device's SMs (one cluster-path CTA each) dealt to the classes in
-        // proportion to their SDs (the multi-pass path's cells, which run beside
+        // proportion to their SDs (the other paths' cells, which run beside
         // them, count too), at least one cluster to each class with cells, at
         // most one per cell and no more than fit at once
         const DevGrids &G = dev_grids();
@@ -1241,7 +1241,7 @@ sdm_status build_plan(sdm_batch *b)
         // the size classes side by side when there is more than one group of
         // work: those whose cells do not fill the device's resident blocks on
         // their own (a class that fills them gains nothing beside another),
-        // and not when the multi-pass path holds more than 2^22 SDs (it then
+        // and not when the larger cells hold more than 2^22 SDs (their path then
         // fills the device by itself, and the classes beside it only slowed
         // it: 1.64e10 against 1.67e10 pair-updates/s on the 1024-box ensemble,
         // while mixes of a few dozen runs stepped a third faster)
@@ -1318,12 +1318,13 @@ sdm_status build_plan(sdm_batch *b)
 }
 
 // n steps (offsets off .. off + n - 1 from each run's device counter) of
-// every cell above the shared-memory threshold: the cluster path and the
-// multi-pass path.  The cluster sizes run side by side and beside the
-// multi-pass path (one fork and one join by events for all n steps; a graph
-// captures the same), each cluster size on its share of the SMs, the
-// multi-pass kernels on the rest; a cluster size's steps follow each other
-// on its stream, and the multi-pass path's on st.
+// every cell above the shared-memory threshold, by the paths that the plan gave
+// them: the bucketed path alone, or the cluster path, the record path and the
+// multi-pass path beside one another.  The cluster sizes run side by side and
+// beside the passes over global memory (one fork and one join by events for all
+// n steps; a graph captures the same), each on its share of the SMs, the others'
+// kernels on the rest; a cluster size's steps follow each other on its stream,
+// the other paths' on st.
 void enqueue_big_steps(const Plan &pl, int64_t off, int32_t n, cudaStream_t st)
 {
     const bool fork = pl.mid_fork != nullptr;

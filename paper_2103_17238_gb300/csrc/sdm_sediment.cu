@@ -33,6 +33,7 @@
 // SDs, one level per step) a step takes 53, 128, 196 us against 94, 147, 202 sorted.
 //
 // With larger cells (a warp would take too long), a stable sort of all SDs:
+//   sed_group_kernel     where the last step went by cells: every slot's group;
 //   sed_move_kernel      per slot (four per thread): the fall, the new group
 //                        of every SD (the cells, then n_cells for outside the
 //                        domain) as a key in SD-id order, counts per new
@@ -571,9 +572,6 @@ __global__ void sed_pad_kernel(int32_t n_groups, const int32_t *__restrict__ ust
     }
 }
 
-// -------------------------------------------------------------------- host
-// The second layout (swapped with the context's after every step, so both
-// sets are freed through their current pointers) and the scratch.
 // ------------------------------------------------- cells of up to kSedByCell
 constexpr int kSedByCell = 1024;  // slots of the largest cell that a warp takes
 constexpr int kSedFewCells = 608, kSedFewLargest = 800; // sdm_sedimentation_step's rule for few cells
@@ -1156,6 +1154,9 @@ __global__ void __launch_bounds__(kSedMergeNT, 9) sed_merge_kernel(const int32_t
     }
 }
 
+// -------------------------------------------------------------------- host
+// The second layout (swapped with the context's after every step, so both
+// sets are freed through their current pointers) and the scratch.
 struct SedBuffers {
     int64_t *xi2 = nullptr;
     double *v2 = nullptr;
@@ -1175,7 +1176,7 @@ struct SedBuffers {
     int32_t *ustart = nullptr;  // n_cells + 2
     ExactBin *precip = nullptr; // the precipitated water's bins (zero between steps), then its sum, the
                                 //   movers' count and the mark of a pile
-    int sorted_left = 0;        // steps that take the sorted path before the movers are counted again
+    int sorted_left = 0;        // steps that take the sorted path before the cells are tried again
     uint32_t *hist = nullptr;   // 256 x tiles, then 256 digit totals
     uint32_t *flags = nullptr;  // flags, then the first bad id (8-byte aligned)
     int32_t *emig = nullptr;    // per SD id: its cell in another piece of the grid after the last step, or -1
