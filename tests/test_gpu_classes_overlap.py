@@ -64,5 +64,9 @@ def test_beside_each_other(env, small, large):
     x, w = run.attributes()
     assert np.array_equal(x, st.xi) and np.array_equal(w, st.v)
     run.close()
-    both, one, other = _time(env, small + large), _time(env, small), _time(env, large)
-    assert both < 0.9 * (one + other), (both, one, other)  # one after the other: 0.99 and more
+    seen = []
+    for _ in range(4):  # (new streams each time: which hardware queues they share is theirs to choose)
+        seen.append((_time(env, small + large), _time(env, small), _time(env, large)))
+        if seen[-1][0] < 0.9 * (seen[-1][1] + seen[-1][2]):  # one after the other: 0.99 and more
+            return
+    assert False, seen
