@@ -48,7 +48,7 @@ struct CondBuffers {
     int64_t layout_version = -1; // the layout the work list was built for
     int32_t n_items = 0;
     CondItem *items = nullptr;
-    int32_t *item_start = nullptr; // n_cells + 1
+    int32_t *item_start = nullptr; // n_cells + 1, with the first work list
     double *partial = nullptr;     // n_items
     double *cond = nullptr;        // n_cells
     // c of each cell, binary32.  A field other than the last is read by the kernel
@@ -288,7 +288,7 @@ void cond_release(sdm_ctx *ctx)
     if (!ctx->cond)
         return;
     CondBuffers &b = *ctx->cond;
-    void *bufs[] = {b.items, b.partial, b.cond}; // (item_start and cf lie behind cond)
+    void *bufs[] = {b.items, b.item_start, b.partial, b.cond, b.cf};
     for (void *p : bufs)
         ctx->mem.put(p, 0);
     for (cudaEvent_t ev : b.cf_done)
@@ -309,10 +309,9 @@ sdm_status cond_prepare(sdm_ctx *ctx)
     if (!ctx->cond) {
         ctx->cond = new CondBuffers();
         CondBuffers &b = *ctx->cond;
-        b.cond = static_cast<double *>(ctx->mem.get(sizeof(double) * nc + sizeof(int32_t) * (nc + 1) + sizeof(float) * nc));
-        b.item_start = reinterpret_cast<int32_t *>(b.cond + nc);
-        b.cf = reinterpret_cast<float *>(b.item_start + nc + 1);
-        if (!b.cond) {
+        b.cond = static_cast<double *>(ctx->mem.get(sizeof(double) * nc));
+        b.cf = static_cast<float *>(ctx->mem.get(sizeof(float) * nc));
+        if (!b.cond || !b.cf) {
             cond_release(ctx);
             return fail(&ctx->error, SDM_ENOMEM, "condensation: device allocation failed");
         }
@@ -329,6 +328,11 @@ sdm_status cond_prepare(sdm_ctx *ctx)
     CondBuffers &b = *ctx->cond;
     if (ctx->largest_cell <= kCondByCell || b.layout_version == ctx->layout_version)
         return SDM_OK;
+    if (!b.item_start) {
+        b.item_start = static_cast<int32_t *>(ctx->mem.get(sizeof(int32_t) * (nc + 1)));
+        if (!b.item_start)
+            return fail(&ctx->error, SDM_ENOMEM, "condensation: device allocation failed");
+    }
     std::vector<CondItem> items;
     std::vector<int32_t> start(nc + 1);
     for (int32_t c = 0; c < nc; ++c) {
