@@ -126,7 +126,8 @@ struct FixedSum {
 // Whether v may enter the fixed-point sums below: positive and normal.  (An
 // evaporating step's rounding can leave a volume at or below zero; such SDs are
 // added in binary64, with their sign.)
-__device__ __forceinline__ bool volume_plain(double v) { return __double2hiint(v) >= 0x00100000; }
+constexpr int kPlainHigh = 0x00100000; // the least high word of such a volume
+__device__ __forceinline__ bool volume_plain(double v) { return __double2hiint(v) >= kPlainHigh; }
 
 // xi v: floor(log2 xi) + floor(log2 v) with v's biased exponent, and the
 // product (its top 62 or 63 bits) in units of 2^(emax - 61 - 1023).
@@ -1638,6 +1639,7 @@ __device__ __forceinline__ void diag_finish(const InstDev *P, const DiagPart *pa
                                             uint32_t *status)
 {
     DiagPart a{0ull, 0ull, 0ull, 0.0};
+    const uint32_t st = threadIdx.x == 0 ? P->status : 0u; // on its way beside the parts
     for (int i = threadIdx.x; i < n_parts; i += kDiagNT) {
         const volatile DiagPart *q = parts + i;
         diag_combine(a, DiagPart{q->live, q->xi_lo, q->xi_hi, q->xv});
@@ -1645,7 +1647,7 @@ __device__ __forceinline__ void diag_finish(const InstDev *P, const DiagPart *pa
     a = diag_block_reduce(a);
     if (threadIdx.x == 0) {
         *out = a;
-        *status = P->status;
+        *status = st;
     }
 }
 
@@ -1672,6 +1674,7 @@ __global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(InstDev *P, int64
             vv[i] = in ? gv[lane + 32 * i] : make_double2(1.0, 1.0);
         }
         uint32_t e = 0u;
+        int least = 0x7FFFFFFF; // of the live SDs' volumes (high words)
 #pragma unroll
         for (int i = 0; i < 2 * Q; ++i) {
             const int64_t x = (i & 1) ? xx[i / 2].y : xx[i / 2].x;
@@ -1679,10 +1682,22 @@ __global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(InstDev *P, int64
             if (x > 0) {
                 a.live += 1ull;
                 add128(a.xi_lo, a.xi_hi, (unsigned long long)x, 0ull);
-                if (volume_plain(v))
-                    e = max(e, xiv_exponent((uint64_t)x, v));
-                else
+                e = max(e, xiv_exponent((uint64_t)x, v));
+                least = min(least, __double2hiint(v));
+            }
+        }
+        if (__any_sync(0xFFFFFFFFu, least < kPlainHigh)) { // seldom: those are taken out of the fixed-point sum
+            e = 0u;
+#pragma unroll
+            for (int i = 0; i < 2 * Q; ++i) {
+                long long &x = (i & 1) ? xx[i / 2].y : xx[i / 2].x;
+                const double v = (i & 1) ? vv[i / 2].y : vv[i / 2].x;
+                if (x > 0 && !volume_plain(v)) {
                     other = __fma_rn(xi2d(x), v, other);
+                    x = 0;
+                } else if (x > 0) {
+                    e = max(e, xiv_exponent((uint64_t)x, v));
+                }
             }
         }
         e = __reduce_max_sync(0xFFFFFFFFu, e);
@@ -1690,9 +1705,8 @@ __global__ void __launch_bounds__(kDiagNT) diag_partial_kernel(InstDev *P, int64
 #pragma unroll
         for (int i = 0; i < 2 * Q; ++i) {
             const int64_t x = (i & 1) ? xx[i / 2].y : xx[i / 2].x;
-            const double v = (i & 1) ? vv[i / 2].y : vv[i / 2].x;
-            if (x > 0 && volume_plain(v))
-                f.add(xiv_fixed((uint64_t)x, v, e));
+            if (x > 0)
+                f.add(xiv_fixed((uint64_t)x, (i & 1) ? vv[i / 2].y : vv[i / 2].x, e));
         }
         xv = __dadd_rn(xv, f.warp_sum((int)e - 61 - 1023));
     }
@@ -1914,9 +1928,11 @@ __device__ __noinline__ double spec_odd(const SpecSmem &S, const SpecTab &T, con
 }
 
 // Adds the SDs of slots [lo, lo + n), n <= kSpecChunk, lo even, and returns
-// the sum of bin `lane`.  Every lane of the warp calls it.
+// the sum of bin `lane`.  Every lane of the warp calls it.  odd: set if the lane
+// met an SD of volume at or below zero, which is left for spec_odd (a call in here
+// would cost all chunks its registers).
 __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, const int64_t *__restrict__ gxi,
-                                             const double *__restrict__ gv, int n)
+                                             const double *__restrict__ gv, int n, bool &odd)
 {
     constexpr int Q = kSpecChunk / 64; // slot pairs per lane
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1924,7 +1940,6 @@ __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, cons
     uint64_t x[2 * Q];
     double v[2 * Q];
     int bin[2 * Q];
-    bool odd = false; // an SD whose volume is not plain
 #pragma unroll
     for (int i = 0; i < Q; ++i) { // every load first
         const int q = lane + 32 * i;
@@ -1942,15 +1957,15 @@ __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, cons
 #pragma unroll
     for (int i = 0; i < 2 * Q; ++i) {
         bin[i] = -1;
-        if ((int64_t)x[i] > 0 && !volume_plain(v[i])) {
-            odd = true;
-        } else if ((int64_t)x[i] > 0) {
-            const int b = spec_bin(S, T, v[i]);
+        if ((int64_t)x[i] > 0) {
+            const int b = spec_bin(S, T, v[i]); // (outside the edges if v is not plain)
             if ((unsigned)b < (unsigned)nb) {
                 bin[i] = b;
                 const uint32_t e = xiv_exponent(x[i], v[i]);
                 if (e > S.emax[warp][b]) // most are not, once one round of lanes is in
                     atomicMax(&S.emax[warp][b], e);
+            } else {
+                odd |= !volume_plain(v[i]);
             }
         }
     }
@@ -1979,10 +1994,7 @@ __device__ __forceinline__ double spec_chunk(SpecSmem &S, const SpecTab &T, cons
     __syncwarp();
     spec_clear(S, warp, lane);
     __syncwarp();
-    double sum = e == 0u ? 0.0 : fixed_to_double<42>(a2, ((uint64_t)a1 << 21) + a0, (int)e - 61 - 1023);
-    if (__any_sync(0xFFFFFFFFu, odd))
-        sum = spec_odd(S, T, gxi, gv, n, sum);
-    return sum;
+    return e == 0u ? 0.0 : fixed_to_double<42>(a2, ((uint64_t)a1 << 21) + a0, (int)e - 61 - 1023);
 }
 
 // x / den by the 64-bit reciprocal (x >= 0): within 0.5 + 2^-9 ulp, where the
@@ -2036,9 +2048,14 @@ __global__ void __launch_bounds__(32 * kSpecWarps, 7) spectrum_total_kernel(Inst
     const int64_t *__restrict__ gxi = P->xi;
     const double *__restrict__ gv = P->v;
     double acc = 0.0;
+    bool odd = false;
     const int64_t step = (int64_t)gridDim.x * kSpecWarps * kSpecChunk;
-    for (int64_t at = ((int64_t)blockIdx.x * kSpecWarps + warp) * kSpecChunk; at < n_slots; at += step)
-        acc = __dadd_rn(acc, spec_chunk(S, T, gxi + at, gv + at, (int)min((int64_t)kSpecChunk, n_slots - at)));
+    const int64_t at0 = ((int64_t)blockIdx.x * kSpecWarps + warp) * kSpecChunk;
+    for (int64_t at = at0; at < n_slots; at += step)
+        acc = __dadd_rn(acc, spec_chunk(S, T, gxi + at, gv + at, (int)min((int64_t)kSpecChunk, n_slots - at), odd));
+    if (__any_sync(0xFFFFFFFFu, odd))
+        for (int64_t at = at0; at < n_slots; at += step)
+            acc = spec_odd(S, T, gxi + at, gv + at, (int)min((int64_t)kSpecChunk, n_slots - at), acc);
     S.part[warp][lane] = acc;
     __syncthreads();
     if (warp == 0) {
@@ -2110,9 +2127,14 @@ __global__ void __launch_bounds__(32 * kSpecWarps) spectrum_cells_kernel(const I
     for (int c = unit; c < n_cells; c += units) {
         const int32_t lo = off[c], hi = off[c + 1];
         double acc = 0.0;
-        for (int32_t at = lo + (block_cells ? warp * kSpecChunk : 0); at < hi;
-             at += block_cells ? kSpecWarps * kSpecChunk : kSpecChunk)
-            acc = __dadd_rn(acc, spec_chunk(S, T, gxi + at, gv + at, min(kSpecChunk, hi - at)));
+        bool odd = false;
+        const int32_t at0 = lo + (block_cells ? warp * kSpecChunk : 0);
+        const int32_t step = block_cells ? kSpecWarps * kSpecChunk : kSpecChunk;
+        for (int32_t at = at0; at < hi; at += step)
+            acc = __dadd_rn(acc, spec_chunk(S, T, gxi + at, gv + at, min(kSpecChunk, hi - at), odd));
+        if (__any_sync(0xFFFFFFFFu, odd))
+            for (int32_t at = at0; at < hi; at += step)
+                acc = spec_odd(S, T, gxi + at, gv + at, min(kSpecChunk, hi - at), acc);
         if (block_cells) { // uniform over the block
             S.part[warp][lane] = acc;
             __syncthreads();

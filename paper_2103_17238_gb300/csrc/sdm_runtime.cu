@@ -1698,7 +1698,8 @@ SpecTab spec_table(const double *e, int32_t n_edges, double vol)
         T.edge[i] = e[i];
         const double v = 4.0 / 3.0 * 3.141592653589793 * e[i] * e[i] * e[i]; // may be 0 or infinite
         const uint32_t lo = high_word(v * (1.0 - 0x1p-17));
-        T.key[i] = make_uint2(lo, std::isfinite(v) ? high_word(v * (1.0 + 0x1p-17)) + 1u : 0xFFFFFFFFu);
+        // (an infinite one: above all finite volumes, below the negative ones, which lie above every edge)
+        T.key[i] = make_uint2(lo, std::isfinite(v) ? high_word(v * (1.0 + 0x1p-17)) + 1u : 0x7FF00000u);
     }
     T.key[n_edges] = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
     T.vol = vol;
